@@ -289,12 +289,10 @@ int smr_set_tensor_cores(smr_ctx* ctx, int enable);
  * counterpart in the paper).  Per level: translation with 8x8 target tiles
  * and the full or half direction chunk, 4x4 tiles, threads along the
  * directions (levels of at most 1024 boxes), or one CTA per direction chunk
- * over the whole level (at most 256 boxes); interpolation by the staged
- * kernel (FP32: child theta-row bands bulk-copied into shared memory) or by
- * the gather kernel with the full or half theta-row tile; anterpolation by
- * the staged kernel (FP32, where its tile fits) or by the gather kernel with
- * the full or half column chunk, 256-thread CTAs or one CTA per parent box
- * (FP32); for SMR_PREC_FP32 also
+ * over the whole level (at most 256 boxes); for SMR_PREC_FP64 interpolation
+ * and anterpolation by their built-in rules or by the gather kernels
+ * (interpolation with the full or half theta-row tile, anterpolation with half
+ * the column chunk or 256-thread CTAs); for SMR_PREC_FP32 also
  * aggregation, receive and the near-field product on the tensor cores or the
  * CUDA cores (the near product on the tensor cores only if at least 5 %
  * faster).  Each variant is timed over three products (CUDA events around
@@ -567,16 +565,13 @@ int smr_copy_level(smr_ctx* ctx, int level, int kind, double* out, size_t n_doub
  *    / half direction chunk, 3 4x4 tiles, 4 threads along the directions, 5
  *    one CTA per direction chunk over every box of the level (levels of at
  *    most a few hundred boxes: each source spectrum read once);
- *  SMR_STEP_INTERPOLATE (into the parent of `level`): 0 built-in rule (in
- *    FP32 the staged kernel, child theta-row bands bulk-copied into shared
- *    memory, where its tile fits), 1 / 2 the gather kernel with the full /
- *    half theta-row tile, 3 the staged kernel whose threads produce two
- *    neighbouring parent columns from one window of child columns (FP32);
- *  SMR_STEP_ANTERPOLATE (into `level`): 0 built-in rule (the gather kernel),
- *    1 half its column chunk, 2 256-thread CTAs, 4 the staged kernel (FP32,
- *    parent band bulk-copied, where its tile fits), 5 the gather kernel with
- *    one CTA per parent box serving its four children (FP32: each parent tap
- *    read once for the four quadrants' shifts).
+ *  SMR_STEP_INTERPOLATE (into the parent of `level`): 0 built-in rule (FP32:
+ *    the marching kernel; FP64: the gather kernel), 1 / 2 the gather kernel
+ *    with the full / half theta-row tile (FP64), 3 the marching kernel;
+ *  SMR_STEP_ANTERPOLATE (into `level`): 0 built-in rule (FP32: the marching
+ *    kernel; FP64: that or the gather kernel by the level's size), 1 the gather
+ *    kernel with half its column chunk, 2 with 256-thread CTAs (FP64), 4 and 5
+ *    the marching kernel.
  * A variant that does not apply to a level falls back to the built-in rule.
  * Drops captured products.  No counterpart in the paper. */
 enum { SMR_STEP_TRANSLATE = 0, SMR_STEP_INTERPOLATE = 1, SMR_STEP_ANTERPOLATE = 2 };

@@ -33,15 +33,12 @@ void free_scene(Ctx* c) {
   for (auto& L : c->lev) {
     dfree(L.d_khat); dfree(L.d_w); dfree(L.d_il_ptr); dfree(L.d_il_src); dfree(L.d_il_off); dfree(L.d_il_pk);
     dfree(L.d_T64); dfree(L.d_T32); dfree(L.d_parent); dfree(L.d_quad); dfree(L.d_ch_ptr);
-    dfree(L.d_ch_idx); dfree(L.d_ch_quad); dfree(L.d_th_src); dfree(L.d_th_refl); dfree(L.d_th_w64);
-    dfree(L.d_th_w32); dfree(L.d_th_pk); dfree(L.d_th_ws64); dfree(L.d_th_ws32); dfree(L.d_ph_src); dfree(L.d_ph_w64); dfree(L.d_ph_w32); dfree(L.d_shift64);
-    dfree(L.d_shift32); dfree(L.d_shift4_32); dfree(L.d_ip2_band); dfree(L.d_an2_lo);
-    dfree(L.d_an2_ttp); dfree(L.d_an2_tw); dfree(L.d_an2_pst2); dfree(L.d_an2_pwp);
-    dfree(L.d_an2_tq); dfree(L.d_an2_twq); dfree(L.d_ant_lo); dfree(L.d_ant_pjp); dfree(L.d_ant_pw64); dfree(L.d_ant_pw32);
-    dfree(L.d_ant_ttp); dfree(L.d_ant_tw64); dfree(L.d_ant_tw32);
-    dfree(L.d_tht_ptr); dfree(L.d_tht_tp); dfree(L.d_tht_refl); dfree(L.d_tht_w64); dfree(L.d_tht_w32);
-    dfree(L.d_pht_ptr); dfree(L.d_pht_jp); dfree(L.d_pht_w64); dfree(L.d_pht_w32); dfree(L.d_wthp64);
-    dfree(L.d_wthp32); dfree(L.d_boxmap); dfree(L.d_offid); dfree(L.d_tiles); dfree(L.d_tiles8);
+    dfree(L.d_ch_idx); dfree(L.d_ch_quad); dfree(L.d_ch4); dfree(L.d_th_pk); dfree(L.d_th_ws64); dfree(L.d_th_ws32);
+    dfree(L.d_ph_src); dfree(L.d_ph_w64); dfree(L.d_ph_w32); dfree(L.d_shift64); dfree(L.d_shiftp64);
+    dfree(L.d_shiftp32); dfree(L.d_shiftw32); dfree(L.d_mi_vlast); dfree(L.d_ma_ptr); dfree(L.d_ma_ent);
+    dfree(L.d_ma_w64); dfree(L.d_ma_w32); dfree(L.d_ma_pst); dfree(L.d_ma_pw64); dfree(L.d_ma_pw32);
+    dfree(L.d_ant_lo); dfree(L.d_ant_pjp); dfree(L.d_ant_pw64); dfree(L.d_ant_ttp); dfree(L.d_ant_tw64);
+    dfree(L.d_wthp64); dfree(L.d_boxmap); dfree(L.d_offid); dfree(L.d_tiles); dfree(L.d_tiles8);
     for (int q = 0; q < 2; ++q) {
       if (L.buf_out[q]) cudaFree(L.buf_out[q]);
       if (L.buf_in[q]) cudaFree(L.buf_in[q]);
@@ -75,13 +72,8 @@ void free_scene(Ctx* c) {
   c->tc_ready = false;
   c->tc_agg_ready = false;
   for (int q = 0; q < 2; ++q) {
-    if (c->G_buf[q]) cudaFree(c->G_buf[q]);
-    c->G_buf[q] = nullptr;
-    c->G_size[q] = 0;
     c->buf_R[q] = 0;
   }
-  c->d_G = nullptr;
-  c->G_bytes = 0;
   c->tmp_elems = 0;
   c->spec_R = 0;
   c->spec_prec = -1;
@@ -168,8 +160,8 @@ int build_interp(Ctx* c, Level& C, const Level& P) {
     }
     lagrange4(nodes, f, &pw[4 * jp]);
   }
-  std::vector<float> tw32(tw.begin(), tw.end()), pw32(pw.begin(), pw.end());
-  // single right-hand-side kernel: source row | reflected << 16, and the
+  std::vector<float> pw32(pw.begin(), pw.end());
+  // FP64 gather kernel: source row | reflected << 16; and the
   // weights with the reflection's sign folded in
   std::vector<int> tpk(4 * P.nth);
   std::vector<double> tws(4 * P.nth);
@@ -182,56 +174,7 @@ int build_interp(Ctx* c, Level& C, const Level& P) {
   if ((rc = upload(c, &C.d_th_pk, tpk)) || (rc = upload(c, &C.d_th_ws64, tws)) ||
       (rc = upload(c, &C.d_th_ws32, tws32)))
     return rc;
-  // staged FP32 interpolation (k_interp2): 256 threads; the phi pass gives a
-  // thread NCP column parts (16 bytes each, 2 per direction) of RPT rows; a
-  // tile of TR parent rows reads the band of child rows its taps name
-  {
-    const int NP = 2 * P.nph;
-    int ng, ncp, rpt;
-    if (NP <= 256) { ncp = 1; ng = 256 / NP; rpt = 6; }
-    else { ncp = (NP + 255) / 256; ng = 1; rpt = std::max(1, 8 / ncp); }
-    int TR = std::min(P.nth, ng * rpt);
-    const size_t rowb = (size_t)C.nph * 32;
-    auto band_of = [&](int t0, int t1, int* r0, int* nr) {
-      int lo = ntc, hi = -1;
-      for (int tp = t0; tp < t1; ++tp)
-        for (int a = 0; a < 4; ++a) { lo = std::min(lo, tsrc[4 * tp + a]); hi = std::max(hi, tsrc[4 * tp + a]); }
-      *r0 = lo;
-      *nr = hi - lo + 1;
-    };
-    // shrink the tile until two bands and the tile's theta-pass rows fit 110 KB
-    for (;;) {
-      int br = 0;
-      for (int t0 = 0; t0 < P.nth; t0 += TR) {
-        int r0, nr;
-        band_of(t0, std::min(P.nth, t0 + TR), &r0, &nr);
-        br = std::max(br, nr);
-      }
-      if (TR == 1 || 2 * (size_t)br * rowb + (size_t)TR * (rowb + 96) <= 110 * 1024) break;
-      TR = std::max(1, TR / 2);
-    }
-    C.ip2_TR = TR;
-    C.ip2_nrt = (P.nth + TR - 1) / TR;
-    // paired phi pass: the windows of columns 2m and 2m + 1 start at most one
-    // column apart and five padded columns from the first stay in the row
-    C.ip2_pair = (P.nph % 2 == 0);
-    for (int m = 0; 2 * m + 1 < P.nph && C.ip2_pair; ++m) {
-      const int ja = psrc[4 * (2 * m) + 1], jb = psrc[4 * (2 * m + 1) + 1];
-      C.ip2_pair = (jb - ja == 0 || jb - ja == 1) && ja <= C.nph - 2;
-    }
-    C.ip2_NCP = ncp;
-    C.ip2_RPT = (TR + ng - 1) / ng;
-    std::vector<int> band(2 * C.ip2_nrt);
-    C.ip2_BR = 0;
-    for (int t = 0; t < C.ip2_nrt; ++t) {
-      band_of(t * TR, std::min(P.nth, (t + 1) * TR), &band[t], &band[C.ip2_nrt + t]);
-      C.ip2_BR = std::max(C.ip2_BR, band[C.ip2_nrt + t]);
-    }
-    if ((rc = upload(c, &C.d_ip2_band, band))) return rc;
-  }
-  if ((rc = upload(c, &C.d_th_src, tsrc)) || (rc = upload(c, &C.d_th_refl, trefl)) ||
-      (rc = upload(c, &C.d_th_w64, tw)) || (rc = upload(c, &C.d_th_w32, tw32)) ||
-      (rc = upload(c, &C.d_ph_src, psrc)) || (rc = upload(c, &C.d_ph_w64, pw)) ||
+  if ((rc = upload(c, &C.d_ph_src, psrc)) || (rc = upload(c, &C.d_ph_w64, pw)) ||
       (rc = upload(c, &C.d_ph_w32, pw32)))
     return rc;
   // separable transposes: theta taps grouped by child row (sign and 1/w_theta(child)
@@ -268,16 +211,79 @@ int build_interp(Ctx* c, Level& C, const Level& P) {
         pjp[e] = jp;
         pww[e] = pw[4 * jp + b] * ratio;
       }
-    std::vector<float> tww32(tww.begin(), tww.end()), pww32(pww.begin(), pww.end()),
-        wpth32(wpth.begin(), wpth.end());
-    if ((rc = upload(c, &C.d_tht_ptr, tptr)) || (rc = upload(c, &C.d_tht_tp, ttp)) ||
-        (rc = upload(c, &C.d_tht_refl, trf)) || (rc = upload(c, &C.d_tht_w64, tww)) ||
-        (rc = upload(c, &C.d_tht_w32, tww32)) || (rc = upload(c, &C.d_pht_ptr, pptr)) ||
-        (rc = upload(c, &C.d_pht_jp, pjp)) || (rc = upload(c, &C.d_pht_w64, pww)) ||
-        (rc = upload(c, &C.d_pht_w32, pww32)) || (rc = upload(c, &C.d_wthp64, wpth)) ||
-        (rc = upload(c, &C.d_wthp32, wpth32)))
-      return rc;
-    // tiles of the fused single right-hand-side anterpolation: child theta
+    if ((rc = upload(c, &C.d_wthp64, wpth))) return rc;
+    // marching kernels (k_march.cu)
+    {
+      std::vector<int> vlast(P.nth);
+      struct Ent { int base, pk; double w[4]; };
+      std::vector<Ent> ent;
+      const int top = std::max(0, ntc - 4);        // last first-row of a window
+      for (int tp = 0; tp < P.nth; ++tp) {
+        const int i0 = (int)(std::upper_bound(thc.begin(), thc.end(), thp[tp]) - thc.begin()) - 1;
+        vlast[tp] = i0 + 2;
+        // the direct part of the stencil, and the part past a pole
+        const int base = std::min(std::max(i0 - 1, 0), top);
+        const bool north = i0 - 1 < 0;
+        Ent d{base, tp, {0, 0, 0, 0}}, r{north ? 0 : top, tp | (1 << 16), {0, 0, 0, 0}};
+        bool refl = false;
+        for (int a = 0; a < 4; ++a) {
+          const int i = tsrc[4 * tp + a];
+          const double v = wpth[tp] * tw[4 * tp + a] / wc[i];
+          if (trefl[4 * tp + a]) { r.w[i - r.base] += -v; refl = true; }
+          else d.w[i - d.base] += v;
+        }
+        ent.push_back(d);
+        if (refl) ent.push_back(r);
+      }
+      std::stable_sort(ent.begin(), ent.end(), [](const Ent& a, const Ent& b) { return a.base < b.base; });
+      const int nb = std::max(1, ntc - 3);
+      std::vector<int> ptr(nb + 1, 0), pk;
+      std::vector<double> w;
+      for (auto& e : ent) {
+        ptr[e.base + 1]++;
+        pk.push_back(e.pk);
+        w.insert(w.end(), e.w, e.w + 4);
+      }
+      for (int b = 0; b < nb; ++b) ptr[b + 1] += ptr[b];
+      std::vector<float> w32(w.begin(), w.end());
+      // phi taps: the child columns of neighbouring parent columns never step
+      // back, so the parent columns that read child column j (before
+      // wrapping: column j + a N) are consecutive
+      C.mi_start.resize(P.nph);
+      for (int jp = 0; jp < P.nph; ++jp) C.mi_start[jp] = psrc[4 * jp + 1] - 1;
+      std::vector<int> first(C.nph, 1 << 30), last(C.nph, -(1 << 30));
+      for (int turn = -1; turn <= 1; ++turn)
+        for (int jp = 0; jp < P.nph; ++jp)
+          for (int b = 0; b < 4; ++b) {
+            const int j = C.mi_start[jp] + b + turn * C.nph;
+            if (j < 0 || j >= C.nph) continue;
+            first[j] = std::min(first[j], jp + turn * P.nph);
+            last[j] = std::max(last[j], jp + turn * P.nph);
+          }
+      // columns no parent column reads take their neighbour's start, weight 0
+      int pm = 7;                                  // narrower stencils are padded (zero weights)
+      for (int j = 0; j < C.nph; ++j) {
+        if (last[j] < first[j]) { first[j] = j ? first[j - 1] : 0; last[j] = first[j]; }
+        pm = std::max(pm, last[j] - first[j] + 1);
+      }
+      C.ma_pm = pm;
+      C.ma_start = first;
+      std::vector<double> pw2((size_t)C.nph * pm, 0.0);
+      for (int j = 0; j < C.nph; ++j)
+        for (int q = 0; q < pm; ++q) {
+          const int u = first[j] + q, jp = ((u % P.nph) + P.nph) % P.nph, turn = (u - jp) / P.nph;
+          for (int b = 0; b < 4; ++b)
+            if (C.mi_start[jp] + b + turn * C.nph == j) pw2[(size_t)j * pm + q] = pw[4 * jp + b] * C.nph / P.nph;
+        }
+      std::vector<float> pw232(pw2.begin(), pw2.end());
+      if ((rc = upload(c, &C.d_ma_pst, first)) || (rc = upload(c, &C.d_ma_pw64, pw2)) ||
+          (rc = upload(c, &C.d_ma_pw32, pw232)))
+        return rc;
+      if ((rc = upload(c, &C.d_mi_vlast, vlast)) || (rc = upload(c, &C.d_ma_ptr, ptr)) ||
+          (rc = upload(c, &C.d_ma_ent, pk)) || (rc = upload(c, &C.d_ma_w64, w)) || (rc = upload(c, &C.d_ma_w32, w32)))
+        return rc;
+    }
+    // tiles of the FP64 gather anterpolation: child theta
     // rows in tiles of TI, each with the range [lo, hi) of parent rows its
     // transposed taps read; GR = the widest range
     C.ant_TI = C.nth <= 24 ? C.nth : 16;
@@ -296,14 +302,8 @@ int build_interp(Ctx* c, Level& C, const Level& P) {
       lohi[C.ant_nit + it] = hi;
       C.ant_GR = std::max(C.ant_GR, hi - lo);
     }
-    // column chunk per precision: GR x 2 JC directions in 48 KB of shared memory
-    for (int q = 0; q < 2; ++q) {
-      int dirb = q == 0 ? 64 : 32;                  // SMR_PREC_FP64, SMR_PREC_FP32
-      int jc = (48 * 1024) / (C.ant_GR * 2 * dirb);
-      C.ant_JC[q] = std::max(1, std::min(C.nph / 2, jc));
-    }
-    // the per-parent FP32 kernel holds four quadrants' rows: 52 KB for four CTAs per SM
-    C.ant_JC5 = std::max(1, std::min(C.nph / 2, (52 * 1024) / (4 * C.ant_GR * 2 * 32)));
+    // column chunk: GR x 2 JC directions in 48 KB of shared memory
+    C.ant_JC = std::max(1, std::min(C.nph / 2, (48 * 1024) / (C.ant_GR * 2 * 64)));
     if ((rc = upload(c, &C.d_ant_lo, lohi))) return rc;
     // padded transposed taps
     int pm = 0, tm = 0;
@@ -335,167 +335,35 @@ int build_interp(Ctx* c, Level& C, const Level& P) {
         tpk[(size_t)i * C.ant_TM + q] = pk;
         tpw[(size_t)i * C.ant_TM + q] = real ? tww[e] : 0.0;
       }
-    // staged FP32 anterpolation (k_anterp2)
-    {
-      const int PM = pm, TM = tm;
-      // phi: the taps of child column j are consecutive parent columns (mod
-      // nphP); unwrap them around j's position and keep PM slots from the first
-      std::vector<int> pst(C.nph);
-      std::vector<float> pw2((size_t)C.nph * PM, 0.f);
-      int padl = 0, padr = 0;
-      for (int j = 0; j < C.nph; ++j) {
-        const int ref = (int)std::lround((double)j * P.nph / C.nph);
-        int dmin = 1 << 30;
-        std::vector<int> dd;
-        for (int e = pptr[j]; e < pptr[j + 1]; ++e) {
-          int d = ((pjp[e] - ref) % P.nph + P.nph) % P.nph;
-          if (d > P.nph / 2) d -= P.nph;
-          dd.push_back(d);
-          dmin = std::min(dmin, d);
-        }
-        if (dd.empty()) dmin = 0;
-        pst[j] = ref + dmin;
-        for (size_t t = 0; t < dd.size(); ++t) {
-          const int slot = dd[t] - dmin;
-          if (slot >= PM) return fail(c, SMR_E_INVALID_ARG, "anterpolation phi taps are not consecutive");
-          pw2[(size_t)j * PM + slot] += (float)pww[pptr[j] + t];
-        }
-        padl = std::max(padl, -pst[j]);
-        padr = std::max(padr, pst[j] + PM - P.nph);
-      }
-      // theta: consecutive parent rows (no pole reflection) from a window start
-      // kept inside [0, nthP - TM]; otherwise the packed taps
-      std::vector<int> tws(C.nth), ttp2((size_t)C.nth * TM);
-      std::vector<float> tw2((size_t)C.nth * TM, 0.f);
-      for (int i = 0; i < C.nth; ++i) {
-        bool refl = false;
-        int first = P.nth;
-        for (int e = tptr[i]; e < tptr[i + 1]; ++e) { refl = refl || trf[e]; first = std::min(first, ttp[e]); }
-        if (tptr[i + 1] == tptr[i]) first = 0;
-        if (!refl && P.nth >= TM) {
-          const int ws = std::min(first, P.nth - TM);
-          tws[i] = ws;
-          for (int e = tptr[i]; e < tptr[i + 1]; ++e) {
-            const int slot = ttp[e] - ws;
-            if (slot < 0 || slot >= TM) return fail(c, SMR_E_INVALID_ARG, "anterpolation theta taps are not consecutive");
-            tw2[(size_t)i * TM + slot] += (float)tww[e];
-          }
-          for (int k = 0; k < TM; ++k) ttp2[(size_t)i * TM + k] = ws + k;
-        } else {
-          tws[i] = -1;
-          for (int k = 0; k < TM; ++k) {
-            const int e = tptr[i] + k;
-            const bool real = e < tptr[i + 1];
-            const int e0 = tptr[i + 1] > tptr[i] ? tptr[i] : -1;
-            ttp2[(size_t)i * TM + k] = real ? (ttp[e] | (trf[e] << 16)) : (e0 >= 0 ? (ttp[e0] | (trf[e0] << 16)) : 0);
-            tw2[(size_t)i * TM + k] = real ? (float)tww[e] : 0.f;
-          }
-        }
-      }
-      // pairs of neighbouring child columns (rows) share one window of loaded
-      // values: dense weights over PM + 2 parent columns (the second column's
-      // taps start 0..2 columns after the first's) and TM + 3 parent rows;
-      // weight rows padded to multiples of 4 for 16-byte loads
-      const int WPM = PM + 2, WTM = TM + 3, WPS = (WPM + 3) & ~3, WTS = (WTM + 3) & ~3;
-      const int npp = C.nph / 2, nqp = (C.nth + 1) / 2;
-      std::vector<int> pst2(npp);
-      std::vector<float> pwp((size_t)npp * 2 * WPS, 0.f);
-      bool pairs_ok = (C.nph % 2) == 0;
-      for (int q = 0; q < npp && pairs_ok; ++q) {
-        const int ja = 2 * q, jb = 2 * q + 1, d = pst[jb] - pst[ja];
-        if (d < 0 || d + PM > WPM) { pairs_ok = false; break; }
-        pst2[q] = pst[ja];
-        for (int k = 0; k < PM; ++k) {
-          pwp[((size_t)q * 2 + 0) * WPS + k] = pw2[(size_t)ja * PM + k];
-          pwp[((size_t)q * 2 + 1) * WPS + d + k] = pw2[(size_t)jb * PM + k];
-        }
-        padl = std::max(padl, -pst2[q]);
-        padr = std::max(padr, pst2[q] + WPM - P.nph);
-      }
-      // row pairs (2q, 2q + 1): window start, or -1 where a row reaches a pole
-      std::vector<int> tq(nqp, -1);
-      std::vector<float> twq((size_t)nqp * 2 * WTS, 0.f);
-      for (int q = 0; q < nqp; ++q) {
-        const int ia = 2 * q, ib = 2 * q + 1;
-        if (tws[ia] < 0 || (ib < C.nth && tws[ib] < 0) || P.nth < WTM) continue;
-        const int ws = std::min(tws[ia], P.nth - WTM);
-        const int da = tws[ia] - ws, db = ib < C.nth ? tws[ib] - ws : 0;
-        if (da < 0 || da + TM > WTM || db < 0 || db + TM > WTM) continue;
-        tq[q] = ws;
-        for (int k = 0; k < TM; ++k) {
-          twq[((size_t)q * 2 + 0) * WTS + da + k] = tw2[(size_t)ia * TM + k];
-          if (ib < C.nth) twq[((size_t)q * 2 + 1) * WTS + db + k] = tw2[(size_t)ib * TM + k];
-        }
-      }
-      // child-row tiles (an even number of rows, so pairs align): the widest
-      // tile whose parent band fits 100 KB (the band as copied, its padded
-      // conjugate-shifted rows, the phi-transposed rows)
-      const size_t per_row = (size_t)P.nph * 32 + (size_t)(P.nph + padl + padr) * 32 + (size_t)C.nph * 32;
-      auto tile_band = [&](int i0, int i1, int* lo, int* hi) {
-        *lo = P.nth; *hi = 0;
-        for (int i = i0; i < i1; ++i) {
-          if (tq[i / 2] >= 0) {
-            *lo = std::min(*lo, tq[i / 2]);
-            *hi = std::max(*hi, tq[i / 2] + WTM);
-          } else {
-            for (int k = 0; k < TM; ++k) {
-              const int tp = ttp2[(size_t)i * TM + k] & 0xffff;
-              *lo = std::min(*lo, tp);
-              *hi = std::max(*hi, tp + 1);
-            }
-          }
-        }
-      };
-      int TI = C.nth, br = 0;
-      for (;; TI = std::max(2, (TI / 2) & ~1)) {
-        br = 0;
-        for (int i0 = 0; i0 < C.nth; i0 += TI) {
-          int lo, hi;
-          tile_band(i0, std::min(C.nth, i0 + TI), &lo, &hi);
-          br = std::max(br, hi - lo);
-        }
-        if (TI == 2 || (size_t)br * per_row <= 100 * 1024) break;
-      }
-      C.an2_TI = TI;
-      C.an2_nit = (C.nth + TI - 1) / TI;
-      C.an2_BR = br;
-      C.an2_PM = PM;
-      C.an2_TM = TM;
-      C.an2_PADL = padl;
-      C.an2_PADR = padr;
-      std::vector<int> lohi2(2 * C.an2_nit);
-      for (int it = 0; it < C.an2_nit; ++it)
-        tile_band(it * TI, std::min(C.nth, (it + 1) * TI), &lohi2[it], &lohi2[C.an2_nit + it]);
-      if ((size_t)br * per_row > 100 * 1024 || !pairs_ok) C.an2_TI = 0;   // does not fit: k_anterp1
-      if ((rc = upload(c, &C.d_an2_lo, lohi2)) ||
-          (rc = upload(c, &C.d_an2_ttp, ttp2)) || (rc = upload(c, &C.d_an2_tw, tw2)) ||
-          (rc = upload(c, &C.d_an2_pst2, pst2)) || (rc = upload(c, &C.d_an2_pwp, pwp)) ||
-          (rc = upload(c, &C.d_an2_tq, tq)) || (rc = upload(c, &C.d_an2_twq, twq)))
-        return rc;
-    }
-    std::vector<float> ppw32(ppw.begin(), ppw.end()), tpw32(tpw.begin(), tpw.end());
     if ((rc = upload(c, &C.d_ant_pjp, ppj)) || (rc = upload(c, &C.d_ant_pw64, ppw)) ||
-        (rc = upload(c, &C.d_ant_pw32, ppw32)) || (rc = upload(c, &C.d_ant_ttp, tpk)) ||
-        (rc = upload(c, &C.d_ant_tw64, tpw)) || (rc = upload(c, &C.d_ant_tw32, tpw32)))
+        (rc = upload(c, &C.d_ant_ttp, tpk)) || (rc = upload(c, &C.d_ant_tw64, tpw)))
       return rc;
   }
   // shift tables exp(j k khat_p . (c_child - c_parent)), child offset (+-1/2) x child box
   std::vector<double2> sh(4 * (size_t)P.K);
-  std::vector<float2> sh32(4 * (size_t)P.K);
   for (int q = 0; q < 4; ++q) {
     double dx = ((q & 1) - 0.5) * C.box, dy = ((q >> 1) - 0.5) * C.box;
     for (int k = 0; k < P.K; ++k) {
       double ph = c->k * (P.khat[3 * k] * dx + P.khat[3 * k + 1] * dy);
       sh[(size_t)q * P.K + k] = make_double2(std::cos(ph), std::sin(ph));
-      sh32[(size_t)q * P.K + k] = make_float2((float)std::cos(ph), (float)std::sin(ph));
     }
   }
-  std::vector<float2> sh4((size_t)4 * P.K);      // quadrant-interleaved per direction
+  std::vector<double2> shp((size_t)2 * P.K);     // quadrants 0 and 1 (3 and 2: their conjugates)
+  std::vector<float2> shp32((size_t)2 * P.K);
   for (int k = 0; k < P.K; ++k)
-    for (int q = 0; q < 4; ++q) sh4[(size_t)4 * k + q] = sh32[(size_t)q * P.K + k];
-  if ((rc = upload(c, &C.d_shift64, sh)) || (rc = upload(c, &C.d_shift32, sh32)) ||
-      (rc = upload(c, &C.d_shift4_32, sh4)))
+    for (int q = 0; q < 2; ++q) {
+      shp[(size_t)2 * k + q] = sh[(size_t)q * P.K + k];
+      shp32[(size_t)2 * k + q] = make_float2((float)shp[(size_t)2 * k + q].x, (float)shp[(size_t)2 * k + q].y);
+    }
+  std::vector<float2> shw32;
+  for (const float2& v : shp32) {
+    shw32.push_back(make_float2(v.x, v.x));
+    shw32.push_back(make_float2(v.y, v.y));
+  }
+  if ((rc = upload(c, &C.d_shiftp64, shp)) || (rc = upload(c, &C.d_shiftp32, shp32)) ||
+      (rc = upload(c, &C.d_shiftw32, shw32)))
     return rc;
+  if ((rc = upload(c, &C.d_shift64, sh))) return rc;
   return SMR_OK;
 }
 
@@ -731,9 +599,16 @@ int set_scene(Ctx* c, int p, const double* centres, const int* shape_ids, const 
       ch[B].push_back({b, C.quad[b]});
     }
     P.ch_ptr.assign(1, 0);
+    std::vector<int> ch4((size_t)4 * P.nbox, -1);
     for (int B = 0; B < P.nbox; ++B) {
+      for (auto& e : ch[B]) ch4[(size_t)4 * B + e.second] = e.first;
       for (auto& e : ch[B]) { P.ch_idx.push_back(e.first); P.ch_quad.push_back(e.second); }
       P.ch_ptr.push_back((int)P.ch_idx.size());
+    }
+    int rc4 = upload(c, &P.d_ch4, ch4);
+    if (rc4) {
+      c->lev = std::move(levs);                  // freed with the scene
+      return rc4;
     }
   }
   c->lev = std::move(levs);
@@ -1618,20 +1493,17 @@ int smr_autotune(smr_ctx* h, int R, int precision, void* stream) {
   // translation: 8x8 tiles (full, half direction chunk) and 4x4 tiles
   std::vector<std::vector<double>> ttr(c->nlev, std::vector<double>(6, 1e30));
   std::vector<std::vector<double>> tip(c->nlev, std::vector<double>(4, 1e30));
-  std::vector<std::vector<double>> tan_(c->nlev, std::vector<double>(6, 1e30));
-  const int anv[6] = {0, 0, 1, 2, 4, 5};       // anterpolation variant timed in trial v
+  std::vector<std::vector<double>> tan_(c->nlev, std::vector<double>(4, 1e30));
   double agg[2] = {1e30, 1e30}, rec[2] = {1e30, 1e30}, nea[2] = {1e30, 1e30};
   const int agg0 = c->tune_tc_agg, rec0 = c->tune_tc_rec, nea0 = c->tune_tc_near;
-  // trial 5 times the per-parent FP32 anterpolation and the whole-level
-  // translation (levels of at most 256 boxes), the rest at their first variants
+  // trial 5 times the whole-level translation (levels of at most 256 boxes),
+  // the FP64 interpolation and anterpolation their gather variants in trials 1
+  // and 2 (FP32 has one kernel for each)
   for (int v = 1; v <= 5; ++v) {
     // variant 4 (few-box kernel) only where a level has at most 1024 boxes
     for (auto& L : c->lev) {
       L.tune_tr[q] = (v == 4 && L.nbox > 1024) || (v == 5 && L.nbox > 256) ? 1 : v;
-      // interpolation: the built-in rule (staged kernel in FP32), k_interp1
-      // with the full or the half theta-row tile
-      L.tune_ip[q] = (v == 2) ? 2 : (v == 3 ? 1 : (v == 5 && q == 1 ? 3 : 0));
-      L.tune_an[q] = anv[v];
+      L.tune_ip[q] = L.tune_an[q] = (q == 0 && v <= 2) ? v : 0;
     }
     c->tune_tc_agg = c->tune_tc_rec = c->tune_tc_near = (v == 3) ? 0 : 1;
     if ((rc = profile_min(h, 1, x, y, precision, 3, stream, t))) break;
@@ -1639,7 +1511,8 @@ int smr_autotune(smr_ctx* h, int R, int precision, void* stream) {
       auto it = t.find({"translate", s});
       if (it != t.end() && c->lev[s].tune_tr[q] == v) ttr[s][v] = it->second;
       auto an = t.find({"anterpolate", s});
-      if (an != t.end()) tan_[s][anv[v]] = std::min(tan_[s][anv[v]], an->second);
+      const int av = c->lev[s].tune_an[q];
+      if (an != t.end()) tan_[s][av] = std::min(tan_[s][av], an->second);
       auto ip = t.find({"interpolate", s});
       const int iv = c->lev[s].tune_ip[q];
       if (ip != t.end()) tip[s][iv] = std::min(tip[s][iv], ip->second);
@@ -1663,7 +1536,7 @@ int smr_autotune(smr_ctx* h, int R, int precision, void* stream) {
       if (tip[s][v] < tip[s][bi]) bi = v;
     L.tune_ip[q] = rc ? 0 : bi;
     int ba = 0;
-    for (int v = 1; v <= 5; ++v)
+    for (int v = 1; v <= 3; ++v)
       if (tan_[s][v] < tan_[s][ba]) ba = v;
     L.tune_an[q] = rc ? 0 : ba;
   }

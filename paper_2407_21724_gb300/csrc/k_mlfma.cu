@@ -202,180 +202,28 @@ __global__ void k_aggregate(int K0, int npsi, int R, int RC, int nkc,
   }
 }
 
-// ------------------------------------------------------------------ interpolation (separable)
-// One warp per row of the output grid; lanes stride over (column, field, r).
-// R1 = (R == 1) lets the compiler turn the column / field split into shifts.
-template <bool R1>
-__device__ __forceinline__ void split_e(int e, int R4, int* j, int* fr) {
-  if (R1) { *j = e >> 2; *fr = e & 3; }
-  else { *j = e / R4; *fr = e - *j * R4; }
-}
-
-// theta pass:  G[c][tp][j][f][r] = sum_a w_a sgn_a F[c][row_a][(j + refl_a N/2) mod N][f][r]
-template <typename T, bool R1>
-__global__ void k_interp_theta(int nrows, int nthP, int nphC, int Kc, int R,
-                               const int* __restrict__ th_src, const int* __restrict__ th_refl,
-                               const T* __restrict__ th_w, const typename CV<T>::V* __restrict__ F,
-                               typename CV<T>::V* __restrict__ G) {
-  typedef typename CV<T>::V V;
-  int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (row >= nrows) return;
-  int c = row / nthP, tp = row - c * nthP;
-  int R4 = 4 * R;
-  int srow[4];
-  T w[4];
-  bool rf[4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    rf[a] = th_refl[tp * 4 + a] != 0;
-    w[a] = rf[a] ? -th_w[tp * 4 + a] : th_w[tp * 4 + a];
-    srow[a] = th_src[tp * 4 + a] * nphC;
-  }
-  const V* src = F + (size_t)c * Kc * R4;
-  V* dst = G + (size_t)row * nphC * R4;
-  int half = nphC >> 1, n = nphC * R4;
-  for (int e = lane; e < n; e += 32) {
-    int j, fr;
-    split_e<R1>(e, R4, &j, &fr);
-    int jr = j + half;
-    jr = jr >= nphC ? jr - nphC : jr;
-    V acc = czero<V>();
-#pragma unroll
-    for (int a = 0; a < 4; ++a) rfma(acc, w[a], src[(size_t)(srow[a] + (rf[a] ? jr : j)) * R4 + fr]);
-    dst[e] = acc;
-  }
-}
-
-// phi pass, shift and child sum:
-//   out[B][tp][jp][f][r] = sum_c shift[q_c][tp, jp] sum_b w_b G[c][tp][col_b][f][r]
-template <typename T, bool R1>
-__global__ void k_interp_phi(int nrows, int nthP, int nphP, int nphC, int R,
-                             const int* __restrict__ ch_ptr, const int* __restrict__ ch_idx,
-                             const int* __restrict__ ch_quad, const int* __restrict__ ph_src,
-                             const T* __restrict__ ph_w, const typename CV<T>::V* __restrict__ shift,
-                             const typename CV<T>::V* __restrict__ G,
-                             typename CV<T>::V* __restrict__ out) {
-  typedef typename CV<T>::V V;
-  int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (row >= nrows) return;
-  int B = row / nthP, tp = row - B * nthP;
-  int Kp = nthP * nphP, R4 = 4 * R;
-  int e0 = ch_ptr[B], e1 = ch_ptr[B + 1];
-  const V* gch[4];
-  const V* sh[4];
-  int nch = e1 - e0;
-  for (int q = 0; q < nch; ++q) {
-    gch[q] = G + ((size_t)ch_idx[e0 + q] * nthP + tp) * nphC * R4;
-    sh[q] = shift + (size_t)ch_quad[e0 + q] * Kp + (size_t)tp * nphP;
-  }
-  V* dst = out + (size_t)row * nphP * R4;
-  int n = nphP * R4;
-  for (int e = lane; e < n; e += 32) {
-    int jp, fr;
-    split_e<R1>(e, R4, &jp, &fr);
-    int col[4];
-    T w[4];
-#pragma unroll
-    for (int b = 0; b < 4; ++b) { col[b] = ph_src[jp * 4 + b] * R4 + fr; w[b] = ph_w[jp * 4 + b]; }
-    V acc = czero<V>();
-    for (int q = 0; q < nch; ++q) {
-      V tsum = czero<V>();
-#pragma unroll
-      for (int b = 0; b < 4; ++b) rfma(tsum, w[b], gch[q][col[b]]);
-      cfma(acc, sh[q][jp], tsum);
-    }
-    dst[e] = acc;
-  }
-}
-
-// Fused interpolation: per parent box and tile of TR parent rows, each child's
-// theta pass goes to shared memory and the phi pass, shift and child sum are
-// accumulated in registers (at most EMAX outputs per thread).
-constexpr int EMAX = 12;
-template <typename T, bool R1>
-__global__ void k_interp_fused(int nthP, int nphP, int nphC, int Kc, int R, int TR, int nrt,
-                               const int* __restrict__ ch_ptr, const int* __restrict__ ch_idx,
-                               const int* __restrict__ ch_quad, const int* __restrict__ th_src,
-                               const int* __restrict__ th_refl, const T* __restrict__ th_w,
-                               const int* __restrict__ ph_src, const T* __restrict__ ph_w,
-                               const typename CV<T>::V* __restrict__ shift,
-                               const typename CV<T>::V* __restrict__ F, typename CV<T>::V* __restrict__ out) {
-  typedef typename CV<T>::V V;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  V* G = reinterpret_cast<V*>(smem_raw);           // [TR][nphC][4R]
-  int B = blockIdx.x / nrt, rt = blockIdx.x % nrt;
-  int tp0 = rt * TR, ntr = min(TR, nthP - tp0);
-  int R4 = 4 * R, Kp = nthP * nphP;
-  int rowG = nphC * R4, rowP = nphP * R4;
-  int nG = ntr * rowG, nel = ntr * rowP;
-  int half = nphC >> 1;
-  V acc[EMAX];
-#pragma unroll
-  for (int i = 0; i < EMAX; ++i) acc[i] = czero<V>();
-  for (int e = ch_ptr[B]; e < ch_ptr[B + 1]; ++e) {
-    const V* src = F + (size_t)ch_idx[e] * Kc * R4;
-    const V* sh = shift + (size_t)ch_quad[e] * Kp + (size_t)tp0 * nphP;
-    __syncthreads();
-    for (int t = threadIdx.x; t < nG; t += blockDim.x) {
-      int tr = t / rowG, rem = t - tr * rowG;
-      int j, fr;
-      split_e<R1>(rem, R4, &j, &fr);
-      int tp = tp0 + tr;
-      int jr = j + half;
-      jr = jr >= nphC ? jr - nphC : jr;
-      V a = czero<V>();
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        int refl = th_refl[tp * 4 + q];
-        T w = refl ? -th_w[tp * 4 + q] : th_w[tp * 4 + q];
-        rfma(a, w, src[(size_t)(th_src[tp * 4 + q] * nphC + (refl ? jr : j)) * R4 + fr]);
-      }
-      G[t] = a;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < EMAX; ++i) {
-      int t = threadIdx.x + i * blockDim.x;
-      if (t < nel) {
-        int tr = t / rowP, rem = t - tr * rowP;
-        int jp, fr;
-        split_e<R1>(rem, R4, &jp, &fr);
-        const V* g = G + tr * rowG + fr;
-        V sum = czero<V>();
-#pragma unroll
-        for (int b = 0; b < 4; ++b) rfma(sum, ph_w[jp * 4 + b], g[ph_src[jp * 4 + b] * R4]);
-        cfma(acc[i], sh[tr * nphP + jp], sum);
-      }
-    }
-  }
-  V* dst = out + ((size_t)B * Kp + (size_t)tp0 * nphP) * R4;
-#pragma unroll
-  for (int i = 0; i < EMAX; ++i) {
-    int t = threadIdx.x + i * blockDim.x;
-    if (t < nel) dst[t] = acc[i];
-  }
-}
-
-
-// Single right-hand side: CTA = (parent box, tile of TR parent theta rows);
+// ------------------------------------------------------------------ FP64 interpolation, one right-hand side
+// The FP64 rate is the bound (two FP64 multiply-adds per clock and SM), and the
+// theta pass first needs the fewest of them: it runs on the child's columns,
+// and rows past a pole cost no extra passes.  CTA = (parent box, tile of TR parent theta rows);
 // each thread owns up to EM1 parent direction parts of the tile across the
 // loop over the children.  Per child: theta pass of the tile's rows into
 // shared memory G[TR][nphC][4] (4 taps, tables read as 16-byte vectors), then
 // phi pass, shift and child sum in registers.
-template <typename T> struct EM1 { static constexpr int v = sizeof(T) == 4 ? 8 : 12; };
-template <typename T>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_interp1(int nthP, int nphP, unsigned mP, int nphC, int Kc, int TR, int nrt,
+constexpr int EM1 = 12;                          // direction parts per thread, at most
+__global__ void __launch_bounds__(256, 2) k_interp1(int nthP, int nphP, unsigned mP, int nphC, int Kc, int TR, int nrt,
                                                  const int* __restrict__ ch_ptr, const int* __restrict__ ch_idx,
                                                  const int* __restrict__ ch_quad, const int* __restrict__ th_pk,
-                                                 const T* __restrict__ th_w,
-                                                 const int* __restrict__ ph_src, const T* __restrict__ ph_w,
-                                                 const typename CV<T>::V* __restrict__ shift,
-                                                 const typename CV<T>::V* __restrict__ F,
-                                                 typename CV<T>::V* __restrict__ out) {
-  typedef typename CV<T>::V V;
+                                                 const double* __restrict__ th_w,
+                                                 const int* __restrict__ ph_src, const double* __restrict__ ph_w,
+                                                 const double2* __restrict__ shift,
+                                                 const double2* __restrict__ F,
+                                                 double2* __restrict__ out) {
+  typedef double T;
+  typedef double2 V;
   typedef Part<T> P;
-  typedef typename P::H H;
-  constexpr int NT = P::NT, EM = EM1<T>::v;
+  typedef P::H H;
+  constexpr int NT = P::NT, EM = EM1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   V* G = reinterpret_cast<V*>(smem_raw);           // [TR][nphC][4]
   int B = blockIdx.x / nrt, rt = blockIdx.x - (blockIdx.x / nrt) * nrt;
@@ -791,75 +639,9 @@ __global__ void __launch_bounds__(256) k_translate_lvl(int K, int nbox, int KCH,
   }
 }
 
-// ------------------------------------------------------------------ anterpolation (separable adjoint)
-// phi-transposed pass (one warp per row (c, tp)), child c in quadrant q of parent B:
-//   Gt[c][tp][j][f][r] = w_theta_p[tp] sum_{(jp, w) in Pt(j)} w conj(shift[q][tp, jp]) in[B][tp][jp][f][r]
-template <typename T, bool R1>
-__global__ void k_anterp_phi(int nrows, int nthP, int nphP, int nphC, int R,
-                             const int* __restrict__ parent, const int* __restrict__ quad,
-                             const int* __restrict__ pht_ptr, const int* __restrict__ pht_jp,
-                             const T* __restrict__ pht_w, const T* __restrict__ wthp,
-                             const typename CV<T>::V* __restrict__ shift,
-                             const typename CV<T>::V* __restrict__ inP,
-                             typename CV<T>::V* __restrict__ Gt) {
-  typedef typename CV<T>::V V;
-  int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (row >= nrows) return;
-  int c = row / nthP, tp = row - c * nthP;
-  int Kp = nthP * nphP, R4 = 4 * R;
-  const V* src = inP + ((size_t)parent[c] * Kp + (size_t)tp * nphP) * R4;
-  const V* sh = shift + (size_t)quad[c] * Kp + (size_t)tp * nphP;
-  T wt = wthp[tp];
-  V* dst = Gt + (size_t)row * nphC * R4;
-  int n = nphC * R4;
-  for (int e = lane; e < n; e += 32) {
-    int j, fr;
-    split_e<R1>(e, R4, &j, &fr);
-    V acc = czero<V>();
-    for (int q = pht_ptr[j]; q < pht_ptr[j + 1]; ++q) {
-      int jp = pht_jp[q];
-      V sv = sh[jp];
-      T w = pht_w[q] * wt;
-      cfma(acc, mkc(w * sv.x, -w * sv.y), src[jp * R4 + fr]);
-    }
-    dst[e] = acc;
-  }
-}
-
-// theta-transposed pass (one warp per child row (c, i)), sign and 1/w_theta_c folded in:
-//   in[c][i][j][f][r] += sum_{(tp, w, refl) in Tt(i)} w Gt[c][tp][(j + refl N/2) mod N][f][r]
-template <typename T, bool R1>
-__global__ void k_anterp_theta(int nrows, int nthC, int nthP, int nphC, int R,
-                               const int* __restrict__ tht_ptr, const int* __restrict__ tht_tp,
-                               const int* __restrict__ tht_refl, const T* __restrict__ tht_w,
-                               const typename CV<T>::V* __restrict__ Gt,
-                               typename CV<T>::V* __restrict__ inC) {
-  typedef typename CV<T>::V V;
-  int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (row >= nrows) return;
-  int c = row / nthC, i = row - c * nthC;
-  int R4 = 4 * R;
-  const V* g = Gt + (size_t)c * nthP * nphC * R4;
-  V* dst = inC + (size_t)row * nphC * R4;
-  int half = nphC >> 1, n = nphC * R4;
-  int q0 = tht_ptr[i], q1 = tht_ptr[i + 1];
-  for (int e = lane; e < n; e += 32) {
-    int j, fr;
-    split_e<R1>(e, R4, &j, &fr);
-    int jr = j + half;
-    jr = jr >= nphC ? jr - nphC : jr;
-    V acc = czero<V>();
-    for (int q = q0; q < q1; ++q)
-      rfma(acc, tht_w[q], g[(size_t)(tht_tp[q] * nphC + (tht_refl[q] ? jr : j)) * R4 + fr]);
-    V cur = dst[e];
-    cur.x += acc.x;
-    cur.y += acc.y;
-    dst[e] = cur;
-  }
-}
-
-
-// Single right-hand side, both adjoint passes fused.  CTA = (child c, tile of
+// ------------------------------------------------------------------ FP64 anterpolation, one right-hand side
+// For levels too small for the marching kernel to fill the SMs (run_level).
+// Both adjoint passes fused.  CTA = (child c, tile of
 // child theta rows [i0, i0 + TI), column chunk [j0, j0 + JC) of the first
 // half of the phi grid together with the same chunk shifted by N/2, so that
 // the pole reflection j -> j + N/2 stays inside the CTA).  The parent rows
@@ -869,19 +651,20 @@ __global__ void k_anterp_theta(int nrows, int nthC, int nthP, int nphC, int R,
 // per child column / row (zero weights), packed as (tp | refl << 16).
 // PMC > 0: tap tables padded to 8 per row (PM = TM = 8) and at most PMC
 // real taps per row, known at compile time (tap loops unrolled)
-template <typename T, int PMC>
+template <int PMC>
 __global__ void __launch_bounds__(256) k_anterp1(int nthC, int nphC, int nthP, int nphP, int TI, int nit,
                                                  int JC, int njc, const int* __restrict__ parent,
                                                  const int* __restrict__ quad, const int* __restrict__ lo_row,
-                                                 int PM, const int* __restrict__ pjp, const T* __restrict__ pw,
-                                                 const T* __restrict__ wthp,
-                                                 const typename CV<T>::V* __restrict__ shift,
-                                                 const typename CV<T>::V* __restrict__ inP, int TM,
-                                                 const int* __restrict__ ttp, const T* __restrict__ tw,
-                                                 typename CV<T>::V* __restrict__ inC) {
-  typedef typename CV<T>::V V;
+                                                 int PM, const int* __restrict__ pjp, const double* __restrict__ pw,
+                                                 const double* __restrict__ wthp,
+                                                 const double2* __restrict__ shift,
+                                                 const double2* __restrict__ inP, int TM,
+                                                 const int* __restrict__ ttp, const double* __restrict__ tw,
+                                                 double2* __restrict__ inC) {
+  typedef double T;
+  typedef double2 V;
   typedef Part<T> P;
-  typedef typename P::H H;
+  typedef P::H H;
   constexpr int NT = P::NT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   V* Gt = reinterpret_cast<V*>(smem_raw);          // [GR][2 JC][4]
@@ -897,11 +680,10 @@ __global__ void __launch_bounds__(256) k_anterp1(int nthC, int nphC, int nthP, i
   int Kp = nthP * nphP, Kc = nthC * nphC;
   const V* srcP = inP + (size_t)parent[c] * Kp * 4;
   const V* sh = shift + (size_t)quad[c] * Kp;
-  // each thread owns PPT consecutive 16-byte parts of a direction (two in
-  // FP64, where a direction has four; one in FP32, where more threads hide
-  // more latency); (row, column) of its tasks stepped by the NTH tasks of
-  // one sweep of the CTA without dividing per task
-  constexpr int PPT = sizeof(T) == 8 ? 2 : 1, NT2 = NT / PPT;
+  // each thread owns PPT consecutive 16-byte parts of a direction's four;
+  // (row, column) of its tasks stepped by the NTH tasks of one sweep of the
+  // CTA without dividing per task
+  constexpr int PPT = 2, NT2 = NT / PPT;
   const int NTH = blockDim.x / NT2, task0 = threadIdx.x / NT2, h = PPT * (threadIdx.x % NT2);
   const int r0 = task0 / W, u0 = task0 - r0 * W;
   const int dq = NTH / W, dr = NTH - dq * W;
@@ -971,111 +753,6 @@ __global__ void __launch_bounds__(256) k_anterp1(int nthC, int nphC, int nthP, i
     if (u >= W) { u -= W; ++il; }
   }
 }
-// FP32, one right-hand side: the anterpolation of k_anterp1 with one CTA per
-// parent box serving all of its children.  Every parent tap of the
-// transposed phi pass is read once and multiplied by the conjugate shifts of
-// the four child quadrants (sh4: per parent direction the four quadrants'
-// shifts, 32 bytes), so four accumulators share one load; the theta pass of
-// each child then reads its quadrant's rows from shared memory.
-template <int PMC>
-__global__ void __launch_bounds__(256, 4) k_anterp4(int nthC, int nphC, int nthP, int nphP, int TI, int nit,
-                                                   int JC, int njc, const int* __restrict__ ch_ptr,
-                                                   const int* __restrict__ ch_idx, const int* __restrict__ ch_quad,
-                                                   const int* __restrict__ lo_row, int PM,
-                                                   const int* __restrict__ pjp, const float* __restrict__ pw,
-                                                   const float* __restrict__ wthp, const float4* __restrict__ sh4,
-                                                   const float2* __restrict__ inP, int TM,
-                                                   const int* __restrict__ ttp, const float* __restrict__ tw,
-                                                   float2* __restrict__ inC) {
-  typedef Part<float> P;
-  typedef P::H H;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  float2* Gt = reinterpret_cast<float2*>(smem_raw);   // [4 quadrants][GR][2 JC][4]
-  int blk = blockIdx.x;
-  const int jcb = blk % njc;
-  blk /= njc;
-  const int it = blk % nit, B = blk / nit;
-  const int i0 = it * TI, ni = min(TI, nthC - i0);
-  const int half = nphC >> 1;
-  const int j0 = jcb * JC, nj = min(JC, half - j0);
-  const int lo = lo_row[it], hi = lo_row[nit + it];
-  const int nr = hi - lo, W = 2 * nj;
-  const int Kp = nthP * nphP, Kc = nthC * nphC;
-  const float2* srcP = inP + (size_t)B * Kp * 4;
-  const int NTH = blockDim.x / 2, task0 = threadIdx.x / 2, h = threadIdx.x % 2;
-  const int r0 = task0 / W, u0 = task0 - r0 * W;
-  const int dq = NTH / W, dr = NTH - dq * W;
-  const size_t qstride = (size_t)nr * W;               // tasks per quadrant
-  for (int r = r0, u = u0, task = task0; r < nr; task += NTH) {
-    const int j = (u < nj) ? j0 + u : j0 + half + (u - nj);
-    const int tp = lo + r;
-    const float wt = wthp[tp];
-    const float2* prow = srcP + (size_t)tp * nphP * 4;
-    const float4* srow = sh4 + (size_t)tp * nphP * 2;
-    H a0 = P::zero(), a1 = P::zero(), a2 = P::zero(), a3 = P::zero();
-    const int pm = PMC > 0 ? 8 : PM;
-#pragma unroll
-    for (int q = 0; q < (PMC > 0 ? PMC : PM); q += 4) {
-      const int4 jj = *reinterpret_cast<const int4*>(pjp + (size_t)j * pm + q);
-      float w[4];
-      P::w4(pw + (size_t)j * pm + q, w);
-      const int js[4] = {jj.x, jj.y, jj.z, jj.w};
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        if (PMC > 0 && q + b >= PMC) break;
-        const H v = ldp<float>(prow, js[b], h);
-        const float4 s01 = srow[2 * js[b]], s23 = srow[2 * js[b] + 1];
-        const float ww = w[b] * wt;
-        P::cfma(a0, make_float2(ww * s01.x, -ww * s01.y), v);
-        P::cfma(a1, make_float2(ww * s01.z, -ww * s01.w), v);
-        P::cfma(a2, make_float2(ww * s23.x, -ww * s23.y), v);
-        P::cfma(a3, make_float2(ww * s23.z, -ww * s23.w), v);
-      }
-    }
-    stp<float>(Gt, task, h, a0);
-    stp<float>(Gt, qstride + task, h, a1);
-    stp<float>(Gt, 2 * qstride + task, h, a2);
-    stp<float>(Gt, 3 * qstride + task, h, a3);
-    u += dr;
-    r += dq;
-    if (u >= W) { u -= W; ++r; }
-  }
-  __syncthreads();
-  const int c0 = ch_ptr[B], nch = ch_ptr[B + 1] - c0;
-  for (int k = 0; k < nch; ++k) {
-    const int cb = ch_idx[c0 + k];
-    const float2* Gq = Gt + (size_t)ch_quad[c0 + k] * qstride * 4;
-    for (int il = r0, u = u0; il < ni;) {
-      const int ur = u < nj ? u + nj : u - nj;           // column j + N/2 (mod N)
-      const int j = (u < nj) ? j0 + u : j0 + half + (u - nj);
-      const int i = i0 + il;
-      H a = P::zero();
-      const int tm = PMC > 0 ? 8 : TM;
-#pragma unroll
-      for (int q = 0; q < (PMC > 0 ? PMC : TM); q += 4) {
-        const int4 pk = *reinterpret_cast<const int4*>(ttp + (size_t)i * tm + q);
-        float w[4];
-        P::w4(tw + (size_t)i * tm + q, w);
-        const int ps[4] = {pk.x, pk.y, pk.z, pk.w};
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          if (PMC > 0 && q + b >= PMC) break;
-          const int rr = (ps[b] & 0xffff) - lo;
-          const size_t g = (size_t)rr * W + ((ps[b] >> 16) ? ur : u);
-          P::rfma(a, w[b], ldp<float>(Gq, g, h));
-        }
-      }
-      const size_t d = (size_t)cb * Kc + (size_t)i * nphC + j;
-      H cur = ldp<float>(inC, d, h);
-      P::add(cur, a);
-      stp<float>(inC, d, h, cur);
-      u += dr;
-      il += dq;
-      if (u >= W) { u -= W; ++il; }
-    }
-  }
-}
-
 // ------------------------------------------------------------------ receive
 // y_e[m] += -jk sum_k w conj(sh) [P_th (z B0 + B3) + P_ph (z B1 - B2)]
 // y_m[m] += -jk sum_k w conj(sh) [P_th (-B1 + B2/z) + P_ph (B0 + B3/z)]   (Eqs. 24-25)
@@ -1228,7 +905,6 @@ int ensure_spectra(Ctx* c, int R, int prec) {
       }
     }
     size_t es = (p == 0) ? sizeof(double2) : sizeof(float2);
-    size_t gmax = 0;
     c->buf_R[p] = 0;
     for (int s = 0; s < c->nlev; ++s) {
       Level& L = c->lev[s];
@@ -1242,8 +918,6 @@ int ensure_spectra(Ctx* c, int R, int prec) {
         return SMR_E_OOM;
       }
       L.buf_bytes[p] = bytes;
-      if (s + 1 < c->nlev)
-        gmax = std::max(gmax, (size_t)L.nbox * c->lev[s + 1].nth * L.nph * 4 * R * es);
     }
     if (c->pspec[p]) cudaFree(c->pspec[p]);
     c->pspec[p] = nullptr;
@@ -1253,14 +927,6 @@ int ensure_spectra(Ctx* c, int R, int prec) {
       c->spec_prec = -1;
       return SMR_E_OOM;
     }
-    if (c->G_buf[p]) cudaFree(c->G_buf[p]);
-    c->G_buf[p] = nullptr;
-    if (gmax && cudaMalloc(&c->G_buf[p], gmax) != cudaSuccess) {
-      c->err = "out of device memory for the separable-pass buffer";
-      c->spec_prec = -1;
-      return SMR_E_OOM;
-    }
-    c->G_size[p] = gmax;
     c->buf_R[p] = R;
   }
   for (auto& L : c->lev) {
@@ -1268,8 +934,6 @@ int ensure_spectra(Ctx* c, int R, int prec) {
     L.d_in = L.buf_in[p];
     L.spec_bytes = L.buf_bytes[p];
   }
-  c->d_G = c->G_buf[p];
-  c->G_bytes = c->G_size[p];
   c->spec_R = R;
   c->spec_prec = prec;
   return SMR_OK;
@@ -1295,22 +959,16 @@ bool translate_lvl_ok(Ctx* c, int s, bool f64) {
   return true;
 }
 
-// The per-parent FP32 anterpolation needs the 8-tap tables and its four
-// quadrants' phi-pass rows within the fixed shared-memory ceiling.
-bool anterp4_ok(Ctx* c, int s) {
-  const Level& Lc = c->lev[s];
-  if (!Lc.d_shift4_32 || Lc.ant_PM != 8 || Lc.ant_TM != 8 || std::max(Lc.ant_PMx, Lc.ant_TMx) > 8) return false;
-  const size_t sm4 = (size_t)4 * Lc.ant_GR * 2 * Lc.ant_JC5 * 4 * sizeof(float2);
-  if (Lc.ant_JC5 < 1 || sm4 > 200 * 1024) return false;
-  static bool attr = false;
-  if (!attr) {
-    // one fixed ceiling for every launch (graph nodes keep their own size)
-    cudaFuncSetAttribute(k_anterp4<7>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    cudaFuncSetAttribute(k_anterp4<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    attr = true;
-  }
-  return true;
-}
+// FP64, one right-hand side: the gather kernels above, or the marching kernels
+// (k_march.cu) where they do less.  All are bound by the FP64 rate.
+// Interpolation: the gather kernel does fewer operations (200x200 lens, level
+// 0: 3.00 ms against 3.59 ms).  Anterpolation: the marching kernel does fewer
+// (4.25 against 5.63 ms), but its CTAs are long; by the directions of the
+// parent level (boxes x K) it wins by 15 % and more from 760,000 on (100x100
+// array), the gather kernel by up to 45 % on small levels (20x20), and at
+// 40x40 (120,000 to 260,000) the two are even.
+static bool march_interp(int v) { return v > 2; }
+static bool march_anterp(const Level& Lp, int v) { return v == 0 ? (size_t)Lp.nbox * Lp.K >= 500000 : v > 2; }
 
 // Finest boxes made of cells.  Box b's outgoing spectrum is the sum of its
 // particles' spectra, and each particle receives its box's incoming
@@ -1494,7 +1152,7 @@ static int far_impl(Ctx* c, int R, const double2* x, double2* y, bool accumulate
     }
     pend(c, st);
   }
-  // upward: separable interpolation, theta then phi (+ shift + child sum)
+  // upward: interpolation, shift and child sum
   for (int s = 0; s + 1 < c->nlev; ++s) {
     if (sd) {
       int rc = fork_translate(s);              // level s's outgoing spectra are complete
@@ -1504,57 +1162,21 @@ static int far_impl(Ctx* c, int R, const double2* x, double2* y, bool accumulate
     pbeg(c, st, "interpolate", s,
          ((double)Lc.nbox * Lc.K + (double)Lp.nbox * Lp.K) * 4 * R_ * es + 4.0 * Lp.K * es,
          (double)Lc.nbox * Lp.nth * Lc.nph * 4 * R_ * 16.0 + (double)Lc.nbox * Lp.K * 4 * R_ * 24.0);
-    if (!f64 && R == 1 && (Lc.tune_ip[1] == 0 || Lc.tune_ip[1] == 3) && interp2_ok(c, s)) {
-      int rc = run_interp2(c, s, st);
-      pend(c, st);
+    if (!f64 || R > 1 || march_interp(Lc.tune_ip[0]) || Lp.nph * Part<double>::NT > 256 * EM1) {
+      int rc = run_interp(c, s, R, f64 ? SMR_PREC_FP64 : SMR_PREC_FP32, st);
       if (rc) return rc;
-      continue;
-    }
-    if (R == 1 && Lp.nph * Part<T>::NT <= 256 * EM1<T>::v) {
-      int TR = std::max(1, std::min(Lp.nth, (256 * EM1<T>::v) / (Lp.nph * Part<T>::NT)));
-      if (Lc.tune_ip[f64 ? 0 : 1] == 2) TR = std::max(1, TR / 2);
+    } else {
+      int TR = std::max(1, std::min(Lp.nth, (256 * EM1) / (Lp.nph * Part<double>::NT)));
+      if (Lc.tune_ip[0] == 2) TR = std::max(1, TR / 2);
       int nrt = (Lp.nth + TR - 1) / TR;
-      size_t sm1 = (size_t)TR * Lc.nph * 4 * sizeof(V);
-      cudaFuncSetAttribute(k_interp1<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
+      size_t sm1 = (size_t)TR * Lc.nph * 4 * sizeof(double2);
+      cudaFuncSetAttribute(k_interp1, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
       const unsigned mP = (unsigned)(((1ull << 32) + (unsigned)Lp.nph - 1) / (unsigned)Lp.nph);
-      k_interp1<T><<<(unsigned)(Lp.nbox * nrt), 256, sm1, st>>>(
+      k_interp1<<<(unsigned)(Lp.nbox * nrt), 256, sm1, st>>>(
           Lp.nth, Lp.nph, mP, Lc.nph, Lc.K, TR, nrt, Lp.d_ch_ptr, Lp.d_ch_idx, Lp.d_ch_quad, Lc.d_th_pk,
-          (const T*)(f64 ? (void*)Lc.d_th_ws64 : (void*)Lc.d_th_ws32), Lc.d_ph_src,
-          (const T*)(f64 ? (void*)Lc.d_ph_w64 : (void*)Lc.d_ph_w32),
-          (const V*)(f64 ? (void*)Lc.d_shift64 : (void*)Lc.d_shift32), (const V*)Lc.d_out, (V*)Lp.d_out);
+          Lc.d_th_ws64, Lc.d_ph_src, Lc.d_ph_w64, Lc.d_shift64, (const double2*)Lc.d_out, (double2*)Lp.d_out);
       SMR_LAUNCH(c);
-      pend(c, st);
-      continue;
     }
-    // fused (shared-memory) version when a tile of parent rows fits
-    int TR = std::max(1, std::min(Lp.nth, (256 * EMAX) / (Lp.nph * 4 * R)));
-    size_t smf = (size_t)TR * Lc.nph * 4 * R * sizeof(V);
-    if (Lp.nph * 4 * R <= 256 * EMAX && smf <= 96 * 1024) {
-      int nrt = (Lp.nth + TR - 1) / TR;
-      auto kf = (R == 1) ? k_interp_fused<T, true> : k_interp_fused<T, false>;
-      cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
-      kf<<<(unsigned)(Lp.nbox * nrt), 256, smf, st>>>(
-          Lp.nth, Lp.nph, Lc.nph, Lc.K, R, TR, nrt, Lp.d_ch_ptr, Lp.d_ch_idx, Lp.d_ch_quad, Lc.d_th_src,
-          Lc.d_th_refl, (const T*)(f64 ? (void*)Lc.d_th_w64 : (void*)Lc.d_th_w32), Lc.d_ph_src,
-          (const T*)(f64 ? (void*)Lc.d_ph_w64 : (void*)Lc.d_ph_w32),
-          (const V*)(f64 ? (void*)Lc.d_shift64 : (void*)Lc.d_shift32), (const V*)Lc.d_out, (V*)Lp.d_out);
-      SMR_LAUNCH(c);
-      pend(c, st);
-      continue;
-    }
-    int rows1 = Lc.nbox * Lp.nth;
-    auto kth = (R == 1) ? k_interp_theta<T, true> : k_interp_theta<T, false>;
-    kth<<<(unsigned)((rows1 + 7) / 8), 256, 0, st>>>(
-        rows1, Lp.nth, Lc.nph, Lc.K, R, Lc.d_th_src, Lc.d_th_refl,
-        (const T*)(f64 ? (void*)Lc.d_th_w64 : (void*)Lc.d_th_w32), (const V*)Lc.d_out, (V*)c->d_G);
-    SMR_LAUNCH(c);
-    int rows2 = Lp.nbox * Lp.nth;
-    auto kph = (R == 1) ? k_interp_phi<T, true> : k_interp_phi<T, false>;
-    kph<<<(unsigned)((rows2 + 7) / 8), 256, 0, st>>>(
-        rows2, Lp.nth, Lp.nph, Lc.nph, R, Lp.d_ch_ptr, Lp.d_ch_idx, Lp.d_ch_quad, Lc.d_ph_src,
-        (const T*)(f64 ? (void*)Lc.d_ph_w64 : (void*)Lc.d_ph_w32),
-        (const V*)(f64 ? (void*)Lc.d_shift64 : (void*)Lc.d_shift32), (const V*)c->d_G, (V*)Lp.d_out);
-    SMR_LAUNCH(c);
     pend(c, st);
   }
   if (sd) {
@@ -1566,7 +1188,7 @@ static int far_impl(Ctx* c, int R, const double2* x, double2* y, bool accumulate
       if (rc) return rc;
     }
   }
-  // downward: separable adjoint, phi-transpose then theta-transpose (accumulates)
+  // downward: the weighted adjoint (accumulates)
   for (int s = c->nlev - 2; s >= 0; --s) {
     if (sd) {
       // the parent level's incoming spectra and this level's translation
@@ -1578,58 +1200,24 @@ static int far_impl(Ctx* c, int R, const double2* x, double2* y, bool accumulate
          ((double)Lp.nbox * Lp.K + 2.0 * Lc.nbox * Lc.K) * 4 * R_ * es + 4.0 * Lp.K * es,
          (double)Lc.nbox * Lp.nth * Lc.nph * 4 * R_ * 8.0 * 2 * (double)Lp.nph / Lc.nph * 4.0 / 4.0 +
              (double)Lc.nbox * Lc.K * 4 * R_ * 16.0 * (double)Lp.nth / Lc.nth);
-    if (!f64 && R == 1 && Lc.tune_an[1] == 4 && anterp2_ok(c, s)) {
-      int rc = run_anterp2(c, s, st);
-      pend(c, st);
+    if (!f64 || R > 1 || march_anterp(Lp, Lc.tune_an[0])) {
+      int rc = run_anterp(c, s, R, f64 ? SMR_PREC_FP64 : SMR_PREC_FP32, st);
       if (rc) return rc;
-      continue;
-    }
-    if (!f64 && R == 1 && Lc.tune_an[1] == 5 && anterp4_ok(c, s)) {
-      const int JC = Lc.ant_JC5;
-      const int njc = (Lc.nph / 2 + JC - 1) / JC;
-      const size_t sm4 = (size_t)4 * Lc.ant_GR * 2 * JC * 4 * sizeof(float2);
-      auto ka = std::max(Lc.ant_PMx, Lc.ant_TMx) <= 7 ? k_anterp4<7> : k_anterp4<8>;
-      ka<<<(unsigned)(Lp.nbox * Lc.ant_nit * njc), 256, sm4, st>>>(
-          Lc.nth, Lc.nph, Lp.nth, Lp.nph, Lc.ant_TI, Lc.ant_nit, JC, njc, Lp.d_ch_ptr, Lp.d_ch_idx, Lp.d_ch_quad,
-          Lc.d_ant_lo, Lc.ant_PM, Lc.d_ant_pjp, Lc.d_ant_pw32, Lc.d_wthp32, (const float4*)Lc.d_shift4_32,
-          (const float2*)Lp.d_in, Lc.ant_TM, Lc.d_ant_ttp, Lc.d_ant_tw32, (float2*)Lc.d_in);
-      SMR_LAUNCH(c);
-      pend(c, st);
-      continue;
-    }
-    if (R == 1) {
-      const int an = Lc.tune_an[f64 ? 0 : 1];
-      int JC = Lc.ant_JC[f64 ? 0 : 1];
+    } else {
+      const int an = Lc.tune_an[0];
+      int JC = Lc.ant_JC;
       if (an == 1) JC = std::max(1, JC / 2);
       int njc = (Lc.nph / 2 + JC - 1) / JC;
-      size_t sm1 = (size_t)Lc.ant_GR * 2 * JC * 4 * sizeof(V);
-      int thr = (an == 2 || Lc.ant_GR * 2 * JC * (Part<T>::NT / (f64 ? 2 : 1)) >= 2048) ? 256 : 128;
-      auto ka = k_anterp1<T, 0>;
-      if (Lc.ant_PM == 8 && Lc.ant_TM == 8) ka = std::max(Lc.ant_PMx, Lc.ant_TMx) <= 7 ? k_anterp1<T, 7> : k_anterp1<T, 8>;
+      size_t sm1 = (size_t)Lc.ant_GR * 2 * JC * 4 * sizeof(double2);
+      int thr = (an == 2 || Lc.ant_GR * 2 * JC * (Part<double>::NT / 2) >= 2048) ? 256 : 128;
+      auto ka = k_anterp1<0>;
+      if (Lc.ant_PM == 8 && Lc.ant_TM == 8) ka = std::max(Lc.ant_PMx, Lc.ant_TMx) <= 7 ? k_anterp1<7> : k_anterp1<8>;
       ka<<<(unsigned)(Lc.nbox * Lc.ant_nit * njc), thr, sm1, st>>>(
           Lc.nth, Lc.nph, Lp.nth, Lp.nph, Lc.ant_TI, Lc.ant_nit, JC, njc, Lc.d_parent, Lc.d_quad, Lc.d_ant_lo,
-          Lc.ant_PM, Lc.d_ant_pjp, (const T*)(f64 ? (void*)Lc.d_ant_pw64 : (void*)Lc.d_ant_pw32),
-          (const T*)(f64 ? (void*)Lc.d_wthp64 : (void*)Lc.d_wthp32),
-          (const V*)(f64 ? (void*)Lc.d_shift64 : (void*)Lc.d_shift32), (const V*)Lp.d_in, Lc.ant_TM,
-          Lc.d_ant_ttp, (const T*)(f64 ? (void*)Lc.d_ant_tw64 : (void*)Lc.d_ant_tw32), (V*)Lc.d_in);
+          Lc.ant_PM, Lc.d_ant_pjp, Lc.d_ant_pw64, Lc.d_wthp64, Lc.d_shift64, (const double2*)Lp.d_in, Lc.ant_TM,
+          Lc.d_ant_ttp, Lc.d_ant_tw64, (double2*)Lc.d_in);
       SMR_LAUNCH(c);
-      pend(c, st);
-      continue;
     }
-    int rows1 = Lc.nbox * Lp.nth;
-    auto kap = (R == 1) ? k_anterp_phi<T, true> : k_anterp_phi<T, false>;
-    kap<<<(unsigned)((rows1 + 7) / 8), 256, 0, st>>>(
-        rows1, Lp.nth, Lp.nph, Lc.nph, R, Lc.d_parent, Lc.d_quad, Lc.d_pht_ptr, Lc.d_pht_jp,
-        (const T*)(f64 ? (void*)Lc.d_pht_w64 : (void*)Lc.d_pht_w32),
-        (const T*)(f64 ? (void*)Lc.d_wthp64 : (void*)Lc.d_wthp32),
-        (const V*)(f64 ? (void*)Lc.d_shift64 : (void*)Lc.d_shift32), (const V*)Lp.d_in, (V*)c->d_G);
-    SMR_LAUNCH(c);
-    int rows2 = Lc.nbox * Lc.nth;
-    auto kat = (R == 1) ? k_anterp_theta<T, true> : k_anterp_theta<T, false>;
-    kat<<<(unsigned)((rows2 + 7) / 8), 256, 0, st>>>(
-        rows2, Lc.nth, Lp.nth, Lc.nph, R, Lc.d_tht_ptr, Lc.d_tht_tp, Lc.d_tht_refl,
-        (const T*)(f64 ? (void*)Lc.d_tht_w64 : (void*)Lc.d_tht_w32), (const V*)c->d_G, (V*)Lc.d_in);
-    SMR_LAUNCH(c);
     pend(c, st);
   }
   // receive
@@ -1798,7 +1386,6 @@ void free_lanes(Ctx* c) {
     Ctx::Lane& a = c->lanes[j];
     for (void* q : a.out) if (q) cudaFree(q);
     for (void* q : a.in) if (q) cudaFree(q);
-    if (a.G) cudaFree(a.G);
     if (a.x32) cudaFree(a.x32);
     if (a.tcn_part) cudaFree(a.tcn_part);
     if (a.s) cudaStreamDestroy(a.s);
@@ -1824,7 +1411,6 @@ int ensure_lanes(Ctx* c, int nl) {
     l0.out[s] = c->lev[s].buf_out[1];
     l0.in[s] = c->lev[s].buf_in[1];
   }
-  l0.G = c->G_buf[1];
   l0.x32 = c->d_x32;
   l0.tcn_part = c->d_tcn_part;
   for (int j = 0; j < nl; ++j) {
@@ -1842,7 +1428,6 @@ int ensure_lanes(Ctx* c, int nl) {
       ok = (a.out[s] || cudaMalloc(&a.out[s], b) == cudaSuccess) &&
            (a.in[s] || cudaMalloc(&a.in[s], b) == cudaSuccess);
     }
-    if (ok && c->G_size[1] && !a.G) ok = cudaMalloc(&a.G, c->G_size[1]) == cudaSuccess;
     if (ok && c->d_x32 && !a.x32)
       ok = cudaMalloc((void**)&a.x32, (size_t)c->p * 2 * c->npsi * sizeof(float2)) == cudaSuccess;
     if (ok && c->d_tcn_part && !a.tcn_part) ok = cudaMalloc((void**)&a.tcn_part, c->tcn_part_bytes) == cudaSuccess;
@@ -1863,7 +1448,6 @@ static void use_lane(Ctx* c, int j) {
     c->lev[s].d_out = a.out[s];
     c->lev[s].d_in = a.in[s];
   }
-  c->d_G = a.G;
   c->d_x32 = a.x32;
   c->d_tcn_part = a.tcn_part;
 }

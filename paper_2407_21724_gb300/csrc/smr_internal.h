@@ -88,15 +88,11 @@ struct Level {
   float2* d_T32 = nullptr;
   int* d_parent = nullptr;
   int* d_quad = nullptr;
-  float2* d_shift4_32 = nullptr;   // [K][4] the four quadrants' shifts per direction (parent level's child tables)
+  int* d_ch4 = nullptr;                  // [nbox][4] child box per quadrant, -1 if absent
   int* d_ch_ptr = nullptr;
   int* d_ch_idx = nullptr;
   int* d_ch_quad = nullptr;
   // interpolation from this level (child) to s+1 (parent) -- stored on the child
-  int* d_th_src = nullptr;               // [nth_p][4] source theta row
-  int* d_th_refl = nullptr;              // [nth_p][4] 1 if reflected through a pole
-  double* d_th_w64 = nullptr;            // [nth_p][4]
-  float* d_th_w32 = nullptr;
   int* d_th_pk = nullptr;                 // [nth_parent][4] source row | reflected << 16
   double* d_th_ws64 = nullptr;            // [nth_parent][4] weights, reflection sign folded in
   float* d_th_ws32 = nullptr;
@@ -104,19 +100,28 @@ struct Level {
   double* d_ph_w64 = nullptr;
   float* d_ph_w32 = nullptr;
   double2* d_shift64 = nullptr;          // [4][K_p] exp(j k khat_p.(c_c - c_p))
-  float2* d_shift32 = nullptr;
-  // separable passes (stored on the child level):
-  int* d_tht_ptr = nullptr;              // [nth+1] theta-transposed taps by child row
-  int* d_tht_tp = nullptr;               //   parent row
-  int* d_tht_refl = nullptr;             //   1 if reflected through a pole
-  double* d_tht_w64 = nullptr;           //   sign x weight / w_theta(child row)
-  float* d_tht_w32 = nullptr;
-  int* d_pht_ptr = nullptr;              // [nph+1] phi-transposed taps by child column
-  int* d_pht_jp = nullptr;               //   parent column
-  double* d_pht_w64 = nullptr;           //   weight x dphi_p / dphi_c
-  float* d_pht_w32 = nullptr;
-  double* d_wthp64 = nullptr;            // [nth_p] parent theta weights
-  float* d_wthp32 = nullptr;
+  // marching kernels (k_march.cu), stored on the child level: the shifts of
+  // quadrants 0 and 1 per parent direction ([K_p][2]; 3 and 2 are their
+  // conjugates); the last virtual child row of every parent row's stencil;
+  // the adjoint's entries (parent row | reflected << 16) by first child row
+  // with the weights of four child rows
+  double2* d_shiftp64 = nullptr;
+  float2* d_shiftp32 = nullptr;
+  float2* d_shiftw32 = nullptr;          // [K_p][4] the same as weight pairs (re, re), (im, im)
+  int* d_mi_vlast = nullptr;
+  int* d_ma_ptr = nullptr;
+  int* d_ma_ent = nullptr;
+  std::vector<int> mi_start;             // [nph_p] child column before the first phi tap (unwrapped)
+  // phi-transposed taps: ma_pm consecutive parent columns from ma_start[j]
+  // (unwrapped) per child column j, weights [nph][ma_pm]
+  std::vector<int> ma_start;
+  int ma_pm = 0;
+  int* d_ma_pst = nullptr;
+  double* d_ma_pw64 = nullptr;
+  float* d_ma_pw32 = nullptr;
+  double* d_ma_w64 = nullptr;
+  float* d_ma_w32 = nullptr;
+  double* d_wthp64 = nullptr;            // [nth_p] parent theta weights (stored on the child level)
   // dense lattice map of the boxes of this level (translation tiles)
   int map_x0 = 0, map_y0 = 0, map_w = 0, map_h = 0;
   int* d_boxmap = nullptr;               // [map_h][map_w] box index or -1
@@ -125,63 +130,31 @@ struct Level {
   int* d_tiles = nullptr;                // non-empty 4x4 translation tiles (ty * ntile_x + tx)
   int ntile8_x = 0, ntile8_ne = 0;
   int* d_tiles8 = nullptr;               // non-empty 8x8 tiles (single right-hand side kernel)
-  // fused single right-hand-side anterpolation into this level: child theta
-  // rows in nit tiles of TI, parent rows [lo, hi) per tile ([2][nit]), GR the
-  // widest range, JC the column chunk per precision (FP64, FP32)
-  int ant_TI = 0, ant_nit = 0, ant_GR = 0;
-  int ant_JC[2] = {0, 0};
-  int ant_JC5 = 0;                       // column chunk of the per-parent FP32 kernel (four quadrants' rows)
+  // FP64 gather anterpolation into this level, one right-hand side (k_anterp1):
+  // child theta rows in nit tiles of TI, parent rows [lo, hi) per tile
+  // ([2][nit]), GR the widest range, JC the column chunk
+  int ant_TI = 0, ant_nit = 0, ant_GR = 0, ant_JC = 0;
   int* d_ant_lo = nullptr;
-  // the transposed taps padded to fixed widths (multiples of 4, zero weights):
-  // phi by child column [nph][PM] (parent column, weight x dphi_p / dphi_c),
-  // theta by child row [nth][TM] (parent row | refl << 16, sign x weight / w_theta)
   // launch variants chosen by smr_autotune per precision (FP64, FP32), one
   // right-hand side; 0 = the built-in rule.  Translation: 1 / 2 = 8x8 target
   // tiles with the full / half direction chunk, 3 = 4x4 tiles, 4 = the
-  // few-box kernel (threads along the directions).  Interpolation
-  // into the parent of this level: 0 = the built-in rule (the staged kernel
-  // k_interp2 in FP32 where its tile fits), 1 = k_interp1 with the full, 2 =
-  // with half the theta-row tile.
+  // few-box kernel (threads along the directions).  FP64 interpolation into
+  // the parent of this level: 1 / 2 = the gather kernel with the full / half
+  // theta-row tile.
   int tune_tr[2] = {0, 0};
   int tune_ip[2] = {0, 0};
-  // anterpolation into this level: 0 = the built-in rule (k_anterp1), 1 =
-  // k_anterp1 with half the column chunk, 2 = with 256 threads, 4 = the
-  // staged kernel k_anterp2 (FP32, where its tile fits)
+  // FP64 anterpolation into this level: 1 / 2 = the gather kernel with half
+  // the column chunk / with 256 threads
   int tune_an[2] = {0, 0};
-  // staged single right-hand-side FP32 interpolation into the parent of this
-  // level (k_interp2): tiles of ip2_TR parent theta rows, each with the band
-  // of child rows [first, first + count) its theta taps read ([2][nrt]);
-  // ip2_BR the widest band; ip2_NCP / ip2_RPT the phi-pass shape (column
-  // parts and rows per thread)
-  int ip2_TR = 0, ip2_nrt = 0, ip2_BR = 0, ip2_NCP = 0, ip2_RPT = 0;
-  bool ip2_pair = false;                 // paired phi pass possible (tap windows of column pairs)
-  int* d_ip2_band = nullptr;
-  // staged single right-hand-side FP32 anterpolation into this level
-  // (k_anterp2): child theta-row tiles of an2_TI rows (even, so row pairs
-  // align), each with the parent rows [lo, hi) it reads ([2][nit], widest
-  // an2_BR); an2_PM / an2_TM the widest phi- / theta-transposed stencil; wrap
-  // padding of the parent rows an2_PADL left and an2_PADR right; the packed
-  // theta taps of each child row (tp | refl << 16) with their weights, used
-  // where a row pair reaches a pole
-  int an2_TI = 0, an2_nit = 0, an2_BR = 0, an2_PM = 0, an2_TM = 0, an2_PADL = 0, an2_PADR = 0;
-  int* d_an2_lo = nullptr;
-  int* d_an2_ttp = nullptr;
-  float* d_an2_tw = nullptr;
-  // pairs of neighbouring child columns / rows (two outputs per thread from one
-  // window): window start and dense weights [pairs][2][(PM + 2) or (TM + 3),
-  // padded to 4]; a row pair's start is -1 where a row reaches a pole
-  int* d_an2_pst2 = nullptr;
-  float* d_an2_pwp = nullptr;
-  int* d_an2_tq = nullptr;
-  float* d_an2_twq = nullptr;
+  // the transposed taps padded to fixed widths (multiples of 4, zero weights):
+  // phi by child column [nph][PM] (parent column, weight x dphi_p / dphi_c),
+  // theta by child row [nth][TM] (parent row | refl << 16, sign x weight / w_theta)
   int ant_PM = 0, ant_TM = 0;             // padded transposed taps per child column / row
   int ant_PMx = 0, ant_TMx = 0;           // real maxima
   int* d_ant_pjp = nullptr;
   double* d_ant_pw64 = nullptr;
-  float* d_ant_pw32 = nullptr;
   int* d_ant_ttp = nullptr;
   double* d_ant_tw64 = nullptr;
-  float* d_ant_tw32 = nullptr;
   // spectra (allocated for the current R and precision)
   void* d_out = nullptr;                 // active spectra (the last product's precision)
   void* d_in = nullptr;
@@ -286,10 +259,6 @@ struct Ctx {
   std::vector<GraphEntry> graphs;
   cudaStream_t capture_stream = nullptr;
   // work buffers
-  void* d_G = nullptr;                  // separable-pass intermediate (active precision)
-  size_t G_bytes = 0;
-  void* G_buf[2] = {nullptr, nullptr};
-  size_t G_size[2] = {0, 0};
   int buf_R[2] = {0, 0};
   int spec_R = 0, spec_prec = -1;
   double2* d_tmp = nullptr;             // [N][R] scratch for split products
@@ -315,7 +284,6 @@ struct Ctx {
   float* d_tc_agg = nullptr;              // [S][M tiles][K chunks][hi | lo][128][32] aggregation images
   // tensor cores for aggregation / receive chosen by smr_autotune (-1: not tuned)
   int tune_tc_agg = -1, tune_tc_rec = -1, tune_tc_near = -1;
-  bool lv2_enable = true;                 // staged level kernels for the FP32 product (smr_set_level_kernels)
   // near product on the tensor cores: block images, and per lattice offset
   // (phase; self blocks first) tiles of up to 128 pairs sharing a block
   bool tcn_ready = false;
@@ -344,7 +312,6 @@ struct Ctx {
   // lanes 1.. own theirs.
   struct Lane {
     std::vector<void*> out, in;           // per level FP32 spectra
-    void* G = nullptr;
     float2* x32 = nullptr;
     float* tcn_part = nullptr;
     cudaStream_t s = nullptr;
@@ -495,12 +462,9 @@ int run_near_tc(Ctx* c, double2* y, cudaStream_t st);
 int prep_x32(Ctx* c, int R, int prec, const double2* x, cudaStream_t st);
 int run_aggregate_tc(Ctx* c, const double2* x, const float2* x32, float2* out0, cudaStream_t st);
 int tc_check(Ctx* c);
-// staged FP32 level kernels (k_levels.cu)
-bool interp2_ok(const Ctx* c, int s);
-int run_interp2(Ctx* c, int s, cudaStream_t st);
-bool interp2_pair_ok(const Ctx* c, int s);
-bool anterp2_ok(const Ctx* c, int s);
-int run_anterp2(Ctx* c, int s, cudaStream_t st);
+// interpolation s -> s + 1 and anterpolation s + 1 -> s (k_march.cu)
+int run_interp(Ctx* c, int s, int R, int prec, cudaStream_t st);
+int run_anterp(Ctx* c, int s, int R, int prec, cudaStream_t st);
 
 // ------------------------------------------------------------------ linear algebra (k_linalg.cu)
 // h[j*R + r] = sum_i conj(V_j[i][r]) w[i][r] for j < J (V_j = V + j*ldv), FP64.
