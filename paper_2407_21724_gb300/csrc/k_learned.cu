@@ -28,119 +28,251 @@ __device__ __forceinline__ float dsilu(float z) {
   float s = 1.f / (1.f + __expf(-z));
   return s * (1.f + z * (1.f - s));
 }
-__device__ __forceinline__ float ld(const float* p) { return *p; }
-__device__ __forceinline__ float ld(const __nv_bfloat16* p) { return __bfloat162float(*p); }
+// ------------------------------------------------------------------ GEMMs
+// C tile of 64 x 64 per CTA, 256 threads of 4 x 4 results each, K in steps of 32
+// through two shared-memory buffers (the next step's values are loaded into
+// registers while this one is multiplied).  FP32 multiply-adds: a split-TF32
+// tensor-core version is a quarter faster, but its accumulators round toward
+// zero, which over a batch's rows put the gradient 6.3e-6 off, against 1.5e-7.
+// Bound: the grids are small (4,096 rows at width 256 make 256 such tiles), so
+// few warps per scheduler hide the shared-memory latency of two reads per 16
+// multiply-adds.  A 4096 x 256 x 256 layer takes 27 us; 8 x 4 results per
+// thread and half the threads 38 us, 8 x 8 (128 tiles of 128 x 64) 45 us.  A
+// batch (4,096 rows, width 256, loss and gradient to the host): 2.68 -> 0.32 ms,
+// against no prefetch, one CTA per tile of the weight gradients (28 CTAs) and
+// serial column and loss sums.
+constexpr int GT = 64, GK = 32, GTHREADS = 256, GP = GT + 4;
 
-// C[M x N] = op(A)[M x K] op(B)[K x N], FP32 accumulation.
-//   A(m, k) = TRA ? A[row(k) * lda + m] : A[row(m) * lda + k],  row(r) = aidx ? aidx[r] : r
-//   B(k, n) = TRB ? B[n * ldb + k]      : B[k * ldb + n]
-template <typename TA, typename TB, bool TRA, bool TRB>
-__global__ void k_gemm(int M, int N, int K, const TA* __restrict__ A, int lda, const int* __restrict__ aidx,
-                       const TB* __restrict__ B, int ldb, float* __restrict__ C, int ldc) {
-  __shared__ float As[16][64 + 4];
-  __shared__ float Bs[16][64 + 4];
-  int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-  float acc[4][4] = {};
-  for (int k0 = 0; k0 < K; k0 += 16) {
-    for (int t = threadIdx.x; t < 64 * 16; t += 256) {
-      int mm = t % 64, kk = t / 64;           // A tile element (m, k)
-      int m = m0 + mm, k = k0 + kk;
-      float va = 0.f;
-      if (m < M && k < K) {
-        if (TRA) va = ld(A + (size_t)(aidx ? aidx[k] : k) * lda + m);
-        else va = ld(A + (size_t)(aidx ? aidx[m] : m) * lda + k);
+// A tile's loader: 64 (rows of the tile) x 32 (k), 8 values per thread in two
+// runs of four.  KC: k is the contiguous index of the matrix, a run is (row
+// q / 8, k 4 (q % 8)); else the tile's row is, a run is (k q / 16, rows
+// 4 (q % 16)).  V4: rows are 16-byte (BF16: 8-byte) aligned and a multiple of
+// four long.
+template <typename T, bool KC, bool V4>
+struct TileLoad {
+  const T* p[2];                               // KC: the run's row; else its column in row 0
+  const int* idx;                              // gathered rows (not KC)
+  int ld, left[2];                             // KC: -1 where the row is outside; else values in the row
+  float v[8];
+  __device__ __forceinline__ TileLoad(const T* src, const int* gather, int ld_, int nrow, int row0)
+      : idx(gather), ld(ld_) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int q = threadIdx.x + u * GTHREADS, r = row0 + (KC ? q >> 3 : 4 * (q & 15));
+      left[u] = KC ? (r < nrow ? 4 : -1) : nrow - r;
+      p[u] = KC ? src + (size_t)(r < nrow ? (gather ? gather[r] : r) : 0) * ld + 4 * (q & 7) : src + r;
+    }
+  }
+  static __device__ __forceinline__ float one(const float* a) { return *a; }
+  static __device__ __forceinline__ float one(const __nv_bfloat16* a) { return __bfloat162float(*a); }
+  // four values from a, of which n exist
+  static __device__ __forceinline__ void run(const T* a, int n, float* o) {
+    if (V4 && n >= 4) {
+      if constexpr (sizeof(T) == 4) {
+        const float4 x = *reinterpret_cast<const float4*>(a);
+        o[0] = x.x; o[1] = x.y; o[2] = x.z; o[3] = x.w;
+      } else {
+        const uint2 x = *reinterpret_cast<const uint2*>(a);
+        o[0] = __uint_as_float(x.x << 16); o[1] = __uint_as_float(x.x & 0xffff0000u);
+        o[2] = __uint_as_float(x.y << 16); o[3] = __uint_as_float(x.y & 0xffff0000u);
       }
-      As[kk][mm] = va;
-      int nn = t % 64;                         // B tile element (k, n)
-      int n = n0 + nn;
-      float vb = 0.f;
-      if (n < N && k < K) vb = TRB ? ld(B + (size_t)n * ldb + k) : ld(B + (size_t)k * ldb + n);
-      Bs[kk][nn] = vb;
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) o[e] = e < n ? one(a + e) : 0.f;
     }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < 16; ++kk) {
-      float a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) { a[i] = As[kk][ty * 4 + i]; b[i] = Bs[kk][tx * 4 + i]; }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-    }
-    __syncthreads();
   }
-  for (int i = 0; i < 4; ++i)
-    for (int j = 0; j < 4; ++j) {
-      int m = m0 + ty * 4 + i, n = n0 + tx * 4 + j;
-      if (m < M && n < N) C[(size_t)m * ldc + n] = acc[i][j];
+  __device__ __forceinline__ void load(int k0, int k1) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int q = threadIdx.x + u * GTHREADS;
+      if (KC) {
+        run(p[u] + k0, left[u] < 0 ? 0 : k1 - k0 - 4 * (q & 7), v + 4 * u);
+      } else {
+        const int k = k0 + (q >> 4);
+        const bool in = k < k1;
+        run(p[u] + (size_t)(in ? (idx ? idx[k] : k) : 0) * ld, in ? left[u] : 0, v + 4 * u);
+      }
     }
+  }
+  __device__ __forceinline__ void store(float (*S)[GP]) const {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int q = threadIdx.x + u * GTHREADS;
+      if (KC) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) S[4 * (q & 7) + e][q >> 3] = v[4 * u + e];
+      } else {
+        *reinterpret_cast<float4*>(&S[q >> 4][4 * (q & 15)]) =
+            make_float4(v[4 * u], v[4 * u + 1], v[4 * u + 2], v[4 * u + 3]);
+      }
+    }
+  }
+};
+
+typedef float TileS[GK][GP];
+
+// This thread's 4 x 4 results: rows 4 (thread / 16) + i, columns 4 (thread % 16) + j
+struct Tile {
+  float2 d[4][2];
+  // f(row, column, value) for every result
+  template <typename Fn> __device__ __forceinline__ void each(Fn f) const {
+    const int r = threadIdx.x >> 4 << 2, c = (threadIdx.x & 15) << 2;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        f(r + i, c + 2 * j, d[i][j].x);
+        f(r + i, c + 2 * j + 1, d[i][j].y);
+      }
+  }
+};
+
+// C += A B over k in [k0, k1); with colsum, db += the sums over k of B's
+// column threadIdx.x
+template <typename LA, typename LB>
+__device__ __forceinline__ void tile_mma(LA& a, LB& b, int k0, int k1, TileS* As, TileS* Bs, Tile& c, bool colsum,
+                                         float* db) {
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  a.load(k0, k1);
+  b.load(k0, k1);
+  int buf = 0;
+  for (int k = k0; k < k1; k += GK, buf ^= 1) {
+    a.store(As[buf]);
+    b.store(Bs[buf]);
+    __syncthreads();
+    if (k + GK < k1) {
+      a.load(k + GK, k1);
+      b.load(k + GK, k1);
+    }
+#pragma unroll
+    for (int q = 0; q < GK; ++q) {
+      const float4 x = *reinterpret_cast<const float4*>(&As[buf][q][4 * ty]);
+      const float4 y = *reinterpret_cast<const float4*>(&Bs[buf][q][4 * tx]);
+      const float2 y0 = make_float2(y.x, y.y), y1 = make_float2(y.z, y.w);
+      const float xs[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float2 xx = make_float2(xs[i], xs[i]);
+        c.d[i][0] = __ffma2_rn(xx, y0, c.d[i][0]);
+        c.d[i][1] = __ffma2_rn(xx, y1, c.d[i][1]);
+      }
+    }
+    if (colsum && threadIdx.x < GT) {
+#pragma unroll
+      for (int q = 0; q < GK; ++q) *db += Bs[buf][q][threadIdx.x];
+    }
+  }
 }
 
-template <typename TA, typename TB, bool TRA, bool TRB>
-int gemm(Ctx* c, int M, int N, int K, const TA* A, int lda, const int* aidx, const TB* B, int ldb, float* C,
-         int ldc, cudaStream_t st) {
-  dim3 g((N + 63) / 64, (M + 63) / 64);
-  k_gemm<TA, TB, TRA, TRB><<<g, 256, 0, st>>>(M, N, K, A, lda, aidx, B, ldb, C, ldc);
-  SMR_LAUNCH(c);
-  return SMR_OK;
-}
-
-// Z += bias (per column); A = silu(Z) when act
-__global__ void k_bias_act(int n, int w, float* __restrict__ Z, const float* __restrict__ bias,
-                           float* __restrict__ A, int act) {
-  long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t >= (long long)n * w) return;
-  float z = Z[t] + bias[t % w];
-  Z[t] = z;
-  if (act) A[t] = silu(z);
-}
-
-// dZ = dA * silu'(Z)
-__global__ void k_act_back(long long n, const float* __restrict__ Z, const float* __restrict__ dA,
-                           float* __restrict__ dZ) {
-  long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t < n) dZ[t] = dA[t] * dsilu(Z[t]);
-}
-
-// db[j] = sum_m dZ[m][j]
-__global__ void k_colsum(int M, int N, const float* __restrict__ dZ, float* __restrict__ db) {
-  int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= N) return;
-  float s = 0.f;
-  for (int m = 0; m < M; ++m) s += dZ[(size_t)m * N + j];
-  db[j] = s;
-}
-
-// mean squared error: dY = 2 (Y - T) / (n O); per-block partial sums of (Y - T)^2
-__global__ void k_mse(int n, int O, const float* __restrict__ Y, const float* __restrict__ T,
-                      const int* __restrict__ tidx, float* __restrict__ dY, double* __restrict__ part) {
-  __shared__ double red[256];
-  long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+// Forward layer: Z = A W + b, and A' = silu(Z) (act), or for the last layer
+// with targets dZ = 2 (Z - T) / (n O) and the CTA's sum of (Z - T)^2.
+template <bool V4>
+__global__ void __launch_bounds__(GTHREADS) k_fwd(int n, int N, int K, const float* __restrict__ A,
+                                                  const int* __restrict__ aidx, const __nv_bfloat16* __restrict__ W,
+                                                  const float* __restrict__ bias, float* __restrict__ Z,
+                                                  float* __restrict__ act, const float* __restrict__ T,
+                                                  const int* __restrict__ tidx, float* __restrict__ dZ,
+                                                  double* __restrict__ part) {
+  __shared__ __align__(16) TileS As[2], Bs[2];
+  __shared__ double red[GTHREADS];
+  const int m0 = blockIdx.y * GT, n0 = blockIdx.x * GT;
+  TileLoad<float, true, V4> a(A, aidx, K, n, m0);
+  TileLoad<__nv_bfloat16, false, V4> b(W, nullptr, N, N, n0);
+  Tile acc = {};
+  tile_mma(a, b, 0, K, As, Bs, acc, false, nullptr);
   double e2 = 0.0;
-  if (t < (long long)n * O) {
-    int m = (int)(t / O), o = (int)(t % O);
-    int row = tidx ? tidx[m] : m;
-    float d = Y[t] - T[(size_t)row * O + o];
-    dY[t] = 2.f * d / ((float)n * (float)O);
-    e2 = (double)d * d;
-  }
+  const float scale = (float)n * (float)N;
+  acc.each([&](int i, int j, float v) {
+    const int m = m0 + i, c = n0 + j;
+    if (m >= n || c >= N) return;
+    const float z = v + bias[c];
+    Z[(size_t)m * N + c] = z;
+    if (act) act[(size_t)m * N + c] = silu(z);
+    if (T) {
+      const float d = z - T[(size_t)(tidx ? tidx[m] : m) * N + c];
+      dZ[(size_t)m * N + c] = 2.f * d / scale;
+      e2 += (double)d * d;
+    }
+  });
+  if (!T) return;
   red[threadIdx.x] = e2;
   __syncthreads();
-  for (int h = 128; h > 0; h >>= 1) {
-    if ((int)threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
+  for (int h = GTHREADS / 2; h > 0; h >>= 1) {
+    if (threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
     __syncthreads();
   }
-  if (threadIdx.x == 0) part[blockIdx.x] = red[0];
+  if (threadIdx.x == 0) part[blockIdx.y * gridDim.x + blockIdx.x] = red[0];
 }
 
+// dZ_{l-1} = (dZ_l W_l^T) silu'(Z_{l-1});  dZ_l [n][K], W_l [N][K]
+template <bool V4>
+__global__ void __launch_bounds__(GTHREADS) k_dx(int n, int N, int K, const float* __restrict__ dZl,
+                                                 const __nv_bfloat16* __restrict__ W, const float* __restrict__ Z,
+                                                 float* __restrict__ out) {
+  __shared__ __align__(16) TileS As[2], Bs[2];
+  const int m0 = blockIdx.y * GT, n0 = blockIdx.x * GT;
+  TileLoad<float, true, V4> a(dZl, nullptr, K, n, m0);
+  TileLoad<__nv_bfloat16, true, V4> b(W, nullptr, K, N, n0);
+  Tile acc = {};
+  tile_mma(a, b, 0, K, As, Bs, acc, false, nullptr);
+  acc.each([&](int i, int j, float v) {
+    const int m = m0 + i, c = n0 + j;
+    if (m < n && c < N) out[(size_t)m * N + c] = v * dsilu(Z[(size_t)m * N + c]);
+  });
+}
+
+// Weight gradients of all layers in one launch: dW_l = A_l^T dZ_l and db_l =
+// the column sums of dZ_l over the rows of split blockIdx.y, into that split's
+// copy of the parameter layout.  Tiles t0[l] .. t0[l + 1] belong to layer l.
+struct GradArgs {
+  const float* A[4];
+  const float* dZ[4];
+  const int* idx;                              // rows of layer 0's input
+  int in[4], out[4], t0[5];
+  long long off[4], np;
+};
+template <bool V4>
+__global__ void __launch_bounds__(GTHREADS) k_dw(GradArgs g, int n, int rows, float* __restrict__ part) {
+  __shared__ __align__(16) TileS As[2], Bs[2];
+  int l = 0;
+  while (l < 3 && (int)blockIdx.x >= g.t0[l + 1]) ++l;
+  const int t = blockIdx.x - g.t0[l], M = g.in[l], N = g.out[l], nx = (N + GT - 1) / GT;
+  const int m0 = t / nx * GT, n0 = t % nx * GT;
+  const int k0 = blockIdx.y * rows, k1 = min(n, k0 + rows);
+  TileLoad<float, false, V4> a(g.A[l], l == 0 ? g.idx : nullptr, M, M, m0);
+  TileLoad<float, false, V4> b(g.dZ[l], nullptr, N, N, n0);
+  Tile acc = {};
+  float db = 0.f;
+  if (k0 < k1) tile_mma(a, b, k0, k1, As, Bs, acc, m0 == 0, &db);
+  float* o = part + (size_t)blockIdx.y * g.np + g.off[l];
+  acc.each([&](int i, int j, float v) {
+    const int m = m0 + i, c = n0 + j;
+    if (m < M && c < N) o[(size_t)m * N + c] = v;
+  });
+  if (m0 == 0 && threadIdx.x < GT && n0 + threadIdx.x < N) o[(size_t)M * N + n0 + threadIdx.x] = db;
+}
+
+// gradient = sum of the splits, in split order
+__global__ void k_split_sum(long long np, int S, const float* __restrict__ part, float* __restrict__ g) {
+  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (i >= np) return;
+  float s = part[i];
+  for (int q = 1; q < S; ++q) s += part[(size_t)q * np + i];
+  g[i] = s;
+}
+
+// loss = scale x the sum of the partial sums (one CTA of 256)
 __global__ void k_sum(int n, const double* __restrict__ part, double scale, double* __restrict__ out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double s = 0.0;
-    for (int i = 0; i < n; ++i) s += part[i];
-    *out = s * scale;
+  __shared__ double red[256];
+  double s = 0.0;
+  for (int i = threadIdx.x; i < n; i += 256) s += part[i];
+  red[threadIdx.x] = s;
+  __syncthreads();
+  for (int h = 128; h > 0; h >>= 1) {
+    if (threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
+    __syncthreads();
   }
+  if (threadIdx.x == 0) *out = red[0] * scale;
 }
 
 __global__ void k_adam(long long n, float* __restrict__ p, __nv_bfloat16* __restrict__ w16,
@@ -241,7 +373,7 @@ long long woff(const NN& nn, int l) {
 void nn_free(Ctx* c) {
   NN& nn = c->nn;
   cudaFree(nn.p32); cudaFree(nn.w16); cudaFree(nn.m); cudaFree(nn.v); cudaFree(nn.g);
-  cudaFree(nn.act); cudaFree(nn.dact); cudaFree(nn.d_loss); cudaFree(nn.d_slots);
+  cudaFree(nn.act); cudaFree(nn.dact); cudaFree(nn.part); cudaFree(nn.d_loss); cudaFree(nn.d_slots);
   nn = NN();
 }
 
@@ -273,8 +405,8 @@ int nn_init(Ctx* c, int width, unsigned long long seed) {
   SMR_CUDA(c, cudaMalloc((void**)&nn.v, nn.np * sizeof(float)));
   SMR_CUDA(c, cudaMalloc((void**)&nn.g, nn.np * sizeof(float)));
   SMR_CUDA(c, cudaMalloc((void**)&nn.act, abytes));
-  SMR_CUDA(c, cudaMalloc((void**)&nn.dact, abytes + (size_t)nn.cap * nn.F * sizeof(float)));
-  SMR_CUDA(c, cudaMalloc((void**)&nn.d_loss, ((size_t)nn.cap * nn.O / 256 + 2) * sizeof(double)));
+  SMR_CUDA(c, cudaMalloc((void**)&nn.dact, (size_t)nn.cap * (3 * (size_t)width + nn.O) * sizeof(float)));
+  SMR_CUDA(c, cudaMalloc((void**)&nn.d_loss, ((size_t)(nn.cap / GT) * ((nn.O + GT - 1) / GT) + 1) * sizeof(double)));
   SMR_CUDA(c, cudaMemcpy(nn.p32, p.data(), nn.np * sizeof(float), cudaMemcpyHostToDevice));
   SMR_CUDA(c, cudaMemset(nn.m, 0, nn.np * sizeof(float)));
   SMR_CUDA(c, cudaMemset(nn.v, 0, nn.np * sizeof(float)));
@@ -331,63 +463,75 @@ int nn_forward_backward(Ctx* c, int n, const float* feat, const int* idx, const 
   NN& nn = c->nn;
   if (!nn.p32) { c->err = "call smr_nn_init first"; return SMR_E_STATE; }
   if (n < 1 || n > nn.cap) { c->err = "batch must be 1..8192 rows"; return SMR_E_INVALID_ARG; }
-  int H = nn.H, O = nn.O;
-  // activation layout: Z1 A1 Z2 A2 Z3 A3 Y
-  float* Z[4];
-  float* A[4];
-  Z[0] = nn.act;
-  A[0] = Z[0] + (size_t)nn.cap * H;
-  Z[1] = A[0] + (size_t)nn.cap * H;
-  A[1] = Z[1] + (size_t)nn.cap * H;
-  Z[2] = A[1] + (size_t)nn.cap * H;
-  A[2] = Z[2] + (size_t)nn.cap * H;
-  Z[3] = A[2] + (size_t)nn.cap * H;   // output Y [n][O]
-  int rc;
+  const int H = nn.H, O = nn.O;
+  // buffers: pre-activations Z and activations A of the three hidden layers,
+  // the output, and the gradients with respect to the pre-activations
+  float *Z[4], *A[4] = {nullptr, nullptr, nullptr, nullptr}, *dZ[4];
+  for (int l = 0; l < 3; ++l) {
+    Z[l] = nn.act + (size_t)(2 * l) * nn.cap * H;
+    A[l] = nn.act + (size_t)(2 * l + 1) * nn.cap * H;
+    dZ[l] = nn.dact + (size_t)nn.cap * O + (size_t)l * nn.cap * H;
+  }
+  Z[3] = nn.act + (size_t)6 * nn.cap * H;
+  dZ[3] = nn.dact;
+  // 16-byte loads where every row of every operand is aligned for them
+  const bool v4 = nn.F % 4 == 0 && H % 4 == 0 && O % 4 == 0 && ((uintptr_t)feat & 15) == 0;
+  const int my = (n + GT - 1) / GT;
+  int nb = 0;
   for (int l = 0; l < 4; ++l) {
-    int in = nn.dims[l], out = nn.dims[l + 1];
+    const int in = nn.dims[l], out = nn.dims[l + 1];
     const __nv_bfloat16* W = nn.w16 + woff(nn, l);
     const float* b = nn.p32 + woff(nn, l) + (long long)in * out;
-    if (l == 0) rc = gemm<float, __nv_bfloat16, false, false>(c, n, out, in, feat, in, idx, W, out, Z[0], out, st);
-    else rc = gemm<float, __nv_bfloat16, false, false>(c, n, out, in, A[l - 1], in, nullptr, W, out, Z[l], out, st);
-    if (rc) return rc;
-    k_bias_act<<<(unsigned)(((long long)n * out + 255) / 256), 256, 0, st>>>(n, out, Z[l], b, l < 3 ? A[l] : nullptr,
-                                                                          l < 3 ? 1 : 0);
+    const dim3 g((out + GT - 1) / GT, my);
+    const bool last = l == 3;
+    if (last) nb = (int)(g.x * g.y);
+    auto k = v4 ? k_fwd<true> : k_fwd<false>;
+    k<<<g, GTHREADS, 0, st>>>(n, out, in, l ? A[l - 1] : feat, l ? nullptr : idx, W, b, Z[l], A[l],
+                              last ? tgt : nullptr, idx, dZ[3], nn.d_loss + 1);
     SMR_LAUNCH(c);
   }
-  // loss and dY
-  float* dZ[4];
-  float* dA = nn.dact;                         // [cap][max(F, H)]
-  dZ[3] = dA + (size_t)nn.cap * std::max(nn.F, H);
-  dZ[2] = dZ[3] + (size_t)nn.cap * O;
-  dZ[1] = dZ[2] + (size_t)nn.cap * H;
-  dZ[0] = dZ[1] + (size_t)nn.cap * H;
   if (!tgt) return SMR_OK;                      // inference only
-  int nb = (int)(((long long)n * O + 255) / 256);
-  k_mse<<<nb, 256, 0, st>>>(n, O, Z[3], tgt, idx, dZ[3], nn.d_loss + 1);
-  SMR_LAUNCH(c);
-  k_sum<<<1, 32, 0, st>>>(nb, nn.d_loss + 1, 1.0 / ((double)n * O), nn.d_loss);
+  k_sum<<<1, 256, 0, st>>>(nb, nn.d_loss + 1, 1.0 / ((double)n * O), nn.d_loss);
   SMR_LAUNCH(c);
   if (backward) {
-    for (int l = 3; l >= 0; --l) {
-      int in = nn.dims[l], out = nn.dims[l + 1];
-      float* gW = nn.g + woff(nn, l);
-      float* gb = gW + (long long)in * out;
-      const float* Ain = l == 0 ? feat : A[l - 1];
-      const int* ai = l == 0 ? idx : nullptr;
-      // dW = A_in^T dZ
-      rc = gemm<float, float, true, false>(c, in, out, n, Ain, in, ai, dZ[l], out, gW, out, st);
-      if (rc) return rc;
-      k_colsum<<<(out + 127) / 128, 128, 0, st>>>(n, out, dZ[l], gb);
+    for (int l = 3; l > 0; --l) {
+      const int in = nn.dims[l], out = nn.dims[l + 1];
+      auto k = v4 ? k_dx<true> : k_dx<false>;
+      k<<<dim3((in + GT - 1) / GT, my), GTHREADS, 0, st>>>(n, in, out, dZ[l], nn.w16 + woff(nn, l), Z[l - 1],
+                                                           dZ[l - 1]);
       SMR_LAUNCH(c);
-      if (l > 0) {
-        // dA_{l-1} = dZ_l W_l^T ; dZ_{l-1} = dA * silu'(Z_{l-1})
-        const __nv_bfloat16* W = nn.w16 + woff(nn, l);
-        rc = gemm<float, __nv_bfloat16, false, true>(c, n, in, out, dZ[l], out, nullptr, W, out, dA, in, st);
-        if (rc) return rc;
-        long long ne = (long long)n * in;
-        k_act_back<<<(unsigned)((ne + 255) / 256), 256, 0, st>>>(ne, Z[l - 1], dA, dZ[l - 1]);
-        SMR_LAUNCH(c);
-      }
+    }
+    GradArgs g;
+    g.idx = idx;
+    g.np = nn.np;
+    g.t0[0] = 0;
+    for (int l = 0; l < 4; ++l) {
+      g.A[l] = l ? A[l - 1] : feat;
+      g.dZ[l] = dZ[l];
+      g.in[l] = nn.dims[l];
+      g.out[l] = nn.dims[l + 1];
+      g.off[l] = woff(nn, l);
+      g.t0[l + 1] = g.t0[l] + (g.in[l] + GT - 1) / GT * ((g.out[l] + GT - 1) / GT);
+    }
+    // the batch's rows in splits: about three CTAs per SM in all, at least 64
+    // rows each (68 tiles at width 256: six splits)
+    int S = std::max(1, std::min(3 * 152 / g.t0[4], n / 64));
+    const int rows = ((n + S - 1) / S + GK - 1) / GK * GK;
+    S = (n + rows - 1) / rows;
+    const size_t need = (size_t)S * nn.np;
+    if (S > 1 && nn.part_elems < need) {
+      cudaFree(nn.part);
+      nn.part = nullptr;
+      nn.part_elems = 0;
+      SMR_CUDA(c, cudaMalloc((void**)&nn.part, need * sizeof(float)));
+      nn.part_elems = need;
+    }
+    auto k = v4 ? k_dw<true> : k_dw<false>;
+    k<<<dim3(g.t0[4], S), GTHREADS, 0, st>>>(g, n, rows, S > 1 ? nn.part : nn.g);
+    SMR_LAUNCH(c);
+    if (S > 1) {
+      k_split_sum<<<(unsigned)((nn.np + 255) / 256), 256, 0, st>>>(nn.np, S, nn.part, nn.g);
+      SMR_LAUNCH(c);
     }
   }
   if (loss_host) {

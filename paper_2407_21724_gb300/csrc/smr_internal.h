@@ -175,6 +175,8 @@ struct NN {
   int cap = 0;                          // rows of the activation buffers
   float* act = nullptr;                 // activations and pre-activations
   float* dact = nullptr;
+  float* part = nullptr;                // weight gradients per split of the batch's rows
+  size_t part_elems = 0;
   double* d_loss = nullptr;
   int* d_slots = nullptr;               // [48][2] neighbour offsets, sorted
 };
