@@ -38,7 +38,7 @@ void free_scene(Ctx* c) {
     dfree(L.d_shiftp32); dfree(L.d_shiftw32); dfree(L.d_mi_vlast); dfree(L.d_ma_ptr); dfree(L.d_ma_ent);
     dfree(L.d_ma_w64); dfree(L.d_ma_w32); dfree(L.d_ma_pst); dfree(L.d_ma_pw64); dfree(L.d_ma_pw32);
     dfree(L.d_ant_lo); dfree(L.d_ant_pjp); dfree(L.d_ant_pw64); dfree(L.d_ant_ttp); dfree(L.d_ant_tw64);
-    dfree(L.d_wthp64); dfree(L.d_boxmap); dfree(L.d_offid); dfree(L.d_tiles); dfree(L.d_tiles8);
+    dfree(L.d_wthp64); dfree(L.d_boxmap); dfree(L.d_offid); dfree(L.d_tiles); dfree(L.d_tiles8); dfree(L.d_tile_tab);
     for (int q = 0; q < 2; ++q) {
       if (L.buf_out[q]) cudaFree(L.buf_out[q]);
       if (L.buf_in[q]) cudaFree(L.buf_in[q]);
@@ -667,7 +667,7 @@ int set_scene(Ctx* c, int p, const double* centres, const int* shape_ids, const 
     if (!pk.empty() && (rc = upload(c, &L.d_il_pk, pk))) return rc;
     if ((rc = upload(c, &L.d_tiles8, tiles8))) return rc;
     if ((rc = upload(c, &L.d_boxmap, bm)) || (rc = upload(c, &L.d_offid, oid)) ||
-        (rc = upload(c, &L.d_tiles, tiles)))
+        (rc = upload(c, &L.d_tiles, tiles)) || (rc = build_translate_tiles(c, L, tiles, bm)))
       return rc;
   }
   // particles grouped by shape, tiles of at most 16
@@ -1490,19 +1490,22 @@ int smr_autotune(smr_ctx* h, int R, int precision, void* stream) {
   double2* y = c->d_tmp + n;
   SMR_CUDA(c, cudaMemsetAsync(x, 0, n * sizeof(double2), (cudaStream_t)stream));
   std::map<std::pair<std::string, int>, double> t;
-  // translation: 8x8 tiles (full, half direction chunk) and 4x4 tiles
+  // FP64 translation: 8x8 tiles (full, half direction chunk), 4x4 tiles, the
+  // few-box and the whole-level kernel
   std::vector<std::vector<double>> ttr(c->nlev, std::vector<double>(6, 1e30));
   std::vector<std::vector<double>> tip(c->nlev, std::vector<double>(4, 1e30));
   std::vector<std::vector<double>> tan_(c->nlev, std::vector<double>(4, 1e30));
   double agg[2] = {1e30, 1e30}, rec[2] = {1e30, 1e30}, nea[2] = {1e30, 1e30};
   const int agg0 = c->tune_tc_agg, rec0 = c->tune_tc_rec, nea0 = c->tune_tc_near;
   // trial 5 times the whole-level translation (levels of at most 256 boxes),
-  // the FP64 interpolation and anterpolation their gather variants in trials 1
-  // and 2 (FP32 has one kernel for each)
+  // trials 1 and 2 the gather variants of the FP64 interpolation and
+  // anterpolation.  FP32 has one kernel for each level step: its trials 1 and 3
+  // time the tensor cores and the CUDA cores
   for (int v = 1; v <= 5; ++v) {
+    if (q == 1 && v != 1 && v != 3) continue;
     // variant 4 (few-box kernel) only where a level has at most 1024 boxes
     for (auto& L : c->lev) {
-      L.tune_tr[q] = (v == 4 && L.nbox > 1024) || (v == 5 && L.nbox > 256) ? 1 : v;
+      L.tune_tr[q] = q == 1 ? 0 : (v == 4 && L.nbox > 1024) || (v == 5 && L.nbox > 256) ? 1 : v;
       L.tune_ip[q] = L.tune_an[q] = (q == 0 && v <= 2) ? v : 0;
     }
     c->tune_tc_agg = c->tune_tc_rec = c->tune_tc_near = (v == 3) ? 0 : 1;
@@ -1530,7 +1533,7 @@ int smr_autotune(smr_ctx* h, int R, int precision, void* stream) {
     int bv = 1;
     for (int v = 2; v <= 5; ++v)
       if (ttr[s][v] < ttr[s][bv]) bv = v;
-    L.tune_tr[q] = rc ? 0 : bv;
+    L.tune_tr[q] = rc || q == 1 ? 0 : bv;
     int bi = 0;
     for (int v = 1; v <= 3; ++v)
       if (tip[s][v] < tip[s][bi]) bi = v;

@@ -445,21 +445,22 @@ __global__ void k_translate(int K, int R, int RC, int KC, int ntx, int ntile, co
   }
 }
 
-// Single right-hand side: each thread owns one 16-byte part of the 2x2
+// FP64, one right-hand side (FP32: k_translate.cu): each thread owns one 16-byte part of the 2x2
 // targets that share one parent, for one direction, and walks the parent's
 // 6x6 source window once; a staged source part is read from shared memory
 // once for all four targets (conflict-free: lanes read consecutive 16-byte
 // parts).  CTA = 8x8 targets (4x4 parents) x KC directions; 16 x KC x NT threads.
-template <typename T, int KC>
+template <int KC>
 __global__ void __launch_bounds__(512, 2) k_translate1(int K, int ntx, int ntile,
                                                     const int* __restrict__ tiles, int map_x0, int map_y0,
                                                     int map_w, int map_h, const int* __restrict__ boxmap,
-                                                    const typename CV<T>::V* __restrict__ Tg,
-                                                    const typename CV<T>::V* __restrict__ out,
-                                                    typename CV<T>::V* __restrict__ in) {
-  typedef typename CV<T>::V V;
+                                                    const double2* __restrict__ Tg,
+                                                    const double2* __restrict__ out,
+                                                    double2* __restrict__ in) {
+  typedef double T;
+  typedef double2 V;
   typedef Part<T> P;
-  typedef typename P::H H;
+  typedef P::H H;
   constexpr int NT = P::NT;
   constexpr int TS = 8, HS = TS + 4;                  // targets per side, halo per side
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -472,12 +473,7 @@ __global__ void __launch_bounds__(512, 2) k_translate1(int K, int ntx, int ntile
   constexpr int W = KC * 4;
   V* S = reinterpret_cast<V*>(smem_raw);              // [HS*HS sources][KC][4]
   V* Ts = S + HS * HS * W;                            // [49 offsets][KC]
-  // FP32: the table entries as (t_r, t_r, -t_i, t_i), so that a complex
-  // multiply-add of two fields is four packed FMAs
-  constexpr bool PK = sizeof(T) == 4;
-  float4* Ts4 = reinterpret_cast<float4*>(Ts);
-  int* bid = reinterpret_cast<int*>(PK ? reinterpret_cast<unsigned char*>(Ts4 + 49 * KC)
-                                       : reinterpret_cast<unsigned char*>(Ts + 49 * KC));   // [HS*HS] source box ids
+  int* bid = reinterpret_cast<int*>(Ts + 49 * KC);    // [HS*HS] source box ids
   int* tb = bid + HS * HS;                            // [TS*TS] target box ids
   for (int t = threadIdx.x; t < HS * HS + TS * TS; t += blockDim.x) {
     int sx, sy;
@@ -504,9 +500,7 @@ __global__ void __launch_bounds__(512, 2) k_translate1(int K, int ntx, int ntile
   }
   for (int t = threadIdx.x; t < 49 * KC; t += blockDim.x) {
     int o = t / KC, kl = t - o * KC;
-    const V tv = (kl < nk) ? Tg[(size_t)o * K + k0 + kl] : czero<V>();
-    if constexpr (PK) Ts4[t] = make_float4((float)tv.x, (float)tv.x, -(float)tv.y, (float)tv.y);
-    else Ts[t] = tv;
+    Ts[t] = (kl < nk) ? Tg[(size_t)o * K + k0 + kl] : czero<V>();
   }
   cp_async_wait_all();
   __syncthreads();
@@ -530,31 +524,11 @@ __global__ void __launch_bounds__(512, 2) k_translate1(int K, int ntx, int ntile
 #pragma unroll
     for (int wx = 0; wx < 6; ++wx) {
       H v = reinterpret_cast<const H*>(Sp + (wy * HS + wx) * W)[h];
-      if constexpr (PK) {
-        // (re, im) += (t_r, t_r) (v_re, v_im) + (-t_i, t_i) (v_im, v_re), per field
-        const float2 v0 = make_float2(v.x, v.y), v1 = make_float2(v.z, v.w);
-        const float2 s0 = make_float2(v.y, v.x), s1 = make_float2(v.w, v.z);
-        const float4* T4 = Ts4 + kl;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int dx = (q & 1) + 2 - wx, dy = (q >> 1) + 2 - wy;
-          if (dx >= -1 && dx <= 1 && dy >= -1 && dy <= 1) continue;
-          const float4 t = T4[((dx + 3) * 7 + (dy + 3)) * KC];
-          const float2 tr = make_float2(t.x, t.y), tn = make_float2(t.z, t.w);
-          float2 a0 = make_float2(acc[q].x, acc[q].y), a1 = make_float2(acc[q].z, acc[q].w);
-          a0 = __ffma2_rn(tr, v0, a0);
-          a0 = __ffma2_rn(tn, s0, a0);
-          a1 = __ffma2_rn(tr, v1, a1);
-          a1 = __ffma2_rn(tn, s1, a1);
-          acc[q] = make_float4(a0.x, a0.y, a1.x, a1.y);
-        }
-      } else {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int dx = (q & 1) + 2 - wx, dy = (q >> 1) + 2 - wy;
-          if (dx >= -1 && dx <= 1 && dy >= -1 && dy <= 1) continue;
-          P::cfma(acc[q], Tp[((dx + 3) * 7 + (dy + 3)) * KC], v);
-        }
+      for (int q = 0; q < 4; ++q) {
+        const int dx = (q & 1) + 2 - wx, dy = (q >> 1) + 2 - wy;
+        if (dx >= -1 && dx <= 1 && dy >= -1 && dy <= 1) continue;
+        P::cfma(acc[q], Tp[((dx + 3) * 7 + (dy + 3)) * KC], v);
       }
     }
   }
@@ -570,15 +544,15 @@ __global__ void __launch_bounds__(512, 2) k_translate1(int K, int ntx, int ntile
 // along the directions (NT 16-byte parts each, coalesced); a CTA takes TG
 // consecutive target boxes and reads each target's interaction list
 // (source box * 64 + table row) uniformly.
-template <typename T>
 __global__ void __launch_bounds__(256) k_translate_few(int K, int nbox, int TG, const int* __restrict__ il_ptr,
                                                        const int* __restrict__ il_pk,
-                                                       const typename CV<T>::V* __restrict__ Tg,
-                                                       const typename CV<T>::V* __restrict__ out,
-                                                       typename CV<T>::V* __restrict__ in) {
-  typedef typename CV<T>::V V;
+                                                       const double2* __restrict__ Tg,
+                                                       const double2* __restrict__ out,
+                                                       double2* __restrict__ in) {
+  typedef double T;
+  typedef double2 V;
   typedef Part<T> P;
-  typedef typename P::H H;
+  typedef P::H H;
   constexpr int NT = P::NT;
   const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const int k = (int)(t / NT), h = (int)(t % NT);
@@ -601,15 +575,15 @@ __global__ void __launch_bounds__(256) k_translate_few(int K, int nbox, int TG, 
 // spectrum is read from memory once instead of once per target that lists
 // it.  Tasks are (target, direction, 16-byte part), the parts of consecutive
 // directions on consecutive threads.
-template <typename T>
 __global__ void __launch_bounds__(256) k_translate_lvl(int K, int nbox, int KCH, const int* __restrict__ il_ptr,
                                                        const int* __restrict__ il_pk,
-                                                       const typename CV<T>::V* __restrict__ Tg,
-                                                       const typename CV<T>::V* __restrict__ out,
-                                                       typename CV<T>::V* __restrict__ in) {
-  typedef typename CV<T>::V V;
+                                                       const double2* __restrict__ Tg,
+                                                       const double2* __restrict__ out,
+                                                       double2* __restrict__ in) {
+  typedef double T;
+  typedef double2 V;
   typedef Part<T> P;
-  typedef typename P::H H;
+  typedef P::H H;
   constexpr int NT = P::NT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   V* S = reinterpret_cast<V*>(smem_raw);                 // [nbox][KCH][4]
@@ -947,13 +921,12 @@ int translate_lvl_chunk(int nbox, size_t vbytes) {
   return 0;
 }
 
-bool translate_lvl_ok(Ctx* c, int s, bool f64) {
+bool translate_lvl_ok(Ctx* c, int s) {
   const Level& L = c->lev[s];
-  if (L.off_dx.empty() || !L.d_il_pk || translate_lvl_chunk(L.nbox, f64 ? 16 : 8) == 0) return false;
+  if (L.off_dx.empty() || !L.d_il_pk || translate_lvl_chunk(L.nbox, sizeof(double2)) == 0) return false;
   static bool attr = false;
   if (!attr) {
-    cudaFuncSetAttribute(k_translate_lvl<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    cudaFuncSetAttribute(k_translate_lvl<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaFuncSetAttribute(k_translate_lvl, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     attr = true;
   }
   return true;
@@ -1063,40 +1036,41 @@ static int far_impl(Ctx* c, int R, const double2* x, double2* y, bool accumulate
     pbeg(c, ts, "translate", s,
          2.0 * L.nbox * L.K * 4 * R_ * es + (double)L.off_dx.size() * L.K * es,
          8.0 * L.il_src.size() * L.K * 4 * R_);
-    // single right-hand side: 8x8-tile register-blocked kernel, except on
+    if (!f64 && R == 1) {
+      int rc = run_translate_tiles(c, s, ts);
+      pend(c, ts);
+      return rc;
+    }
+    // FP64, one right-hand side: 8x8-tile register-blocked kernel, except on
     // levels whose few boxes would leave most of one 8x8 tile idle (or as tuned)
-    const int tv = (R == 1) ? L.tune_tr[f64 ? 0 : 1] : 0;
-    if (tv == 5 && translate_lvl_ok(c, s, f64)) {
-      const int KCH = translate_lvl_chunk(L.nbox, sizeof(V));
-      const size_t sml = ((size_t)L.nbox * KCH * 4 + (size_t)49 * KCH) * sizeof(V);
-      k_translate_lvl<T><<<(unsigned)((L.K + KCH - 1) / KCH), 256, sml, ts>>>(
-          L.K, L.nbox, KCH, L.d_il_ptr, L.d_il_pk, (const V*)(f64 ? (void*)L.d_T64 : (void*)L.d_T32),
-          (const V*)L.d_out, (V*)L.d_in);
+    const int tv = (R == 1) ? L.tune_tr[0] : 0;
+    if (R == 1 && tv == 5 && translate_lvl_ok(c, s)) {
+      const int KCH = translate_lvl_chunk(L.nbox, sizeof(double2));
+      const size_t sml = ((size_t)L.nbox * KCH * 4 + (size_t)49 * KCH) * sizeof(double2);
+      k_translate_lvl<<<(unsigned)((L.K + KCH - 1) / KCH), 256, sml, ts>>>(
+          L.K, L.nbox, KCH, L.d_il_ptr, L.d_il_pk, L.d_T64, (const double2*)L.d_out, (double2*)L.d_in);
       SMR_LAUNCH(c);
       pend(c, ts);
       return SMR_OK;
     }
-    const bool few = (tv == 4) || (tv == 0 && R == 1 && L.nbox <= 64);
-    const bool use8 = (tv == 0) ? (R == 1 && !(L.ntile8_ne == 1 && L.nbox < 32)) : (tv != 3);
+    const bool few = R == 1 && (tv == 4 || (tv == 0 && L.nbox <= 64));
+    const bool use8 = R == 1 && (tv == 0 ? !(L.ntile8_ne == 1 && L.nbox < 32) : tv != 3);
     if (few) {
       const int TG = 8;
-      dim3 g((unsigned)(((long long)L.K * Part<T>::NT + 255) / 256), (unsigned)((L.nbox + TG - 1) / TG));
-      k_translate_few<T><<<g, 256, 0, ts>>>(L.K, L.nbox, TG, L.d_il_ptr, L.d_il_pk,
-                                             (const V*)(f64 ? (void*)L.d_T64 : (void*)L.d_T32), (const V*)L.d_out,
-                                             (V*)L.d_in);
+      dim3 g((unsigned)(((long long)L.K * Part<double>::NT + 255) / 256), (unsigned)((L.nbox + TG - 1) / TG));
+      k_translate_few<<<g, 256, 0, ts>>>(L.K, L.nbox, TG, L.d_il_ptr, L.d_il_pk, L.d_T64, (const double2*)L.d_out,
+                                         (double2*)L.d_in);
     } else if (use8) {
-      // direction chunk: 16 (FP32) or 8 (FP64) directions, halved by the tuner
+      // 8 directions per CTA, halved by the tuner
       const bool halfc = (tv == 2);
-      int KC1 = (f64 ? 8 : 16) / (halfc ? 2 : 1);
+      int KC1 = 8 / (halfc ? 2 : 1);
       int nk1 = (L.K + KC1 - 1) / KC1;
-      // FP32 tables are staged as 16-byte (t_r, t_r, -t_i, t_i) entries
-      size_t sm1 = ((size_t)144 * KC1 * 4) * sizeof(V) + (size_t)49 * KC1 * (f64 ? sizeof(V) : 16) +
-                   (144 + 64) * sizeof(int);
-      auto kt = halfc ? k_translate1<T, (sizeof(T) == 8 ? 4 : 8)> : k_translate1<T, (sizeof(T) == 8 ? 8 : 16)>;
+      size_t sm1 = ((size_t)144 * KC1 * 4 + (size_t)49 * KC1) * sizeof(double2) + (144 + 64) * sizeof(int);
+      auto kt = halfc ? k_translate1<4> : k_translate1<8>;
       cudaFuncSetAttribute(kt, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-      kt<<<(unsigned)(L.ntile8_ne * nk1), 16 * KC1 * Part<T>::NT, sm1, ts>>>(
+      kt<<<(unsigned)(L.ntile8_ne * nk1), 16 * KC1 * Part<double>::NT, sm1, ts>>>(
           L.K, L.ntile8_x, L.ntile8_ne, L.d_tiles8, L.map_x0, L.map_y0, L.map_w, L.map_h, L.d_boxmap,
-          (const V*)(f64 ? (void*)L.d_T64 : (void*)L.d_T32), (const V*)L.d_out, (V*)L.d_in);
+          L.d_T64, (const double2*)L.d_out, (double2*)L.d_in);
     } else {
       k_translate<T><<<(unsigned)(L.ntile_ne * nkch * nrct), 256, sm, ts>>>(
           L.K, R, RCt, KC, L.ntile_x, L.ntile_ne, L.d_tiles, L.map_x0, L.map_y0, L.map_w, L.map_h, noff,

@@ -128,6 +128,7 @@ struct Level {
   int* d_offid = nullptr;                // [7][7] offset (dx+3, dy+3) -> table row or -1
   int ntile_x = 0, ntile_y = 0, ntile_ne = 0;
   int* d_tiles = nullptr;                // non-empty 4x4 translation tiles (ty * ntile_x + tx)
+  int* d_tile_tab = nullptr;             // per non-empty 4x4 tile: 64 source and 16 target boxes (k_translate.cu)
   int ntile8_x = 0, ntile8_ne = 0;
   int* d_tiles8 = nullptr;               // non-empty 8x8 tiles (single right-hand side kernel)
   // FP64 gather anterpolation into this level, one right-hand side (k_anterp1):
@@ -464,6 +465,9 @@ int run_near_tc(Ctx* c, double2* y, cudaStream_t st);
 int prep_x32(Ctx* c, int R, int prec, const double2* x, cudaStream_t st);
 int run_aggregate_tc(Ctx* c, const double2* x, const float2* x32, float2* out0, cudaStream_t st);
 int tc_check(Ctx* c);
+// FP32 translation of one right-hand side (k_translate.cu)
+int build_translate_tiles(Ctx* c, Level& L, const std::vector<int>& tiles, const std::vector<int>& boxmap);
+int run_translate_tiles(Ctx* c, int s, cudaStream_t st);
 // interpolation s -> s + 1 and anterpolation s + 1 -> s (k_march.cu)
 int run_interp(Ctx* c, int s, int R, int prec, cudaStream_t st);
 int run_anterp(Ctx* c, int s, int R, int prec, cudaStream_t st);
