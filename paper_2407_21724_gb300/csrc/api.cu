@@ -57,7 +57,7 @@ void free_scene(Ctx* c) {
   c->multi = 0;
   dfree(c->d_B64); dfree(c->d_B32); dfree(c->d_tcn_img); dfree(c->d_tcn_blk); dfree(c->d_tcn_start);
   dfree(c->d_tcn_count); dfree(c->d_tcn_nu); dfree(c->d_tcn_mu); dfree(c->d_x32);
-  dfree(c->d_tcn_mask); dfree(c->d_tcn_part); dfree(c->d_Pinv64); dfree(c->d_Pinv32); dfree(c->d_pc_ptr);
+  dfree(c->d_tcn_mask); dfree(c->d_tcn_part); dfree(c->d_tc_part); dfree(c->d_Pinv64); dfree(c->d_Pinv32); dfree(c->d_pc_ptr);
   dfree(c->d_pc_col); dfree(c->d_pc_blk); dfree(c->d_tmp);
   dfree(c->d_arr);
   dfree(c->d_tile_shape); dfree(c->d_tile_start); dfree(c->d_tile_count); dfree(c->d_perm);

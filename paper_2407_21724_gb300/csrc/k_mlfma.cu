@@ -1196,7 +1196,6 @@ static int far_impl(Ctx* c, int R, const double2* x, double2* y, bool accumulate
   }
   // receive
   if (sd) SMR_CUDA(c, cudaStreamWaitEvent(st, sd->etr[0], 0));
-  if (c->near_ev) SMR_CUDA(c, cudaStreamWaitEvent(st, c->near_ev, 0));
   {
     int thr = c->npsi * 8;
     size_t sm = ((size_t)32 * 2 * c->npsi + 32 * 16 * 4) * sizeof(V);
@@ -1220,10 +1219,11 @@ static int far_impl(Ctx* c, int R, const double2* x, double2* y, bool accumulate
       inc = part;
     }
     if (tc) {
-      int rc = run_receive_tc(c, (const float2*)inc, y, accumulate, st);
+      int rc = run_receive_tc(c, (const float2*)inc, y, accumulate, c->near_ev, st);
       pend(c, st);
       return rc;
     }
+    if (c->near_ev) SMR_CUDA(c, cudaStreamWaitEvent(st, c->near_ev, 0));
     int nsub = (16 + std::max(1, 16 / RC) - 1) / std::max(1, 16 / RC);
     cudaFuncSetAttribute(k_receive<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     k_receive<T><<<(unsigned)(c->ntile * nsub * nrc), thr, sm, st>>>(
@@ -1362,6 +1362,7 @@ void free_lanes(Ctx* c) {
     for (void* q : a.in) if (q) cudaFree(q);
     if (a.x32) cudaFree(a.x32);
     if (a.tcn_part) cudaFree(a.tcn_part);
+    if (a.tc_part) cudaFree(a.tc_part);
     if (a.s) cudaStreamDestroy(a.s);
   }
   for (auto& a : c->lanes)
@@ -1387,6 +1388,7 @@ int ensure_lanes(Ctx* c, int nl) {
   }
   l0.x32 = c->d_x32;
   l0.tcn_part = c->d_tcn_part;
+  l0.tc_part = c->d_tc_part;
   for (int j = 0; j < nl; ++j) {
     Ctx::Lane& a = c->lanes[j];
     if (!a.ev) SMR_CUDA(c, cudaEventCreateWithFlags(&a.ev, cudaEventDisableTiming));
@@ -1404,6 +1406,7 @@ int ensure_lanes(Ctx* c, int nl) {
     }
     if (ok && c->d_x32 && !a.x32)
       ok = cudaMalloc((void**)&a.x32, (size_t)c->p * 2 * c->npsi * sizeof(float2)) == cudaSuccess;
+    if (ok && c->d_tc_part && !a.tc_part) ok = cudaMalloc((void**)&a.tc_part, c->tc_part_bytes) == cudaSuccess;
     if (ok && c->d_tcn_part && !a.tcn_part) ok = cudaMalloc((void**)&a.tcn_part, c->tcn_part_bytes) == cudaSuccess;
     if (!ok) {
       cudaGetLastError();
@@ -1424,6 +1427,7 @@ static void use_lane(Ctx* c, int j) {
   }
   c->d_x32 = a.x32;
   c->d_tcn_part = a.tcn_part;
+  c->d_tc_part = a.tc_part;
 }
 
 // one lane where products use the shared per-particle spectra (several

@@ -47,6 +47,9 @@ constexpr int TC_BBYTES = TC_NP * TC_KC * 4;   // one spectrum chunk, one split:
 constexpr int TC_STAGE = 2 * TC_ABYTES + 2 * TC_BBYTES;
 constexpr int TC_NSTAGE = 3;
 constexpr int TC_PF = 3;                       // spectrum chunks of loads in flight per producer
+constexpr int TC_PW = 16;                      // producer warps of the receive kernel
+constexpr int TC_PT = 32 * TC_PW;              // producer threads
+constexpr int TC_PQ = TC_NP * 8 / TC_PT;       // 16-byte pieces of a chunk per producer
 constexpr size_t TC_SMEM = (size_t)TC_NSTAGE * TC_STAGE + 1024 + 2048;   // + alignment, barriers, ids
 constexpr uint32_t TC_SPIN = 1u << 24;         // default polling limit; also the drain bound
 constexpr int NEAR_NPH = 9;                    // near-product phases: self blocks + 8 lattice offsets
@@ -151,13 +154,18 @@ __device__ __forceinline__ void tmem_ld32(uint32_t t, float* v) {
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// Receive on the tensor cores: CTA = up to 128 particles of one shape, 256
-// threads.  K runs in chunks of 32 through a ring of TC_NSTAGE shared-memory
-// stages: the coefficient chunk arrives by one bulk copy issued a chunk ahead;
-// the spectrum chunk (128 rows x 128 bytes, read 4 rows per warp instruction)
-// is loaded two chunks ahead into registers, then split into TF32 hi / lo and
-// stored swizzled.  Thread 0 issues the 12 MMAs of a chunk (4 K steps x 3
-// products) and commits them to the stage's barrier.
+// Receive on the tensor cores: CTA = up to 128 particles of one shape, 16
+// producer warps and a control warp.  K runs in chunks of 32 through a ring of
+// TC_NSTAGE shared-memory stages: the coefficient chunk arrives by one bulk
+// copy issued a chunk ahead; the spectrum chunk (128 rows x 128 bytes, read 4
+// rows per warp instruction) is loaded three chunks ahead into registers, then
+// split into TF32 hi / lo and stored swizzled.  One thread issues the 12 MMAs of
+// a chunk (4 K steps x 3 products) and commits them to the stage's barrier.
+// Bound: the producers' instructions (a warp takes about 80 for each 512-byte
+// row group of a chunk, at the latency of a few warps per scheduler); 8
+// producer warps instead of 16 take 248 us on the 200x200 lens against 235.
+// CTA (tile, s) of a grid with several s takes chunks s nK / S .. (s + 1) nK / S
+// and writes its partial rows (no accumulation) to y + s ystride.
 // A = coefficient images [nK][hi | lo][128 rows][32] (swizzled), one per
 // tile (tshape); in0 = B rows [.][K8] (FP32), gathered by perm; y [.][M4]
 // (FP64), rows yperm.  Receive: A per shape, in0 the level-0 incoming
@@ -166,8 +174,8 @@ __device__ __forceinline__ void tmem_ld32(uint32_t t, float* v) {
 __device__ __forceinline__ void ld_chunk(const float* __restrict__ in0, int K8, const int* mus, int c, int tid,
                                          float4* r) {
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    int idx = tid + 256 * j, row = idx >> 3, q = idx & 7;
+  for (int j = 0; j < TC_PQ; ++j) {
+    int idx = tid + TC_PT * j, row = idx >> 3, q = idx & 7;
     int mu = mus[row], kk = c * TC_KC + 4 * q;
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
     if (mu >= 0) {
@@ -188,8 +196,8 @@ __device__ __forceinline__ void st_chunk(unsigned char* S, int tid, const float4
   float* Bh = reinterpret_cast<float*>(S + 2 * TC_ABYTES);
   float* Bl = reinterpret_cast<float*>(S + 2 * TC_ABYTES + TC_BBYTES);
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    int idx = tid + 256 * j, row = idx >> 3, q = idx & 7;
+  for (int j = 0; j < TC_PQ; ++j) {
+    int idx = tid + TC_PT * j, row = idx >> 3, q = idx & 7;
     float4 v = r[j];
     float4 h = make_float4(tf32r(v.x), tf32r(v.y), tf32r(v.z), tf32r(v.w));
     float4 l = make_float4(tf32r(v.x - h.x), tf32r(v.y - h.y), tf32r(v.z - h.z), tf32r(v.w - h.w));
@@ -200,16 +208,17 @@ __device__ __forceinline__ void st_chunk(unsigned char* S, int tid, const float4
 }
 
 template <typename YT>
-__global__ void __launch_bounds__(288, 1) k_receive_tc(int nK, int K8, int M4, const int* __restrict__ tshape,
+__global__ void __launch_bounds__(TC_PT + 32, 1) k_receive_tc(int nKall, int K8, int M4, const int* __restrict__ tshape,
                                                        const int* __restrict__ tstart,
                                                        const int* __restrict__ tcount,
                                                        const int* __restrict__ perm,
                                                        const int* __restrict__ yperm, const float* __restrict__ A,
-                                                       const float* __restrict__ in0, YT* __restrict__ y,
-                                                       int accumulate, uint32_t spin, int* __restrict__ err) {
+                                                       const float* __restrict__ in0, YT* __restrict__ y0,
+                                                       size_t ystride, int accumulate, uint32_t spin,
+                                                       int* __restrict__ err) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* sm = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  // barriers: fullA[NS] (bulk copy bytes), fullB[NS] (8 producer warps), done[NS] (MMA commit)
+  // barriers: fullA[NS] (bulk copy bytes), fullB[NS] (producer warps), done[NS] (MMA commit)
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm + TC_NSTAGE * TC_STAGE);
   uint32_t* slot = reinterpret_cast<uint32_t*>(bars + 3 * TC_NSTAGE);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(slot + 1);
@@ -222,12 +231,15 @@ __global__ void __launch_bounds__(288, 1) k_receive_tc(int nK, int K8, int M4, c
   auto fullA = [&](int st) { return saddr(bars + st); };
   auto fullB = [&](int st) { return saddr(bars + TC_NSTAGE + st); };
   auto done = [&](int st) { return saddr(bars + 2 * TC_NSTAGE + st); };
-  const float* As = A + (size_t)s * nK * (2 * 128 * TC_KC);
+  const int cbeg = (int)((long long)nKall * blockIdx.y / gridDim.y);
+  const int nK = (int)((long long)nKall * (blockIdx.y + 1) / gridDim.y) - cbeg;   // this CTA's chunks
+  YT* y = y0 + blockIdx.y * ystride;
+  const float* As = A + ((size_t)s * nKall + cbeg) * (2 * 128 * TC_KC);
   if (warp == 0) tmem_alloc(saddr(slot), TC_NP);
   if (tid == 0) {
     for (int i = 0; i < TC_NSTAGE; ++i) {
       mbar_init(fullA(i), 1);
-      mbar_init(fullB(i), 8);
+      mbar_init(fullB(i), TC_PW);
       mbar_init(done(i), 1);
     }
     *abort_flag = 0;
@@ -242,14 +254,14 @@ __global__ void __launch_bounds__(288, 1) k_receive_tc(int nK, int K8, int M4, c
   tc_after();
   const uint32_t tmem = *slot;
   bool bad = false;
-  if (warp < 8) {
+  if (warp < TC_PW) {
     // ---- producers: spectrum chunks, TC_PF chunks of loads in flight (the
     // loop is unrolled by TC_PF so that each register buffer is only read a
     // full round after its loads were issued)
-    float4 r[TC_PF][4];
+    float4 r[TC_PF][TC_PQ];
 #pragma unroll
     for (int b = 0; b < TC_PF; ++b)
-      if (b < nK) ld_chunk(in0, K8, mus, b, tid, r[b]);
+      if (b < nK) ld_chunk(in0, K8, mus, cbeg + b, tid, r[b]);
 #pragma unroll 1
     for (int cb = 0; cb < nK && !bad; cb += TC_PF) {
 #pragma unroll
@@ -271,7 +283,7 @@ __global__ void __launch_bounds__(288, 1) k_receive_tc(int nK, int K8, int M4, c
             __syncwarp();
             if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(fullB(st)) : "memory");
             // the next loads go out after the fence, so it does not wait for them
-            if (c + TC_PF < nK) ld_chunk(in0, K8, mus, c + TC_PF, tid, r[b]);
+            if (c + TC_PF < nK) ld_chunk(in0, K8, mus, cbeg + c + TC_PF, tid, r[b]);
           }
         }
       }
@@ -327,28 +339,29 @@ __global__ void __launch_bounds__(288, 1) k_receive_tc(int nK, int K8, int M4, c
     }
   }
   bad = __syncthreads_or(bad) != 0;
-  if (!bad && warp < 8) {
+  if (!bad && warp < TC_PW) {
     tc_after();
-    const int q4 = warp & 3, half = warp >> 2;         // lane quarter, column half
+    const int q4 = warp & 3, g = warp >> 2;            // lane quarter, 32 columns
     const int row = q4 * 32 + lane;                    // m'
-#pragma unroll 1
-    for (int g = half * 2; g < half * 2 + 2; ++g) {
-      if (g * 32 >= cnt) break;                        // uniform per warp
+    if (g * 32 < cnt) {                                // uniform per warp
       float v[32];
       tmem_ld32(tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(g * 32), v);
       if (row < M4) {
         if (accumulate) {
-          // the 32 columns are distinct y rows: all loads first, then stores
-          YT yo[32];
+          // the columns are distinct y rows: 16 loads in flight, then the stores
 #pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            int col = g * 32 + j;
-            yo[j] = col < cnt ? y[(size_t)ys[col] * M4 + row] : YT(0);
-          }
+          for (int j0 = 0; j0 < 32; j0 += 16) {
+            YT yo[16];
 #pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            int col = g * 32 + j;
-            if (col < cnt) y[(size_t)ys[col] * M4 + row] = yo[j] + (YT)v[j];
+            for (int j = 0; j < 16; ++j) {
+              int col = g * 32 + j0 + j;
+              yo[j] = col < cnt ? y[(size_t)ys[col] * M4 + row] : YT(0);
+            }
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              int col = g * 32 + j0 + j;
+              if (col < cnt) y[(size_t)ys[col] * M4 + row] = yo[j] + (YT)v[j0 + j];
+            }
           }
         } else {
 #pragma unroll
@@ -378,18 +391,20 @@ __global__ void __launch_bounds__(288, 1) k_receive_tc(int nK, int K8, int M4, c
 // [128 (t >> 1), 128 (t >> 1) + 128) of it, and reads only that current's
 // K chunks (half of K).  Consecutive tiles write the two halves of the same
 // output sectors.
-// CTA = up to 128 particles of one shape, 288 threads.  The 8 producer
-// warps load the tile's coefficients once (FP64 -> split TF32, swizzled,
-// resident for the whole CTA) and then drain the accumulators; one control
-// thread streams the coefficient images of the M tiles through a bulk-copy
-// ring and issues the MMAs into two alternating tensor-memory accumulators,
-// so the epilogue of one M tile overlaps the MMAs of the next.
+// CTA = up to 128 particles of one shape and a range of M tile pairs, 16 worker
+// warps and a control warp.  The workers load the tile's coefficients once
+// (split TF32, swizzled, resident for the whole CTA) and then drain the
+// accumulators; one control thread streams the coefficient images of the M
+// tiles through a bulk-copy ring and issues the MMAs into two alternating
+// tensor-memory accumulators, so the epilogue of one M tile overlaps the MMAs
+// of the next.  Bound: the epilogue's stores (187 us on the 200x200 lens with 8
+// workers, 161 with 16).
 constexpr int AG_NS = 3;                       // coefficient-image stages
 constexpr int AG_KCMAX = 4;                    // K chunks (K' <= 128)
 constexpr size_t AG_SMEM = (size_t)2 * AG_KCMAX * TC_BBYTES + (size_t)AG_NS * 2 * TC_ABYTES + 1024 + 1024;
 
 template <typename XT>
-__global__ void __launch_bounds__(288, 1) k_aggregate_tc(int nMT, int nKc, int K4, int npsi2,
+__global__ void __launch_bounds__(TC_PT + 32, 1) k_aggregate_tc(int nMTall, int nKc, int K4, int npsi2,
                                                          const int* __restrict__ tshape,
                                                          const int* __restrict__ tstart,
                                                          const int* __restrict__ tcount,
@@ -415,7 +430,10 @@ __global__ void __launch_bounds__(288, 1) k_aggregate_tc(int nMT, int nKc, int K
   auto accFull = [&](int b) { return saddr(bars + 2 * AG_NS + b); };
   auto accEmpty = [&](int b) { return saddr(bars + 2 * AG_NS + 2 + b); };
   const size_t tileA = (size_t)nKc * 2 * 128 * TC_KC;                   // floats per M tile image
-  const float* As = A + (size_t)s * nMT * tileA;
+  // this CTA's M tiles: whole pairs (the two currents of 128 rows)
+  const int tb = 2 * (int)((long long)(nMTall / 2) * blockIdx.y / gridDim.y);
+  const int nMT = 2 * (int)((long long)(nMTall / 2) * (blockIdx.y + 1) / gridDim.y) - tb;
+  const float* As = A + ((size_t)s * nMTall + tb) * tileA;
   if (warp == 0) tmem_alloc(saddr(slot), 2 * TC_NP);
   if (tid == 0) {
     for (int i = 0; i < AG_NS; ++i) {
@@ -424,7 +442,7 @@ __global__ void __launch_bounds__(288, 1) k_aggregate_tc(int nMT, int nKc, int K
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(accFull(b), 1);
-      mbar_init(accEmpty(b), 8);
+      mbar_init(accEmpty(b), TC_PW);
     }
     *abort_flag = 0;
     mbar_fence_init();
@@ -442,17 +460,17 @@ __global__ void __launch_bounds__(288, 1) k_aggregate_tc(int nMT, int nKc, int K
     bulk_g2s(ar0 + st * 2 * TC_ABYTES, As + t * tileA + (size_t)c * 2 * 128 * TC_KC, 2 * TC_ABYTES, aFull(st));
     ++ncopy;
   };
-  if (tid == 288 - 32) {
+  if (tid == TC_PT) {
     // control thread: first coefficient chunks while the producers load x
     for (int g = 0; g < AG_NS - 1 && g < total; ++g) copy_chunk(g);
   }
-  if (warp < 8) {
+  if (warp < TC_PW) {
     // the tile's coefficients: row = particle; item = 4 consecutive values of
     // one current's (mode, re/im) run, padded to nKc chunks of 32
     const int per_cur = nKc * 8;                     // items per current and row
     const int ngrp = 128 * 2 * per_cur;
     const int Kx = 2 * npsi2;
-    for (int g = tid; g < ngrp; g += 256) {
+    for (int g = tid; g < ngrp; g += TC_PT) {
       const int row = g / (2 * per_cur), rem = g - row * (2 * per_cur);
       const int cur = rem / per_cur, q4 = rem - cur * per_cur;
       const int mu = mus[row], kl = 4 * q4;
@@ -498,9 +516,9 @@ __global__ void __launch_bounds__(288, 1) k_aggregate_tc(int nMT, int nKc, int K
   }
   __syncthreads();
   bool bad = false;
-  if (warp < 8) {
+  if (warp < TC_PW) {
     // ---- epilogue warps: drain the accumulator of each M tile
-    const int q4 = warp & 3, half = warp >> 2;
+    const int q4 = warp & 3, g = warp >> 2;            // lane quarter, 32 columns
     for (int t = 0; t < nMT && !bad; ++t) {
       const int b = t & 1;
       bool ok = false;
@@ -512,11 +530,9 @@ __global__ void __launch_bounds__(288, 1) k_aggregate_tc(int nMT, int nKc, int K
         break;
       }
       tc_after();
-      const int rc = (t >> 1) * 128 + q4 * 32 + lane;   // (direction, component, re/im) of current t & 1
+      const int rc = ((t + tb) >> 1) * 128 + q4 * 32 + lane;   // (direction, component, re/im) of current t & 1
       const int oi = (rc >> 2) * 8 + (t & 1) * 4 + (rc & 3);
-#pragma unroll 1
-      for (int g = half * 2; g < half * 2 + 2; ++g) {
-        if (g * 32 >= cnt) break;                      // uniform per warp
+      if (g * 32 < cnt) {                              // uniform per warp
         float v[32];
         tmem_ld32(tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(b * TC_NP + g * 32), v);
         if (rc < K4) {
@@ -689,6 +705,18 @@ int build_tc(Ctx* c) {
   if (!agg.empty()) {
     if ((rc = upload(c, &c->d_tc_agg, agg))) return rc;
     c->tc_nMT = nMT;
+    // CTAs along the M tile pairs of a particle tile, the number that finishes
+    // first: a CTA costs its M tiles plus about three for its coefficients
+    // (1,600 particles in 18 tiles: one 32 us, eight 20.6 us)
+    const int pairs = nMT / 2, ntile = (int)tsh.size();
+    long long cost = -1;
+    for (int m = 1; m <= pairs; ++m) {
+      const long long t = ((long long)ntile * m + 151) / 152 * (2 * ((pairs + m - 1) / m) + 3);
+      if (cost < 0 || t < cost) {
+        cost = t;
+        c->tc_nmsplit = m;
+      }
+    }
     c->tc_nKc = nKc;
     c->tc_agg_ready = true;
   }
@@ -700,6 +728,24 @@ int build_tc(Ctx* c) {
   SMR_CUDA(c, cudaMemset(c->d_tc_err, 0, sizeof(int)));
   c->tc_nK = nK;
   c->tc_ntile = (int)tsh.size();
+  // Splits of the receive's K chunks: with few tiles most SMs would idle while
+  // each CTA walks through all 61 chunks.  The number that finishes first,
+  // a split costing about six chunks of start and epilogue and the sum of the
+  // partial rows about ten (1,600 particles in 18 tiles: one split 76 us, eight
+  // 24.5 us; 24x24 with six tiles 90 and 30.5 us).
+  c->tc_nsplit = 1;
+  long long cost = -1;
+  for (int S = 1; S <= std::max(1, std::min(32, nK / 2)); ++S) {
+    const long long t = ((long long)c->tc_ntile * S + 151) / 152 * ((nK + S - 1) / S + 6) + (S > 1 ? 10 : 0);
+    if (cost < 0 || t < cost) {
+      cost = t;
+      c->tc_nsplit = S;
+    }
+  }
+  if (c->d_tc_part) cudaFree(c->d_tc_part);
+  c->d_tc_part = nullptr;
+  c->tc_part_bytes = c->tc_nsplit > 1 ? (size_t)c->tc_nsplit * c->p * M4 * sizeof(float) : 0;
+  if (c->tc_part_bytes) SMR_CUDA(c, cudaMalloc((void**)&c->d_tc_part, c->tc_part_bytes));
   c->tc_ready = true;
   return SMR_OK;
 }
@@ -708,12 +754,49 @@ int build_tc(Ctx* c) {
 // box sum and broadcast around them apply the shifts
 bool tc_receive_ok(const Ctx* c, int R) { return c->tc_enable && c->tc_ready && R == 1; }
 
-int run_receive_tc(Ctx* c, const float2* in0, double2* y, bool accumulate, cudaStream_t st) {
-  cudaFuncSetAttribute(k_receive_tc<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM);
-  k_receive_tc<double><<<(unsigned)c->tc_ntile, 288, TC_SMEM, st>>>(
-      c->tc_nK, 8 * c->lev[0].K, 4 * c->npsi, c->d_tc_shape, c->d_tc_start, c->d_tc_count, c->d_tc_perm,
-      c->d_tc_perm, c->d_tc_rec, reinterpret_cast<const float*>(in0), reinterpret_cast<double*>(y), accumulate ? 1 : 0,
-      c->tc_spin, c->d_tc_err);
+// y (+)= the sum of S partial rows (FP32, in split order), added in FP64.
+// Thread = 4 consecutive values.
+__global__ void k_receive_sum(long long n4, int S, const float4* __restrict__ part, double2* __restrict__ y,
+                              int accumulate) {
+  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (t >= n4) return;
+  float4 a = part[t];
+  for (int s = 1; s < S; ++s) {
+    const float4 v = part[(size_t)s * n4 + t];
+    a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
+  }
+  double2 lo = make_double2(a.x, a.y), hi = make_double2(a.z, a.w);
+  if (accumulate) {
+    const double2 l = y[2 * t], h = y[2 * t + 1];
+    lo.x += l.x; lo.y += l.y; hi.x += h.x; hi.y += h.y;
+  }
+  y[2 * t] = lo;
+  y[2 * t + 1] = hi;
+}
+
+// ready: an event the first write of y waits for (null: none)
+int run_receive_tc(Ctx* c, const float2* in0, double2* y, bool accumulate, cudaEvent_t ready, cudaStream_t st) {
+  const int S = c->tc_nsplit, K8 = 8 * c->lev[0].K, M4 = 4 * c->npsi;
+  const float* B = reinterpret_cast<const float*>(in0);
+  if (S == 1) {
+    if (ready) SMR_CUDA(c, cudaStreamWaitEvent(st, ready, 0));
+    cudaFuncSetAttribute(k_receive_tc<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM);
+    k_receive_tc<double><<<(unsigned)c->tc_ntile, TC_PT + 32, TC_SMEM, st>>>(
+        c->tc_nK, K8, M4, c->d_tc_shape, c->d_tc_start, c->d_tc_count, c->d_tc_perm, c->d_tc_perm, c->d_tc_rec, B,
+        reinterpret_cast<double*>(y), 0, accumulate ? 1 : 0, c->tc_spin, c->d_tc_err);
+    SMR_LAUNCH(c);
+    return SMR_OK;
+  }
+  const size_t n = (size_t)c->p * M4;
+  cudaFuncSetAttribute(k_receive_tc<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM);
+  k_receive_tc<float><<<dim3(c->tc_ntile, S), TC_PT + 32, TC_SMEM, st>>>(
+      c->tc_nK, K8, M4, c->d_tc_shape, c->d_tc_start, c->d_tc_count, c->d_tc_perm, c->d_tc_perm, c->d_tc_rec, B,
+      c->d_tc_part, n, 0, c->tc_spin, c->d_tc_err);
+  SMR_LAUNCH(c);
+  if (ready) SMR_CUDA(c, cudaStreamWaitEvent(st, ready, 0));
+  k_receive_sum<<<(unsigned)((n / 4 + 255) / 256), 256, 0, st>>>((long long)(n / 4), S,
+                                                                reinterpret_cast<const float4*>(c->d_tc_part), y,
+                                                                accumulate ? 1 : 0);
   SMR_LAUNCH(c);
   return SMR_OK;
 }
@@ -726,13 +809,13 @@ bool tc_aggregate_ok(const Ctx* c, int R) {
 int run_aggregate_tc(Ctx* c, const double2* x, const float2* x32, float2* out0, cudaStream_t st) {
   if (x32) {
     cudaFuncSetAttribute(k_aggregate_tc<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AG_SMEM);
-    k_aggregate_tc<float><<<(unsigned)c->tc_ntile, 288, AG_SMEM, st>>>(
+    k_aggregate_tc<float><<<dim3(c->tc_ntile, c->tc_nmsplit), TC_PT + 32, AG_SMEM, st>>>(
         c->tc_nMT, c->tc_nKc, 4 * c->lev[0].K, 2 * c->npsi, c->d_tc_shape, c->d_tc_start, c->d_tc_count,
         c->d_tc_perm, c->d_tc_agg, reinterpret_cast<const float*>(x32), reinterpret_cast<float*>(out0),
         c->tc_spin, c->d_tc_err);
   } else {
     cudaFuncSetAttribute(k_aggregate_tc<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AG_SMEM);
-    k_aggregate_tc<double><<<(unsigned)c->tc_ntile, 288, AG_SMEM, st>>>(
+    k_aggregate_tc<double><<<dim3(c->tc_ntile, c->tc_nmsplit), TC_PT + 32, AG_SMEM, st>>>(
         c->tc_nMT, c->tc_nKc, 4 * c->lev[0].K, 2 * c->npsi, c->d_tc_shape, c->d_tc_start, c->d_tc_count,
         c->d_tc_perm, c->d_tc_agg, reinterpret_cast<const double*>(x), reinterpret_cast<float*>(out0),
         c->tc_spin, c->d_tc_err);
@@ -897,9 +980,9 @@ int run_near_tc(Ctx* c, double2* y, cudaStream_t st) {
   }
   cudaFuncSetAttribute(k_receive_tc<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM);
   pbeg(c, st, "near", -1, bytes, flops);
-  k_receive_tc<float><<<(unsigned)nt, 288, TC_SMEM, st>>>(
+  k_receive_tc<float><<<(unsigned)nt, TC_PT + 32, TC_SMEM, st>>>(
       c->tcn_nK, M4, M4, c->d_tcn_blk, c->d_tcn_start, c->d_tcn_count, c->d_tcn_nu, c->d_tcn_mu,
-      c->d_tcn_img, reinterpret_cast<const float*>(c->d_x32), c->d_tcn_part, 0, c->tc_spin, c->d_tc_err);
+      c->d_tcn_img, reinterpret_cast<const float*>(c->d_x32), c->d_tcn_part, 0, 0, c->tc_spin, c->d_tc_err);
   SMR_LAUNCH(c);
   pend(c, st);
   const long long nm = (long long)c->p * M4, nt4 = nm / 4;

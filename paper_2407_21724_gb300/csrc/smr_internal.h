@@ -275,6 +275,9 @@ struct Ctx {
   // tensor-core receive and aggregation (FP32 product, one right-hand side)
   bool tc_enable = true, tc_ready = false;
   int tc_nK = 0, tc_ntile = 0;
+  int tc_nsplit = 1;                      // splits of the receive's K chunks
+  float* d_tc_part = nullptr;             // [tc_nsplit][p][4 n_psi] partial rows (null for one split)
+  size_t tc_part_bytes = 0;
   float* d_tc_rec = nullptr;              // [S][nK][hi | lo][128][32] swizzled coefficient images
   int* d_tc_perm = nullptr;
   int* d_tc_shape = nullptr;
@@ -284,6 +287,7 @@ struct Ctx {
   uint32_t tc_spin = 1u << 24;            // polling limit of the pipeline waits (smr_set_wait_limit)
   bool tc_agg_ready = false;
   int tc_nMT = 0, tc_nKc = 0;
+  int tc_nmsplit = 1;                     // CTAs along a tile's M tile pairs
   float* d_tc_agg = nullptr;              // [S][M tiles][K chunks][hi | lo][128][32] aggregation images
   // tensor cores for aggregation / receive chosen by smr_autotune (-1: not tuned)
   int tune_tc_agg = -1, tune_tc_rec = -1, tune_tc_near = -1;
@@ -317,6 +321,7 @@ struct Ctx {
     std::vector<void*> out, in;           // per level FP32 spectra
     float2* x32 = nullptr;
     float* tcn_part = nullptr;
+    float* tc_part = nullptr;
     cudaStream_t s = nullptr;
     cudaEvent_t ev = nullptr;             // end of the lane's columns
   };
@@ -457,7 +462,7 @@ void free_side(Ctx* c);
 // tensor-core receive and aggregation (k_tc.cu)
 int build_tc(Ctx* c);
 bool tc_receive_ok(const Ctx* c, int R);
-int run_receive_tc(Ctx* c, const float2* in0, double2* y, bool accumulate, cudaStream_t st);
+int run_receive_tc(Ctx* c, const float2* in0, double2* y, bool accumulate, cudaEvent_t ready, cudaStream_t st);
 bool tc_aggregate_ok(const Ctx* c, int R);
 int build_near_tc(Ctx* c);
 bool tc_near_ok(const Ctx* c, int R);
