@@ -10,7 +10,12 @@
 // with particles of one shape as the N dimension.  FP32 accuracy comes from
 // split TF32: a = a_hi + a_lo with a_hi = tf32(a), a_lo = tf32(a - a_hi), and
 // A B ~ A_hi B_hi + A_hi B_lo + A_lo B_hi (three MMAs per K step, FP32
-// accumulation in tensor memory).
+// accumulation in tensor memory).  The accumulator truncates at every step, a
+// bias that grows with the length of the chain: the hi x hi products therefore
+// take turns on TC_NACC accumulators and the small cross terms have one of
+// their own, added in the epilogue (a 40 x 40 product's error against FP64:
+// one accumulator 2.9e-6, these four 1.9e-7, CUDA cores 2.2e-7; 0.7 % of the
+// lens product's time).
 //
 // The near-field product (block-sparse, Eq. 16 blocks) runs through the same
 // kernel: pairs (mu, nu) that share a block are one GEMM with the block's real
@@ -46,6 +51,7 @@ constexpr int TC_ABYTES = 128 * TC_KC * 4;     // one coefficient chunk, one spl
 constexpr int TC_BBYTES = TC_NP * TC_KC * 4;   // one spectrum chunk, one split: 16 KB
 constexpr int TC_STAGE = 2 * TC_ABYTES + 2 * TC_BBYTES;
 constexpr int TC_NSTAGE = 3;
+constexpr int TC_NACC = 3;                     // accumulators of the hi x hi products; one more for the cross terms
 constexpr int TC_PF = 3;                       // spectrum chunks of loads in flight per producer
 constexpr int TC_PW = 16;                      // producer warps of the receive kernel
 constexpr int TC_PT = 32 * TC_PW;              // producer threads
@@ -154,6 +160,19 @@ __device__ __forceinline__ void tmem_ld32(uint32_t t, float* v) {
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// the same columns of NA accumulators, TC_NP columns apart, added
+template <int NA>
+__device__ __forceinline__ void tmem_sum32(uint32_t t, float* v) {
+  tmem_ld32(t + (NA - 1) * TC_NP, v);              // the cross terms first: the smallest
+#pragma unroll
+  for (int a = 0; a < NA - 1; ++a) {
+    float w[32];
+    tmem_ld32(t + a * TC_NP, w);
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[i] += w[i];
+  }
+}
+
 // Receive on the tensor cores: CTA = up to 128 particles of one shape, 16
 // producer warps and a control warp.  K runs in chunks of 32 through a ring of
 // TC_NSTAGE shared-memory stages: the coefficient chunk arrives by one bulk
@@ -163,7 +182,7 @@ __device__ __forceinline__ void tmem_ld32(uint32_t t, float* v) {
 // a chunk (4 K steps x 3 products) and commits them to the stage's barrier.
 // Bound: the producers' instructions (a warp takes about 80 for each 512-byte
 // row group of a chunk, at the latency of a few warps per scheduler); 8
-// producer warps instead of 16 take 248 us on the 200x200 lens against 235.
+// producer warps instead of 16 take 248 us on the 200x200 lens against 243.
 // CTA (tile, s) of a grid with several s takes chunks s nK / S .. (s + 1) nK / S
 // and writes its partial rows (no accumulation) to y + s ystride.
 // A = coefficient images [nK][hi | lo][128 rows][32] (swizzled), one per
@@ -235,7 +254,7 @@ __global__ void __launch_bounds__(TC_PT + 32, 1) k_receive_tc(int nKall, int K8,
   const int nK = (int)((long long)nKall * (blockIdx.y + 1) / gridDim.y) - cbeg;   // this CTA's chunks
   YT* y = y0 + blockIdx.y * ystride;
   const float* As = A + ((size_t)s * nKall + cbeg) * (2 * 128 * TC_KC);
-  if (warp == 0) tmem_alloc(saddr(slot), TC_NP);
+  if (warp == 0) tmem_alloc(saddr(slot), (TC_NACC + 1) * TC_NP);
   if (tid == 0) {
     for (int i = 0; i < TC_NSTAGE; ++i) {
       mbar_init(fullA(i), 1);
@@ -313,9 +332,10 @@ __global__ void __launch_bounds__(TC_PT + 32, 1) k_receive_tc(int nKall, int K8,
         uint64_t ah = sdesc_sw128(Sa + 32 * k), al = sdesc_sw128(Sa + TC_ABYTES + 32 * k);
         uint64_t bh = sdesc_sw128(Sa + 2 * TC_ABYTES + 32 * k);
         uint64_t bl = sdesc_sw128(Sa + 2 * TC_ABYTES + TC_BBYTES + 32 * k);
-        mma_tf32(tmem, ah, bh, idesc, (c > 0 || k > 0) ? 1u : 0u);
-        mma_tf32(tmem, ah, bl, idesc, 1u);
-        mma_tf32(tmem, al, bh, idesc, 1u);
+        const int ks = c * (TC_KC / 8) + k;
+        mma_tf32(tmem + (uint32_t)(ks % TC_NACC * TC_NP), ah, bh, idesc, ks >= TC_NACC ? 1u : 0u);
+        mma_tf32(tmem + TC_NACC * TC_NP, ah, bl, idesc, ks > 0 ? 1u : 0u);
+        mma_tf32(tmem + TC_NACC * TC_NP, al, bh, idesc, 1u);
       }
       mma_commit(done(st));
       issued = c;
@@ -345,7 +365,7 @@ __global__ void __launch_bounds__(TC_PT + 32, 1) k_receive_tc(int nKall, int K8,
     const int row = q4 * 32 + lane;                    // m'
     if (g * 32 < cnt) {                                // uniform per warp
       float v[32];
-      tmem_ld32(tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(g * 32), v);
+      tmem_sum32<TC_NACC + 1>(tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(g * 32), v);
       if (row < M4) {
         if (accumulate) {
           // the columns are distinct y rows: 16 loads in flight, then the stores
@@ -379,7 +399,7 @@ __global__ void __launch_bounds__(TC_PT + 32, 1) k_receive_tc(int nKall, int K8,
   __syncthreads();
   if (warp == 0) {
     tc_after();
-    tmem_dealloc(tmem, TC_NP);
+    tmem_dealloc(tmem, (TC_NACC + 1) * TC_NP);
   }
 }
 
@@ -398,7 +418,7 @@ __global__ void __launch_bounds__(TC_PT + 32, 1) k_receive_tc(int nKall, int K8,
 // tiles through a bulk-copy ring and issues the MMAs into two alternating
 // tensor-memory accumulators, so the epilogue of one M tile overlaps the MMAs
 // of the next.  Bound: the epilogue's stores (187 us on the 200x200 lens with 8
-// workers, 161 with 16).
+// workers, 167 with 16).
 constexpr int AG_NS = 3;                       // coefficient-image stages
 constexpr int AG_KCMAX = 4;                    // K chunks (K' <= 128)
 constexpr size_t AG_SMEM = (size_t)2 * AG_KCMAX * TC_BBYTES + (size_t)AG_NS * 2 * TC_ABYTES + 1024 + 1024;
@@ -434,7 +454,7 @@ __global__ void __launch_bounds__(TC_PT + 32, 1) k_aggregate_tc(int nMTall, int 
   const int tb = 2 * (int)((long long)(nMTall / 2) * blockIdx.y / gridDim.y);
   const int nMT = 2 * (int)((long long)(nMTall / 2) * (blockIdx.y + 1) / gridDim.y) - tb;
   const float* As = A + ((size_t)s * nMTall + tb) * tileA;
-  if (warp == 0) tmem_alloc(saddr(slot), 2 * TC_NP);
+  if (warp == 0) tmem_alloc(saddr(slot), 4 * TC_NP);
   if (tid == 0) {
     for (int i = 0; i < AG_NS; ++i) {
       mbar_init(aFull(i), 1);
@@ -534,7 +554,7 @@ __global__ void __launch_bounds__(TC_PT + 32, 1) k_aggregate_tc(int nMTall, int 
       const int oi = (rc >> 2) * 8 + (t & 1) * 4 + (rc & 3);
       if (g * 32 < cnt) {                              // uniform per warp
         float v[32];
-        tmem_ld32(tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(b * TC_NP + g * 32), v);
+        tmem_sum32<2>(tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(b * 2 * TC_NP + g * 32), v);
         if (rc < K4) {
 #pragma unroll
           for (int j = 0; j < 32; ++j) {
@@ -558,7 +578,7 @@ __global__ void __launch_bounds__(TC_PT + 32, 1) k_aggregate_tc(int nMTall, int 
       const int b = t & 1;
       if (t >= 2 && !mbar_wait_or_abort(accEmpty(b), ((t >> 1) - 1) & 1, spin, abort_flag)) { bad = true; break; }
       tc_after();
-      const uint32_t d = tmem + (uint32_t)(b * TC_NP);
+      const uint32_t d = tmem + (uint32_t)(b * 2 * TC_NP);
       for (int c = 0; c < nKc; ++c) {
         const int st = g % AG_NS;
         if (!mbar_wait_or_abort(aFull(st), (g / AG_NS) & 1, spin, abort_flag)) { bad = true; break; }
@@ -570,8 +590,8 @@ __global__ void __launch_bounds__(TC_PT + 32, 1) k_aggregate_tc(int nMTall, int 
           const int cb = (t & 1) * nKc + c;            // this current's K chunk of the coefficients
           uint64_t bh = sdesc_sw128(bh0 + cb * TC_BBYTES + 32 * k), bl = sdesc_sw128(bl0 + cb * TC_BBYTES + 32 * k);
           mma_tf32(d, ah, bh, idesc, (c > 0 || k > 0) ? 1u : 0u);
-          mma_tf32(d, ah, bl, idesc, 1u);
-          mma_tf32(d, al, bh, idesc, 1u);
+          mma_tf32(d + TC_NP, ah, bl, idesc, (c > 0 || k > 0) ? 1u : 0u);
+          mma_tf32(d + TC_NP, al, bh, idesc, 1u);
         }
         mma_commit(aDone(st));
         last_bar = aDone(st);
@@ -605,7 +625,7 @@ __global__ void __launch_bounds__(TC_PT + 32, 1) k_aggregate_tc(int nMTall, int 
   __syncthreads();
   if (warp == 0) {
     tc_after();
-    tmem_dealloc(tmem, 2 * TC_NP);
+    tmem_dealloc(tmem, 4 * TC_NP);
   }
 }
 
