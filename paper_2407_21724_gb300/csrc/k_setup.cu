@@ -1,7 +1,6 @@
 // FP64 setup kernels: mode sampling, k-space patterns (Eq. 26), translation
-// tables (Eq. 23), near blocks (Eq. 16), right-hand sides (Eqs. 18-19), far
-// and near fields.  Everything here runs once per scene (or per output
-// request) in FP64; the hot path reads FP64 or FP32 copies of these tables.
+// tables (Eq. 23), near blocks (Eq. 16), right-hand sides (Eqs. 18-19).
+// Everything here runs once per scene (or per right-hand side) in FP64; the hot path reads FP64 or FP32 copies of these tables.
 #include <cmath>
 #include <cstring>
 #include <map>
@@ -607,285 +606,6 @@ int launch_rhs_scratch(Ctx* c, int R, const double* d_khat, const double2* d_pol
   long long t2 = (long long)c->p * 2 * c->npsi * R;
   k_rhs_scatter<<<(unsigned)((t2 + 255) / 256), 256, 0, st>>>(c->p, c->npsi, R, c->d_sid, c->d_centres,
                                                              d_khat, Sv, c->k, b);
-  SMR_LAUNCH(c);
-  return SMR_OK;
-}
-
-// ------------------------------------------------------------------ far field
-// Rv[s][n][d][3] = sum_q w psi_n(q) exp(+j k rhat_d . r_q)   (radiation vectors)
-__global__ void k_radvec(int S, int npsi, int Q, int nd, const double* __restrict__ modes,
-                         const double* __restrict__ rq, const double* __restrict__ dirs, double kw,
-                         double2* __restrict__ Rv) {
-  long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t >= (long long)S * npsi * nd) return;
-  int d = (int)(t % nd), n = (int)((t / nd) % npsi), s = (int)(t / ((long long)nd * npsi));
-  const double* u = dirs + 3 * d;
-  const double* M = modes + ((size_t)s * npsi + n) * Q * 4;
-  const double* Rr = rq + (size_t)s * Q * 4;
-  double2 a[3] = {make_double2(0, 0), make_double2(0, 0), make_double2(0, 0)};
-  for (int q = 0; q < Q; ++q) {
-    const double* p = Rr + 4 * q;
-    double sn, cs;
-    sincos(kw * (u[0] * p[0] + u[1] * p[1] + u[2] * p[2]), &sn, &cs);
-    for (int i = 0; i < 3; ++i) {
-      double v = p[3] * M[4 * q + i];
-      a[i].x += v * cs;
-      a[i].y += v * sn;
-    }
-  }
-  for (int i = 0; i < 3; ++i) Rv[t * 3 + i] = a[i];
-}
-
-// F[d][3][r]: CTA per (d, r); threads stride over particles; block reduction.
-__global__ void k_farfield(int p, int npsi, int nd, int R, const int* __restrict__ sid,
-                           const double* __restrict__ cen, const double* __restrict__ dirs,
-                           const double2* __restrict__ Rv, const double2* __restrict__ x,
-                           double kw, double zeta, double2* __restrict__ F) {
-  int d = blockIdx.x / R, r = blockIdx.x % R;
-  const double* u = dirs + 3 * d;
-  double2 J[3] = {make_double2(0, 0), make_double2(0, 0), make_double2(0, 0)};
-  double2 M[3] = {make_double2(0, 0), make_double2(0, 0), make_double2(0, 0)};
-  for (int mu = threadIdx.x; mu < p; mu += blockDim.x) {
-    const double* cc = cen + 3 * mu;
-    double sn, cs;
-    sincos(kw * (u[0] * cc[0] + u[1] * cc[1] + u[2] * cc[2]), &sn, &cs);
-    int s = sid[mu];
-    double2 je[3] = {make_double2(0, 0), make_double2(0, 0), make_double2(0, 0)};
-    double2 jm[3] = {make_double2(0, 0), make_double2(0, 0), make_double2(0, 0)};
-    for (int n = 0; n < npsi; ++n) {
-      double2 ae = x[((size_t)mu * 2 * npsi + n) * R + r];
-      double2 am = x[((size_t)mu * 2 * npsi + npsi + n) * R + r];
-      const double2* rv = Rv + (((size_t)s * npsi + n) * nd + d) * 3;
-      for (int i = 0; i < 3; ++i) {
-        je[i].x += ae.x * rv[i].x - ae.y * rv[i].y; je[i].y += ae.x * rv[i].y + ae.y * rv[i].x;
-        jm[i].x += am.x * rv[i].x - am.y * rv[i].y; jm[i].y += am.x * rv[i].y + am.y * rv[i].x;
-      }
-    }
-    for (int i = 0; i < 3; ++i) {
-      J[i].x += je[i].x * cs - je[i].y * sn; J[i].y += je[i].x * sn + je[i].y * cs;
-      M[i].x += jm[i].x * cs - jm[i].y * sn; M[i].y += jm[i].x * sn + jm[i].y * cs;
-    }
-  }
-  __shared__ double red[12][256];
-  for (int i = 0; i < 3; ++i) {
-    red[2 * i][threadIdx.x] = J[i].x; red[2 * i + 1][threadIdx.x] = J[i].y;
-    red[6 + 2 * i][threadIdx.x] = M[i].x; red[7 + 2 * i][threadIdx.x] = M[i].y;
-  }
-  __syncthreads();
-  for (int h = blockDim.x / 2; h > 0; h >>= 1) {
-    if ((int)threadIdx.x < h)
-      for (int q = 0; q < 12; ++q) red[q][threadIdx.x] += red[q][threadIdx.x + h];
-    __syncthreads();
-  }
-  if (threadIdx.x != 0) return;
-  double2 Jt[3], Mt[3];
-  for (int i = 0; i < 3; ++i) {
-    Jt[i] = make_double2(red[2 * i][0], red[2 * i + 1][0]);
-    Mt[i] = make_double2(red[6 + 2 * i][0], red[7 + 2 * i][0]);
-  }
-  double2 rj = make_double2(u[0] * Jt[0].x + u[1] * Jt[1].x + u[2] * Jt[2].x,
-                            u[0] * Jt[0].y + u[1] * Jt[1].y + u[2] * Jt[2].y);
-  double2 rxm[3];
-  rxm[0] = make_double2(u[1] * Mt[2].x - u[2] * Mt[1].x, u[1] * Mt[2].y - u[2] * Mt[1].y);
-  rxm[1] = make_double2(u[2] * Mt[0].x - u[0] * Mt[2].x, u[2] * Mt[0].y - u[0] * Mt[2].y);
-  rxm[2] = make_double2(u[0] * Mt[1].x - u[1] * Mt[0].x, u[0] * Mt[1].y - u[1] * Mt[0].y);
-  double pre = kw / (4.0 * PI);  // F = j pre [ zeta (J - u (u.J)) - u x M ]
-  for (int i = 0; i < 3; ++i) {
-    double vx = zeta * (Jt[i].x - u[i] * rj.x) - rxm[i].x;
-    double vy = zeta * (Jt[i].y - u[i] * rj.y) - rxm[i].y;
-    F[((size_t)d * 3 + i) * R + r] = make_double2(-pre * vy, pre * vx);
-  }
-}
-
-int launch_far_field(Ctx* c, int R, const double2* x, int nd, const double* d_dirs, double2* F,
-                     cudaStream_t st) {
-  double2* Rv = nullptr;
-  SMR_CUDA(c, cudaMallocAsync((void**)&Rv, (size_t)c->S * c->npsi * nd * 3 * sizeof(double2), st));
-  long long t1 = (long long)c->S * c->npsi * nd;
-  k_radvec<<<(unsigned)((t1 + 127) / 128), 128, 0, st>>>(c->S, c->npsi, c->Q, nd, c->d_modes, c->d_rq,
-                                                        d_dirs, c->k, Rv);
-  SMR_LAUNCH(c);
-  k_farfield<<<(unsigned)(nd * R), 256, 0, st>>>(c->p, c->npsi, nd, R, c->d_sid, c->d_centres, d_dirs,
-                                                 Rv, x, c->k, c->zeta, F);
-  SMR_LAUNCH(c);
-  SMR_CUDA(c, cudaFreeAsync(Rv, st));
-  return SMR_OK;
-}
-
-// Cross sections from far-field amplitudes F[nd][3][R].  CTA per column r:
-// the first n_sca directions carry quadrature weights W (scattered power
-// over the sphere, Sec. V); direction n_sca + r is column r's own incident
-// direction, where the optical theorem gives the extinction.  cs[2r] = C_sca,
-// cs[2r + 1] = C_ext.
-__global__ void k_cross_sections(int n_sca, int R, const double2* __restrict__ F,
-                                 const double* __restrict__ W, const double2* __restrict__ pol,
-                                 double kw, double* __restrict__ cs) {
-  __shared__ double red[256];
-  int r = blockIdx.x;
-  double acc = 0;
-  for (int d = threadIdx.x; d < n_sca; d += blockDim.x) {
-    double e = 0;
-    for (int i = 0; i < 3; ++i) {
-      double2 f = F[((size_t)d * 3 + i) * R + r];
-      e += f.x * f.x + f.y * f.y;
-    }
-    acc += W[d] * e;
-  }
-  red[threadIdx.x] = acc;
-  __syncthreads();
-  for (int h = blockDim.x / 2; h > 0; h >>= 1) {
-    if (threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    // Im(conj(e) . F) / |e|^2 at the forward direction.
-    double im = 0, nn = 0;
-    for (int i = 0; i < 3; ++i) {
-      double2 e = pol[(size_t)r * 3 + i];
-      double2 f = F[((size_t)(n_sca + r) * 3 + i) * R + r];
-      im += e.x * f.y - e.y * f.x;
-      nn += e.x * e.x + e.y * e.y;
-    }
-    cs[2 * r] = red[0];
-    cs[2 * r + 1] = -(4.0 * M_PI / kw) * im / nn;
-  }
-}
-
-int launch_cross_sections(Ctx* c, int R, const double2* x, int n_sca, const double* d_dirs,
-                          const double* d_w, const double2* d_pol, double* d_cs, cudaStream_t st) {
-  int nd = n_sca + R;
-  double2* F = nullptr;
-  SMR_CUDA(c, cudaMallocAsync((void**)&F, (size_t)nd * 3 * R * sizeof(double2), st));
-  int rc = launch_far_field(c, R, x, nd, d_dirs, F, st);
-  if (rc == SMR_OK) {
-    k_cross_sections<<<R, 256, 0, st>>>(n_sca, R, F, d_w, d_pol, c->k, d_cs);
-    SMR_LAUNCH(c);
-  }
-  SMR_CUDA(c, cudaFreeAsync(F, st));
-  return rc;
-}
-
-// ------------------------------------------------------------------ near field
-// CTA per particle mu (and right-hand side r): currents at the quadrature
-// points staged in shared memory; threads stride over field points and add
-// their particle's contribution with atomics.
-// Field points in groups of blockDim (one point per thread, blockIdx.z),
-// one right-hand side per blockIdx.y; the blocks of a group stride over the
-// units (particle, chunk of at most QC surface points): each unit's currents
-// are staged in shared memory and every thread adds their field at its point
-// in registers.  One atomic add per block and field component at the end.
-__global__ void k_nearfield(int p, int npsi, int Q, int QC, int npt, int R, const int* __restrict__ sid,
-                            const double* __restrict__ cen, const double* __restrict__ modes,
-                            const double* __restrict__ rq, const double2* __restrict__ x,
-                            const double* __restrict__ pts, double kw, double zeta,
-                            double* __restrict__ EH) {
-  extern __shared__ double sm[];   // [QC][8 complex] J xyz, divJ, M xyz, divM  + [QC][4] point
-  const int nch = (Q + QC - 1) / QC;
-  const int r = blockIdx.y;
-  const int ip = blockIdx.z * blockDim.x + threadIdx.x;
-  const bool act = ip < npt;
-  double2* cur = reinterpret_cast<double2*>(sm);
-  double* pq = sm + (size_t)QC * 16;
-  double P[3] = {0, 0, 0};
-  if (act)
-    for (int d = 0; d < 3; ++d) P[d] = pts[3 * ip + d];
-  double2 E[3], H[3];
-  for (int i = 0; i < 3; ++i) { E[i] = make_double2(0, 0); H[i] = make_double2(0, 0); }
-  for (long long u = blockIdx.x; u < (long long)p * nch; u += gridDim.x) {
-    const int mu = (int)(u / nch), ch = (int)(u % nch);
-    const int s = sid[mu];
-    const int q0 = ch * QC, nq = min(QC, Q - q0);
-    const double* Ms = modes + (size_t)s * npsi * Q * 4 + (size_t)q0 * 4;
-    for (int q = threadIdx.x; q < nq; q += blockDim.x) {
-      double2 a[8];
-      for (int i = 0; i < 8; ++i) a[i] = make_double2(0, 0);
-      for (int n = 0; n < npsi; ++n) {
-        double2 ae = x[((size_t)mu * 2 * npsi + n) * R + r];
-        double2 am = x[((size_t)mu * 2 * npsi + npsi + n) * R + r];
-        const double* m = Ms + ((size_t)n * Q + q) * 4;
-        for (int i = 0; i < 4; ++i) {
-          a[i].x += ae.x * m[i]; a[i].y += ae.y * m[i];
-          a[4 + i].x += am.x * m[i]; a[4 + i].y += am.y * m[i];
-        }
-      }
-      for (int i = 0; i < 8; ++i) cur[(size_t)q * 8 + i] = a[i];
-      const double* rr = rq + ((size_t)s * Q + q0 + q) * 4;
-      pq[4 * q] = rr[0] + cen[3 * mu];
-      pq[4 * q + 1] = rr[1] + cen[3 * mu + 1];
-      pq[4 * q + 2] = rr[2] + cen[3 * mu + 2];
-      pq[4 * q + 3] = rr[3];
-    }
-    __syncthreads();
-    if (act) {
-      for (int q = 0; q < nq; ++q) {
-        double d[3] = {P[0] - pq[4 * q], P[1] - pq[4 * q + 1], P[2] - pq[4 * q + 2]};
-        double R2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-        double Rr = sqrt(R2), iR = 1.0 / Rr;
-        double sn, cs;
-        sincos(-kw * Rr, &sn, &cs);
-        double w = pq[4 * q + 3];
-        double g = w * iR / (4.0 * PI);
-        double2 G = make_double2(g * cs, g * sn);
-        // grad_r g = -(d) (1 + jkR) e / (4 pi R^3)   (times w)
-        double g3 = g * iR * iR;
-        double2 D = make_double2(-g3 * (cs - kw * Rr * sn), -g3 * (sn + kw * Rr * cs));
-        const double2* c8 = cur + (size_t)q * 8;
-        for (int which = 0; which < 2; ++which) {
-          const double2* X = c8 + 4 * which;
-          // L{X} = -jk G X - (j/k) grad g (div X)
-          // K{X} = grad g x X
-          double2 Lv[3], Kv[3];
-          double2 DX = make_double2(D.x * X[3].x - D.y * X[3].y, D.x * X[3].y + D.y * X[3].x);
-          for (int i = 0; i < 3; ++i) {
-            double2 GX = make_double2(G.x * X[i].x - G.y * X[i].y, G.x * X[i].y + G.y * X[i].x);
-            // -jk GX - (j/k) d_i DX
-            Lv[i] = make_double2(kw * GX.y + d[i] * DX.y / kw, -kw * GX.x - d[i] * DX.x / kw);
-          }
-          // (d x X) * D
-          double2 cxX[3];
-          cxX[0] = make_double2(d[1] * X[2].x - d[2] * X[1].x, d[1] * X[2].y - d[2] * X[1].y);
-          cxX[1] = make_double2(d[2] * X[0].x - d[0] * X[2].x, d[2] * X[0].y - d[0] * X[2].y);
-          cxX[2] = make_double2(d[0] * X[1].x - d[1] * X[0].x, d[0] * X[1].y - d[1] * X[0].y);
-          for (int i = 0; i < 3; ++i)
-            Kv[i] = make_double2(D.x * cxX[i].x - D.y * cxX[i].y, D.x * cxX[i].y + D.y * cxX[i].x);
-          if (which == 0) {  // J: E += -zeta L{J}, H += -K{J}
-            for (int i = 0; i < 3; ++i) {
-              E[i].x -= zeta * Lv[i].x; E[i].y -= zeta * Lv[i].y;
-              H[i].x -= Kv[i].x; H[i].y -= Kv[i].y;
-            }
-          } else {           // M: E += K{M}, H += -L{M}/zeta
-            for (int i = 0; i < 3; ++i) {
-              E[i].x += Kv[i].x; E[i].y += Kv[i].y;
-              H[i].x -= Lv[i].x / zeta; H[i].y -= Lv[i].y / zeta;
-            }
-          }
-        }
-      }
-    }
-    __syncthreads();
-  }
-  if (act) {
-    double* o = EH + (((size_t)ip * 6) * R + r) * 2;
-    for (int i = 0; i < 3; ++i) {
-      atomicAdd(o + ((size_t)i * R) * 2, E[i].x);
-      atomicAdd(o + ((size_t)i * R) * 2 + 1, E[i].y);
-      atomicAdd(o + ((size_t)(3 + i) * R) * 2, H[i].x);
-      atomicAdd(o + ((size_t)(3 + i) * R) * 2 + 1, H[i].y);
-    }
-  }
-}
-
-int launch_near_field(Ctx* c, int R, const double2* x, int npt, const double* d_pts, double2* EH,
-                      cudaStream_t st) {
-  SMR_CUDA(c, cudaMemsetAsync(EH, 0, (size_t)npt * 6 * R * sizeof(double2), st));
-  const int QC = std::min(c->Q, 1024);
-  const int nch = (c->Q + QC - 1) / QC;
-  size_t sm = (size_t)QC * (16 + 4) * sizeof(double);
-  SMR_CUDA(c, cudaFuncSetAttribute(k_nearfield, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-  const long long units = (long long)c->p * nch;
-  dim3 grid((unsigned)std::min<long long>(units, 1216), (unsigned)R, (unsigned)((npt + 255) / 256));
-  k_nearfield<<<grid, 256, sm, st>>>(c->p, c->npsi, c->Q, QC, npt, R, c->d_sid, c->d_centres, c->d_modes,
-                                     c->d_rq, x, d_pts, c->k, c->zeta, (double*)EH);
   SMR_LAUNCH(c);
   return SMR_OK;
 }

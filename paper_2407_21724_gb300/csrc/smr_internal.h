@@ -415,6 +415,8 @@ int launch_rhs(Ctx* c, int R, const double* d_khat, const double2* d_pol, double
 int launch_rhs_arrays(Ctx* c, const double* d_khat, const double2* d_pol, double2* b, cudaStream_t st);
 int launch_rhs_scratch(Ctx* c, int R, const double* d_khat, const double2* d_pol, double2* Sv,
                        double2* b, cudaStream_t st);
+
+// ------------------------------------------------------------------ fields (k_fields.cu)
 int launch_far_field(Ctx* c, int R, const double2* x, int nd, const double* d_dirs,
                      double2* F, cudaStream_t st);
 int launch_cross_sections(Ctx* c, int R, const double2* x, int n_sca, const double* d_dirs,
