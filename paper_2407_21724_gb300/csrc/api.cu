@@ -35,7 +35,7 @@ void free_scene(Ctx* c) {
     dfree(L.d_T64); dfree(L.d_T32); dfree(L.d_parent); dfree(L.d_quad); dfree(L.d_ch_ptr);
     dfree(L.d_ch_idx); dfree(L.d_ch_quad); dfree(L.d_ch4); dfree(L.d_th_pk); dfree(L.d_th_ws64); dfree(L.d_th_ws32);
     dfree(L.d_ph_src); dfree(L.d_ph_w64); dfree(L.d_ph_w32); dfree(L.d_shift64); dfree(L.d_shiftp64);
-    dfree(L.d_shiftp32); dfree(L.d_shiftw32); dfree(L.d_mi_vlast); dfree(L.d_ma_ptr); dfree(L.d_ma_ent);
+    dfree(L.d_shiftp32); dfree(L.d_mi_vlast); dfree(L.d_ma_ptr); dfree(L.d_ma_ent);
     dfree(L.d_ma_w64); dfree(L.d_ma_w32); dfree(L.d_ma_pst); dfree(L.d_ma_pw64); dfree(L.d_ma_pw32);
     dfree(L.d_ant_lo); dfree(L.d_ant_pjp); dfree(L.d_ant_pw64); dfree(L.d_ant_ttp); dfree(L.d_ant_tw64);
     dfree(L.d_wthp64); dfree(L.d_boxmap); dfree(L.d_offid); dfree(L.d_tiles); dfree(L.d_tiles8); dfree(L.d_tile_tab);
@@ -47,7 +47,8 @@ void free_scene(Ctx* c) {
     L.d_out = L.d_in = nullptr;
   }
   c->lev.clear();
-  dfree(c->d_modes); dfree(c->d_rq); dfree(c->d_P64); dfree(c->d_P32); dfree(c->d_sid);
+  dfree(c->d_modes); dfree(c->d_rq); dfree(c->d_P64); dfree(c->d_Pd64); dfree(c->d_Pd32);
+  dfree(c->d_Pm64); dfree(c->d_Pm32); dfree(c->d_xs[0]); dfree(c->d_xs[1]); dfree(c->d_sid);
   dfree(c->d_centres); dfree(c->d_dshift); dfree(c->d_nr_ptr); dfree(c->d_nr_col); dfree(c->d_nr_blk);
   dfree(c->d_cell_of); dfree(c->d_cell_ptr); dfree(c->d_cell_idx);
   for (int q = 0; q < 2; ++q) {
@@ -355,14 +356,7 @@ int build_interp(Ctx* c, Level& C, const Level& P) {
       shp[(size_t)2 * k + q] = sh[(size_t)q * P.K + k];
       shp32[(size_t)2 * k + q] = make_float2((float)shp[(size_t)2 * k + q].x, (float)shp[(size_t)2 * k + q].y);
     }
-  std::vector<float2> shw32;
-  for (const float2& v : shp32) {
-    shw32.push_back(make_float2(v.x, v.x));
-    shw32.push_back(make_float2(v.y, v.y));
-  }
-  if ((rc = upload(c, &C.d_shiftp64, shp)) || (rc = upload(c, &C.d_shiftp32, shp32)) ||
-      (rc = upload(c, &C.d_shiftw32, shw32)))
-    return rc;
+  if ((rc = upload(c, &C.d_shiftp64, shp)) || (rc = upload(c, &C.d_shiftp32, shp32))) return rc;
   if ((rc = upload(c, &C.d_shift64, sh))) return rc;
   return SMR_OK;
 }
@@ -1117,7 +1111,7 @@ int smr_info(smr_ctx* h, smr_info_t* info) {
     info->K[s] = L.K;
     info->n_box[s] = L.nbox;
     info->n_il[s] = (int)L.il_src.size();
-    bytes += 2.0 * L.nbox * L.K * 4 * 16 + (double)L.off_dx.size() * L.K * 24;
+    bytes += 2.0 * L.nbox * L.K * NF * 16 + (double)L.off_dx.size() * L.K * 24;
   }
   info->n_near_pairs = (long long)c->nr_col.size();
   info->n_near_blocks = c->nblk;
@@ -1775,16 +1769,7 @@ int smr_copy_level(smr_ctx* h, int level, int kind, double* out, size_t n_double
   Level& L = c->lev[level];
   size_t elems = (size_t)L.nbox * L.K * 4 * c->spec_R;
   if (n_doubles < 2 * elems) return fail(c, SMR_E_INVALID_ARG, "output buffer too small");
-  const void* src = kind == 0 ? L.d_out : L.d_in;
-  cudaDeviceSynchronize();
-  if (c->spec_prec == SMR_PREC_FP64) {
-    SMR_CUDA(c, cudaMemcpy(out, src, elems * sizeof(double2), cudaMemcpyDeviceToHost));
-  } else {
-    std::vector<float2> t(elems);
-    SMR_CUDA(c, cudaMemcpy(t.data(), src, elems * sizeof(float2), cudaMemcpyDeviceToHost));
-    for (size_t i = 0; i < elems; ++i) { out[2 * i] = t[i].x; out[2 * i + 1] = t[i].y; }
-  }
-  return SMR_OK;
+  return copy_fields(c, level, kind, out);
 }
 
 }  // extern "C"

@@ -4,7 +4,7 @@
 //
 // Both stencils are separable, real and narrow: 4 theta rows times 4 phi
 // columns.  A thread owns one phi column of its output grid (one 16-byte part
-// of it: part h of the NT parts a direction's 4 R complex fields make) for
+// of it: part h of the NT parts a direction's NF R complex fields make) for
 // the four children of a parent box, and marches along theta with the 4-row
 // stencil window in registers, so every theta tap after the first is a
 // register read.  All lanes are at the same theta position, which makes the
@@ -22,14 +22,17 @@
 //
 // Bound: instruction issue and shared-memory reads, both near half of their
 // peak with 12 to 14 warps per SM (the windows take the registers).  On the
-// 200x200 lens in FP32 (algorithmic bytes 517 and 827 MB at level 0, of
-// measured 6.68 TB/s): interpolation level 0 262 -> 168 us, six levels 955 ->
-// 597 us; anterpolation level 0 356 -> 235 us, six levels 1369 -> 808 us,
-// against kernels that kept the phi-pass rows in shared memory (a barrier and
-// a round trip per row, 7 gathered taps per output).  A thread per child pair
-// instead of four children (half the registers, twice the warps) measured 696
-// and 1021 us; CTAs that run on over several boxes 873 and 1062 us, the ring's
-// bookkeeping costing more than its restarts.
+// 200x200 lens in FP32 (algorithmic bytes 259 and 414 MB at level 0, of
+// measured 6.68 TB/s): interpolation level 0 96 us, six levels 352 us;
+// anterpolation level 0 121 us, six levels 407 us.  With four fields a direction
+// these took 168, 597, 235 and 808 us, and kernels that kept the phi-pass rows in
+// shared memory (a barrier and a round trip per row, 7 gathered taps per output)
+// 262, 955, 356 and 1369 us.  Measured with four fields: a thread per child pair
+// instead of four children (half the registers, twice the warps) 696 and 1021
+// us; CTAs that run on over several boxes 873 and 1062 us, the ring's
+// bookkeeping costing more than its restarts.  The adjoint's shifts, read by every
+// tap, stay packed as they lie in memory (Mp<float>::G): staged as the weight pairs
+// the packed multiply-add takes for two fields they took 649 us.
 #include <algorithm>
 
 #include "smr_internal.h"
@@ -58,11 +61,41 @@ template <> struct Mp<float> {
   typedef float2 W;                            // a weight as the pair the packed multiply-add takes
   typedef float2 C;                            // a complex value
   typedef float4 S;                            // a direction's two shifts
-  struct __align__(16) W4 { float2 w[4]; };    // the same as weights
-  static __device__ __forceinline__ H scale(float w, H v) {
+  // Re and Im sums of both conjugate pairs, [component][pair]: the packed
+  // multiply-add takes a pair's Re and Im weights as they lie in memory, where one
+  // weight for both fields would have to be read or moved into a pair first
+  struct G { float2 c[4][2]; };
+  static __device__ __forceinline__ void gzero(G& g) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) g.c[i][0] = g.c[i][1] = make_float2(0.f, 0.f);
+  }
+  // g += (Re, Im of both shifts) w v
+  static __device__ __forceinline__ void tap(G& g, float w, H v, const S* sp) {
+    const float4 s = *sp;
+    const float e[4] = {w * v.x, w * v.y, w * v.z, w * v.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float2 d = make_float2(e[i], e[i]);
+      g.c[i][0] = __ffma2_rn(d, make_float2(s.x, s.y), g.c[i][0]);
+      g.c[i][1] = __ffma2_rn(d, make_float2(s.z, s.w), g.c[i][1]);
+    }
+  }
+  static __device__ __forceinline__ void scatter(G& a, float w, const G& g) {
     const float2 w2 = make_float2(w, w);
-    const float2 lo = __fmul2_rn(w2, make_float2(v.x, v.y)), hi = __fmul2_rn(w2, make_float2(v.z, v.w));
-    return make_float4(lo.x, lo.y, hi.x, hi.y);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      a.c[i][0] = __ffma2_rn(w2, g.c[i][0], a.c[i][0]);
+      a.c[i][1] = __ffma2_rn(w2, g.c[i][1], a.c[i][1]);
+    }
+  }
+  // conj(s_q) v of the four children: Re - i Im for 0 and 1, Re + i Im for 3 and 2
+  static __device__ __forceinline__ void children(const G& a, H* d) {
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      const float2 x = a.c[0][p], y = a.c[1][p], z = a.c[2][p], w = a.c[3][p];
+      d[p] = make_float4(x.x + y.y, y.x - x.y, z.x + w.y, w.x - z.y);
+      d[3 - p] = make_float4(x.x - y.y, y.x + x.y, z.x - w.y, w.x + z.y);
+    }
   }
   // the four children's values += d, as reductions in the L2 (one addend per
   // element, so the result does not depend on their order)
@@ -81,7 +114,7 @@ template <> struct Mp<float> {
     const float4 v = *p;
     s[0] = v.x; s[1] = v.y; s[2] = v.z; s[3] = v.w;
   }
-  static constexpr int HN = 2;                 // parts of a direction a CTA takes (R = 1: all of them)
+  static constexpr int HN = NF / 2;            // parts of a direction a CTA takes (R = 1: all of them)
   static __device__ __forceinline__ H zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
   static __device__ __forceinline__ W wt(float w) { return make_float2(w, w); }
   static __device__ __forceinline__ void fma(H& a, W w, H v) {
@@ -124,8 +157,26 @@ template <> struct Mp<double> {
   typedef double W;
   typedef double2 C;
   struct S { double2 a, b; };
-  typedef S W4;
-  static __device__ __forceinline__ H scale(double w, H v) { return make_double2(w * v.x, w * v.y); }
+  struct G { double2 x[4]; };                  // Re 03, Im 03, Re 12, Im 12
+  static __device__ __forceinline__ void gzero(G& g) {
+#pragma unroll
+    for (int x = 0; x < 4; ++x) g.x[x] = zero();
+  }
+  static __device__ __forceinline__ void tap(G& g, double w, H r, const S* sp) {
+    double s[4];
+    unpack(sp, s);
+    const H v = make_double2(w * r.x, w * r.y);
+#pragma unroll
+    for (int x = 0; x < 4; ++x) fma(g.x[x], s[x], v);
+  }
+  static __device__ __forceinline__ void scatter(G& a, double w, const G& g) {
+#pragma unroll
+    for (int x = 0; x < 4; ++x) fma(a.x[x], w, g.x[x]);
+  }
+  static __device__ __forceinline__ void children(const G& a, H* d) {
+    const H i03 = itimes(a.x[1]), i12 = itimes(a.x[3]);
+    d[0] = sub(a.x[0], i03); d[1] = sub(a.x[2], i12); d[2] = add(a.x[2], i12); d[3] = add(a.x[0], i03);
+  }
   static __device__ __forceinline__ void add_to(const bool* has, H* base, const unsigned* kid, unsigned ro, int NT,
                                                 const H* d) {
     H cur[4];
@@ -139,7 +190,7 @@ template <> struct Mp<double> {
     const double2 a = p->a, b = p->b;
     s[0] = a.x; s[1] = a.y; s[2] = b.x; s[3] = b.y;
   }
-  static constexpr int HN = 4;
+  static constexpr int HN = NF;
   static __device__ __forceinline__ H zero() { return make_double2(0.0, 0.0); }
   static __device__ __forceinline__ W wt(double w) { return w; }
   static __device__ __forceinline__ void fma(H& a, W w, H v) { a.x = ::fma(w, v.x, a.x); a.y = ::fma(w, v.y, a.y); }
@@ -343,17 +394,17 @@ __global__ void __launch_bounds__(INTERP_THREADS, INTERP_CTAS) k_interp_march(
 // ptw) give the thread's child column the Re- and Im-weighted sums of both
 // conjugate pairs; the window scatters them to four child rows, and a row
 // that no later entry reaches is added to the four children's incoming
-// spectra.  The shifts are staged as the weights the multiply-adds take.
+// spectra. 
 template <typename T, int PM, int NK = ANTERP_NK>
 __global__ void __launch_bounds__(ANTERP_THREADS, ANTERP_CTAS) k_anterp_march(
     int nbox, int nthC, int nphC, int nthP, int nphP, int NT, int TI, MarchTile m, const int4* __restrict__ ch4,
     const int* __restrict__ ent_ptr, const int* __restrict__ ent, const T* __restrict__ entw,
-    const int* __restrict__ pst, const T* __restrict__ ptw, int pm, const typename Mp<T>::W4* __restrict__ shiftw,
+    const int* __restrict__ pst, const T* __restrict__ ptw, int pm, const typename Mp<T>::S* __restrict__ shift,
     const typename Mp<T>::H* __restrict__ inP, typename Mp<T>::H* __restrict__ inC) {
   typedef Mp<T> P;
   typedef typename P::H H;
-  typedef typename P::W W;
-  typedef typename P::W4 W4;
+  typedef typename P::S S;
+  typedef typename P::G G;
   constexpr int HN = P::HN;
   extern __shared__ __align__(128) unsigned char smem[];
   const int tid = threadIdx.x;
@@ -363,7 +414,7 @@ __global__ void __launch_bounds__(ANTERP_THREADS, ANTERP_CTAS) k_anterp_march(
   bx -= bg * m.nck * m.nhk;
   const int ck = bx / m.nhk, h0 = (bx - ck * m.nhk) * HN, p0 = ck * m.ncol, B0 = bg * m.nbx;
   const int jp0 = pst[p0];                      // first staged parent column (before wrapping)
-  constexpr int SP = sizeof(W4) / 16;           // 16-byte pieces of a direction's shifts
+  constexpr int SP = sizeof(S) / 16;            // 16-byte pieces of a direction's shifts
   const int h = tid & (HN - 1);
   // chunk e of a row = (box, column, part), then the row's shifts
   const int Ev = m.nbx * m.cc * HN, E = Ev + m.cc * SP;
@@ -383,7 +434,7 @@ __global__ void __launch_bounds__(ANTERP_THREADS, ANTERP_CTAS) k_anterp_march(
     int j = jp0 + (int)(ec - lb * m.cc);
     j = j < 0 ? j + nphP : j >= nphP ? j - nphP : j;
     const bool ok = c < (unsigned)E && B0 + (int)lb < nbox && j >= 0 && j < nphP;
-    rc.at[k] = sh ? reinterpret_cast<const char*>(shiftw + j) + (c - Ev) % SP * 16
+    rc.at[k] = sh ? reinterpret_cast<const char*>(shift + j) + (c - Ev) % SP * 16
                   : reinterpret_cast<const char*>(inP + ((size_t)(B0 + lb) * nthP * nphP + j) * NT + h0 + h);
     if (ok) rc.have |= 1u << k;
     if (j >= (nphP >> 1)) rc.over |= 1u << k;
@@ -428,17 +479,15 @@ __global__ void __launch_bounds__(ANTERP_THREADS, ANTERP_CTAS) k_anterp_march(
   const bool has[4] = {c4.x >= 0, c4.y >= 0, c4.z >= 0, c4.w >= 0};
   const int tcol = pst[j] - jp0;
   const H* tap = reinterpret_cast<const H*>(smem) + ((act ? lb : 0) * m.cc + tcol) * HN + h;
-  const int stap = (Ev - ((act ? lb : 0) * m.cc + tcol) * HN - h) * 16 + tcol * (int)sizeof(W4);
+  const int stap = (Ev - ((act ? lb : 0) * m.cc + tcol) * HN - h) * 16 + tcol * (int)sizeof(S);
   T w[PM > 0 ? PM : 1];
   if (PM > 0) {
 #pragma unroll
     for (int q = 0; q < PM; ++q) w[q] = ptw[(size_t)j * pm + q];
   }
-  H acc[4][4];                                  // [child row mod 4][Re 03, Im 03, Re 12, Im 12]
+  G acc[4];                                     // [child row mod 4]
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int x = 0; x < 4; ++x) acc[a][x] = P::zero();
+  for (int a = 0; a < 4; ++a) P::gzero(acc[a]);
   int e1 = ent_ptr[min(b0 + 1, nb)];
   // child row b = bb + ph: ph the window slot
   for (int bb = b0;; bb += 4) {
@@ -454,37 +503,23 @@ __global__ void __launch_bounds__(ANTERP_THREADS, ANTERP_CTAS) k_anterp_march(
         __syncthreads();                        // this entry's row landed; the previous one's slot is free
         stage(e + 3);
         const H* r = tap + (e & 3) * E;
-        const W4* rs = reinterpret_cast<const W4*>(reinterpret_cast<const char*>(r) + stap);
-        H g[4];
+        const S* rs = reinterpret_cast<const S*>(reinterpret_cast<const char*>(r) + stap);
+        G g;
+        P::gzero(g);
 #pragma unroll
-        for (int x = 0; x < 4; ++x) g[x] = P::zero();
+        for (int q = 0; q < (PM > 0 ? PM : pm); ++q)
+          P::tap(g, PM > 0 ? w[PM > 0 ? q : 0] : ptw[(size_t)j * pm + q], r[q * HN], rs + q);
 #pragma unroll
-        for (int q = 0; q < (PM > 0 ? PM : pm); ++q) {
-          const T wq = PM > 0 ? w[PM > 0 ? q : 0] : ptw[(size_t)j * pm + q];
-          const H v = P::scale(wq, r[q * HN]);
-          W s[4];
-          P::w4(reinterpret_cast<const W*>(rs + q), s);
-#pragma unroll
-          for (int x = 0; x < 4; ++x) P::fma(g[x], s[x], v);
-        }
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-          const W ww = P::wt(tw[a]);
-#pragma unroll
-          for (int x = 0; x < 4; ++x) P::fma(acc[(ph + a) & 3][x], ww, g[x]);
-        }
+        for (int a = 0; a < 4; ++a) P::scatter(acc[(ph + a) & 3], tw[a], g);
       }
       e1 = e2;
       if (b >= i0) {
-        // conj(s_q) v of the four children: Re - i Im for 0 and 1, Re + i Im for 3 and 2
         const unsigned ro = (unsigned)(b * nphC);
-        const H i03 = P::itimes(acc[ph][1]), i12 = P::itimes(acc[ph][3]);
-        const H d[4] = {P::sub(acc[ph][0], i03), P::sub(acc[ph][2], i12), P::add(acc[ph][2], i12),
-                        P::add(acc[ph][0], i03)};
+        H d[4];
+        P::children(acc[ph], d);
         P::add_to(has, Ch, kid, ro, NT, d);
       }
-#pragma unroll
-      for (int x = 0; x < 4; ++x) acc[ph][x] = P::zero();
+      P::gzero(acc[ph]);
     }
   }
 }
@@ -571,7 +606,7 @@ int anterp_impl(Ctx* c, int s, int R, cudaStream_t st) {
   typedef Mp<T> P;
   const bool f64 = sizeof(T) == 8;
   const Level &Lc = c->lev[s], &Lp = c->lev[s + 1];
-  const int NT = P::HN * R, sp = (int)sizeof(typename P::W4) / 16;
+  const int NT = P::HN * R, sp = (int)sizeof(typename P::S) / 16;
   const MarchTile m = march_tile(ANTERP_THREADS, Lc.ma_pm <= 8 ? ANTERP_NK : 16, P::HN, P::HN, !f64, Lp.nbox,
                                  Lc.nph, NT, Lc.ma_start, Lc.ma_pm, 1, sp);
   const int TI = march_rows(m, Lc.nth, f64 ? 1 : 65536 / (168 * m.T), Lc.nth);
@@ -582,7 +617,7 @@ int anterp_impl(Ctx* c, int s, int R, cudaStream_t st) {
   k<<<g, m.T, sm, st>>>(Lp.nbox, Lc.nth, Lc.nph, Lp.nth, Lp.nph, NT, TI, m, (const int4*)Lp.d_ch4, Lc.d_ma_ptr,
                         Lc.d_ma_ent, (const T*)(f64 ? (void*)Lc.d_ma_w64 : (void*)Lc.d_ma_w32), Lc.d_ma_pst,
                         (const T*)(f64 ? (void*)Lc.d_ma_pw64 : (void*)Lc.d_ma_pw32), Lc.ma_pm,
-                        (const typename P::W4*)(f64 ? (void*)Lc.d_shiftp64 : (void*)Lc.d_shiftw32),
+                        (const typename P::S*)(f64 ? (void*)Lc.d_shiftp64 : (void*)Lc.d_shiftp32),
                         (const typename P::H*)Lp.d_in, (typename P::H*)Lc.d_in);
   SMR_LAUNCH(c);
   return SMR_OK;

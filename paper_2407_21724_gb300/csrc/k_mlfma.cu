@@ -56,53 +56,15 @@ template <typename V> __device__ __forceinline__ V cmul(V a, V b) {
   return r;
 }
 
-// the 4 fields of one direction (single right-hand side): 32 or 64 bytes
-__device__ __forceinline__ void ld_dir(const float2* p, float2* v) {
-  float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1];
-  v[0] = make_float2(a.x, a.y); v[1] = make_float2(a.z, a.w);
-  v[2] = make_float2(b.x, b.y); v[3] = make_float2(b.z, b.w);
-}
-__device__ __forceinline__ void ld_dir(const double2* p, double2* v) {
-  v[0] = p[0]; v[1] = p[1]; v[2] = p[2]; v[3] = p[3];
-}
-__device__ __forceinline__ void st_dir(float2* p, const float2* v) {
-  reinterpret_cast<float4*>(p)[0] = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
-  reinterpret_cast<float4*>(p)[1] = make_float4(v[2].x, v[2].y, v[3].x, v[3].y);
-}
-__device__ __forceinline__ void st_dir(double2* p, const double2* v) {
-  p[0] = v[0]; p[1] = v[1]; p[2] = v[2]; p[3] = v[3];
-}
-
-
 // ------------------------------------------------------------------ 16-byte direction parts
-// Single right-hand side kernels give each thread one 16-byte part of a
-// direction's 4 fields (FP32: 2 fields as a float4, FP64: 1 field), so that
+// The FP64 single right-hand side kernels give each thread one 16-byte part of a
+// direction (one field), so that
 // a warp instruction reads or writes one contiguous 512-byte run and shared
 // memory is accessed without bank conflicts.  NT threads share a direction.
 template <typename T> struct Part;
-template <> struct Part<float> {
-  typedef float4 H;
-  static constexpr int NT = 2, FPT = 2;
-  static __device__ __forceinline__ H zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
-  static __device__ __forceinline__ void rfma(H& a, float w, H v) {
-    a.x = fmaf(w, v.x, a.x); a.y = fmaf(w, v.y, a.y); a.z = fmaf(w, v.z, a.z); a.w = fmaf(w, v.w, a.w);
-  }
-  // a += s * v for each complex field of v
-  static __device__ __forceinline__ void cfma(H& a, float2 s, H v) {
-    a.x = fmaf(s.x, v.x, a.x); a.x = fmaf(-s.y, v.y, a.x);
-    a.y = fmaf(s.x, v.y, a.y); a.y = fmaf(s.y, v.x, a.y);
-    a.z = fmaf(s.x, v.z, a.z); a.z = fmaf(-s.y, v.w, a.z);
-    a.w = fmaf(s.x, v.w, a.w); a.w = fmaf(s.y, v.z, a.w);
-  }
-  static __device__ __forceinline__ void add(H& a, H v) { a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w; }
-  static __device__ __forceinline__ void w4(const float* p, float* w) {
-    float4 a = *reinterpret_cast<const float4*>(p);
-    w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w;
-  }
-};
 template <> struct Part<double> {
   typedef double2 H;
-  static constexpr int NT = 4, FPT = 1;
+  static constexpr int NT = NF;
   static __device__ __forceinline__ H zero() { return make_double2(0.0, 0.0); }
   static __device__ __forceinline__ void rfma(H& a, double w, H v) { a.x = fma(w, v.x, a.x); a.y = fma(w, v.y, a.y); }
   static __device__ __forceinline__ void cfma(H& a, double2 s, H v) {
@@ -117,89 +79,84 @@ template <> struct Part<double> {
 };
 template <typename T>
 __device__ __forceinline__ typename Part<T>::H ldp(const typename CV<T>::V* base, size_t dir, int h) {
-  return reinterpret_cast<const typename Part<T>::H*>(base + dir * 4)[h];
+  return reinterpret_cast<const typename Part<T>::H*>(base + dir * NF)[h];
 }
 template <typename T>
 __device__ __forceinline__ void stp(typename CV<T>::V* base, size_t dir, int h, typename Part<T>::H v) {
-  reinterpret_cast<typename Part<T>::H*>(base + dir * 4)[h] = v;
+  reinterpret_cast<typename Part<T>::H*>(base + dir * NF)[h] = v;
 }
 
 // ------------------------------------------------------------------ aggregation
-// out0[mu][k][f][r] = shift * sum_n conj(P[s][n][comp f][k]) x[mu][cur f][n][r]
-// One CTA = a tile of up to 16 particles of one shape (x in shared memory) x a
-// chunk of 64 directions; each pattern value is reused for the tile's columns.
+// out0[mu][k][f][r] = shift * sum_n conj(P_f[s][n][k]) (e_n +- (j/z) m_n), e and m
+// the particle's electric and magnetic coefficients, P_+- = P_th +- j P_ph.
+// The modes are real, so the pattern of the opposite direction k' is the
+// conjugate one: with P = a + j b and x = u + j v the sums of a u, b v, a v and
+// b u give both directions, 8 real multiply-adds a mode and pair of directions
+// (both fields) where 4 fields of every direction take 32.
+// CTA = one column (particle, r) x 128 pairs of directions, the modes in two
+// halves: what bounds it in FP64 is the FP64 rate, and a CTA per column keeps
+// every SM at it from some 100 columns on (64 particles: 104 us on 16 CTAs of 16
+// columns and 4 fields before, 12.3 us now; 1,600 particles 424 and 105 us).
+constexpr int AGC_PAIRS = 128;
 template <typename T>
-__global__ void k_aggregate(int K0, int npsi, int R, int RC, int nkc,
-                            const int* __restrict__ tile_shape, const int* __restrict__ tile_start,
-                            const int* __restrict__ tile_count, const int* __restrict__ perm,
-                            const double2* __restrict__ x, const typename CV<T>::V* __restrict__ P,
-                            const double* __restrict__ dshift, int any_dshift,
-                            const double* __restrict__ khat, double k,
-                            typename CV<T>::V* __restrict__ out) {
+__global__ void __launch_bounds__(2 * AGC_PAIRS) k_aggregate(
+    int K0, int nph, int npsi, int R, int nchunk, const int* __restrict__ perm, const int* __restrict__ sid,
+    const double2* __restrict__ x, const typename CV<T>::V* __restrict__ Pd, const double* __restrict__ dshift,
+    int any_dshift, const double* __restrict__ khat, double k, double iz, typename CV<T>::V* __restrict__ out) {
   typedef typename CV<T>::V V;
-  extern __shared__ unsigned char smem_raw[];
-  V* xs = reinterpret_cast<V*>(smem_raw);          // [col][2][npsi]
-  int nrc = (R + RC - 1) / RC;
-  int TP = max(1, 16 / RC);                        // particles per column group
-  int nsub = (16 + TP - 1) / TP;
-  int tile = blockIdx.x / (nsub * nkc * nrc);
-  int rest = blockIdx.x % (nsub * nkc * nrc);
-  int sub = rest / (nkc * nrc);
-  rest %= nkc * nrc;
-  int kc = rest / nrc, r0 = (rest % nrc) * RC;
-  int nr = min(RC, R - r0);
-  int s = tile_shape[tile], tp = tile_count[tile];
-  int t0 = tile_start[tile] + sub * TP;
-  int np_ = min(tp - sub * TP, TP);
-  if (np_ <= 0) return;
-  int ncol = np_ * nr;
-  // stage x for the tile's columns (particle, r)
-  for (int t = threadIdx.x; t < ncol * 2 * npsi; t += blockDim.x) {
-    int n = t % npsi, cc = (t / npsi) % 2, col = t / (2 * npsi);
-    int mu = perm[t0 + col / nr], r = r0 + col % nr;
-    xs[(col * 2 + cc) * npsi + n] = cvt2(x[((size_t)mu * 2 * npsi + cc * npsi + n) * R + r], V());
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  V* xs = reinterpret_cast<V*>(smem_raw);          // [npsi][2]
+  V* red = xs + 2 * npsi;                          // [2 halves][4][AGC_PAIRS]
+  const int chunk = blockIdx.x % nchunk, col = blockIdx.x / nchunk;
+  const int mu = perm[col / R], r = col % R, s = sid[mu];
+  for (int n = threadIdx.x; n < npsi; n += blockDim.x) {
+    const double2 e = x[((size_t)mu * 2 * npsi + n) * R + r], m = x[((size_t)mu * 2 * npsi + npsi + n) * R + r];
+    xs[2 * n] = cvt2(make_double2(fma(-iz, m.y, e.x), fma(iz, m.x, e.y)), V());
+    xs[2 * n + 1] = cvt2(make_double2(fma(iz, m.y, e.x), fma(-iz, m.x, e.y)), V());
   }
   __syncthreads();
-  int kl = threadIdx.x & 63, g = threadIdx.x >> 6;   // 64 directions x 4 column groups
-  int kk = kc * 64 + kl;
-  if (kk >= K0) return;
-  const V* Ps = P + (size_t)s * npsi * 2 * K0 + kk;
-  V acc[4][4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q)
-#pragma unroll
-    for (int f = 0; f < 4; ++f) acc[q][f] = czero<V>();
-  for (int n = 0; n < npsi; ++n) {
-    V pt = Ps[(size_t)(2 * n) * K0], pp = Ps[(size_t)(2 * n + 1) * K0];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      int col = g + 4 * q;
-      if (col < ncol) {
-        V e = xs[(col * 2) * npsi + n], m = xs[(col * 2 + 1) * npsi + n];
-        cfmac(acc[q][0], pt, e);
-        cfmac(acc[q][1], pp, e);
-        cfmac(acc[q][2], pt, m);
-        cfmac(acc[q][3], pp, m);
-      }
+  const int K2 = K0 / 2, kl = threadIdx.x % AGC_PAIRS, half = threadIdx.x / AGC_PAIRS;
+  const int q = chunk * AGC_PAIRS + kl;
+  {
+    const V* Pp = Pd + (size_t)s * 2 * npsi * K2 + min(q, K2 - 1);
+    const V* Pm = Pp + (size_t)npsi * K2;
+    V ap = czero<V>(), bp = czero<V>(), am = czero<V>(), bm = czero<V>();   // a x, b x of both fields
+#pragma unroll 4
+    for (int n = half; n < npsi; n += 2) {
+      const V p = Pp[(size_t)n * K2], m = Pm[(size_t)n * K2], xp = xs[2 * n], xm = xs[2 * n + 1];
+      rfma(ap, p.x, xp);
+      rfma(bp, p.y, xp);
+      rfma(am, m.x, xm);
+      rfma(bm, m.y, xm);
     }
+    V* o = red + (size_t)half * 4 * AGC_PAIRS + kl;
+    o[0] = ap; o[AGC_PAIRS] = bp; o[2 * AGC_PAIRS] = am; o[3 * AGC_PAIRS] = bm;
   }
+  __syncthreads();
+  if (q >= K2) return;
+  V t[4];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    int col = g + 4 * q;
-    if (col >= ncol) continue;
-    int mu = perm[t0 + col / nr], r = r0 + col % nr;
-    if (any_dshift) {
-      const double* d = dshift + 3 * mu;
-      const double* kh = khat + 3 * kk;
-      double ph = k * (kh[0] * d[0] + kh[1] * d[1] + kh[2] * d[2]);
-      double sn, cs;
-      sincos(ph, &sn, &cs);
-      V sh = mkc((T)cs, (T)sn);
-      for (int f = 0; f < 4; ++f) acc[q][f] = cmul(acc[q][f], sh);
-    }
-    V* o = out + ((size_t)mu * K0 + kk) * 4 * R + r;
-    o[0] = acc[q][0]; o[R] = acc[q][1]; o[2 * R] = acc[q][2]; o[3 * R] = acc[q][3];
+  for (int i = 0; i < 4; ++i) {
+    const V a = red[i * AGC_PAIRS + kl], b = red[(4 + i) * AGC_PAIRS + kl];
+    t[i] = mkc(a.x + b.x, a.y + b.y);
   }
+  // one half of the threads takes the directions of the table, the other their opposites
+  const T sg = half ? (T)-1 : (T)1;                // conj(P) x = (au + bv) + j (av - bu); P x the other signs
+  V w0 = mkc(t[0].x + sg * t[1].y, t[0].y - sg * t[1].x), w1 = mkc(t[2].x + sg * t[3].y, t[2].y - sg * t[3].x);
+  const int i = q / nph, j = q - i * nph;
+  const int kk = half ? (K0 / nph - 1 - i) * nph + (j + nph / 2 < nph ? j + nph / 2 : j - nph / 2) : q;
+  if (any_dshift) {
+    const double* d = dshift + 3 * mu;
+    const double* kh = khat + 3 * kk;
+    double sn, cs;
+    sincos(k * (kh[0] * d[0] + kh[1] * d[1] + kh[2] * d[2]), &sn, &cs);
+    const V sh = mkc((T)cs, (T)sn);
+    w0 = cmul(w0, sh);
+    w1 = cmul(w1, sh);
+  }
+  V* o = out + ((size_t)mu * K0 + kk) * NF * R + r;
+  o[0] = w0;
+  o[R] = w1;
 }
 
 // ------------------------------------------------------------------ FP64 interpolation, one right-hand side
@@ -208,9 +165,9 @@ __global__ void k_aggregate(int K0, int npsi, int R, int RC, int nkc,
 // and rows past a pole cost no extra passes.  CTA = (parent box, tile of TR parent theta rows);
 // each thread owns up to EM1 parent direction parts of the tile across the
 // loop over the children.  Per child: theta pass of the tile's rows into
-// shared memory G[TR][nphC][4] (4 taps, tables read as 16-byte vectors), then
+// shared memory G[TR][nphC][NF] (4 taps, tables read as 16-byte vectors), then
 // phi pass, shift and child sum in registers.
-constexpr int EM1 = 12;                          // direction parts per thread, at most
+constexpr int EM1 = 6;                           // direction parts per thread, at most
 __global__ void __launch_bounds__(256, 2) k_interp1(int nthP, int nphP, unsigned mP, int nphC, int Kc, int TR, int nrt,
                                                  const int* __restrict__ ch_ptr, const int* __restrict__ ch_idx,
                                                  const int* __restrict__ ch_quad, const int* __restrict__ th_pk,
@@ -225,7 +182,7 @@ __global__ void __launch_bounds__(256, 2) k_interp1(int nthP, int nphP, unsigned
   typedef P::H H;
   constexpr int NT = P::NT, EM = EM1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  V* G = reinterpret_cast<V*>(smem_raw);           // [TR][nphC][4]
+  V* G = reinterpret_cast<V*>(smem_raw);           // [TR][nphC][NF]
   int B = blockIdx.x / nrt, rt = blockIdx.x - (blockIdx.x / nrt) * nrt;
   int tp0 = rt * TR, ntr = min(TR, nthP - tp0);
   int Kp = nthP * nphP;
@@ -240,7 +197,7 @@ __global__ void __launch_bounds__(256, 2) k_interp1(int nthP, int nphP, unsigned
 #pragma unroll
   for (int i = 0; i < EM; ++i) acc[i] = P::zero();
   for (int e = ch_ptr[B]; e < ch_ptr[B + 1]; ++e) {
-    const V* src = F + (size_t)ch_idx[e] * Kc * 4;
+    const V* src = F + (size_t)ch_idx[e] * Kc * NF;
     const V* sh = shift + (size_t)ch_quad[e] * Kp + (size_t)tp0 * nphP;
     __syncthreads();
     for (int tr = trG0, j = jG0, task = task0; tr < ntr; task += NTH) {
@@ -280,7 +237,7 @@ __global__ void __launch_bounds__(256, 2) k_interp1(int nthP, int nphP, unsigned
       }
     }
   }
-  V* dst = out + ((size_t)B * Kp + (size_t)tp0 * nphP) * 4;
+  V* dst = out + ((size_t)B * Kp + (size_t)tp0 * nphP) * NF;
 #pragma unroll
   for (int i = 0; i < EM; ++i) {
     int t = threadIdx.x + i * blockDim.x;
@@ -301,16 +258,6 @@ __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.wait_group 0;\n" ::);
 }
 
-// 4 consecutive complex values (the 4 fields of one direction) from shared memory
-__device__ __forceinline__ void load4(const float2* p, float2* v) {
-  float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1];
-  v[0] = make_float2(a.x, a.y); v[1] = make_float2(a.z, a.w);
-  v[2] = make_float2(b.x, b.y); v[3] = make_float2(b.z, b.w);
-}
-__device__ __forceinline__ void load4(const double2* p, double2* v) {
-  v[0] = p[0]; v[1] = p[1]; v[2] = p[2]; v[3] = p[3];
-}
-
 template <typename T>
 __global__ void k_translate(int K, int R, int RC, int KC, int ntx, int ntile, const int* __restrict__ tiles,
                             int map_x0, int map_y0, int map_w, int map_h, int noff,
@@ -329,8 +276,8 @@ __global__ void k_translate(int K, int R, int RC, int KC, int ntx, int ntile, co
   int ax0 = ((map_x0 >> 2) + tx) * 4, ay0 = ((map_y0 >> 2) + ty) * 4;
   int k0 = kch * KC, r0 = rch * RC;
   int nk = min(KC, K - k0), nr = min(RC, R - r0);
-  int W = KC * 4 * RC;                                // V per source box in the chunk
-  V* S = reinterpret_cast<V*>(smem_raw);              // [64 sources][KC][4][RC]
+  int W = KC * NF * RC;                               // V per source box in the chunk
+  V* S = reinterpret_cast<V*>(smem_raw);              // [64 sources][KC][NF][RC]
   V* Ts = S + 64 * W;                                 // [noff][KC]
   int* bid = reinterpret_cast<int*>(Ts + max(noff, 1) * KC);   // [64] source box ids
   int* tgt = bid + 64;                                // [16] target box ids
@@ -346,14 +293,14 @@ __global__ void k_translate(int K, int R, int RC, int KC, int ntx, int ntile, co
     // each source box's chunk is contiguous in global memory: asynchronous
     // 16-byte copies, zero-filled for missing boxes and past the last direction
     int per = W * (int)sizeof(V) / 16;
-    int valid = nk * 4 * R * (int)sizeof(V);
+    int valid = nk * NF * R * (int)sizeof(V);
     for (int t = threadIdx.x; t < 64 * per; t += blockDim.x) {
       int sb = t / per, pc = t - sb * per;
       int b = bid[sb];
       const char* g = reinterpret_cast<const char*>(out);
       int nb = 0;
       if (b >= 0 && pc * 16 < valid) {
-        g += ((size_t)b * K + k0) * 4 * R * sizeof(V) + (size_t)pc * 16;
+        g += ((size_t)b * K + k0) * NF * R * sizeof(V) + (size_t)pc * 16;
         nb = 16;
       }
       cp_async16(reinterpret_cast<char*>(S + (size_t)sb * W) + pc * 16, g, nb);
@@ -363,17 +310,17 @@ __global__ void k_translate(int K, int R, int RC, int KC, int ntx, int ntile, co
     // columns (aligned: R and RC span whole 16-byte pieces), zero-filled for
     // missing boxes, past the last direction and past the last column
     int pr = RC * (int)sizeof(V) / 16;               // pieces per run
-    int per = KC * 4 * pr;                           // pieces per source box
+    int per = KC * NF * pr;                          // pieces per source box
     for (int t = threadIdx.x; t < 64 * per; t += blockDim.x) {
       int sb = t / per, e = t - sb * per;
-      int run = e / pr, pc = e - run * pr;           // run = kl * 4 + f
-      int kl = run >> 2;
+      int run = e / pr, pc = e - run * pr;           // run = kl * NF + f
+      int kl = run / NF;
       int b = bid[sb];
       const char* g = reinterpret_cast<const char*>(out);
       int nb = 0;
       int col = pc * 16 / (int)sizeof(V);            // first column of the piece
       if (b >= 0 && kl < nk && col < nr) {
-        g += ((((size_t)b * K + k0 + kl) * 4 + (run & 3)) * R + r0) * sizeof(V) + (size_t)pc * 16;
+        g += ((((size_t)b * K + k0 + kl) * NF + run % NF) * R + r0) * sizeof(V) + (size_t)pc * 16;
         nb = 16;
       }
       cp_async16(reinterpret_cast<char*>(S + (size_t)sb * W + (size_t)run * RC) + pc * 16, g, nb);
@@ -381,9 +328,9 @@ __global__ void k_translate(int K, int R, int RC, int KC, int ntx, int ntile, co
   } else {
     for (int t = threadIdx.x; t < 64 * W; t += blockDim.x) {
       int sb = t / W, e = t % W;
-      int rl = e % RC, kl = e / (4 * RC), f = (e / RC) % 4;
+      int rl = e % RC, kl = e / (NF * RC), f = (e / RC) % NF;
       int b = bid[sb];
-      S[t] = (b >= 0 && kl < nk && rl < nr) ? out[(((size_t)b * K + k0 + kl) * 4 + f) * R + r0 + rl]
+      S[t] = (b >= 0 && kl < nk && rl < nr) ? out[(((size_t)b * K + k0 + kl) * NF + f) * R + r0 + rl]
                                            : czero<V>();
     }
   }
@@ -415,33 +362,25 @@ __global__ void k_translate(int K, int R, int RC, int KC, int ntx, int ntile, co
   }
   cp_async_wait_all();
   __syncthreads();
-  // outputs: 16 targets x nk directions x nr columns, 4 fields each
+  // outputs: 16 targets x nk directions x nr columns, NF fields each
   int nout = 16 * nk * nr;
   for (int t = threadIdx.x; t < nout; t += blockDim.x) {
     int rl = t % nr, kl = (t / nr) % nk, tg = t / (nr * nk);
     int b = tgt[tg];
     if (b < 0) continue;
-    V acc[4] = {czero<V>(), czero<V>(), czero<V>(), czero<V>()};
+    V acc[NF] = {czero<V>(), czero<V>()};
     int n = cnt[tg];
     const int2* L = lst + tg * 27;
-    int kr = kl * 4 * RC + rl;
+    int kr = kl * NF * RC + rl;
     for (int e = 0; e < n; ++e) {
       int2 so = L[e];
       V tv = Ts[so.y + kl];
       const V* sv = S + so.x + kr;
-      V v[4];
-      if (RC == 1) {
-        load4(sv, v);
-      } else {
-        v[0] = sv[0]; v[1] = sv[RC]; v[2] = sv[2 * RC]; v[3] = sv[3 * RC];
-      }
-      cfma(acc[0], tv, v[0]);
-      cfma(acc[1], tv, v[1]);
-      cfma(acc[2], tv, v[2]);
-      cfma(acc[3], tv, v[3]);
+      cfma(acc[0], tv, sv[0]);
+      cfma(acc[1], tv, sv[RC]);
     }
-    V* o = in + ((size_t)b * K + k0 + kl) * 4 * R + r0 + rl;
-    for (int f = 0; f < 4; ++f) o[f * R] = acc[f];
+    V* o = in + ((size_t)b * K + k0 + kl) * NF * R + r0 + rl;
+    for (int f = 0; f < NF; ++f) o[f * R] = acc[f];
   }
 }
 
@@ -470,8 +409,8 @@ __global__ void __launch_bounds__(512, 2) k_translate1(int K, int ntx, int ntile
   int ax0 = ((map_x0 >> 3) + tx) * TS, ay0 = ((map_y0 >> 3) + ty) * TS;
   int k0 = kch * KC;
   int nk = min(KC, K - k0);
-  constexpr int W = KC * 4;
-  V* S = reinterpret_cast<V*>(smem_raw);              // [HS*HS sources][KC][4]
+  constexpr int W = KC * NF;
+  V* S = reinterpret_cast<V*>(smem_raw);              // [HS*HS sources][KC][NF]
   V* Ts = S + HS * HS * W;                            // [49 offsets][KC]
   int* bid = reinterpret_cast<int*>(Ts + 49 * KC);    // [HS*HS] source box ids
   int* tb = bid + HS * HS;                            // [TS*TS] target box ids
@@ -485,14 +424,14 @@ __global__ void __launch_bounds__(512, 2) k_translate1(int K, int ntx, int ntile
   __syncthreads();
   {
     constexpr int per = W * (int)sizeof(V) / 16;      // 16-byte pieces per source row
-    int valid = nk * 4 * (int)sizeof(V);
+    int valid = nk * NF * (int)sizeof(V);
     for (int t = threadIdx.x; t < HS * HS * per; t += blockDim.x) {
       int sb = t / per, pc = t - sb * per;
       int b = bid[sb];
       const char* g = reinterpret_cast<const char*>(out);
       int nb = 0;
       if (b >= 0 && pc * 16 < valid) {
-        g += ((size_t)b * K + k0) * 4 * sizeof(V) + (size_t)pc * 16;
+        g += ((size_t)b * K + k0) * NF * sizeof(V) + (size_t)pc * 16;
         nb = 16;
       }
       cp_async16(reinterpret_cast<char*>(S + (size_t)sb * W) + pc * 16, g, nb);
@@ -512,7 +451,7 @@ __global__ void __launch_bounds__(512, 2) k_translate1(int K, int ntx, int ntile
 #pragma unroll
   for (int q = 0; q < 4; ++q) any |= tb[(pyo + (q >> 1)) * TS + (pxo + (q & 1))] >= 0;
   if (!any) return;
-  const V* Sp = S + (size_t)(pyo * HS + pxo) * W + kl * 4;   // window origin
+  const V* Sp = S + (size_t)(pyo * HS + pxo) * W + kl * NF;   // window origin
   const V* Tp = Ts + kl;
   H acc[4];
 #pragma unroll
@@ -586,10 +525,10 @@ __global__ void __launch_bounds__(256) k_translate_lvl(int K, int nbox, int KCH,
   typedef P::H H;
   constexpr int NT = P::NT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  V* S = reinterpret_cast<V*>(smem_raw);                 // [nbox][KCH][4]
-  V* Ts = S + (size_t)nbox * KCH * 4;                    // [49][KCH]
+  V* S = reinterpret_cast<V*>(smem_raw);                 // [nbox][KCH][NF]
+  V* Ts = S + (size_t)nbox * KCH * NF;                   // [49][KCH]
   const int k0 = blockIdx.x * KCH, kn = min(KCH, K - k0);
-  // stage: every box's 4 fields for the chunk, and the tables
+  // stage: every box's fields for the chunk, and the tables
   for (int i = threadIdx.x; i < nbox * KCH * NT; i += blockDim.x) {
     const int b = i / (KCH * NT), r = i - b * (KCH * NT), kl = r / NT, h = r - kl * NT;
     H v = P::zero();
@@ -641,7 +580,7 @@ __global__ void __launch_bounds__(256) k_anterp1(int nthC, int nphC, int nthP, i
   typedef P::H H;
   constexpr int NT = P::NT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  V* Gt = reinterpret_cast<V*>(smem_raw);          // [GR][2 JC][4]
+  V* Gt = reinterpret_cast<V*>(smem_raw);          // [GR][2 JC][NF]
   int blk = blockIdx.x;
   int jcb = blk % njc;
   blk /= njc;
@@ -652,9 +591,9 @@ __global__ void __launch_bounds__(256) k_anterp1(int nthC, int nphC, int nthP, i
   int lo = lo_row[it], hi = lo_row[nit + it];
   int nr = hi - lo, W = 2 * nj;
   int Kp = nthP * nphP, Kc = nthC * nphC;
-  const V* srcP = inP + (size_t)parent[c] * Kp * 4;
+  const V* srcP = inP + (size_t)parent[c] * Kp * NF;
   const V* sh = shift + (size_t)quad[c] * Kp;
-  // each thread owns PPT consecutive 16-byte parts of a direction's four;
+  // each thread owns PPT consecutive 16-byte parts of a direction;
   // (row, column) of its tasks stepped by the NTH tasks of one sweep of the
   // CTA without dividing per task
   constexpr int PPT = 2, NT2 = NT / PPT;
@@ -665,7 +604,7 @@ __global__ void __launch_bounds__(256) k_anterp1(int nthC, int nphC, int nthP, i
     int j = (u < nj) ? j0 + u : j0 + half + (u - nj);
     int tp = lo + r;
     T wt = wthp[tp];
-    const V* prow = srcP + (size_t)tp * nphP * 4;
+    const V* prow = srcP + (size_t)tp * nphP * NF;
     const V* srow = sh + (size_t)tp * nphP;
     H a = P::zero(), a1 = P::zero();
     const int pm = PMC > 0 ? 8 : PM;
@@ -728,101 +667,82 @@ __global__ void __launch_bounds__(256) k_anterp1(int nthC, int nphC, int nthP, i
   }
 }
 // ------------------------------------------------------------------ receive
-// y_e[m] += -jk sum_k w conj(sh) [P_th (z B0 + B3) + P_ph (z B1 - B2)]
-// y_m[m] += -jk sum_k w conj(sh) [P_th (-B1 + B2/z) + P_ph (B0 + B3/z)]   (Eqs. 24-25)
-// One CTA = a tile of up to 16 (particle, r) columns of one shape; threads are
-// (mode, column pair); pattern and combined spectra chunks staged in shared memory.
+// Y_f[n] = sum_k w conj(sh) P_f[n][k] W_f[k];  y_e += -jk z (Y_+ + Y_-) / 2,
+// y_m += -(k / 2) (Y_+ - Y_-)   (Eqs. 24-25 in the circular components).
+// Opposite directions k, k' together: P W + conj(P) W' = a (W + W') + j b (W - W'),
+// 8 real multiply-adds a mode and pair of directions.  CTA = one column; threads
+// are (mode, every KS-th pair), the sums and differences of 64 pairs staged in
+// shared memory.  Bound by the FP64 rate (64 particles 426 us on 4 CTAs of 16
+// columns and 4 fields before, 16.4 us now; 1,600 particles 543 and 102 us).
+constexpr int RCV_PAIRS = 64;
 template <typename T>
-__global__ void k_receive(int K0, int npsi, int R, int RC, const int* __restrict__ tile_shape,
-                          const int* __restrict__ tile_start, const int* __restrict__ tile_count,
-                          const int* __restrict__ perm, const typename CV<T>::V* __restrict__ in0,
-                          const typename CV<T>::V* __restrict__ P, const double* __restrict__ w0,
-                          const double* __restrict__ dshift, int any_dshift,
-                          const double* __restrict__ khat, double k, double zeta,
-                          double2* __restrict__ y, int accumulate) {
+__global__ void k_receive(int K0, int nph, int npsi, int R, const int* __restrict__ perm, const int* __restrict__ sid,
+                          const typename CV<T>::V* __restrict__ in0, const typename CV<T>::V* __restrict__ Pm,
+                          const double* __restrict__ w0, const double* __restrict__ dshift, int any_dshift,
+                          const double* __restrict__ khat, double k, double zeta, double2* __restrict__ y,
+                          int accumulate) {
   typedef typename CV<T>::V V;
-  const int KC = 32;
-  extern __shared__ unsigned char smem_raw[];
-  V* Ps = reinterpret_cast<V*>(smem_raw);          // [KC][2][npsi]
-  V* Cs = Ps + KC * 2 * npsi;                      // [KC][16 cols][4]
-  int nrc = (R + RC - 1) / RC;
-  int TP = max(1, 16 / RC);
-  int nsub = (16 + TP - 1) / TP;
-  int tile = blockIdx.x / (nsub * nrc);
-  int sub = (blockIdx.x / nrc) % nsub, r0 = (blockIdx.x % nrc) * RC;
-  int nr = min(RC, R - r0);
-  int s = tile_shape[tile], tp = tile_count[tile];
-  int t0 = tile_start[tile] + sub * TP;
-  int ncol = max(0, min(tp - sub * TP, TP)) * nr;
-  if (ncol == 0) return;                           // uniform per block: no barrier skipped
-  int m = threadIdx.x % npsi, g = threadIdx.x / npsi;   // g in [0, 8): columns g, g + 8
-  T z = (T)zeta, iz = (T)(1.0 / zeta);
-  V ye[2] = {czero<V>(), czero<V>()}, ym[2] = {czero<V>(), czero<V>()};
-  const V* Pg = P + (size_t)s * npsi * 2 * K0;
-  for (int k0 = 0; k0 < K0; k0 += KC) {
-    int nk = min(KC, K0 - k0);
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  V* sd = reinterpret_cast<V*>(smem_raw);          // [RCV_PAIRS][2 fields][sum, difference]
+  V* red = sd + 4 * RCV_PAIRS;                     // [2 fields][threads]
+  const int mu = perm[blockIdx.x / R], r = blockIdx.x % R, s = sid[mu];
+  const int K2 = K0 / 2, KS = blockDim.x / npsi, m = threadIdx.x % npsi, ks = threadIdx.x / npsi;
+  const V* Pp = Pm + (size_t)s * 2 * K2 * npsi + m;
+  const V* Pn = Pp + (size_t)K2 * npsi;
+  V yp = czero<V>(), yn = czero<V>();
+  for (int q0 = 0; q0 < K2; q0 += RCV_PAIRS) {
+    const int nq = min(RCV_PAIRS, K2 - q0);
     __syncthreads();
-    for (int t = threadIdx.x; t < nk * 2 * npsi; t += blockDim.x) {
-      int kl = t % nk, comp = (t / nk) % 2, mm = t / (2 * nk);
-      Ps[(kl * 2 + comp) * npsi + mm] = Pg[((size_t)mm * 2 + comp) * K0 + k0 + kl];
-    }
-    for (int t = threadIdx.x; t < nk * ncol; t += blockDim.x) {
-      int kl = t % nk, col = t / nk;
-      int mu = perm[t0 + col / nr], r = r0 + col % nr;
-      int kk = k0 + kl;
-      const V* b = in0 + ((size_t)mu * K0 + kk) * 4 * R + r;
-      V B0 = b[0], B1 = b[R], B2 = b[2 * R], B3 = b[3 * R];
-      T wk = (T)w0[kk];
-      V sh = mkc(wk, (T)0);
+    for (int t = threadIdx.x; t < 2 * nq; t += blockDim.x) {
+      const int f = t & 1, q = q0 + (t >> 1), i = q / nph, j = q - i * nph;
+      const int kk = (K0 / nph - 1 - i) * nph + (j + nph / 2 < nph ? j + nph / 2 : j - nph / 2);
+      V a = in0[(((size_t)mu * K0 + q) * NF + f) * R + r], b = in0[(((size_t)mu * K0 + kk) * NF + f) * R + r];
       if (any_dshift) {
         const double* d = dshift + 3 * mu;
-        const double* kh = khat + 3 * kk;
-        double ph = -k * (kh[0] * d[0] + kh[1] * d[1] + kh[2] * d[2]);
+        const double* kh = khat + 3 * q;
         double sn, cs;
-        sincos(ph, &sn, &cs);
-        sh = mkc((T)(w0[kk] * cs), (T)(w0[kk] * sn));
+        sincos(-k * (kh[0] * d[0] + kh[1] * d[1] + kh[2] * d[2]), &sn, &cs);
+        a = cmul(a, mkc((T)cs, (T)sn));
+        b = cmul(b, mkc((T)cs, (T)-sn));
       }
-      V* cc = Cs + ((size_t)kl * 16 + col) * 4;
-      cc[0] = cmul(sh, mkc(z * B0.x + B3.x, z * B0.y + B3.y));
-      cc[1] = cmul(sh, mkc(z * B1.x - B2.x, z * B1.y - B2.y));
-      cc[2] = cmul(sh, mkc(-B1.x + iz * B2.x, -B1.y + iz * B2.y));
-      cc[3] = cmul(sh, mkc(B0.x + iz * B3.x, B0.y + iz * B3.y));
+      const T w = (T)w0[q];
+      sd[2 * t] = mkc(w * (a.x + b.x), w * (a.y + b.y));
+      sd[2 * t + 1] = mkc(w * (a.x - b.x), w * (a.y - b.y));
     }
     __syncthreads();
-    if (g < 8) {
-      for (int kl = 0; kl < nk; ++kl) {
-        V pt = Ps[(kl * 2) * npsi + m], pp = Ps[(kl * 2 + 1) * npsi + m];
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          int col = g + 8 * q;
-          if (col < ncol) {
-            const V* cc = Cs + ((size_t)kl * 16 + col) * 4;
-            cfma(ye[q], pt, cc[0]);
-            cfma(ye[q], pp, cc[1]);
-            cfma(ym[q], pt, cc[2]);
-            cfma(ym[q], pp, cc[3]);
-          }
-        }
-      }
+#pragma unroll 4
+    for (int q = ks; q < nq; q += KS) {
+      const V p = Pp[(size_t)(q0 + q) * npsi], n = Pn[(size_t)(q0 + q) * npsi];
+      const V* c = sd + 4 * q;
+      rfma(yp, p.x, c[0]);
+      yp.x = fma(-p.y, c[1].y, yp.x);
+      yp.y = fma(p.y, c[1].x, yp.y);
+      rfma(yn, n.x, c[2]);
+      yn.x = fma(-n.y, c[3].y, yn.x);
+      yn.y = fma(n.y, c[3].x, yn.y);
     }
   }
-  if (g >= 8) return;
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    int col = g + 8 * q;
-    if (col >= ncol) continue;
-    int mu = perm[t0 + col / nr], r = r0 + col % nr;
-    double2 oe = make_double2(k * (double)ye[q].y, -k * (double)ye[q].x);   // -j k
-    double2 om = make_double2(k * (double)ym[q].y, -k * (double)ym[q].x);
-    double2* pe = y + ((size_t)mu * 2 * npsi + m) * R + r;
-    double2* pm = pe + (size_t)npsi * R;
-    if (accumulate) {
-      double2 a = *pe, b = *pm;
-      oe.x += a.x; oe.y += a.y; om.x += b.x; om.y += b.y;
-    }
-    *pe = oe;
-    *pm = om;
+  red[threadIdx.x] = yp;
+  red[blockDim.x + threadIdx.x] = yn;
+  __syncthreads();
+  if (ks) return;
+  for (int t = 1; t < KS; ++t) {
+    const V a = red[t * npsi + m], b = red[blockDim.x + t * npsi + m];
+    yp.x += a.x; yp.y += a.y;
+    yn.x += b.x; yn.y += b.y;
   }
+  const double h = 0.5 * k, hz = h * zeta;
+  const double2 p = to64(yp), n = to64(yn);
+  double2 oe = make_double2(hz * (p.y + n.y), -hz * (p.x + n.x));
+  double2 om = make_double2(-h * (p.x - n.x), -h * (p.y - n.y));
+  double2* pe = y + ((size_t)mu * 2 * npsi + m) * R + r;
+  double2* pm = pe + (size_t)npsi * R;
+  if (accumulate) {
+    const double2 a = *pe, b = *pm;
+    oe.x += a.x; oe.y += a.y; om.x += b.x; om.y += b.y;
+  }
+  *pe = oe;
+  *pm = om;
 }
 
 // ------------------------------------------------------------------ block-sparse product
@@ -885,7 +805,7 @@ int ensure_spectra(Ctx* c, int R, int prec) {
       if (L.buf_out[p]) cudaFree(L.buf_out[p]);
       if (L.buf_in[p]) cudaFree(L.buf_in[p]);
       L.buf_out[p] = L.buf_in[p] = nullptr;
-      size_t bytes = (size_t)L.nbox * L.K * 4 * R * es;
+      size_t bytes = (size_t)L.nbox * L.K * NF * R * es;
       if (cudaMalloc(&L.buf_out[p], bytes) != cudaSuccess || cudaMalloc(&L.buf_in[p], bytes) != cudaSuccess) {
         c->err = "out of device memory for level spectra";
         c->spec_prec = -1;
@@ -896,8 +816,16 @@ int ensure_spectra(Ctx* c, int R, int prec) {
     if (c->pspec[p]) cudaFree(c->pspec[p]);
     c->pspec[p] = nullptr;
     if ((c->multi || c->any_dshift) &&
-        cudaMalloc(&c->pspec[p], (size_t)c->p * c->lev[0].K * 4 * R * es) != cudaSuccess) {
+        cudaMalloc(&c->pspec[p], (size_t)c->p * c->lev[0].K * NF * R * es) != cudaSuccess) {
       c->err = "out of device memory for the per-particle spectra";
+      c->spec_prec = -1;
+      return SMR_E_OOM;
+    }
+    if (c->d_xs[p]) cudaFree(c->d_xs[p]);
+    c->d_xs[p] = nullptr;
+    if (cudaMalloc((void**)&c->d_xs[p], (size_t)c->p * 2 * c->npsi * R * sizeof(double2)) != cudaSuccess) {
+      cudaGetLastError();
+      c->err = "out of device memory for the spectra's coefficients";
       c->spec_prec = -1;
       return SMR_E_OOM;
     }
@@ -917,7 +845,7 @@ int ensure_spectra(Ctx* c, int R, int prec) {
 // up to 32 whose staged spectra and tables fit in 96 KB (0: none fits).
 int translate_lvl_chunk(int nbox, size_t vbytes) {
   for (int kch = 32; kch >= 4; kch /= 2)
-    if (((size_t)nbox * kch * 4 + (size_t)49 * kch) * vbytes <= 96 * 1024) return kch;
+    if (((size_t)nbox * kch * NF + (size_t)49 * kch) * vbytes <= 96 * 1024) return kch;
   return 0;
 }
 
@@ -945,7 +873,7 @@ static bool march_anterp(const Level& Lp, int v) { return v == 0 ? (size_t)Lp.nb
 
 // Finest boxes made of cells.  Box b's outgoing spectrum is the sum of its
 // particles' spectra, and each particle receives its box's incoming
-// spectrum; a row is one box's or one particle's [K0][4][R] spectrum.  With
+// spectrum; a row is one box's or one particle's [K0][NF][R] spectrum.  With
 // `shift` set the kernels also carry each particle's displacement d from
 // its box centre: e^{+jk khat.d} into the sum, e^{-jk khat.d} out of the
 // broadcast (the tensor-core aggregation and receive work on unshifted
@@ -978,7 +906,7 @@ __global__ void k_cell_sum(int nbox, long long row, int R, const int* __restrict
   const int b = blockIdx.x;
   const long long e = blockIdx.y * (long long)blockDim.x + threadIdx.x;
   if (b >= nbox || e >= row) return;
-  const int kk = (int)(e / (4LL * R));
+  const int kk = (int)(e / ((long long)NF * R));
   V acc = mkc((T)0, (T)0);
   for (int t = ptr[b]; t < ptr[b + 1]; ++t) {
     const int mu = idx[t];
@@ -999,7 +927,7 @@ __global__ void k_cell_bcast(int p, long long row, int R, const int* __restrict_
   const long long e = blockIdx.y * (long long)blockDim.x + threadIdx.x;
   if (mu >= p || e >= row) return;
   V v = box[(size_t)cell[mu] * row + e];
-  if (shift) v = cmul(v, shift_phase<T>(dshift + 3 * mu, khat + 3 * (int)(e / (4LL * R)), k, -1.0));
+  if (shift) v = cmul(v, shift_phase<T>(dshift + 3 * mu, khat + 3 * (int)(e / ((long long)NF * R)), k, -1.0));
   part[(size_t)mu * row + e] = v;
 }
 
@@ -1009,14 +937,21 @@ static int far_impl(Ctx* c, int R, const double2* x, double2* y, bool accumulate
   const bool f64 = sizeof(T) == 8;
   const double es = sizeof(V), R_ = R;
   Level& L0 = c->lev[0];
-  int RC = std::min(R, 16);
-  int nrc = (R + RC - 1) / RC;
   // Overlap: the translation of each level runs on a side stream after an
   // event that marks its outgoing spectra, and the anterpolation into a level
   // waits for that level's translation; the receive waits for the near
   // product when run_product put it on a side stream (c->near_ev).
   Ctx::Side* sd = (c->overlap && !c->prof && c->cur_side < (int)c->side.size()) ? &c->side[c->cur_side] : nullptr;
   if (sd && (!sd->tr || c->nlev > (int)sd->eout.size())) sd = nullptr;
+  // the coefficients stay with the spectra (smr_copy_level's fields come from both)
+  if (!c->keep_x) {
+    const size_t bytes = (size_t)c->p * 2 * c->npsi * R * sizeof(double2);
+    if (sd) {
+      SMR_CUDA(c, cudaEventRecord(sd->efork, st));
+      SMR_CUDA(c, cudaStreamWaitEvent(sd->tr, sd->efork, 0));
+    }
+    SMR_CUDA(c, cudaMemcpyAsync(c->d_xs[f64 ? 0 : 1], x, bytes, cudaMemcpyDeviceToDevice, sd ? sd->tr : st));
+  }
   // translation at every level (in the upward loop when it overlaps)
   auto translate = [&](int s, cudaStream_t ts) -> int {
     Level& L = c->lev[s];
@@ -1030,12 +965,12 @@ static int far_impl(Ctx* c, int R, const double2* x, double2* y, bool accumulate
     int KC = std::max(1, cap / RCt);
     int nkch = (L.K + KC - 1) / KC;
     int nrct = (R + RCt - 1) / RCt;
-    size_t sm = ((size_t)64 * KC * 4 * RCt + (size_t)std::max(noff, 1) * KC) * sizeof(V) +
+    size_t sm = ((size_t)64 * KC * NF * RCt + (size_t)std::max(noff, 1) * KC) * sizeof(V) +
                 (64 + 16 + 16) * sizeof(int) + 16 * 27 * sizeof(int2);
     cudaFuncSetAttribute(k_translate<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     pbeg(c, ts, "translate", s,
-         2.0 * L.nbox * L.K * 4 * R_ * es + (double)L.off_dx.size() * L.K * es,
-         8.0 * L.il_src.size() * L.K * 4 * R_);
+         2.0 * L.nbox * L.K * NF * R_ * es + (double)L.off_dx.size() * L.K * es,
+         8.0 * L.il_src.size() * L.K * NF * R_);
     if (!f64 && R == 1) {
       int rc = run_translate_tiles(c, s, ts);
       pend(c, ts);
@@ -1046,7 +981,7 @@ static int far_impl(Ctx* c, int R, const double2* x, double2* y, bool accumulate
     const int tv = (R == 1) ? L.tune_tr[0] : 0;
     if (R == 1 && tv == 5 && translate_lvl_ok(c, s)) {
       const int KCH = translate_lvl_chunk(L.nbox, sizeof(double2));
-      const size_t sml = ((size_t)L.nbox * KCH * 4 + (size_t)49 * KCH) * sizeof(double2);
+      const size_t sml = ((size_t)L.nbox * KCH * NF + (size_t)49 * KCH) * sizeof(double2);
       k_translate_lvl<<<(unsigned)((L.K + KCH - 1) / KCH), 256, sml, ts>>>(
           L.K, L.nbox, KCH, L.d_il_ptr, L.d_il_pk, L.d_T64, (const double2*)L.d_out, (double2*)L.d_in);
       SMR_LAUNCH(c);
@@ -1061,12 +996,12 @@ static int far_impl(Ctx* c, int R, const double2* x, double2* y, bool accumulate
       k_translate_few<<<g, 256, 0, ts>>>(L.K, L.nbox, TG, L.d_il_ptr, L.d_il_pk, L.d_T64, (const double2*)L.d_out,
                                          (double2*)L.d_in);
     } else if (use8) {
-      // 8 directions per CTA, halved by the tuner
+      // 16 directions per CTA, halved by the tuner
       const bool halfc = (tv == 2);
-      int KC1 = 8 / (halfc ? 2 : 1);
+      int KC1 = 16 / (halfc ? 2 : 1);
       int nk1 = (L.K + KC1 - 1) / KC1;
-      size_t sm1 = ((size_t)144 * KC1 * 4 + (size_t)49 * KC1) * sizeof(double2) + (144 + 64) * sizeof(int);
-      auto kt = halfc ? k_translate1<4> : k_translate1<8>;
+      size_t sm1 = ((size_t)144 * KC1 * NF + (size_t)49 * KC1) * sizeof(double2) + (144 + 64) * sizeof(int);
+      auto kt = halfc ? k_translate1<8> : k_translate1<16>;
       cudaFuncSetAttribute(kt, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
       kt<<<(unsigned)(L.ntile8_ne * nk1), 16 * KC1 * Part<double>::NT, sm1, ts>>>(
           L.K, L.ntile8_x, L.ntile8_ne, L.d_tiles8, L.map_x0, L.map_y0, L.map_w, L.map_h, L.d_boxmap,
@@ -1091,12 +1026,10 @@ static int far_impl(Ctx* c, int R, const double2* x, double2* y, bool accumulate
   };
   // aggregation
   {
-    int nkc = (L0.K + 63) / 64;
-    size_t sm = (size_t)16 * 2 * c->npsi * sizeof(V);
     pbeg(c, st, "aggregate", 0,
          (double)c->p * 2 * c->npsi * R_ * 16 + (double)c->S * c->npsi * 2 * L0.K * es +
-             (double)c->p * L0.K * 4 * R_ * es,
-         32.0 * c->npsi * c->p * L0.K * R_);
+             (double)c->p * L0.K * NF * R_ * es,
+         16.0 * c->npsi * c->p * L0.K * R_);
     // per-particle spectra go through the box sum where boxes hold several
     // particles, or where the tensor cores aggregate displaced particles
     // (the sum then applies the displacement shifts)
@@ -1110,15 +1043,16 @@ static int far_impl(Ctx* c, int R, const double2* x, double2* y, bool accumulate
         return rc;
       }
     } else {
-      int nsub = (16 + std::max(1, 16 / RC) - 1) / std::max(1, 16 / RC);
-      k_aggregate<T><<<(unsigned)(c->ntile * nsub * nkc * nrc), 256, sm, st>>>(
-          L0.K, c->npsi, R, RC, nkc, c->d_tile_shape, c->d_tile_start, c->d_tile_count, c->d_perm, x,
-          (const V*)(f64 ? (void*)c->d_P64 : (void*)c->d_P32), c->d_dshift, c->any_dshift, L0.d_khat,
-          c->k, agg);
+      const int nchunk = (L0.K / 2 + AGC_PAIRS - 1) / AGC_PAIRS;
+      const size_t sm = (size_t)(2 * c->npsi + 8 * AGC_PAIRS) * sizeof(V);
+      k_aggregate<T><<<(unsigned)((long long)c->p * R * nchunk), 2 * AGC_PAIRS, sm, st>>>(
+          L0.K, L0.nph, c->npsi, R, nchunk, c->d_perm, c->d_sid, x,
+          (const V*)(f64 ? (void*)c->d_Pd64 : (void*)c->d_Pd32), c->d_dshift, c->any_dshift, L0.d_khat, c->k,
+          1.0 / c->zeta, agg);
       SMR_LAUNCH(c);
     }
     if (cells) {
-      const long long row = (long long)L0.K * 4 * R;
+      const long long row = (long long)L0.K * NF * R;
       k_cell_sum<T><<<dim3((unsigned)L0.nbox, (unsigned)((row + 255) / 256)), 256, 0, st>>>(
           L0.nbox, row, R, c->d_cell_ptr, c->d_cell_idx, (tc && c->any_dshift) ? 1 : 0, c->d_dshift,
           L0.d_khat, c->k, agg, (V*)L0.d_out);
@@ -1134,8 +1068,8 @@ static int far_impl(Ctx* c, int R, const double2* x, double2* y, bool accumulate
     }
     Level &Lc = c->lev[s], &Lp = c->lev[s + 1];
     pbeg(c, st, "interpolate", s,
-         ((double)Lc.nbox * Lc.K + (double)Lp.nbox * Lp.K) * 4 * R_ * es + 4.0 * Lp.K * es,
-         (double)Lc.nbox * Lp.nth * Lc.nph * 4 * R_ * 16.0 + (double)Lc.nbox * Lp.K * 4 * R_ * 24.0);
+         ((double)Lc.nbox * Lc.K + (double)Lp.nbox * Lp.K) * NF * R_ * es + 4.0 * Lp.K * es,
+         (double)Lc.nbox * Lp.nth * Lc.nph * NF * R_ * 16.0 + (double)Lc.nbox * Lp.K * NF * R_ * 24.0);
     if (!f64 || R > 1 || march_interp(Lc.tune_ip[0]) || Lp.nph * Part<double>::NT > 256 * EM1) {
       int rc = run_interp(c, s, R, f64 ? SMR_PREC_FP64 : SMR_PREC_FP32, st);
       if (rc) return rc;
@@ -1143,7 +1077,7 @@ static int far_impl(Ctx* c, int R, const double2* x, double2* y, bool accumulate
       int TR = std::max(1, std::min(Lp.nth, (256 * EM1) / (Lp.nph * Part<double>::NT)));
       if (Lc.tune_ip[0] == 2) TR = std::max(1, TR / 2);
       int nrt = (Lp.nth + TR - 1) / TR;
-      size_t sm1 = (size_t)TR * Lc.nph * 4 * sizeof(double2);
+      size_t sm1 = (size_t)TR * Lc.nph * NF * sizeof(double2);
       cudaFuncSetAttribute(k_interp1, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
       const unsigned mP = (unsigned)(((1ull << 32) + (unsigned)Lp.nph - 1) / (unsigned)Lp.nph);
       k_interp1<<<(unsigned)(Lp.nbox * nrt), 256, sm1, st>>>(
@@ -1171,9 +1105,9 @@ static int far_impl(Ctx* c, int R, const double2* x, double2* y, bool accumulate
     }
     Level &Lc = c->lev[s], &Lp = c->lev[s + 1];
     pbeg(c, st, "anterpolate", s,
-         ((double)Lp.nbox * Lp.K + 2.0 * Lc.nbox * Lc.K) * 4 * R_ * es + 4.0 * Lp.K * es,
-         (double)Lc.nbox * Lp.nth * Lc.nph * 4 * R_ * 8.0 * 2 * (double)Lp.nph / Lc.nph * 4.0 / 4.0 +
-             (double)Lc.nbox * Lc.K * 4 * R_ * 16.0 * (double)Lp.nth / Lc.nth);
+         ((double)Lp.nbox * Lp.K + 2.0 * Lc.nbox * Lc.K) * NF * R_ * es + 4.0 * Lp.K * es,
+         (double)Lc.nbox * Lp.nth * Lc.nph * NF * R_ * 8.0 * 2 * (double)Lp.nph / Lc.nph * 4.0 / 4.0 +
+             (double)Lc.nbox * Lc.K * NF * R_ * 16.0 * (double)Lp.nth / Lc.nth);
     if (!f64 || R > 1 || march_anterp(Lp, Lc.tune_an[0])) {
       int rc = run_anterp(c, s, R, f64 ? SMR_PREC_FP64 : SMR_PREC_FP32, st);
       if (rc) return rc;
@@ -1182,7 +1116,7 @@ static int far_impl(Ctx* c, int R, const double2* x, double2* y, bool accumulate
       int JC = Lc.ant_JC;
       if (an == 1) JC = std::max(1, JC / 2);
       int njc = (Lc.nph / 2 + JC - 1) / JC;
-      size_t sm1 = (size_t)Lc.ant_GR * 2 * JC * 4 * sizeof(double2);
+      size_t sm1 = (size_t)Lc.ant_GR * 2 * JC * NF * sizeof(double2);
       int thr = (an == 2 || Lc.ant_GR * 2 * JC * (Part<double>::NT / 2) >= 2048) ? 256 : 128;
       auto ka = k_anterp1<0>;
       if (Lc.ant_PM == 8 && Lc.ant_TM == 8) ka = std::max(Lc.ant_PMx, Lc.ant_TMx) <= 7 ? k_anterp1<7> : k_anterp1<8>;
@@ -1197,12 +1131,10 @@ static int far_impl(Ctx* c, int R, const double2* x, double2* y, bool accumulate
   // receive
   if (sd) SMR_CUDA(c, cudaStreamWaitEvent(st, sd->etr[0], 0));
   {
-    int thr = c->npsi * 8;
-    size_t sm = ((size_t)32 * 2 * c->npsi + 32 * 16 * 4) * sizeof(V);
     pbeg(c, st, "receive", 0,
-         (double)c->p * L0.K * 4 * R_ * es + (double)c->S * c->npsi * 2 * L0.K * es +
+         (double)c->p * L0.K * NF * R_ * es + (double)c->S * c->npsi * 2 * L0.K * es +
              (accumulate ? 2.0 : 1.0) * c->p * 2 * c->npsi * R_ * 16,
-         48.0 * c->p * c->npsi * L0.K * R_);
+         16.0 * c->p * c->npsi * L0.K * R_);
     // per-particle incoming spectra where boxes hold several particles, or
     // where the tensor cores receive for displaced particles (the broadcast
     // then applies the displacement shifts)
@@ -1210,7 +1142,7 @@ static int far_impl(Ctx* c, int R, const double2* x, double2* y, bool accumulate
     const bool cells = c->multi || (tc && c->any_dshift);
     const V* inc = (const V*)L0.d_in;
     if (cells) {
-      const long long row = (long long)L0.K * 4 * R;
+      const long long row = (long long)L0.K * NF * R;
       V* part = (V*)c->pspec[f64 ? 0 : 1];
       k_cell_bcast<T><<<dim3((unsigned)c->p, (unsigned)((row + 255) / 256)), 256, 0, st>>>(
           c->p, row, R, c->d_cell_of, (tc && c->any_dshift) ? 1 : 0, c->d_dshift, L0.d_khat, c->k,
@@ -1224,12 +1156,10 @@ static int far_impl(Ctx* c, int R, const double2* x, double2* y, bool accumulate
       return rc;
     }
     if (c->near_ev) SMR_CUDA(c, cudaStreamWaitEvent(st, c->near_ev, 0));
-    int nsub = (16 + std::max(1, 16 / RC) - 1) / std::max(1, 16 / RC);
-    cudaFuncSetAttribute(k_receive<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    k_receive<T><<<(unsigned)(c->ntile * nsub * nrc), thr, sm, st>>>(
-        L0.K, c->npsi, R, RC, c->d_tile_shape, c->d_tile_start, c->d_tile_count, c->d_perm,
-        inc, (const V*)(f64 ? (void*)c->d_P64 : (void*)c->d_P32), L0.d_w, c->d_dshift,
-        c->any_dshift, L0.d_khat, c->k, c->zeta, y, accumulate ? 1 : 0);
+    const int thr = c->npsi * std::max(1, 256 / c->npsi);
+    k_receive<T><<<(unsigned)((long long)c->p * R), thr, (size_t)(4 * RCV_PAIRS + 2 * thr) * sizeof(V), st>>>(
+        L0.K, L0.nph, c->npsi, R, c->d_perm, c->d_sid, inc, (const V*)(f64 ? (void*)c->d_Pm64 : (void*)c->d_Pm32),
+        L0.d_w, c->d_dshift, c->any_dshift, L0.d_khat, c->k, c->zeta, y, accumulate ? 1 : 0);
     SMR_LAUNCH(c);
     pend(c, st);
   }
@@ -1448,6 +1378,7 @@ int ensure_side(Ctx* c, int n) {
     SMR_CUDA(c, cudaStreamCreateWithFlags(&d.nr, cudaStreamNonBlocking));
     SMR_CUDA(c, cudaEventCreateWithFlags(&d.ex, cudaEventDisableTiming));
     SMR_CUDA(c, cudaEventCreateWithFlags(&d.enear, cudaEventDisableTiming));
+    SMR_CUDA(c, cudaEventCreateWithFlags(&d.efork, cudaEventDisableTiming));
     d.eout.assign(32, nullptr);
     d.etr.assign(32, nullptr);
     for (int s = 0; s < 32; ++s) {
@@ -1464,6 +1395,7 @@ void free_side(Ctx* c) {
     if (d.nr) cudaStreamDestroy(d.nr);
     if (d.ex) cudaEventDestroy(d.ex);
     if (d.enear) cudaEventDestroy(d.enear);
+    if (d.efork) cudaEventDestroy(d.efork);
     for (auto e : d.eout) if (e) cudaEventDestroy(e);
     for (auto e : d.etr) if (e) cudaEventDestroy(e);
   }
@@ -1529,6 +1461,7 @@ int run_product(Ctx* c, int R, int prec, const double2* x, double2* y, cudaStrea
     cudaStream_t sj = j ? c->lanes[j].s : st;
     use_lane(c, j);
     c->cur_side = j;
+    c->keep_x = j > 0 || r + nl < R;             // lane 0's last column is the one that stays
     rc = prep_x32(c, 1, prec, xs + (size_t)r * n, sj);
     if (!rc) rc = near_step(c, 1, prec, xs + (size_t)r * n, ys + (size_t)r * n, sj, j);
     if (!rc) rc = far_impl<float>(c, 1, xs + (size_t)r * n, ys + (size_t)r * n, true, sj);
@@ -1536,6 +1469,7 @@ int run_product(Ctx* c, int R, int prec, const double2* x, double2* y, cudaStrea
   }
   use_lane(c, 0);
   c->cur_side = 0;
+  c->keep_x = false;
   c->x32_of = nullptr;
   // every forked lane is joined, also after an error, so that a capture ends cleanly
   for (int j = 1; j < nl; ++j) {
@@ -1622,6 +1556,76 @@ int run_precond(Ctx* c, int R, int prec, const double2* r, double2* z, cudaStrea
   if (prec == SMR_PREC_FP64)
     return bs_impl<double>(c, c->p, R, c->d_pc_ptr, c->d_pc_col, c->d_pc_blk, c->d_Pinv64, r, z, false, st);
   return bs_impl<float>(c, c->p, R, c->d_pc_ptr, c->d_pc_col, c->d_pc_blk, c->d_Pinv32, r, z, false, st);
+}
+
+// current `cur`'s coefficients of x, zeros for the other's
+__global__ void k_one_current(long long n, int run, int cur, const double2* __restrict__ x, double2* __restrict__ o) {
+  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (i < n) o[i] = (int)(i / run & 1) == cur ? x[i] : make_double2(0.0, 0.0);
+}
+
+// A level's spectra of the last product in the four fields (theta and phi of
+// the electric and of the magnetic current's radiation), which the two circular
+// fields do not tell apart: the far pass once more for each current alone.
+int copy_fields(Ctx* c, int level, int kind, double* out) {
+  const int prec = c->spec_prec, R = c->spec_R;
+  const Level& L = c->lev[level];
+  const long long n = (long long)c->p * 2 * c->npsi * R;
+  const size_t elems = (size_t)L.nbox * L.K * NF * R;
+  double2* buf = nullptr;
+  SMR_CUDA(c, cudaDeviceSynchronize());
+  if (cudaMalloc((void**)&buf, 2 * n * sizeof(double2)) != cudaSuccess) {
+    cudaGetLastError();
+    c->err = "out of device memory for a level's fields";
+    return SMR_E_OOM;
+  }
+  int rc = ensure_side(c, 1);
+  std::vector<double2> w[2];
+  std::vector<ProfRec>* prof = c->prof;
+  c->prof = nullptr;
+  c->cur_side = 0;
+  c->keep_x = true;
+  for (int cur = 0; cur < 2 && !rc; ++cur) {
+    w[cur].resize(elems);
+    k_one_current<<<(unsigned)((n + 255) / 256), 256>>>(n, c->npsi * R, cur, c->d_xs[prec == SMR_PREC_FP64 ? 0 : 1], buf);
+    rc = run_far(c, R, prec, buf, buf + n, false, nullptr);
+    cudaError_t e = cudaDeviceSynchronize();
+    const void* src = kind == 0 ? L.d_out : L.d_in;
+    if (e == cudaSuccess && prec == SMR_PREC_FP64) {
+      e = cudaMemcpy(w[cur].data(), src, elems * sizeof(double2), cudaMemcpyDeviceToHost);
+    } else if (e == cudaSuccess) {
+      std::vector<float2> t(elems);
+      e = cudaMemcpy(t.data(), src, elems * sizeof(float2), cudaMemcpyDeviceToHost);
+      for (size_t i = 0; i < elems; ++i) w[cur][i] = make_double2(t[i].x, t[i].y);
+    }
+    if (!rc && e != cudaSuccess) {
+      c->err = std::string("level fields: ") + cudaGetErrorString(e);
+      rc = SMR_E_CUDA;
+    }
+  }
+  c->keep_x = false;
+  c->prof = prof;
+  cudaFree(buf);
+  if (rc) return rc;
+  // electric current: W_+- = B0 -+ j B1; magnetic: W_+- = +-(j / z) (B2 -+ j B3)
+  for (size_t d = 0; d < (size_t)L.nbox * L.K; ++d)
+    for (int r = 0; r < R; ++r) {
+      double* o = out + 2 * (d * 4 * R + r);
+      for (int cur = 0; cur < 2; ++cur) {
+        double2 p = w[cur][d * NF * R + r], q = w[cur][(d * NF + 1) * R + r];
+        if (cur) {
+          p = make_double2(c->zeta * p.y, -c->zeta * p.x);    // -j z W_+
+          q = make_double2(-c->zeta * q.y, c->zeta * q.x);    // +j z W_-
+        }
+        const double2 v[2] = {make_double2(0.5 * (p.x + q.x), 0.5 * (p.y + q.y)),
+                              make_double2(0.5 * (q.y - p.y), -0.5 * (q.x - p.x))};
+        for (int f = 0; f < 2; ++f) {
+          o[2 * (size_t)(2 * cur + f) * R] = v[f].x;
+          o[2 * (size_t)(2 * cur + f) * R + 1] = v[f].y;
+        }
+      }
+    }
+  return SMR_OK;
 }
 
 }  // namespace smr

@@ -143,6 +143,23 @@ __global__ void k_patterns(int S, int npsi, int Q, int K0, const double* __restr
   P[(((size_t)s * npsi + n) * 2 + 1) * K0 + kk] = ap;
 }
 
+// Pd[s][f][n][q] = Pm[s][f][q][n] = P_th +- j P_ph of direction q, the first half of
+// the grid: direction q's opposite is in the other half, and its pattern is the
+// conjugate (real modes; theta unit vectors of opposite directions are equal, phi ones
+// opposite)
+__global__ void k_circular(long long n, int npsi, int K0, const double2* __restrict__ P, double2* __restrict__ Pd,
+                           double2* __restrict__ Pm) {
+  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (t >= n) return;
+  const int K2 = K0 / 2, q = (int)(t % K2), m = (int)(t / K2 % npsi);
+  const long long sf = t / ((long long)K2 * npsi);
+  const double2* p = P + ((sf / 2 * npsi + m) * 2) * K0 + q;
+  const double2 a = p[0], b = p[K0];
+  const double2 v = sf & 1 ? make_double2(a.x + b.y, a.y - b.x) : make_double2(a.x - b.y, a.y + b.x);
+  Pd[t] = v;
+  Pm[(sf * K2 + q) * npsi + m] = v;
+}
+
 int build_patterns(Ctx* c) {
   Level& L0 = c->lev[0];
   long long n = (long long)c->S * c->npsi * 2 * L0.K;
@@ -153,7 +170,19 @@ int build_patterns(Ctx* c) {
   k_patterns<<<(unsigned)((tot + 127) / 128), 128>>>(c->S, c->npsi, c->Q, L0.K, c->d_modes, c->d_rq,
                                                     L0.d_khat, c->k, c->d_P64);
   SMR_LAUNCH(c);
-  return copy32(c, c->d_P64, &c->d_P32, n);
+  // the circular patterns P_th +- j P_ph over one direction of each opposite pair,
+  // directions fastest for the aggregation, modes fastest for the receive
+  const int K2 = L0.K / 2;
+  const long long n2 = (long long)c->S * 2 * c->npsi * K2;
+  for (double2** q : {&c->d_Pd64, &c->d_Pm64}) {
+    if (*q) cudaFree(*q);
+    *q = nullptr;
+    SMR_CUDA(c, cudaMalloc((void**)q, n2 * sizeof(double2)));
+  }
+  k_circular<<<(unsigned)((n2 + 255) / 256), 256>>>(n2, c->npsi, L0.K, c->d_P64, c->d_Pd64, c->d_Pm64);
+  SMR_LAUNCH(c);
+  int rc = copy32(c, c->d_Pd64, &c->d_Pd32, n2);
+  return rc ? rc : copy32(c, c->d_Pm64, &c->d_Pm32, n2);
 }
 
 // ------------------------------------------------------------------ translation (Eq. 23)

@@ -1,11 +1,11 @@
 // Dense per-shape contractions of the FP32 product on the 5th-generation
 // tensor cores (tcgen05 MMA, accumulators in tensor memory).
 //
-// Receive (Eqs. 24-25) with the combination of the four incoming fields
+// Receive (Eqs. 24-25) with the combination of the two incoming fields
 // folded into a per-shape coefficient matrix is a real GEMM
 //   y[mu][m'] += sum_k' A_s[m'][k'] B[mu][k'],
 //   m' = (current, mode, re/im)          (4 N_psi <= 128 rows: one MMA M tile)
-//   k' = (direction, field, re/im)       (8 K_0: the level-0 incoming spectrum
+//   k' = (direction, field, re/im)       (4 K_0: the level-0 incoming spectrum
 //                                          of particle mu, contiguous in HBM)
 // with particles of one shape as the N dimension.  FP32 accuracy comes from
 // split TF32: a = a_hi + a_lo with a_hi = tf32(a), a_lo = tf32(a - a_hi), and
@@ -186,11 +186,11 @@ __device__ __forceinline__ void tmem_sum32(uint32_t t, float* v) {
 // CTA (tile, s) of a grid with several s takes chunks s nK / S .. (s + 1) nK / S
 // and writes its partial rows (no accumulation) to y + s ystride.
 // A = coefficient images [nK][hi | lo][128 rows][32] (swizzled), one per
-// tile (tshape); in0 = B rows [.][K8] (FP32), gathered by perm; y [.][M4]
+// tile (tshape); in0 = B rows [.][KB] (FP32), gathered by perm; y [.][M4]
 // (FP64), rows yperm.  Receive: A per shape, in0 the level-0 incoming
 // spectra, perm = yperm = particles.  Near: A per block, in0 = x (FP32),
 // perm = nu, yperm = mu.
-__device__ __forceinline__ void ld_chunk(const float* __restrict__ in0, int K8, const int* mus, int c, int tid,
+__device__ __forceinline__ void ld_chunk(const float* __restrict__ in0, int KB, const int* mus, int c, int tid,
                                          float4* r) {
 #pragma unroll
   for (int j = 0; j < TC_PQ; ++j) {
@@ -198,13 +198,13 @@ __device__ __forceinline__ void ld_chunk(const float* __restrict__ in0, int K8, 
     int mu = mus[row], kk = c * TC_KC + 4 * q;
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
     if (mu >= 0) {
-      const float* b = in0 + (size_t)mu * K8 + kk;
-      if (kk + 3 < K8) {
+      const float* b = in0 + (size_t)mu * KB + kk;
+      if (kk + 3 < KB) {
         v = *reinterpret_cast<const float4*>(b);
       } else {
-        if (kk < K8) v.x = b[0];
-        if (kk + 1 < K8) v.y = b[1];
-        if (kk + 2 < K8) v.z = b[2];
+        if (kk < KB) v.x = b[0];
+        if (kk + 1 < KB) v.y = b[1];
+        if (kk + 2 < KB) v.z = b[2];
       }
     }
     r[j] = v;
@@ -227,7 +227,7 @@ __device__ __forceinline__ void st_chunk(unsigned char* S, int tid, const float4
 }
 
 template <typename YT>
-__global__ void __launch_bounds__(TC_PT + 32, 1) k_receive_tc(int nKall, int K8, int M4, const int* __restrict__ tshape,
+__global__ void __launch_bounds__(TC_PT + 32, 1) k_receive_tc(int nKall, int KB, int M4, const int* __restrict__ tshape,
                                                        const int* __restrict__ tstart,
                                                        const int* __restrict__ tcount,
                                                        const int* __restrict__ perm,
@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(TC_PT + 32, 1) k_receive_tc(int nKall, int K8,
     float4 r[TC_PF][TC_PQ];
 #pragma unroll
     for (int b = 0; b < TC_PF; ++b)
-      if (b < nK) ld_chunk(in0, K8, mus, cbeg + b, tid, r[b]);
+      if (b < nK) ld_chunk(in0, KB, mus, cbeg + b, tid, r[b]);
 #pragma unroll 1
     for (int cb = 0; cb < nK && !bad; cb += TC_PF) {
 #pragma unroll
@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(TC_PT + 32, 1) k_receive_tc(int nKall, int K8,
             __syncwarp();
             if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(fullB(st)) : "memory");
             // the next loads go out after the fence, so it does not wait for them
-            if (c + TC_PF < nK) ld_chunk(in0, K8, mus, cbeg + c + TC_PF, tid, r[b]);
+            if (c + TC_PF < nK) ld_chunk(in0, KB, mus, cbeg + c + TC_PF, tid, r[b]);
           }
         }
       }
@@ -406,12 +406,7 @@ __global__ void __launch_bounds__(TC_PT + 32, 1) k_receive_tc(int nKall, int K8,
 // Aggregation on the tensor cores (Eq. 26 patterns times coefficients):
 //   out0[mu][(direction, field, re/im)] = sum_k' A_s[.][k'] x[mu][k'],
 //   k' = (current, mode, re/im) (4 N_psi <= 128: the coefficients of mu).
-// A field belongs to one current, so the rows are taken current by current:
-// M tile t covers current t & 1 and the rows (direction, component, re/im)
-// [128 (t >> 1), 128 (t >> 1) + 128) of it, and reads only that current's
-// K chunks (half of K).  Consecutive tiles write the two halves of the same
-// output sectors.
-// CTA = up to 128 particles of one shape and a range of M tile pairs, 16 worker
+// CTA = up to 128 particles of one shape and a range of M tiles, 16 worker
 // warps and a control warp.  The workers load the tile's coefficients once
 // (split TF32, swizzled, resident for the whole CTA) and then drain the
 // accumulators; one control thread streams the coefficient images of the M
@@ -449,10 +444,11 @@ __global__ void __launch_bounds__(TC_PT + 32, 1) k_aggregate_tc(int nMTall, int 
   auto aDone = [&](int st) { return saddr(bars + AG_NS + st); };
   auto accFull = [&](int b) { return saddr(bars + 2 * AG_NS + b); };
   auto accEmpty = [&](int b) { return saddr(bars + 2 * AG_NS + 2 + b); };
-  const size_t tileA = (size_t)nKc * 2 * 128 * TC_KC;                   // floats per M tile image
-  // this CTA's M tiles: whole pairs (the two currents of 128 rows)
-  const int tb = 2 * (int)((long long)(nMTall / 2) * blockIdx.y / gridDim.y);
-  const int nMT = 2 * (int)((long long)(nMTall / 2) * (blockIdx.y + 1) / gridDim.y) - tb;
+  const size_t tileA = (size_t)2 * nKc * 2 * 128 * TC_KC;               // floats per M tile image
+  // this CTA's M tiles
+  const int tb = (int)((long long)nMTall * blockIdx.y / gridDim.y);
+  const int nMT = (int)((long long)nMTall * (blockIdx.y + 1) / gridDim.y) - tb;
+  const int nKt = 2 * nKc;                            // K chunks of both currents
   const float* As = A + ((size_t)s * nMTall + tb) * tileA;
   if (warp == 0) tmem_alloc(saddr(slot), 4 * TC_NP);
   if (tid == 0) {
@@ -472,10 +468,10 @@ __global__ void __launch_bounds__(TC_PT + 32, 1) k_aggregate_tc(int nMTall, int 
   __syncthreads();
   tc_after();
   const uint32_t tmem = *slot;
-  const int total = nMT * nKc;                        // coefficient chunks in order (M tile, K chunk)
+  const int total = nMT * nKt;                        // coefficient chunks in order (M tile, K chunk)
   int ncopy = 0;                                      // chunks whose bulk copy was issued (control thread)
   auto copy_chunk = [&](int g) {
-    const int t = g / nKc, c = g % nKc, st = g % AG_NS;
+    const int t = g / nKt, c = g % nKt, st = g % AG_NS;
     mbar_expect_tx(aFull(st), 2 * TC_ABYTES);
     bulk_g2s(ar0 + st * 2 * TC_ABYTES, As + t * tileA + (size_t)c * 2 * 128 * TC_KC, 2 * TC_ABYTES, aFull(st));
     ++ncopy;
@@ -550,8 +546,7 @@ __global__ void __launch_bounds__(TC_PT + 32, 1) k_aggregate_tc(int nMTall, int 
         break;
       }
       tc_after();
-      const int rc = ((t + tb) >> 1) * 128 + q4 * 32 + lane;   // (direction, component, re/im) of current t & 1
-      const int oi = (rc >> 2) * 8 + (t & 1) * 4 + (rc & 3);
+      const int rc = (t + tb) * 128 + q4 * 32 + lane;  // (direction, field, re/im)
       if (g * 32 < cnt) {                              // uniform per warp
         float v[32];
         tmem_sum32<2>(tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(b * 2 * TC_NP + g * 32), v);
@@ -559,7 +554,7 @@ __global__ void __launch_bounds__(TC_PT + 32, 1) k_aggregate_tc(int nMTall, int 
 #pragma unroll
           for (int j = 0; j < 32; ++j) {
             int col = g * 32 + j;
-            if (col < cnt) out0[(size_t)mus[col] * (2 * K4) + oi] = v[j];
+            if (col < cnt) out0[(size_t)mus[col] * K4 + rc] = v[j];
           }
         }
       }
@@ -579,7 +574,7 @@ __global__ void __launch_bounds__(TC_PT + 32, 1) k_aggregate_tc(int nMTall, int 
       if (t >= 2 && !mbar_wait_or_abort(accEmpty(b), ((t >> 1) - 1) & 1, spin, abort_flag)) { bad = true; break; }
       tc_after();
       const uint32_t d = tmem + (uint32_t)(b * 2 * TC_NP);
-      for (int c = 0; c < nKc; ++c) {
+      for (int c = 0; c < nKt; ++c) {
         const int st = g % AG_NS;
         if (!mbar_wait_or_abort(aFull(st), (g / AG_NS) & 1, spin, abort_flag)) { bad = true; break; }
         tc_after();
@@ -587,8 +582,7 @@ __global__ void __launch_bounds__(TC_PT + 32, 1) k_aggregate_tc(int nMTall, int 
 #pragma unroll
         for (int k = 0; k < TC_KC / 8; ++k) {
           uint64_t ah = sdesc_sw128(Sa + 32 * k), al = sdesc_sw128(Sa + TC_ABYTES + 32 * k);
-          const int cb = (t & 1) * nKc + c;            // this current's K chunk of the coefficients
-          uint64_t bh = sdesc_sw128(bh0 + cb * TC_BBYTES + 32 * k), bl = sdesc_sw128(bl0 + cb * TC_BBYTES + 32 * k);
+          uint64_t bh = sdesc_sw128(bh0 + c * TC_BBYTES + 32 * k), bl = sdesc_sw128(bl0 + c * TC_BBYTES + 32 * k);
           mma_tf32(d, ah, bh, idesc, (c > 0 || k > 0) ? 1u : 0u);
           mma_tf32(d + TC_NP, ah, bl, idesc, (c > 0 || k > 0) ? 1u : 0u);
           mma_tf32(d + TC_NP, al, bh, idesc, 1u);
@@ -643,34 +637,31 @@ float tf32_host(float x) {
 
 // Coefficient images of the tensor-core receive for every shape, from the
 // FP64 patterns: row m' = (current, mode, re/im), column k' = (direction,
-// field, re/im); entry = the real form of -j k w_k c(current, field) P(mode,
-// field's component, k), c from Eqs. 24-25 (zeta B0 + B3, zeta B1 - B2,
-// -B1 + B2/zeta, B0 + B3/zeta for the electric rows and the magnetic ones).
+// field, re/im); entry = the real form of w_k P_+-(mode, k) times -j k zeta / 2
+// for the electric rows and -+ k / 2 for the magnetic ones (k_receive).
 int build_tc(Ctx* c) {
   c->tc_ready = false;
   Level& L0 = c->lev[0];
   int npsi = c->npsi, K0 = L0.K, S = c->S;
-  int M4 = 4 * npsi, K8 = 8 * K0;
+  int M4 = 4 * npsi, K4 = 4 * K0;
   if (M4 > 128) return SMR_OK;                       // more than one M tile: CUDA-core paths
-  int nK = (K8 + TC_KC - 1) / TC_KC;
+  int nK = (K4 + TC_KC - 1) / TC_KC;
   size_t nP = (size_t)S * npsi * 2 * K0;
   std::vector<double2> P(nP);
   SMR_CUDA(c, cudaMemcpy(P.data(), c->d_P64, nP * sizeof(double2), cudaMemcpyDeviceToHost));
   std::vector<float> img((size_t)S * nK * 2 * 128 * TC_KC, 0.f);
   typedef std::complex<double> cx;
-  const cx mjk(0.0, -c->k);
-  const double z = c->zeta, iz = 1.0 / c->zeta;
   for (int s = 0; s < S; ++s)
     for (int row = 0; row < M4; ++row) {
       int cur = row / (2 * npsi), m = (row / 2) % npsi, ro = row & 1;
-      for (int kp = 0; kp < K8; ++kp) {
-        int k = kp / 8, f = (kp / 2) & 3, ri = kp & 1;
+      for (int kp = 0; kp < K4; ++kp) {
+        int k = kp / 4, f = (kp / 2) & 1, ri = kp & 1;
         const double2 pt = P[(((size_t)s * npsi + m) * 2 + 0) * K0 + k];
         const double2 pp = P[(((size_t)s * npsi + m) * 2 + 1) * K0 + k];
-        cx Pt(pt.x, pt.y), Pp(pp.x, pp.y), cf;
-        if (cur == 0) cf = f == 0 ? z * Pt : f == 1 ? z * Pp : f == 2 ? -Pp : Pt;
-        else cf = f == 0 ? Pp : f == 1 ? -Pt : f == 2 ? iz * Pt : iz * Pp;
-        cf *= mjk * L0.w[k];
+        // y_e = -jk z/2 (Y_+ + Y_-), y_m = -k/2 (Y_+ - Y_-)
+        const double sf = f ? -1.0 : 1.0;
+        const cx Pf = cx(pt.x, pt.y) + cx(0.0, sf) * cx(pp.x, pp.y);
+        const cx cf = (cur == 0 ? cx(0.0, -0.5 * c->k * c->zeta) : cx(-0.5 * sf * c->k, 0.0)) * L0.w[k] * Pf;
         double v = ro == 0 ? (ri == 0 ? cf.real() : -cf.imag()) : (ri == 0 ? cf.imag() : cf.real());
         float hi = tf32_host((float)v);
         float lo = tf32_host((float)(v - (double)hi));
@@ -682,24 +673,28 @@ int build_tc(Ctx* c) {
       }
     }
   // aggregation images: row m' = (direction, field, re/im), column k' =
-  // (current, mode, re/im); entry = the real form of conj(P(mode, field's
-  // component, direction)) where the field's current matches, else 0
-  int K4 = 4 * K0, npsi2 = 2 * npsi;
-  int nKc = (npsi2 + TC_KC - 1) / TC_KC, nMT = 2 * ((K4 + 127) / 128);
+  // (current, mode, re/im), each current padded to nKc chunks; entry = the real
+  // form of conj(P_+-(mode, direction)) times 1 or +-j / zeta
+  int npsi2 = 2 * npsi;
+  int nKc = (npsi2 + TC_KC - 1) / TC_KC, nMT = (K4 + 127) / 128;
   std::vector<float> agg;
   if (2 * nKc <= AG_KCMAX && npsi % 2 == 0) {
-    size_t tileA = (size_t)nKc * 2 * 128 * TC_KC;
+    size_t tileA = (size_t)2 * nKc * 2 * 128 * TC_KC;
     agg.assign((size_t)S * nMT * tileA, 0.f);
     for (int s = 0; s < S; ++s)
       for (int t = 0; t < nMT; ++t)
         for (int rl = 0; rl < 128; ++rl) {
-          int rc = (t >> 1) * 128 + rl;
+          int rc = t * 128 + rl;
           if (rc >= K4) break;
-          int k = rc / 4, comp = (rc / 2) & 1, ro = rc & 1;
-          for (int kl = 0; kl < npsi2; ++kl) {
-            int n = kl / 2, ri = kl & 1;
-            const double2 pv = P[(((size_t)s * npsi + n) * 2 + comp) * K0 + k];
-            double v = ro == 0 ? (ri == 0 ? pv.x : pv.y) : (ri == 0 ? -pv.y : pv.x);
+          int k = rc / 4, ro = rc & 1;
+          const double sf = rc & 2 ? -1.0 : 1.0;
+          for (int kp = 0; kp < 2 * npsi2; ++kp) {
+            int cur = kp / npsi2, n = kp % npsi2 / 2, ri = kp & 1, kl = cur * nKc * TC_KC + kp % npsi2;
+            const double2 pt = P[(((size_t)s * npsi + n) * 2 + 0) * K0 + k];
+            const double2 pp = P[(((size_t)s * npsi + n) * 2 + 1) * K0 + k];
+            cx cf = std::conj(cx(pt.x, pt.y) + cx(0.0, sf) * cx(pp.x, pp.y));
+            if (cur) cf *= cx(0.0, sf / c->zeta);
+            double v = ro == 0 ? (ri == 0 ? cf.real() : -cf.imag()) : (ri == 0 ? cf.imag() : cf.real());
             float hi = tf32_host((float)v);
             float lo = tf32_host((float)(v - (double)hi));
             int ch = kl / TC_KC, kk = kl % TC_KC, q = kk >> 2, e = kk & 3;
@@ -725,13 +720,13 @@ int build_tc(Ctx* c) {
   if (!agg.empty()) {
     if ((rc = upload(c, &c->d_tc_agg, agg))) return rc;
     c->tc_nMT = nMT;
-    // CTAs along the M tile pairs of a particle tile, the number that finishes
+    // CTAs along the M tiles of a particle tile, the number that finishes
     // first: a CTA costs its M tiles plus about three for its coefficients
-    // (1,600 particles in 18 tiles: one 32 us, eight 20.6 us)
-    const int pairs = nMT / 2, ntile = (int)tsh.size();
+    // (1,600 particles in 18 tiles, 16 M tiles then: one 32 us, eight 20.6 us)
+    const int ntile = (int)tsh.size();
     long long cost = -1;
-    for (int m = 1; m <= pairs; ++m) {
-      const long long t = ((long long)ntile * m + 151) / 152 * (2 * ((pairs + m - 1) / m) + 3);
+    for (int m = 1; m <= nMT; ++m) {
+      const long long t = ((long long)ntile * m + 151) / 152 * ((nMT + m - 1) / m + 3);
       if (cost < 0 || t < cost) {
         cost = t;
         c->tc_nmsplit = m;
@@ -796,13 +791,13 @@ __global__ void k_receive_sum(long long n4, int S, const float4* __restrict__ pa
 
 // ready: an event the first write of y waits for (null: none)
 int run_receive_tc(Ctx* c, const float2* in0, double2* y, bool accumulate, cudaEvent_t ready, cudaStream_t st) {
-  const int S = c->tc_nsplit, K8 = 8 * c->lev[0].K, M4 = 4 * c->npsi;
+  const int S = c->tc_nsplit, KB = 4 * c->lev[0].K, M4 = 4 * c->npsi;
   const float* B = reinterpret_cast<const float*>(in0);
   if (S == 1) {
     if (ready) SMR_CUDA(c, cudaStreamWaitEvent(st, ready, 0));
     cudaFuncSetAttribute(k_receive_tc<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM);
     k_receive_tc<double><<<(unsigned)c->tc_ntile, TC_PT + 32, TC_SMEM, st>>>(
-        c->tc_nK, K8, M4, c->d_tc_shape, c->d_tc_start, c->d_tc_count, c->d_tc_perm, c->d_tc_perm, c->d_tc_rec, B,
+        c->tc_nK, KB, M4, c->d_tc_shape, c->d_tc_start, c->d_tc_count, c->d_tc_perm, c->d_tc_perm, c->d_tc_rec, B,
         reinterpret_cast<double*>(y), 0, accumulate ? 1 : 0, c->tc_spin, c->d_tc_err);
     SMR_LAUNCH(c);
     return SMR_OK;
@@ -810,7 +805,7 @@ int run_receive_tc(Ctx* c, const float2* in0, double2* y, bool accumulate, cudaE
   const size_t n = (size_t)c->p * M4;
   cudaFuncSetAttribute(k_receive_tc<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM);
   k_receive_tc<float><<<dim3(c->tc_ntile, S), TC_PT + 32, TC_SMEM, st>>>(
-      c->tc_nK, K8, M4, c->d_tc_shape, c->d_tc_start, c->d_tc_count, c->d_tc_perm, c->d_tc_perm, c->d_tc_rec, B,
+      c->tc_nK, KB, M4, c->d_tc_shape, c->d_tc_start, c->d_tc_count, c->d_tc_perm, c->d_tc_perm, c->d_tc_rec, B,
       c->d_tc_part, n, 0, c->tc_spin, c->d_tc_err);
   SMR_LAUNCH(c);
   if (ready) SMR_CUDA(c, cudaStreamWaitEvent(st, ready, 0));

@@ -13,6 +13,14 @@
 
 namespace smr {
 
+// Fields of a direction's spectrum.  A particle's radiation has four, the theta
+// and phi components of both currents' (B0, B1 electric, B2, B3 magnetic), and the
+// receive takes them in two combinations only, v = B0 + B3 / z and u = -B1 + B2 / z
+// (Eqs. 24-25).  The product carries the circular ones, W_+- = v +- j u: every step
+// between is the same linear map for all fields, the patterns of the aggregation and
+// the receive become P_th +- j P_ph, and the two never mix.
+constexpr int NF = 2;
+
 typedef std::complex<double> cd;
 
 // ------------------------------------------------------------------ host math
@@ -107,7 +115,6 @@ struct Level {
   // with the weights of four child rows
   double2* d_shiftp64 = nullptr;
   float2* d_shiftp32 = nullptr;
-  float2* d_shiftw32 = nullptr;          // [K_p][4] the same as weight pairs (re, re), (im, im)
   int* d_mi_vlast = nullptr;
   int* d_ma_ptr = nullptr;
   int* d_ma_ent = nullptr;
@@ -212,7 +219,10 @@ struct Ctx {
   double* d_rq = nullptr;               // [S][Q][4]: point xyz, weight
   // patterns [S][npsi][2][K0]
   double2* d_P64 = nullptr;
-  float2* d_P32 = nullptr;
+  // circular patterns P_th +- j P_ph, half of the directions: [S][2][npsi][K0 / 2]
+  // and [S][2][K0 / 2][npsi]
+  double2 *d_Pd64 = nullptr, *d_Pm64 = nullptr;
+  float2 *d_Pd32 = nullptr, *d_Pm32 = nullptr;
   // particles
   int* d_sid = nullptr;
   std::vector<int> arr;                 // [p] array id of each particle
@@ -264,6 +274,8 @@ struct Ctx {
   // work buffers
   int buf_R[2] = {0, 0};
   int spec_R = 0, spec_prec = -1;
+  double2* d_xs[2] = {nullptr, nullptr}; // per precision: the coefficients the spectra belong to
+  bool keep_x = false;                   // a product that leaves d_xs alone
   double2* d_tmp = nullptr;             // [N][R] scratch for split products
   size_t tmp_elems = 0;
   // solver scratch
@@ -287,7 +299,7 @@ struct Ctx {
   uint32_t tc_spin = 1u << 24;            // polling limit of the pipeline waits (smr_set_wait_limit)
   bool tc_agg_ready = false;
   int tc_nMT = 0, tc_nKc = 0;
-  int tc_nmsplit = 1;                     // CTAs along a tile's M tile pairs
+  int tc_nmsplit = 1;                     // CTAs along a tile's M tiles
   float* d_tc_agg = nullptr;              // [S][M tiles][K chunks][hi | lo][128][32] aggregation images
   // tensor cores for aggregation / receive chosen by smr_autotune (-1: not tuned)
   int tune_tc_agg = -1, tune_tc_rec = -1, tune_tc_near = -1;
@@ -330,7 +342,7 @@ struct Ctx {
   // translations, one for the near product, and the events that order them
   struct Side {
     cudaStream_t tr = nullptr, nr = nullptr;
-    cudaEvent_t ex = nullptr, enear = nullptr;
+    cudaEvent_t ex = nullptr, enear = nullptr, efork = nullptr;
     std::vector<cudaEvent_t> eout, etr;   // per level: outgoing spectra ready, translation done
   };
   std::vector<Side> side;
@@ -405,7 +417,7 @@ inline void pend(Ctx* c, cudaStream_t st) {
 
 // ------------------------------------------------------------------ setup (k_setup.cu)
 int build_modes(Ctx* c);          // d_modes, d_rq (host evaluation, upload)
-int build_patterns(Ctx* c);       // d_P64 / d_P32 on the GPU (FP64)
+int build_patterns(Ctx* c);       // d_P64, d_Pd* and d_Pm* on the GPU (FP64)
 int build_translations(Ctx* c);   // per level d_T64 / d_T32 on the GPU (FP64)
 int build_near(Ctx* c);           // d_B64 / d_B32 on the GPU (FP64) + self blocks
 int launch_rhs(Ctx* c, int R, const double* d_khat, const double2* d_pol, double2* b,
@@ -415,6 +427,8 @@ int launch_rhs(Ctx* c, int R, const double* d_khat, const double2* d_pol, double
 int launch_rhs_arrays(Ctx* c, const double* d_khat, const double2* d_pol, double2* b, cudaStream_t st);
 int launch_rhs_scratch(Ctx* c, int R, const double* d_khat, const double2* d_pol, double2* Sv,
                        double2* b, cudaStream_t st);
+
+int copy_fields(Ctx* c, int level, int kind, double* out);   // k_mlfma.cu
 
 // ------------------------------------------------------------------ fields (k_fields.cu)
 int launch_far_field(Ctx* c, int R, const double2* x, int nd, const double* d_dirs,
