@@ -159,15 +159,16 @@ __global__ void __launch_bounds__(256) k_gs_dot(int J, long long n, const double
     long long i = i0 + 32 * q;
     wr[q] = (full || i < n) ? w[i] : make_double2(0, 0);
   }
-  if (with_norm) {
+  if (with_norm && blockIdx.y == 0) {
     double s = 0;
 #pragma unroll
     for (int q = 0; q < GS_RPL; ++q) s += wr[q].x * wr[q].x + wr[q].y * wr[q].y;
     s = warp_sum(s);
     if (lane == 0) part[(size_t)J * nseg + g] = make_double2(s, 0);
   }
-  int j = 0;
-  for (; j + 2 <= J; j += 2) {
+  const int G = gridDim.y, per = 2 * (((J + 1) / 2 + G - 1) / G), j1 = min(J, per * ((int)blockIdx.y + 1));
+  int j = per * blockIdx.y;
+  for (; j + 2 <= j1; j += 2) {
     const double2* v0 = V + (size_t)j * ldv + i0;
     const double2* v1 = v0 + ldv;
     double2 a[GS_RPL], b[GS_RPL];
@@ -202,7 +203,7 @@ __global__ void __launch_bounds__(256) k_gs_dot(int J, long long n, const double
       part[(size_t)(j + 1) * nseg + g] = make_double2(bx, by);
     }
   }
-  if (j < J) {
+  if (j < j1) {
     const double2* v0 = V + (size_t)j * ldv + i0;
     double ax = 0, ay = 0;
 #pragma unroll
@@ -218,58 +219,51 @@ __global__ void __launch_bounds__(256) k_gs_dot(int J, long long n, const double
 }
 
 // w += sign * sum_j V_j h[j] on the warp's rows; with part_norm, also
-// part_norm[g] = sum |w_new|^2 over those rows.
+// part_norm[g] = sum |w_new|^2 over those rows.  A lane holds RPL rows and reads
+// 16 / RPL basis vectors at a time.
+template <int RPL>
 __global__ void __launch_bounds__(256) k_gs_axpy(int J, long long n, const double2* __restrict__ V,
                                                  long long ldv, const double2* __restrict__ h,
                                                  double2* __restrict__ w, double sign,
                                                  double2* __restrict__ part_norm, int nseg) {
+  constexpr int JU = 16 / RPL, SEG = 32 * RPL;
   int g = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
   int lane = threadIdx.x & 31;
   if (g >= nseg) return;
-  long long i0 = (long long)g * GS_SEG + lane;
-  bool full = (long long)(g + 1) * GS_SEG <= n;
-  double2 acc[GS_RPL];
+  long long i0 = (long long)g * SEG + lane;
+  bool full = (long long)(g + 1) * SEG <= n;
+  double2 acc[RPL];
 #pragma unroll
-  for (int q = 0; q < GS_RPL; ++q) acc[q] = make_double2(0, 0);
+  for (int q = 0; q < RPL; ++q) acc[q] = make_double2(0, 0);
+  auto ld = [&](int jj, int q) {
+    return full || i0 + 32 * q < n ? V[(size_t)jj * ldv + i0 + 32 * q] : make_double2(0, 0);
+  };
+  auto add = [&](double2& o, double2 a, double2 c0) {
+    o.x += a.x * c0.x - a.y * c0.y;
+    o.y += a.x * c0.y + a.y * c0.x;
+  };
   int j = 0;
-  for (; j + 2 <= J; j += 2) {
-    const double2* v0 = V + (size_t)j * ldv + i0;
-    const double2* v1 = v0 + ldv;
-    double2 a[GS_RPL], b[GS_RPL];
-    if (full) {
+  for (; j + JU <= J; j += JU) {
+    double2 a[JU][RPL];
 #pragma unroll
-      for (int q = 0; q < GS_RPL; ++q) {
-        a[q] = v0[32 * q];
-        b[q] = v1[32 * q];
-      }
-    } else {
+    for (int u = 0; u < JU; ++u)
 #pragma unroll
-      for (int q = 0; q < GS_RPL; ++q) {
-        bool in = i0 + 32 * q < n;
-        a[q] = in ? v0[32 * q] : make_double2(0, 0);
-        b[q] = in ? v1[32 * q] : make_double2(0, 0);
-      }
-    }
-    double2 c0 = h[j], c1 = h[j + 1];
+      for (int q = 0; q < RPL; ++q) a[u][q] = ld(j + u, q);
 #pragma unroll
-    for (int q = 0; q < GS_RPL; ++q) {
-      acc[q].x += a[q].x * c0.x - a[q].y * c0.y + b[q].x * c1.x - b[q].y * c1.y;
-      acc[q].y += a[q].x * c0.y + a[q].y * c0.x + b[q].x * c1.y + b[q].y * c1.x;
+    for (int u = 0; u < JU; ++u) {
+      const double2 c0 = h[j + u];
+#pragma unroll
+      for (int q = 0; q < RPL; ++q) add(acc[q], a[u][q], c0);
     }
   }
-  if (j < J) {
-    const double2* v0 = V + (size_t)j * ldv + i0;
-    double2 c0 = h[j];
+  for (; j < J; ++j) {
+    const double2 c0 = h[j];
 #pragma unroll
-    for (int q = 0; q < GS_RPL; ++q) {
-      double2 a = (full || i0 + 32 * q < n) ? v0[32 * q] : make_double2(0, 0);
-      acc[q].x += a.x * c0.x - a.y * c0.y;
-      acc[q].y += a.x * c0.y + a.y * c0.x;
-    }
+    for (int q = 0; q < RPL; ++q) add(acc[q], ld(j, q), c0);
   }
   double s = 0;
 #pragma unroll
-  for (int q = 0; q < GS_RPL; ++q) {
+  for (int q = 0; q < RPL; ++q) {
     long long i = i0 + 32 * q;
     if (full || i < n) {
       double2 o = w[i];
@@ -319,13 +313,22 @@ __global__ void k_gs_final(int nseg, const double2* __restrict__ part, int na, d
 static inline int gs_nseg(long long n) { return (int)((n + GS_SEG - 1) / GS_SEG); }
 static inline unsigned gs_grid(int nseg) { return (unsigned)((nseg + 7) / 8); }
 
+// CTAs along the basis vectors of an inner-product pass: as many as make two CTAs an
+// SM, at most one per `most` units.  A solve of 1,600 particles, 107 steps on an FP32
+// basis: 9.6 ms of Gram-Schmidt with 25 CTAs for all vectors, 5.3 with the split and
+// with one row pair a lane in the update below 152 CTAs of eight
+static inline unsigned gs_split(unsigned ctas, int most) {
+  return std::max(1u, std::min((unsigned)std::max(1, most), 304u / std::max(1u, ctas)));
+}
+
 // h[0..J) = V^H w and, when d_norm is given, *d_norm = ||w||^2 (one pass).
 static int gs_dot(Ctx* c, int J, long long n, const double2* V, long long ldv, const double2* w,
                   double2* d_h, double2* d_norm, double2* d_part, cudaStream_t st) {
   int nseg = gs_nseg(n);
   int rows = J + (d_norm ? 1 : 0);
   if (rows == 0) return SMR_OK;
-  k_gs_dot<<<gs_grid(nseg), 256, 0, st>>>(J, n, V, ldv, w, d_part, nseg, d_norm ? 1 : 0);
+  const dim3 grid(gs_grid(nseg), gs_split(gs_grid(nseg), (J + 1) / 2));
+  k_gs_dot<<<grid, 256, 0, st>>>(J, n, V, ldv, w, d_part, nseg, d_norm ? 1 : 0);
   SMR_LAUNCH(c);
   k_gs_final<<<rows, 256, 0, st>>>(nseg, d_part, J, d_h, d_norm, nullptr);
   SMR_LAUNCH(c);
@@ -335,8 +338,11 @@ static int gs_dot(Ctx* c, int J, long long n, const double2* V, long long ldv, c
 // w += sign V h and, when d_norm is given, *d_norm = ||w_new||^2 (one pass).
 static int gs_axpy(Ctx* c, int J, long long n, const double2* V, long long ldv, const double2* d_h,
                    double2* w, double sign, double2* d_norm, double2* d_part, cudaStream_t st) {
-  int nseg = gs_nseg(n);
-  k_gs_axpy<<<gs_grid(nseg), 256, 0, st>>>(J, n, V, ldv, d_h, w, sign, d_norm ? d_part : nullptr, nseg);
+  // one row a lane where eight leave SMs idle (as in gs32_axpy)
+  const bool few = gs_grid(gs_nseg(n)) < 152;
+  const int nseg = few ? (int)((n + 31) / 32) : gs_nseg(n);
+  auto k = few ? k_gs_axpy<1> : k_gs_axpy<GS_RPL>;
+  k<<<gs_grid(nseg), 256, 0, st>>>(J, n, V, ldv, d_h, w, sign, d_norm ? d_part : nullptr, nseg);
   SMR_LAUNCH(c);
   if (d_norm) {
     k_gs_final<<<1, 256, 0, st>>>(nseg, d_part, 0, nullptr, d_norm, nullptr);
@@ -371,11 +377,13 @@ __device__ __forceinline__ float4 ld_pair(const float2* __restrict__ v, long lon
 }
 
 // part[j][g] = conj(V_j) . w over the warp's rows (j < J); with with_norm,
-// part[J][g] = sum |w|^2 (FP64).
+// part[J][g] = sum |w|^2 (FP64).  The basis vectors are divided over blockIdx.y: with
+// a warp per segment for all of them, short vectors leave most SMs idle (1,600
+// particles: 200 warps; figures at gs_split).
 __global__ void __launch_bounds__(256) k_gs32_dot(int J, long long n, const float2* __restrict__ V,
                                                   long long ldv, const double2* __restrict__ w,
                                                   double2* __restrict__ part, int nseg, int with_norm) {
-  int g = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
+  const int g = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
   int lane = threadIdx.x & 31;
   if (g >= nseg) return;
   long long i0 = (long long)g * G32_SEG + 2 * lane;
@@ -390,12 +398,14 @@ __global__ void __launch_bounds__(256) k_gs32_dot(int J, long long n, const floa
     s += w0.x * w0.x + w0.y * w0.y + w1.x * w1.x + w1.y * w1.y;
     wf[q] = make_float4((float)w0.x, (float)w0.y, (float)w1.x, (float)w1.y);
   }
-  if (with_norm) {
+  if (with_norm && blockIdx.y == 0) {
     s = warp_sum(s);
     if (lane == 0) part[(size_t)J * nseg + g] = make_double2(s, 0);
   }
-  int j = 0;
-  for (; j + 2 <= J; j += 2) {
+  // this CTA's basis vectors, an even number of them but for the last
+  const int G = gridDim.y, per = 2 * (((J + 1) / 2 + G - 1) / G), j1 = min(J, per * ((int)blockIdx.y + 1));
+  int j = per * blockIdx.y;
+  for (; j + 2 <= j1; j += 2) {
     const float2* v0 = V + (size_t)j * ldv;
     const float2* v1 = v0 + ldv;
     float4 a[G32_RPL], b[G32_RPL];
@@ -422,7 +432,7 @@ __global__ void __launch_bounds__(256) k_gs32_dot(int J, long long n, const floa
       part[(size_t)(j + 1) * nseg + g] = make_double2(bx, by);
     }
   }
-  if (j < J) {
+  if (j < j1) {
     const float2* v0 = V + (size_t)j * ldv;
     float ax = 0, ay = 0;
 #pragma unroll
@@ -438,53 +448,50 @@ __global__ void __launch_bounds__(256) k_gs32_dot(int J, long long n, const floa
 }
 
 // w += sign * sum_j V_j hf[j] (FP32 products and sums, FP64 update of w);
-// with part_norm, part_norm[g] = sum |w_new|^2 over the warp's rows.
+// with part_norm, part_norm[g] = sum |w_new|^2 over the warp's rows.  A lane holds
+// RPL row pairs and reads 16 / RPL basis vectors at a time.
+template <int RPL>
 __global__ void __launch_bounds__(256) k_gs32_axpy(int J, long long n, const float2* __restrict__ V,
                                                    long long ldv, const float2* __restrict__ hf,
                                                    double2* __restrict__ w, double sign,
                                                    double2* __restrict__ part_norm, int nseg) {
+  constexpr int JU = 16 / RPL, SEG = 64 * RPL;
   int g = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
   int lane = threadIdx.x & 31;
   if (g >= nseg) return;
-  long long i0 = (long long)g * G32_SEG + 2 * lane;
-  bool full = (long long)(g + 1) * G32_SEG <= n;
-  float4 acc[G32_RPL];
+  long long i0 = (long long)g * SEG + 2 * lane;
+  bool full = (long long)(g + 1) * SEG <= n;
+  float4 acc[RPL];
 #pragma unroll
-  for (int q = 0; q < G32_RPL; ++q) acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int q = 0; q < RPL; ++q) acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto add = [&](float4& o, float4 a, float2 c0) {
+    o.x += a.x * c0.x - a.y * c0.y;
+    o.y += a.x * c0.y + a.y * c0.x;
+    o.z += a.z * c0.x - a.w * c0.y;
+    o.w += a.z * c0.y + a.w * c0.x;
+  };
   int j = 0;
-  for (; j + 2 <= J; j += 2) {
-    const float2* v0 = V + (size_t)j * ldv;
-    const float2* v1 = v0 + ldv;
-    float4 a[G32_RPL], b[G32_RPL];
+  for (; j + JU <= J; j += JU) {
+    float4 a[JU][RPL];
 #pragma unroll
-    for (int q = 0; q < G32_RPL; ++q) {
-      a[q] = ld_pair(v0, i0 + 64 * q, n, full);
-      b[q] = ld_pair(v1, i0 + 64 * q, n, full);
-    }
-    float2 c0 = hf[j], c1 = hf[j + 1];
+    for (int u = 0; u < JU; ++u)
 #pragma unroll
-    for (int q = 0; q < G32_RPL; ++q) {
-      acc[q].x += a[q].x * c0.x - a[q].y * c0.y + b[q].x * c1.x - b[q].y * c1.y;
-      acc[q].y += a[q].x * c0.y + a[q].y * c0.x + b[q].x * c1.y + b[q].y * c1.x;
-      acc[q].z += a[q].z * c0.x - a[q].w * c0.y + b[q].z * c1.x - b[q].w * c1.y;
-      acc[q].w += a[q].z * c0.y + a[q].w * c0.x + b[q].z * c1.y + b[q].w * c1.x;
+      for (int q = 0; q < RPL; ++q) a[u][q] = ld_pair(V + (size_t)(j + u) * ldv, i0 + 64 * q, n, full);
+#pragma unroll
+    for (int u = 0; u < JU; ++u) {
+      const float2 c0 = hf[j + u];
+#pragma unroll
+      for (int q = 0; q < RPL; ++q) add(acc[q], a[u][q], c0);
     }
   }
-  if (j < J) {
-    const float2* v0 = V + (size_t)j * ldv;
-    float2 c0 = hf[j];
+  for (; j < J; ++j) {
+    const float2 c0 = hf[j];
 #pragma unroll
-    for (int q = 0; q < G32_RPL; ++q) {
-      float4 a = ld_pair(v0, i0 + 64 * q, n, full);
-      acc[q].x += a.x * c0.x - a.y * c0.y;
-      acc[q].y += a.x * c0.y + a.y * c0.x;
-      acc[q].z += a.z * c0.x - a.w * c0.y;
-      acc[q].w += a.z * c0.y + a.w * c0.x;
-    }
+    for (int q = 0; q < RPL; ++q) add(acc[q], ld_pair(V + (size_t)j * ldv, i0 + 64 * q, n, full), c0);
   }
   double s = 0;
 #pragma unroll
-  for (int q = 0; q < G32_RPL; ++q) {
+  for (int q = 0; q < RPL; ++q) {
     long long i = i0 + 64 * q;
     if (full || i < n) {
       double2 o = w[i];
@@ -617,7 +624,8 @@ static int gs32_dot(Ctx* c, int J, long long n, const float2* V, long long ldv, 
   int nseg = g32_nseg(n);
   int rows = J + (d_norm ? 1 : 0);
   if (rows == 0) return SMR_OK;
-  k_gs32_dot<<<gs_grid(nseg), 256, 0, st>>>(J, n, V, ldv, w, d_part, nseg, d_norm ? 1 : 0);
+  const dim3 grid(gs_grid(nseg), gs_split(gs_grid(nseg), (J + 1) / 2));
+  k_gs32_dot<<<grid, 256, 0, st>>>(J, n, V, ldv, w, d_part, nseg, d_norm ? 1 : 0);
   SMR_LAUNCH(c);
   k_gs_final<<<rows, 256, 0, st>>>(nseg, d_part, J, d_h, d_norm, d_hf);
   SMR_LAUNCH(c);
@@ -626,8 +634,11 @@ static int gs32_dot(Ctx* c, int J, long long n, const float2* V, long long ldv, 
 
 static int gs32_axpy(Ctx* c, int J, long long n, const float2* V, long long ldv, const float2* d_hf,
                      double2* w, double sign, double2* d_norm, double2* d_part, cudaStream_t st) {
-  int nseg = g32_nseg(n);
-  k_gs32_axpy<<<gs_grid(nseg), 256, 0, st>>>(J, n, V, ldv, d_hf, w, sign, d_norm ? d_part : nullptr, nseg);
+  // one row pair a lane where eight leave SMs idle (figures at gs_split)
+  const bool few = gs_grid(g32_nseg(n)) < 152;
+  const int nseg = few ? (int)((n + 63) / 64) : g32_nseg(n);
+  auto k = few ? k_gs32_axpy<1> : k_gs32_axpy<G32_RPL>;
+  k<<<gs_grid(nseg), 256, 0, st>>>(J, n, V, ldv, d_hf, w, sign, d_norm ? d_part : nullptr, nseg);
   SMR_LAUNCH(c);
   if (d_norm) {
     k_gs_final<<<1, 256, 0, st>>>(nseg, d_part, 0, nullptr, d_norm, nullptr);
@@ -641,7 +652,7 @@ static size_t part_elems(long long n, int R, int J) {
   int rl, nchunk;
   long long per;
   chunking(n, R, &rl, &nchunk, &per);
-  return std::max((size_t)J * nchunk * R, (size_t)(J + 1) * gs_nseg(n));
+  return std::max(std::max((size_t)J * nchunk * R, (size_t)(J + 1) * gs_nseg(n)), (size_t)((n + 31) / 32));
 }
 
 // d_h[J][R] on the device.
@@ -1044,8 +1055,12 @@ static int gmres_core(Ctx* c, int R, int prec, int precond, const double2* rhs, 
   float2* dh1f = W.coef_f;
   float2* dh2f = W.coef_f + (size_t)(m + 1) * R;
   float2* dyf = W.coef_f + (size_t)2 * (m + 1) * R;
-  // host Hessenberg storage per column (rotated), rotations, rhs g
-  std::vector<std::complex<double>> H((size_t)(m + 1) * m * R), g((size_t)(m + 1) * R);
+  // host Hessenberg storage (rotated), rotations, rhs g.  Column j of right-hand side
+  // r has j + 2 entries and the columns are packed as they come: with the full
+  // (m + 1) x m an unrestarted solve (m = maxit = 2,000) clears 64 MB for each
+  // right-hand side, 3.6 ms each
+  std::vector<std::complex<double>> H, g((size_t)(m + 1) * R);
+  auto hcol = [&](int r, int j) { return (size_t)R * j * (j + 3) / 2 + (size_t)r * (j + 2); };
   std::vector<std::complex<double>> cs((size_t)m * R), sn((size_t)m * R);
   // pinned host mirror of the coefficient area; each iteration copies only
   // the live part (j + 1 coefficients per column and the two norms)
@@ -1150,9 +1165,10 @@ static int gmres_core(Ctx* c, int R, int prec, int precond, const double2* rhs, 
       rc = store_basis(j + 1, W.w);
       if (rc) return rc;
       bool any = false;
+      if (H.size() < hcol(0, j + 1)) H.resize(std::max(2 * H.size(), hcol(0, j + 1)));
       for (int r = 0; r < R; ++r) {
         if (!active[r]) continue;
-        std::complex<double>* Hc = &H[((size_t)r * m + j) * (m + 1)];   // column j of column-set r
+        std::complex<double>* Hc = &H[hcol(r, j)];
         for (int i = 0; i <= j; ++i) {
           double2 a = hbuf[(size_t)i * R + r], b = hbuf[(size_t)(m + 1) * R + (size_t)i * R + r];
           Hc[i] = std::complex<double>(a.x + b.x, a.y + b.y);
@@ -1201,8 +1217,8 @@ static int gmres_core(Ctx* c, int R, int prec, int precond, const double2* rhs, 
       std::vector<std::complex<double>> y(J);
       for (int i = J - 1; i >= 0; --i) {
         std::complex<double> s = g[(size_t)r * (m + 1) + i];
-        for (int q = i + 1; q < J; ++q) s -= H[((size_t)r * m + q) * (m + 1) + i] * y[q];
-        std::complex<double> diag = H[((size_t)r * m + i) * (m + 1) + i];
+        for (int q = i + 1; q < J; ++q) s -= H[hcol(r, q) + i] * y[q];
+        std::complex<double> diag = H[hcol(r, i) + i];
         y[i] = (diag != 0.0) ? s / diag : 0.0;
       }
       for (int i = 0; i < J; ++i) ycoef[(size_t)i * R + r] = make_double2(y[i].real(), y[i].imag());
