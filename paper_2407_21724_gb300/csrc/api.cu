@@ -56,7 +56,7 @@ void free_scene(Ctx* c) {
     c->pspec[q] = nullptr;
   }
   c->multi = 0;
-  dfree(c->d_B64); dfree(c->d_B32); dfree(c->d_tcn_img); dfree(c->d_tcn_blk); dfree(c->d_tcn_start);
+  dfree(c->d_Bs64); dfree(c->d_Bc64); dfree(c->d_Bs32); dfree(c->d_Bc32); dfree(c->d_tcn_img); dfree(c->d_tcn_blk); dfree(c->d_tcn_start);
   dfree(c->d_tcn_count); dfree(c->d_tcn_nu); dfree(c->d_tcn_mu); dfree(c->d_x32);
   dfree(c->d_tcn_mask); dfree(c->d_tcn_part); dfree(c->d_tc_part); dfree(c->d_Pinv64); dfree(c->d_Pinv32); dfree(c->d_pc_ptr);
   dfree(c->d_pc_col); dfree(c->d_pc_blk); dfree(c->d_tmp);
@@ -1115,7 +1115,7 @@ int smr_info(smr_ctx* h, smr_info_t* info) {
   }
   info->n_near_pairs = (long long)c->nr_col.size();
   info->n_near_blocks = c->nblk;
-  bytes += (double)c->nblk * 4 * c->npsi * c->npsi * 24;
+  bytes += (double)(c->nblk + c->S) * 2 * c->npsi * c->npsi * 24;
   info->device_bytes = bytes;
   info->column_lanes = c->n_lanes;
   return SMR_OK;
@@ -1718,23 +1718,28 @@ int smr_copy_translation(smr_ctx* h, int level, int dx, int dy, double* out) {
   return fail(c, SMR_E_INVALID_ARG, "offset not in this level's interaction lists");
 }
 
+// near block b, row-major
+static int copy_block(Ctx* c, int b, double* out) {
+  const int n = c->npsi, n2 = 2 * n;
+  const bool self = b < c->S;
+  std::vector<double2> t((size_t)n2 * (self ? n2 : n));
+  const double2* src = self ? c->d_Bs64 + (size_t)b * t.size() : c->d_Bc64 + (size_t)(b - c->S) * t.size();
+  SMR_CUDA(c, cudaMemcpy(t.data(), src, t.size() * sizeof(double2), cudaMemcpyDeviceToHost));
+  for (int i = 0; i < n2; ++i)
+    for (int j = 0; j < n2; ++j) {
+      const double2 v = near_entry(t.data(), t.data(), self ? 1 : 0, n, c->zeta, 0, i, j);
+      out[2 * ((size_t)i * n2 + j)] = v.x;
+      out[2 * ((size_t)i * n2 + j) + 1] = v.y;
+    }
+  return SMR_OK;
+}
+
 int smr_copy_near_block(smr_ctx* h, int sm, int sn, int dx, int dy, double* out) {
   if (!h || !out) return SMR_E_INVALID_ARG;
   Ctx* c = &h->c;
   if (!check_scene(c)) return SMR_E_STATE;
-  int n2 = 2 * c->npsi;
   for (int b = 0; b < c->nblk; ++b)
-    if (c->blk_sm[b] == sm && c->blk_sn[b] == sn && c->blk_dx[b] == dx && c->blk_dy[b] == dy) {
-      std::vector<double2> t((size_t)n2 * n2);
-      SMR_CUDA(c, cudaMemcpy(t.data(), c->d_B64 + (size_t)b * n2 * n2, t.size() * sizeof(double2),
-                             cudaMemcpyDeviceToHost));
-      for (int i = 0; i < n2; ++i)
-        for (int j = 0; j < n2; ++j) {
-          out[2 * ((size_t)i * n2 + j)] = t[(size_t)j * n2 + i].x;
-          out[2 * ((size_t)i * n2 + j) + 1] = t[(size_t)j * n2 + i].y;
-        }
-      return SMR_OK;
-    }
+    if (c->blk_sm[b] == sm && c->blk_sn[b] == sn && c->blk_dx[b] == dx && c->blk_dy[b] == dy) return copy_block(c, b, out);
   return fail(c, SMR_E_INVALID_ARG, "no such near block in this scene");
 }
 
@@ -1743,19 +1748,8 @@ int smr_copy_pair_block(smr_ctx* h, int mu, int nu, double* out) {
   Ctx* c = &h->c;
   if (!check_scene(c)) return SMR_E_STATE;
   if (mu < 0 || mu >= c->p || nu < 0 || nu >= c->p) return fail(c, SMR_E_INVALID_ARG, "particle index out of range");
-  const int n2 = 2 * c->npsi;
-  for (int e = c->nr_ptr[mu]; e < c->nr_ptr[mu + 1]; ++e) {
-    if (c->nr_col[e] != nu) continue;
-    std::vector<double2> t((size_t)n2 * n2);
-    SMR_CUDA(c, cudaMemcpy(t.data(), c->d_B64 + (size_t)c->nr_blk[e] * n2 * n2, t.size() * sizeof(double2),
-                           cudaMemcpyDeviceToHost));
-    for (int i = 0; i < n2; ++i)
-      for (int j = 0; j < n2; ++j) {
-        out[2 * ((size_t)i * n2 + j)] = t[(size_t)j * n2 + i].x;
-        out[2 * ((size_t)i * n2 + j) + 1] = t[(size_t)j * n2 + i].y;
-      }
-    return SMR_OK;
-  }
+  for (int e = c->nr_ptr[mu]; e < c->nr_ptr[mu + 1]; ++e)
+    if (c->nr_col[e] == nu) return copy_block(c, c->nr_blk[e], out);
   return fail(c, SMR_E_INVALID_ARG, "the two particles are not a near pair");
 }
 

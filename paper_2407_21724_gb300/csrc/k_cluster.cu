@@ -30,7 +30,8 @@ __device__ inline double2 cmul2(double2 a, double2 b) {
 // blocks are stored transposed, Bt[col * m + row].
 __global__ void k_cluster_assemble(int c0, int nb, int m, const int* __restrict__ mem,
                                    const int* __restrict__ ptr, const int* __restrict__ col,
-                                   const int* __restrict__ blk, const double2* __restrict__ Bt,
+                                   const int* __restrict__ blk, const double2* __restrict__ Bs,
+                                   const double2* __restrict__ Bc, int S, double zeta,
                                    double2* __restrict__ A) {
   const int b = blockIdx.x;
   if (b >= nb) return;
@@ -53,7 +54,7 @@ __global__ void k_cluster_assemble(int c0, int nb, int m, const int* __restrict_
     const int a = i / m, bb = j / m, ii = i % m, jj = j % m;
     const int id = bid[4 * a + bb];
     double2 v = make_double2(0.0, 0.0);
-    if (id >= 0) v = Bt[(size_t)id * m * m + (size_t)jj * m + ii];
+    if (id >= 0) v = near_entry(Bs, Bc, S, m / 2, zeta, id, ii, jj);
     else if (i == j && mem[4 * cl + a] < 0) v = make_double2(1.0, 0.0);
     Ab[idx] = v;
   }
@@ -263,7 +264,8 @@ int build_clusters(Ctx* c) {
                                        (int)(N * sizeof(double2)));
   for (int c0 = 0; c0 < ncl && e == cudaSuccess; c0 += batch) {
     const int nb = std::min(batch, ncl - c0);
-    k_cluster_assemble<<<nb, 256>>>(c0, nb, m, d_mem, c->d_nr_ptr, c->d_nr_col, c->d_nr_blk, c->d_B64, scratch);
+    k_cluster_assemble<<<nb, 256>>>(c0, nb, m, d_mem, c->d_nr_ptr, c->d_nr_col, c->d_nr_blk, c->d_Bs64, c->d_Bc64,
+                                      c->S, c->zeta, scratch);
     e = cudaGetLastError();
     if (e != cudaSuccess) break;
     k_cluster_invert<<<nb, 256, N * sizeof(double2)>>>(c0, nb, N, scratch, inv64, inv32, d_bad);

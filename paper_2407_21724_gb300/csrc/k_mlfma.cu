@@ -5,10 +5,11 @@
 //
 // Layouts (complex, interleaved):
 //   x, y              [p][2][n_psi][R]
-//   patterns P        [S][n_psi][2][K0]       (theta, phi components, Eq. 26)
-//   spectra out/in    [n_box][K_s][4][R]      fields A_e.th, A_e.ph, A_m.th, A_m.ph
+//   patterns Pd, Pm   [S][2][n_psi][K0 / 2], [S][2][K0 / 2][n_psi]  (P_th +- j P_ph, Eq. 26)
+//   spectra out/in    [n_box][K_s][NF][R]     circular fields (smr_internal.h)
 //   translation T     [n_offset][K_s]         (Eq. 23)
-//   near blocks       [n_blk][2 n_psi (col j)][2 n_psi (row i)]  (transposed)
+//   self blocks       [S][2 n_psi (col j)][2 n_psi (row i)]  (transposed)
+//   exterior blocks   [n_blk - S][n_psi (col j)][+, -][n_psi (row i)]  (k_near_rows)
 #include <algorithm>
 
 #include "smr_internal.h"
@@ -745,13 +746,80 @@ __global__ void k_receive(int K0, int nph, int npsi, int R, const int* __restric
   *pm = om;
 }
 
+// ------------------------------------------------------------------ near product
+// y[mu] = sum_{e in row mu} B[blk_e] x[col_e].  An exterior block [z T, K; -K, T / z]
+// couples the circular combinations x_+- = e +- (j/z) m and Y_+- = y_e / z +- j y_m
+// only with themselves, Y_+- = (T -+ j K) x_+-: half the multiply-adds and half the
+// block.  Self blocks (blk < S) carry the interior medium as well and stay whole.
+// CTA = one row (particle, r); threads are (output row, every KS-th column), the
+// vectors of up to NR_PAIRS pairs staged in shared memory.  Bound in FP64 by the
+// FP64 rate (1,600 particles 428 -> 236 us, 64 particles 94 -> 27), with one block a pair (displaced particles) by the blocks' bytes
+// (24x24 in FP32 84.6 -> 27.5 us).
+constexpr int NR_PAIRS = 9;
+template <typename T, typename XV>
+__global__ void k_near_rows(int n, int R, int S, const int* __restrict__ ptr, const int* __restrict__ col,
+                            const int* __restrict__ blk, const typename CV<T>::V* __restrict__ Bs,
+                            const typename CV<T>::V* __restrict__ Bc, double zeta, const XV* __restrict__ x,
+                            double2* __restrict__ y) {
+  typedef typename CV<T>::V V;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int n2 = 2 * n, KS = blockDim.x / n2, t = threadIdx.x % n2, ks = threadIdx.x / n2;
+  V* xs = reinterpret_cast<V*>(smem_raw);          // [NR_PAIRS][2][n]: + and -, or e and m
+  V* red = xs + NR_PAIRS * n2;                     // [2][threads]
+  const int mu = blockIdx.x / R, r = blockIdx.x % R;
+  const double iz = 1.0 / zeta;
+  const int sg = t >= n ? n : 0;                   // this row's circular component
+  V full = czero<V>(), circ = czero<V>();
+  const int e1 = ptr[mu + 1];
+  for (int e0 = ptr[mu]; e0 < e1; e0 += NR_PAIRS) {
+    const int ne = min(NR_PAIRS, e1 - e0);
+    __syncthreads();
+    for (int u = threadIdx.x; u < ne * n; u += blockDim.x) {
+      const int q = u / n, j = u - q * n;
+      const XV* xv = x + (size_t)col[e0 + q] * n2 * R + r;
+      const double2 a = to64(xv[(size_t)j * R]), b = to64(xv[(size_t)(n + j) * R]);
+      const bool self = blk[e0 + q] < S;
+      xs[q * n2 + j] = cvt2(self ? a : make_double2(fma(-iz, b.y, a.x), fma(iz, b.x, a.y)), V());
+      xs[q * n2 + n + j] = cvt2(self ? b : make_double2(fma(iz, b.y, a.x), fma(-iz, b.x, a.y)), V());
+    }
+    __syncthreads();
+    for (int q = 0; q < ne; ++q) {
+      const int b = blk[e0 + q];
+      if (b < S) {
+        const V* B = Bs + (size_t)b * n2 * n2 + t;
+#pragma unroll 4
+        for (int j = ks; j < n2; j += KS) cfma(full, B[(size_t)j * n2], xs[q * n2 + j]);
+      } else {
+        const V* B = Bc + (size_t)(b - S) * n * n2 + t;
+#pragma unroll 8
+        for (int j = ks; j < n; j += KS) cfma(circ, B[(size_t)j * n2], xs[q * n2 + sg + j]);
+      }
+    }
+  }
+  red[threadIdx.x] = full;
+  red[blockDim.x + threadIdx.x] = circ;
+  __syncthreads();
+  if (threadIdx.x >= n) return;
+  double2 f[2] = {}, c[2] = {};
+  for (int h = 0; h < 2; ++h)
+    for (int k = 0; k < KS; ++k) {
+      const double2 a = to64(red[k * n2 + h * n + t]), b = to64(red[blockDim.x + k * n2 + h * n + t]);
+      f[h].x += a.x; f[h].y += a.y;
+      c[h].x += b.x; c[h].y += b.y;
+    }
+  const double hz = 0.5 * zeta;
+  double2* o = y + ((size_t)mu * n2 + t) * R + r;
+  o[0] = make_double2(fma(hz, c[0].x + c[1].x, f[0].x), fma(hz, c[0].y + c[1].y, f[0].y));
+  o[(size_t)n * R] = make_double2(fma(0.5, c[0].y - c[1].y, f[1].x), fma(-0.5, c[0].x - c[1].x, f[1].y));
+}
+
 // ------------------------------------------------------------------ block-sparse product
 // y[mu][i][r] (+)= sum_{e in row mu} sum_j B[blk_e][i][j] x[col_e][j][r]
-template <typename T, typename XV = double2>
+template <typename T>
 __global__ void k_blocksparse(int nrow, int n2, int R, int rc, int nrc, const int* __restrict__ ptr,
                               const int* __restrict__ col, const int* __restrict__ blk,
                               const typename CV<T>::V* __restrict__ Bt,
-                              const XV* __restrict__ x, double2* __restrict__ y,
+                              const double2* __restrict__ x, double2* __restrict__ y,
                               int accumulate) {
   typedef typename CV<T>::V V;
   extern __shared__ unsigned char smem_raw[];
@@ -762,7 +830,7 @@ __global__ void k_blocksparse(int nrow, int n2, int R, int rc, int nrc, const in
   bool active = (i < n2) && (rl < nr);
   V acc = czero<V>();
   for (int e = ptr[mu]; e < ptr[mu + 1]; ++e) {
-    const XV* xv = x + (size_t)col[e] * n2 * R + r0;
+    const double2* xv = x + (size_t)col[e] * n2 * R + r0;
     __syncthreads();
     for (int t = threadIdx.x; t < n2 * nr; t += blockDim.x) {
       int jl = t / nr, q = t % nr;
@@ -1221,22 +1289,24 @@ int run_near(Ctx* c, int R, int prec, const double2* x, double2* y, cudaStream_t
   }
   double n2 = 2.0 * c->npsi, es = prec == SMR_PREC_FP64 ? 16 : 8;
   const bool x32 = prec == SMR_PREC_FP32 && R == 1 && c->x32_of == x;
-  pbeg(c, st, "near", -1, c->p * n2 * R * (x32 ? 8 + 16 : 16 + 16) + (double)c->nblk * n2 * n2 * es,
-       8.0 * n2 * n2 * c->nr_col.size() * R);
-  int rc;
-  if (x32) {
-    const int n2i = 2 * c->npsi;
-    k_blocksparse<float, float2><<<(unsigned)c->p, n2i, (size_t)n2i * sizeof(float2), st>>>(
-        c->p, n2i, 1, 1, 1, c->d_nr_ptr, c->d_nr_col, c->d_nr_blk, c->d_B32, c->d_x32, y, 0);
-    SMR_LAUNCH(c);
-    rc = SMR_OK;
-  } else {
-    rc = (prec == SMR_PREC_FP64)
-             ? bs_impl<double>(c, c->p, R, c->d_nr_ptr, c->d_nr_col, c->d_nr_blk, c->d_B64, x, y, false, st)
-             : bs_impl<float>(c, c->p, R, c->d_nr_ptr, c->d_nr_col, c->d_nr_blk, c->d_B32, x, y, false, st);
-  }
+  pbeg(c, st, "near", -1, c->p * n2 * R * (x32 ? 8 + 16 : 16 + 16) + (c->nblk + c->S) * 0.5 * n2 * n2 * es,
+       4.0 * n2 * n2 * (c->nr_col.size() + c->p) * R);
+  const int n = c->npsi, thr = 2 * n * std::max(1, 256 / (2 * n));
+  const size_t vb = prec == SMR_PREC_FP64 ? sizeof(double2) : sizeof(float2);
+  const size_t sm = ((size_t)NR_PAIRS * 2 * n + 2 * thr) * vb;
+  const unsigned g = (unsigned)((long long)c->p * R);
+  if (prec == SMR_PREC_FP64)
+    k_near_rows<double, double2><<<g, thr, sm, st>>>(n, R, c->S, c->d_nr_ptr, c->d_nr_col, c->d_nr_blk, c->d_Bs64,
+                                                     c->d_Bc64, c->zeta, x, y);
+  else if (x32)
+    k_near_rows<float, float2><<<g, thr, sm, st>>>(n, R, c->S, c->d_nr_ptr, c->d_nr_col, c->d_nr_blk, c->d_Bs32,
+                                                   c->d_Bc32, c->zeta, c->d_x32, y);
+  else
+    k_near_rows<float, double2><<<g, thr, sm, st>>>(n, R, c->S, c->d_nr_ptr, c->d_nr_col, c->d_nr_blk, c->d_Bs32,
+                                                    c->d_Bc32, c->zeta, x, y);
+  SMR_LAUNCH(c);
   pend(c, st);
-  return rc;
+  return SMR_OK;
 }
 
 // out[c][i] = in[i][c] for in [rows][cols] (tiles of 32 x 32 through shared

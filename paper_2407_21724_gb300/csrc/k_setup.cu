@@ -305,11 +305,12 @@ __global__ void k_near_f(int nb, int npsi, int Q, const int* __restrict__ bsm,
 }
 
 // Stage 2: T_mn = -jk sum_q w psi_m . Fv_n + (j/k) sum_q w div_m Fd_n,
-//          K_mn = - sum_q w psi_m . FK_n;  block [zT, K; -K, T/z], stored transposed.
+//          K_mn = - sum_q w psi_m . FK_n;  block [zT, K; -K, T/z], stored as its circular
+//          halves T -+ j K, column by column.
 __global__ void k_near_z(int nb, int npsi, int Q, const int* __restrict__ bsm,
                          const double* __restrict__ modes, const double* __restrict__ rq,
-                         const double2* __restrict__ F, double kw, double zeta,
-                         double2* __restrict__ Bt, const int* __restrict__ bidx) {
+                         const double2* __restrict__ F, double kw, double2* __restrict__ Bc,
+                         const int* __restrict__ bidx) {
   int b = blockIdx.y;
   int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= npsi * npsi) return;
@@ -333,30 +334,23 @@ __global__ void k_near_z(int nb, int npsi, int Q, const int* __restrict__ bsm,
   double2 T = make_double2(kw * v.y - d.y / kw, -kw * v.x + d.x / kw);
   double2 K = make_double2(-kk.x, -kk.y);
   int n2 = 2 * npsi;
-  double2* B = Bt + (size_t)bidx[b] * n2 * n2;
-  // B stored transposed: B[col * n2 + row]
-  B[(size_t)n * n2 + m] = make_double2(zeta * T.x, zeta * T.y);
-  B[(size_t)(npsi + n) * n2 + m] = K;
-  B[(size_t)n * n2 + npsi + m] = make_double2(-K.x, -K.y);
-  B[(size_t)(npsi + n) * n2 + npsi + m] = make_double2(T.x / zeta, T.y / zeta);
+  double2* B = Bc + ((size_t)bidx[b] * npsi + n) * n2 + m;
+  B[0] = make_double2(T.x + K.y, T.y - K.x);         // T - j K
+  B[npsi] = make_double2(T.x - K.y, T.y + K.x);      // T + j K
 }
 
 // Reciprocity of the exterior blocks: T and K are symmetric bilinear forms
 // (the Green's function and the triple product under the swap of source and
-// test), so Z^{nu mu} = [T_nm^T ...] follows from Z^{mu nu} = [z T, K; -K, T/z]
-// as Z^{nu mu}(r, c) = s_r s_c Z^{mu nu}(c, r), s = +1 on the electric rows
-// and -1 on the magnetic ones.  Grid: (element chunks of 256, pairs); both
-// blocks stored transposed (B[col * n2 + row]).
+// test), so the swapped pair's T and K are the transposed ones, and its circular
+// halves too.  Grid: (element chunks of 256, pairs).
 __global__ void k_near_mirror(int nd, int npsi, const int* __restrict__ dst, const int* __restrict__ src,
-                              double2* __restrict__ Bt) {
+                              double2* __restrict__ Bc) {
   const int b = blockIdx.y;
   const int n2 = 2 * npsi;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= nd || t >= n2 * n2) return;
-  const int i = t / n2, j = t % n2;             // A(row j, col i) is A[i * n2 + j]
-  const double2 a = Bt[(size_t)src[b] * n2 * n2 + (size_t)i * n2 + j];
-  const double sg = ((i < npsi) == (j < npsi)) ? 1.0 : -1.0;
-  Bt[(size_t)dst[b] * n2 * n2 + (size_t)j * n2 + i] = make_double2(sg * a.x, sg * a.y);
+  if (b >= nd || t >= n2 * npsi) return;
+  const int i = t % npsi, f = t / npsi % 2, j = t / n2;
+  Bc[((size_t)dst[b] * npsi + j) * n2 + f * npsi + i] = Bc[((size_t)src[b] * npsi + i) * n2 + f * npsi + j];
 }
 
 // Closed-form self block of a sphere (Eq. 16 with delta = 1): per (l, m) the
@@ -438,16 +432,15 @@ int build_near(Ctx* c) {
         invT[s * bsz + (size_t)j * n2 + i] = make_double2(Zi[(size_t)i * n2 + j].real(), Zi[(size_t)i * n2 + j].imag());
       }
   }
-  if (c->d_B64) cudaFree(c->d_B64);
-  c->d_B64 = nullptr;
-  SMR_CUDA(c, cudaMalloc((void**)&c->d_B64, (size_t)nb_total * bsz * sizeof(double2)));
-  SMR_CUDA(c, cudaMemcpy(c->d_B64, selfT.data(), (size_t)S * bsz * sizeof(double2), cudaMemcpyHostToDevice));
-  int rc = upload(c, &c->d_Pinv64, invT);
-  if (rc) return rc;
+  int rc;
+  if ((rc = upload(c, &c->d_Bs64, selfT)) || (rc = upload(c, &c->d_Pinv64, invT))) return rc;
+  if (c->d_Bc64) cudaFree(c->d_Bc64);
+  c->d_Bc64 = nullptr;
   // exterior blocks: a block whose swapped pair (shapes exchanged, offset
   // negated) is also stored is computed once and mirrored into the other
   int nex = nb_total - S;
   if (nex > 0) {
+    SMR_CUDA(c, cudaMalloc((void**)&c->d_Bc64, (size_t)nex * bsz / 2 * sizeof(double2)));
     auto bits = [](double v) {
       if (v == 0.0) v = 0.0;                   // -0 and +0 are one key
       unsigned long long u;
@@ -469,8 +462,8 @@ int build_near(Ctx* c) {
                                bits(-off(b, 2))));
       if (it != index.end() && !done[it->second]) {
         done[it->second] = 1;
-        mdst.push_back(S + it->second);
-        msrc.push_back(S + b);
+        mdst.push_back(it->second);
+        msrc.push_back(b);
       }
     }
     const int np = (int)prim.size();
@@ -480,7 +473,7 @@ int build_near(Ctx* c) {
       const int b = prim[i];
       bsm[i] = c->blk_sm[S + b];
       bsn[i] = c->blk_sn[S + b];
-      bid[i] = S + b;
+      bid[i] = b;
       for (int d = 0; d < 3; ++d) bdc[3 * (size_t)i + d] = off(b, d);
     }
     int *d_bsm = nullptr, *d_bsn = nullptr, *d_bid = nullptr, *d_md = nullptr, *d_ms = nullptr;
@@ -499,15 +492,15 @@ int build_near(Ctx* c) {
                            c->k, d_F);
       SMR_LAUNCH(c);
       dim3 g2((n * n + 127) / 128, nbc);
-      k_near_z<<<g2, 128>>>(nbc, n, c->Q, d_bsm + b0, c->d_modes, c->d_rq, d_F, c->k, c->zeta,
-                            c->d_B64, d_bid + b0);
+      k_near_z<<<g2, 128>>>(nbc, n, c->Q, d_bsm + b0, c->d_modes, c->d_rq, d_F, c->k, c->d_Bc64,
+                            d_bid + b0);
       SMR_LAUNCH(c);
     }
     const int nm = (int)mdst.size();
     for (int m0 = 0; m0 < nm; m0 += 65535) {
       const int nd = std::min(65535, nm - m0);
-      dim3 g3((unsigned)((4 * n * n + 255) / 256), (unsigned)nd);
-      k_near_mirror<<<g3, 256>>>(nd, n, d_md + m0, d_ms + m0, c->d_B64);
+      dim3 g3((unsigned)((2 * n * n + 255) / 256), (unsigned)nd);
+      k_near_mirror<<<g3, 256>>>(nd, n, d_md + m0, d_ms + m0, c->d_Bc64);
       SMR_LAUNCH(c);
     }
     SMR_CUDA(c, cudaDeviceSynchronize());
@@ -519,8 +512,9 @@ int build_near(Ctx* c) {
     cudaFree(d_md);
     cudaFree(d_ms);
   }
-  rc = copy32(c, c->d_B64, &c->d_B32, (long long)nb_total * bsz);
-  if (rc) return rc;
+  if ((rc = copy32(c, c->d_Bs64, &c->d_Bs32, (long long)S * bsz)) ||
+      (rc = copy32(c, c->d_Bc64, &c->d_Bc32, (long long)nex * bsz / 2)))
+    return rc;
   return copy32(c, c->d_Pinv64, &c->d_Pinv32, (long long)S * bsz);
 }
 

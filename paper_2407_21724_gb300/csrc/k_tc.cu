@@ -839,8 +839,7 @@ int run_aggregate_tc(Ctx* c, const double2* x, const float2* x32, float2* out0, 
   return SMR_OK;
 }
 
-// Near product on the tensor cores.  Block b (n2 x n2 complex, stored
-// column-major in d_B64) in real form: row (i, re/im) of y, column (j, re/im)
+// Near product on the tensor cores.  Block b (n2 x n2 complex) in real form: row (i, re/im) of y, column (j, re/im)
 // of x, entries [Re, -Im; Im, Re] of B_ij; split into TF32 hi / lo and laid
 // out like the receive images.  Pairs go to phases by lattice offset (self
 // blocks first), and within a phase into tiles of up to TC_NP pairs sharing
@@ -854,14 +853,15 @@ int build_near_tc(Ctx* c) {
   if (M4 > 128 || c->p == 0) return SMR_OK;          // more than one M tile: CUDA-core path
   const int nK = (M4 + TC_KC - 1) / TC_KC;
   const size_t bsz = (size_t)n2 * n2;
-  std::vector<double2> B((size_t)nb * bsz);
-  SMR_CUDA(c, cudaMemcpy(B.data(), c->d_B64, B.size() * sizeof(double2), cudaMemcpyDeviceToHost));
+  std::vector<double2> Bs((size_t)S * bsz), Bc((size_t)(nb - S) * bsz / 2);
+  SMR_CUDA(c, cudaMemcpy(Bs.data(), c->d_Bs64, Bs.size() * sizeof(double2), cudaMemcpyDeviceToHost));
+  if (!Bc.empty()) SMR_CUDA(c, cudaMemcpy(Bc.data(), c->d_Bc64, Bc.size() * sizeof(double2), cudaMemcpyDeviceToHost));
   const size_t per = (size_t)nK * 2 * 128 * TC_KC;
   std::vector<float> img((size_t)nb * per, 0.f);
   for (int b = 0; b < nb; ++b)
     for (int j = 0; j < n2; ++j)
       for (int i = 0; i < n2; ++i) {
-        const double2 z = B[(size_t)b * bsz + (size_t)j * n2 + i];
+        const double2 z = near_entry(Bs.data(), Bc.data(), S, c->npsi, c->zeta, b, i, j);
         for (int ro = 0; ro < 2; ++ro)
           for (int ri = 0; ri < 2; ++ri) {
             const int row = 2 * i + ro, kp = 2 * j + ri;

@@ -246,8 +246,10 @@ struct Ctx {
   int nblk = 0;
   std::vector<int> blk_sm, blk_sn, blk_dx, blk_dy;  // key of each block
   std::vector<double> blk_off;            // [nblk][3] r_mu - r_nu of each block
-  double2* d_B64 = nullptr;
-  float2* d_B32 = nullptr;
+  // self blocks [S][2 npsi (col)][2 npsi (row)], and the circular halves of the exterior
+  // ones [nblk - S][npsi (col)][+, -][npsi (row)] (k_near_rows)
+  double2 *d_Bs64 = nullptr, *d_Bc64 = nullptr;
+  float2 *d_Bs32 = nullptr, *d_Bc32 = nullptr;
   // preconditioner: inverse self blocks, transposed [S][2n][2n]
   bool pinv_ok = true;                  // every self block was invertible
   double2* d_Pinv64 = nullptr;
@@ -419,7 +421,22 @@ inline void pend(Ctx* c, cudaStream_t st) {
 int build_modes(Ctx* c);          // d_modes, d_rq (host evaluation, upload)
 int build_patterns(Ctx* c);       // d_P64, d_Pd* and d_Pm* on the GPU (FP64)
 int build_translations(Ctx* c);   // per level d_T64 / d_T32 on the GPU (FP64)
-int build_near(Ctx* c);           // d_B64 / d_B32 on the GPU (FP64) + self blocks
+int build_near(Ctx* c);           // d_Bs*, d_Bc* on the GPU (FP64) + self blocks
+// Entry (row i, column j) of near block b from its stored form: an exterior block
+// is [z T, K; -K, T / z], stored as T -+ j K
+__host__ __device__ inline double2 near_entry(const double2* self, const double2* circ, int S, int n, double z, int b,
+                                              int i, int j) {
+  const int n2 = 2 * n;
+  if (b < S) return self[((size_t)b * n2 + j) * n2 + i];
+  const double2* q = circ + ((size_t)(b - S) * n + j % n) * n2 + i % n;
+  const double2 p = q[0], m = q[n];
+  if (i / n == j / n) {
+    const double f = i < n ? 0.5 * z : 0.5 / z;
+    return make_double2(f * (p.x + m.x), f * (p.y + m.y));
+  }
+  const double f = i < n ? 0.5 : -0.5;             // K = j (B+ - B-) / 2
+  return make_double2(-f * (p.y - m.y), f * (p.x - m.x));
+}
 int launch_rhs(Ctx* c, int R, const double* d_khat, const double2* d_pol, double2* b,
                cudaStream_t st);
 // R = 1 right-hand side with incidence number arr[mu] for particle mu
