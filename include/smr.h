@@ -286,10 +286,7 @@ int smr_set_tensor_cores(smr_ctx* ctx, int enable);
 
 /* Times the launch variants of the product for one right-hand side in
  * `precision` on this scene and keeps the fastest for later products (no
- * counterpart in the paper).  For SMR_PREC_FP64, per level: translation with
- * 8x8 target tiles and the full or half direction chunk, 4x4 tiles, threads
- * along the directions (levels of at most 1024 boxes), or one CTA per
- * direction chunk over the whole level (at most 256 boxes); interpolation and
+ * counterpart in the paper).  For SMR_PREC_FP64, per level: interpolation and
  * anterpolation by their built-in rules or by the gather kernels
  * (interpolation with the full or half theta-row tile, anterpolation with half
  * the column chunk or 256-thread CTAs).  For SMR_PREC_FP32
@@ -561,10 +558,7 @@ int smr_copy_level(smr_ctx* ctx, int level, int kind, double* out, size_t n_doub
 /* Parity access to the launch variants (the choices smr_autotune makes),
  * for one level (0 .. n_levels - 1) or every level (-1), for products in
  * `precision` with one right-hand side:
- *  SMR_STEP_TRANSLATE: 0 built-in rule, in FP64 1 / 2 8x8 target tiles with
- *    the full / half direction chunk, 3 4x4 tiles, 4 threads along the
- *    directions, 5 one CTA per direction chunk over every box of the level
- *    (levels of at most a few hundred boxes: each source spectrum read once);
+ *  SMR_STEP_TRANSLATE: 0 to 5, all the one kernel of the precision;
  *  SMR_STEP_INTERPOLATE (into the parent of `level`): 0 built-in rule (FP32:
  *    the marching kernel; FP64: the gather kernel), 1 / 2 the gather kernel
  *    with the full / half theta-row tile (FP64), 3 the marching kernel;

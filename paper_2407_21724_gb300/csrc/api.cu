@@ -38,7 +38,7 @@ void free_scene(Ctx* c) {
     dfree(L.d_shiftp32); dfree(L.d_mi_vlast); dfree(L.d_ma_ptr); dfree(L.d_ma_ent);
     dfree(L.d_ma_w64); dfree(L.d_ma_w32); dfree(L.d_ma_pst); dfree(L.d_ma_pw64); dfree(L.d_ma_pw32);
     dfree(L.d_ant_lo); dfree(L.d_ant_pjp); dfree(L.d_ant_pw64); dfree(L.d_ant_ttp); dfree(L.d_ant_tw64);
-    dfree(L.d_wthp64); dfree(L.d_boxmap); dfree(L.d_offid); dfree(L.d_tiles); dfree(L.d_tiles8); dfree(L.d_tile_tab);
+    dfree(L.d_wthp64); dfree(L.d_boxmap); dfree(L.d_offid); dfree(L.d_tiles); dfree(L.d_tile_tab);
     for (int q = 0; q < 2; ++q) {
       if (L.buf_out[q]) cudaFree(L.buf_out[q]);
       if (L.buf_in[q]) cudaFree(L.buf_in[q]);
@@ -644,22 +644,12 @@ int set_scene(Ctx* c, int p, const double* centres, const int* shape_ids, const 
     for (size_t t = 0; t < used.size(); ++t)
       if (used[t]) tiles.push_back((int)t);
     L.ntile_ne = (int)tiles.size();
-    L.ntile8_x = ((x0 + L.map_w - 1) >> 3) - (x0 >> 3) + 1;
-    int nt8y = ((y0 + L.map_h - 1) >> 3) - (y0 >> 3) + 1;
-    std::vector<char> used8((size_t)L.ntile8_x * nt8y, 0);
-    for (int b = 0; b < L.nbox; ++b)
-      used8[(size_t)((L.bj[b] >> 3) - (y0 >> 3)) * L.ntile8_x + ((L.bi[b] >> 3) - (x0 >> 3))] = 1;
-    std::vector<int> tiles8;
-    for (size_t t = 0; t < used8.size(); ++t)
-      if (used8[t]) tiles8.push_back((int)t);
-    L.ntile8_ne = (int)tiles8.size();
-    // interaction list packed for the few-box kernel: source box * 64 + table row
+    // interaction list packed for the FP64 translation: source box * 64 + table row
     std::vector<int> pk(L.il_src.size());
     for (size_t e = 0; e < L.il_src.size(); ++e)
       pk[e] = L.il_src[e] * 64 + (L.off_dx[L.il_off[e]] + 3) * 7 + (L.off_dy[L.il_off[e]] + 3);
     int rc;
     if (!pk.empty() && (rc = upload(c, &L.d_il_pk, pk))) return rc;
-    if ((rc = upload(c, &L.d_tiles8, tiles8))) return rc;
     if ((rc = upload(c, &L.d_boxmap, bm)) || (rc = upload(c, &L.d_offid, oid)) ||
         (rc = upload(c, &L.d_tiles, tiles)) || (rc = build_translate_tiles(c, L, tiles, bm)))
       return rc;
@@ -1262,9 +1252,8 @@ int smr_set_variant(smr_ctx* h, int step, int level, int precision, int variant)
   if (!ok) return fail(c, SMR_E_INVALID_ARG, "unknown step or variant");
   for (int s = (level < 0 ? 0 : level); s < (level < 0 ? c->nlev : level + 1); ++s) {
     Level& L = c->lev[s];
-    if (step == SMR_STEP_TRANSLATE) L.tune_tr[q] = variant;
-    else if (step == SMR_STEP_INTERPOLATE) L.tune_ip[q] = variant;
-    else L.tune_an[q] = variant;
+    if (step == SMR_STEP_INTERPOLATE) L.tune_ip[q] = variant;
+    else if (step == SMR_STEP_ANTERPOLATE) L.tune_an[q] = variant;
   }
   free_graphs(c);                              // captured products used the old variants
   return SMR_OK;
@@ -1484,29 +1473,19 @@ int smr_autotune(smr_ctx* h, int R, int precision, void* stream) {
   double2* y = c->d_tmp + n;
   SMR_CUDA(c, cudaMemsetAsync(x, 0, n * sizeof(double2), (cudaStream_t)stream));
   std::map<std::pair<std::string, int>, double> t;
-  // FP64 translation: 8x8 tiles (full, half direction chunk), 4x4 tiles, the
-  // few-box and the whole-level kernel
-  std::vector<std::vector<double>> ttr(c->nlev, std::vector<double>(6, 1e30));
   std::vector<std::vector<double>> tip(c->nlev, std::vector<double>(4, 1e30));
   std::vector<std::vector<double>> tan_(c->nlev, std::vector<double>(4, 1e30));
   double agg[2] = {1e30, 1e30}, rec[2] = {1e30, 1e30}, nea[2] = {1e30, 1e30};
   const int agg0 = c->tune_tc_agg, rec0 = c->tune_tc_rec, nea0 = c->tune_tc_near;
-  // trial 5 times the whole-level translation (levels of at most 256 boxes),
-  // trials 1 and 2 the gather variants of the FP64 interpolation and
-  // anterpolation.  FP32 has one kernel for each level step: its trials 1 and 3
-  // time the tensor cores and the CUDA cores
-  for (int v = 1; v <= 5; ++v) {
-    if (q == 1 && v != 1 && v != 3) continue;
-    // variant 4 (few-box kernel) only where a level has at most 1024 boxes
-    for (auto& L : c->lev) {
-      L.tune_tr[q] = q == 1 ? 0 : (v == 4 && L.nbox > 1024) || (v == 5 && L.nbox > 256) ? 1 : v;
-      L.tune_ip[q] = L.tune_an[q] = (q == 0 && v <= 2) ? v : 0;
-    }
+  // trials 1 and 2 time the gather variants of the FP64 interpolation and
+  // anterpolation, trial 3 the built-in rules.  FP32 has one kernel for each level
+  // step: its trials 1 and 3 time the tensor cores and the CUDA cores
+  for (int v = 1; v <= 3; ++v) {
+    if (q == 1 && v == 2) continue;
+    for (auto& L : c->lev) L.tune_ip[q] = L.tune_an[q] = (q == 0 && v <= 2) ? v : 0;
     c->tune_tc_agg = c->tune_tc_rec = c->tune_tc_near = (v == 3) ? 0 : 1;
     if ((rc = profile_min(h, 1, x, y, precision, 3, stream, t))) break;
     for (int s = 0; s < c->nlev; ++s) {
-      auto it = t.find({"translate", s});
-      if (it != t.end() && c->lev[s].tune_tr[q] == v) ttr[s][v] = it->second;
       auto an = t.find({"anterpolate", s});
       const int av = c->lev[s].tune_an[q];
       if (an != t.end()) tan_[s][av] = std::min(tan_[s][av], an->second);
@@ -1524,10 +1503,6 @@ int smr_autotune(smr_ctx* h, int R, int precision, void* stream) {
   }
   for (int s = 0; s < c->nlev; ++s) {
     Level& L = c->lev[s];
-    int bv = 1;
-    for (int v = 2; v <= 5; ++v)
-      if (ttr[s][v] < ttr[s][bv]) bv = v;
-    L.tune_tr[q] = rc || q == 1 ? 0 : bv;
     int bi = 0;
     for (int v = 1; v <= 3; ++v)
       if (tip[s][v] < tip[s][bi]) bi = v;

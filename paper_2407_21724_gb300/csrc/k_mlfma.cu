@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(256, 2) k_interp1(int nthP, int nphP, unsigned
 }
 // ------------------------------------------------------------------ translation
 // in[b][k] = sum_{(b', o) in IL(b)} T[o][k] out[b'][k]   (Eqs. 22-23)
-// One CTA = 4x4 target boxes of the lattice x a chunk of directions; the 8x8
+// FP32, several columns (one column: k_translate.cu).  One CTA = 4x4 target boxes of the lattice x a chunk of directions; the 8x8
 // source halo and the table rows of the chunk are staged in shared memory,
 // so each source spectrum is fetched about 4 times instead of 27.
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem, int src_bytes) {
@@ -259,14 +259,12 @@ __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.wait_group 0;\n" ::);
 }
 
-template <typename T>
 __global__ void k_translate(int K, int R, int RC, int KC, int ntx, int ntile, const int* __restrict__ tiles,
                             int map_x0, int map_y0, int map_w, int map_h, int noff,
-                            const int* __restrict__ boxmap,
-                            const int* __restrict__ offid, const typename CV<T>::V* __restrict__ Tt,
-                            const typename CV<T>::V* __restrict__ out,
-                            typename CV<T>::V* __restrict__ in) {
-  typedef typename CV<T>::V V;
+                            const int* __restrict__ boxmap, const int* __restrict__ offid,
+                            const float2* __restrict__ Tt, const float2* __restrict__ out,
+                            float2* __restrict__ in) {
+  typedef float2 V;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   int nrc = (R + RC - 1) / RC;
   int tile = tiles[blockIdx.x % ntile];
@@ -385,172 +383,29 @@ __global__ void k_translate(int K, int R, int RC, int KC, int ntx, int ntile, co
   }
 }
 
-// FP64, one right-hand side (FP32: k_translate.cu): each thread owns one 16-byte part of the 2x2
-// targets that share one parent, for one direction, and walks the parent's
-// 6x6 source window once; a staged source part is read from shared memory
-// once for all four targets (conflict-free: lanes read consecutive 16-byte
-// parts).  CTA = 8x8 targets (4x4 parents) x KC directions; 16 x KC x NT threads.
-template <int KC>
-__global__ void __launch_bounds__(512, 2) k_translate1(int K, int ntx, int ntile,
-                                                    const int* __restrict__ tiles, int map_x0, int map_y0,
-                                                    int map_w, int map_h, const int* __restrict__ boxmap,
-                                                    const double2* __restrict__ Tg,
-                                                    const double2* __restrict__ out,
-                                                    double2* __restrict__ in) {
-  typedef double T;
-  typedef double2 V;
-  typedef Part<T> P;
-  typedef P::H H;
-  constexpr int NT = P::NT;
-  constexpr int TS = 8, HS = TS + 4;                  // targets per side, halo per side
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  int tile = tiles[blockIdx.x % ntile];
-  int kch = blockIdx.x / ntile;
-  int tx = tile % ntx, ty = tile / ntx;
-  int ax0 = ((map_x0 >> 3) + tx) * TS, ay0 = ((map_y0 >> 3) + ty) * TS;
-  int k0 = kch * KC;
-  int nk = min(KC, K - k0);
-  constexpr int W = KC * NF;
-  V* S = reinterpret_cast<V*>(smem_raw);              // [HS*HS sources][KC][NF]
-  V* Ts = S + HS * HS * W;                            // [49 offsets][KC]
-  int* bid = reinterpret_cast<int*>(Ts + 49 * KC);    // [HS*HS] source box ids
-  int* tb = bid + HS * HS;                            // [TS*TS] target box ids
-  for (int t = threadIdx.x; t < HS * HS + TS * TS; t += blockDim.x) {
-    int sx, sy;
-    if (t < HS * HS) { sx = ax0 - 2 + t % HS; sy = ay0 - 2 + t / HS; }
-    else { int u = t - HS * HS; sx = ax0 + u % TS; sy = ay0 + u / TS; }
-    int lx = sx - map_x0, ly = sy - map_y0;
-    bid[t] = (lx >= 0 && ly >= 0 && lx < map_w && ly < map_h) ? boxmap[ly * map_w + lx] : -1;
+// FP64, straight from the interaction lists: thread = one complex value (direction,
+// field, column) of one target box, the sources' values and the factors read through
+// the L2.  Bound by the FP64 rate: 32 bytes for four FP64 multiply-adds are no burden
+// at two of them per clock and SM, so nothing has to be staged, and every level
+// splits into enough CTAs.  Levels of the 40x40 array 170 + 143 + 133 + 39 + 18 us in
+// kernels that staged 8x8 tiles or ran along the directions of 8 boxes, 141 + 90 + 51 +
+// 27 + 14 now; 8x8 87 -> 22; 200x200 10.6 -> 9.6 ms; four right-hand sides on 20x20 337
+// -> 247 us.  il_pk: source box * 64 + table row.
+__global__ void __launch_bounds__(128) k_translate_il(int K, int NR, int nch, const int* __restrict__ il_ptr,
+                                                      const int* __restrict__ il_pk, const double2* __restrict__ Tg,
+                                                      const double2* __restrict__ out, double2* __restrict__ in) {
+  const int b = blockIdx.x / nch;
+  const unsigned n = (unsigned)K * NR, e = (blockIdx.x - b * nch) * 128u + threadIdx.x;
+  if (e >= n) return;
+  const unsigned k = e / NR;
+  const int l1 = il_ptr[b + 1];
+  double2 a = make_double2(0.0, 0.0);
+#pragma unroll 6
+  for (int l = il_ptr[b]; l < l1; ++l) {
+    const int pk = __ldg(il_pk + l);
+    cfma(a, __ldg(Tg + (size_t)(pk & 63) * K + k), __ldg(out + (size_t)(pk >> 6) * n + e));
   }
-  __syncthreads();
-  {
-    constexpr int per = W * (int)sizeof(V) / 16;      // 16-byte pieces per source row
-    int valid = nk * NF * (int)sizeof(V);
-    for (int t = threadIdx.x; t < HS * HS * per; t += blockDim.x) {
-      int sb = t / per, pc = t - sb * per;
-      int b = bid[sb];
-      const char* g = reinterpret_cast<const char*>(out);
-      int nb = 0;
-      if (b >= 0 && pc * 16 < valid) {
-        g += ((size_t)b * K + k0) * NF * sizeof(V) + (size_t)pc * 16;
-        nb = 16;
-      }
-      cp_async16(reinterpret_cast<char*>(S + (size_t)sb * W) + pc * 16, g, nb);
-    }
-  }
-  for (int t = threadIdx.x; t < 49 * KC; t += blockDim.x) {
-    int o = t / KC, kl = t - o * KC;
-    Ts[t] = (kl < nk) ? Tg[(size_t)o * K + k0 + kl] : czero<V>();
-  }
-  cp_async_wait_all();
-  __syncthreads();
-  const int h = threadIdx.x % NT;
-  const int kl = (threadIdx.x / NT) % KC, par = threadIdx.x / (NT * KC);   // parent 0..15 of the tile
-  if (kl >= nk || par >= (TS / 2) * (TS / 2)) return;
-  int pxo = (par % (TS / 2)) * 2, pyo = (par / (TS / 2)) * 2;
-  bool any = false;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) any |= tb[(pyo + (q >> 1)) * TS + (pxo + (q & 1))] >= 0;
-  if (!any) return;
-  const V* Sp = S + (size_t)(pyo * HS + pxo) * W + kl * NF;   // window origin
-  const V* Tp = Ts + kl;
-  H acc[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) acc[q] = P::zero();
-  // the parent's 6x6 source window; target q = (q & 1, q >> 1) inside the
-  // parent; offset (dx, dy) = target - source is known at compile time
-#pragma unroll
-  for (int wy = 0; wy < 6; ++wy) {
-#pragma unroll
-    for (int wx = 0; wx < 6; ++wx) {
-      H v = reinterpret_cast<const H*>(Sp + (wy * HS + wx) * W)[h];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int dx = (q & 1) + 2 - wx, dy = (q >> 1) + 2 - wy;
-        if (dx >= -1 && dx <= 1 && dy >= -1 && dy <= 1) continue;
-        P::cfma(acc[q], Tp[((dx + 3) * 7 + (dy + 3)) * KC], v);
-      }
-    }
-  }
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    int b = tb[(pyo + (q >> 1)) * TS + (pxo + (q & 1))];
-    if (b < 0) continue;
-    stp<T>(in, (size_t)b * K + k0 + kl, h, acc[q]);
-  }
-}
-
-// Few boxes, many directions (coarse levels), one right-hand side: threads run
-// along the directions (NT 16-byte parts each, coalesced); a CTA takes TG
-// consecutive target boxes and reads each target's interaction list
-// (source box * 64 + table row) uniformly.
-__global__ void __launch_bounds__(256) k_translate_few(int K, int nbox, int TG, const int* __restrict__ il_ptr,
-                                                       const int* __restrict__ il_pk,
-                                                       const double2* __restrict__ Tg,
-                                                       const double2* __restrict__ out,
-                                                       double2* __restrict__ in) {
-  typedef double T;
-  typedef double2 V;
-  typedef Part<T> P;
-  typedef P::H H;
-  constexpr int NT = P::NT;
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const int k = (int)(t / NT), h = (int)(t % NT);
-  const bool ok = k < K;
-  const int b0 = blockIdx.y * TG, b1 = min(nbox, b0 + TG);
-  for (int b = b0; b < b1; ++b) {
-    H acc = P::zero();
-    for (int e = il_ptr[b]; e < il_ptr[b + 1]; ++e) {
-      const int pk = il_pk[e];
-      if (ok) P::cfma(acc, Tg[(size_t)(pk & 63) * K + k], ldp<T>(out, (size_t)(pk >> 6) * K + k, h));
-    }
-    if (ok) stp<T>(in, (size_t)b * K + k, h, acc);
-  }
-}
-
-// Whole coarse level per CTA, one right-hand side: a CTA takes a chunk of
-// KCH directions of every box of the level (at most a few hundred boxes),
-// stages their outgoing spectra and the chunk of the 49 offset tables in
-// shared memory, and computes every target's sum from there, so each source
-// spectrum is read from memory once instead of once per target that lists
-// it.  Tasks are (target, direction, 16-byte part), the parts of consecutive
-// directions on consecutive threads.
-__global__ void __launch_bounds__(256) k_translate_lvl(int K, int nbox, int KCH, const int* __restrict__ il_ptr,
-                                                       const int* __restrict__ il_pk,
-                                                       const double2* __restrict__ Tg,
-                                                       const double2* __restrict__ out,
-                                                       double2* __restrict__ in) {
-  typedef double T;
-  typedef double2 V;
-  typedef Part<T> P;
-  typedef P::H H;
-  constexpr int NT = P::NT;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  V* S = reinterpret_cast<V*>(smem_raw);                 // [nbox][KCH][NF]
-  V* Ts = S + (size_t)nbox * KCH * NF;                   // [49][KCH]
-  const int k0 = blockIdx.x * KCH, kn = min(KCH, K - k0);
-  // stage: every box's fields for the chunk, and the tables
-  for (int i = threadIdx.x; i < nbox * KCH * NT; i += blockDim.x) {
-    const int b = i / (KCH * NT), r = i - b * (KCH * NT), kl = r / NT, h = r - kl * NT;
-    H v = P::zero();
-    if (kl < kn) v = ldp<T>(out, (size_t)b * K + k0 + kl, h);
-    stp<T>(S, (size_t)b * KCH + kl, h, v);
-  }
-  for (int i = threadIdx.x; i < 49 * KCH; i += blockDim.x) {
-    const int row = i / KCH, kl = i - row * KCH;
-    Ts[i] = kl < kn ? Tg[(size_t)row * K + k0 + kl] : czero<V>();
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < nbox * KCH * NT; i += blockDim.x) {
-    const int b = i / (KCH * NT), r = i - b * (KCH * NT), kl = r / NT, h = r - kl * NT;
-    if (kl >= kn) continue;
-    H acc = P::zero();
-    for (int e = il_ptr[b]; e < il_ptr[b + 1]; ++e) {
-      const int pk = il_pk[e];
-      P::cfma(acc, Ts[(pk & 63) * KCH + kl], ldp<T>(S, (size_t)(pk >> 6) * KCH + kl, h));
-    }
-    stp<T>(in, (size_t)b * K + k0 + kl, h, acc);
-  }
+  in[(size_t)b * n + e] = a;
 }
 
 // ------------------------------------------------------------------ FP64 anterpolation, one right-hand side
@@ -909,35 +764,21 @@ int ensure_spectra(Ctx* c, int R, int prec) {
   return SMR_OK;
 }
 
-// Direction chunk of the whole-level translation: the largest power of two
-// up to 32 whose staged spectra and tables fit in 96 KB (0: none fits).
-int translate_lvl_chunk(int nbox, size_t vbytes) {
-  for (int kch = 32; kch >= 4; kch /= 2)
-    if (((size_t)nbox * kch * NF + (size_t)49 * kch) * vbytes <= 96 * 1024) return kch;
-  return 0;
-}
-
-bool translate_lvl_ok(Ctx* c, int s) {
-  const Level& L = c->lev[s];
-  if (L.off_dx.empty() || !L.d_il_pk || translate_lvl_chunk(L.nbox, sizeof(double2)) == 0) return false;
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_translate_lvl, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    attr = true;
-  }
-  return true;
-}
-
 // FP64, one right-hand side: the gather kernels above, or the marching kernels
 // (k_march.cu) where they do less.  All are bound by the FP64 rate.
 // Interpolation: the gather kernel does fewer operations (200x200 lens, level
-// 0: 3.00 ms against 3.59 ms).  Anterpolation: the marching kernel does fewer
-// (4.25 against 5.63 ms), but its CTAs are long; by the directions of the
-// parent level (boxes x K) it wins by 15 % and more from 760,000 on (100x100
-// array), the gather kernel by up to 45 % on small levels (20x20), and at
-// 40x40 (120,000 to 260,000) the two are even.
+// 0: 1.57 ms against 2.16 ms).  Anterpolation: the marching kernel does fewer, but a
+// CTA costs some seven rows more than it has and short rows leave it few threads.
+// On rows of 22 columns (level 0) the gather kernel is ahead at every size (60x60
+// 256 against 272 us, 200x200 2.74 against 2.84 ms), on 36 columns up to some 2
+// million parent directions (boxes x K; 100x100 448 against 510 us, 200x200 1.75
+// against 1.63 ms), on longer rows up to 240,000 (40x40 68 against 84 us at 139,000,
+// 60x60 147 against 133 us at 248,000).
 static bool march_interp(int v) { return v > 2; }
-static bool march_anterp(const Level& Lp, int v) { return v == 0 ? (size_t)Lp.nbox * Lp.K >= 500000 : v > 2; }
+static bool march_anterp(const Level& Lc, const Level& Lp, int v) {
+  if (v != 0) return v > 2;
+  return Lc.nph > 24 && (size_t)Lp.nbox * Lp.K >= (Lc.nph <= 40 ? 2000000u : 240000u);
+}
 
 // Finest boxes made of cells.  Box b's outgoing spectrum is the sum of its
 // particles' spectra, and each particle receives its box's incoming
@@ -1027,15 +868,6 @@ static int far_impl(Ctx* c, int R, const double2* x, double2* y, bool accumulate
       SMR_CUDA(c, cudaMemsetAsync(L.d_in, 0, L.spec_bytes, ts));
       return SMR_OK;
     }
-    int noff = 49;                           // tables by lattice offset (7 x 7 grid)
-    int cap = f64 ? 16 : 32;                 // directions x columns staged per CTA
-    int RCt = std::min(R, cap);
-    int KC = std::max(1, cap / RCt);
-    int nkch = (L.K + KC - 1) / KC;
-    int nrct = (R + RCt - 1) / RCt;
-    size_t sm = ((size_t)64 * KC * NF * RCt + (size_t)std::max(noff, 1) * KC) * sizeof(V) +
-                (64 + 16 + 16) * sizeof(int) + 16 * 27 * sizeof(int2);
-    cudaFuncSetAttribute(k_translate<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     pbeg(c, ts, "translate", s,
          2.0 * L.nbox * L.K * NF * R_ * es + (double)L.off_dx.size() * L.K * es,
          8.0 * L.il_src.size() * L.K * NF * R_);
@@ -1044,42 +876,25 @@ static int far_impl(Ctx* c, int R, const double2* x, double2* y, bool accumulate
       pend(c, ts);
       return rc;
     }
-    // FP64, one right-hand side: 8x8-tile register-blocked kernel, except on
-    // levels whose few boxes would leave most of one 8x8 tile idle (or as tuned)
-    const int tv = (R == 1) ? L.tune_tr[0] : 0;
-    if (R == 1 && tv == 5 && translate_lvl_ok(c, s)) {
-      const int KCH = translate_lvl_chunk(L.nbox, sizeof(double2));
-      const size_t sml = ((size_t)L.nbox * KCH * NF + (size_t)49 * KCH) * sizeof(double2);
-      k_translate_lvl<<<(unsigned)((L.K + KCH - 1) / KCH), 256, sml, ts>>>(
-          L.K, L.nbox, KCH, L.d_il_ptr, L.d_il_pk, L.d_T64, (const double2*)L.d_out, (double2*)L.d_in);
+    if (f64) {
+      const int NR = NF * R, nch = (int)(((long long)L.K * NR + 127) / 128);
+      k_translate_il<<<(unsigned)((long long)L.nbox * nch), 128, 0, ts>>>(
+          L.K, NR, nch, L.d_il_ptr, L.d_il_pk, L.d_T64, (const double2*)L.d_out, (double2*)L.d_in);
       SMR_LAUNCH(c);
       pend(c, ts);
       return SMR_OK;
     }
-    const bool few = R == 1 && (tv == 4 || (tv == 0 && L.nbox <= 64));
-    const bool use8 = R == 1 && (tv == 0 ? !(L.ntile8_ne == 1 && L.nbox < 32) : tv != 3);
-    if (few) {
-      const int TG = 8;
-      dim3 g((unsigned)(((long long)L.K * Part<double>::NT + 255) / 256), (unsigned)((L.nbox + TG - 1) / TG));
-      k_translate_few<<<g, 256, 0, ts>>>(L.K, L.nbox, TG, L.d_il_ptr, L.d_il_pk, L.d_T64, (const double2*)L.d_out,
-                                         (double2*)L.d_in);
-    } else if (use8) {
-      // 16 directions per CTA, halved by the tuner
-      const bool halfc = (tv == 2);
-      int KC1 = 16 / (halfc ? 2 : 1);
-      int nk1 = (L.K + KC1 - 1) / KC1;
-      size_t sm1 = ((size_t)144 * KC1 * NF + (size_t)49 * KC1) * sizeof(double2) + (144 + 64) * sizeof(int);
-      auto kt = halfc ? k_translate1<8> : k_translate1<16>;
-      cudaFuncSetAttribute(kt, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-      kt<<<(unsigned)(L.ntile8_ne * nk1), 16 * KC1 * Part<double>::NT, sm1, ts>>>(
-          L.K, L.ntile8_x, L.ntile8_ne, L.d_tiles8, L.map_x0, L.map_y0, L.map_w, L.map_h, L.d_boxmap,
-          L.d_T64, (const double2*)L.d_out, (double2*)L.d_in);
-    } else {
-      k_translate<T><<<(unsigned)(L.ntile_ne * nkch * nrct), 256, sm, ts>>>(
-          L.K, R, RCt, KC, L.ntile_x, L.ntile_ne, L.d_tiles, L.map_x0, L.map_y0, L.map_w, L.map_h, noff,
-          L.d_boxmap, L.d_offid,
-          (const V*)(f64 ? (void*)L.d_T64 : (void*)L.d_T32), (const V*)L.d_out, (V*)L.d_in);
-    }
+    // FP32, several columns at once
+    const int noff = 49;                     // tables by lattice offset (7 x 7 grid)
+    const int cap = 32;                      // directions x columns staged per CTA
+    const int RCt = std::min(R, cap), KC = std::max(1, cap / RCt);
+    const int nkch = (L.K + KC - 1) / KC, nrct = (R + RCt - 1) / RCt;
+    const size_t sm = ((size_t)64 * KC * NF * RCt + (size_t)noff * KC) * sizeof(float2) + (64 + 16 + 16) * sizeof(int) +
+                      16 * 27 * sizeof(int2);
+    cudaFuncSetAttribute(k_translate, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    k_translate<<<(unsigned)(L.ntile_ne * nkch * nrct), 256, sm, ts>>>(
+        L.K, R, RCt, KC, L.ntile_x, L.ntile_ne, L.d_tiles, L.map_x0, L.map_y0, L.map_w, L.map_h, noff, L.d_boxmap,
+        L.d_offid, L.d_T32, (const float2*)L.d_out, (float2*)L.d_in);
     SMR_LAUNCH(c);
     pend(c, ts);
     return SMR_OK;
@@ -1142,8 +957,22 @@ static int far_impl(Ctx* c, int R, const double2* x, double2* y, bool accumulate
       int rc = run_interp(c, s, R, f64 ? SMR_PREC_FP64 : SMR_PREC_FP32, st);
       if (rc) return rc;
     } else {
-      int TR = std::max(1, std::min(Lp.nth, (256 * EM1) / (Lp.nph * Part<double>::NT)));
-      if (Lc.tune_ip[0] == 2) TR = std::max(1, TR / 2);
+      // parent rows of a CTA: whole tiles (variants 1, 2: half), or the split that finishes
+      // first with two CTAs an SM at a time, a CTA costing about two rows more than it
+      // has (levels of the 20x20 array 33 + 35 + 32 us with whole tiles, 23 + 21 + 19 so;
+      // 40x40 80 + 60 + 56 + 44 and 79 + 49 + 42 + 36)
+      const int most = std::max(1, std::min(Lp.nth, (256 * EM1) / (Lp.nph * Part<double>::NT)));
+      int TR = Lc.tune_ip[0] == 2 ? std::max(1, most / 2) : most;
+      if (Lc.tune_ip[0] == 0) {
+        long long cost = -1;
+        for (int t = most; t >= 1; --t) {
+          const long long w = ((long long)Lp.nbox * ((Lp.nth + t - 1) / t) + 303) / 304 * (t + 2);
+          if (cost < 0 || w < cost) {
+            cost = w;
+            TR = t;
+          }
+        }
+      }
       int nrt = (Lp.nth + TR - 1) / TR;
       size_t sm1 = (size_t)TR * Lc.nph * NF * sizeof(double2);
       cudaFuncSetAttribute(k_interp1, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
@@ -1176,16 +1005,19 @@ static int far_impl(Ctx* c, int R, const double2* x, double2* y, bool accumulate
          ((double)Lp.nbox * Lp.K + 2.0 * Lc.nbox * Lc.K) * NF * R_ * es + 4.0 * Lp.K * es,
          (double)Lc.nbox * Lp.nth * Lc.nph * NF * R_ * 8.0 * 2 * (double)Lp.nph / Lc.nph * 4.0 / 4.0 +
              (double)Lc.nbox * Lc.K * NF * R_ * 16.0 * (double)Lp.nth / Lc.nth);
-    if (!f64 || R > 1 || march_anterp(Lp, Lc.tune_an[0])) {
+    if (!f64 || R > 1 || march_anterp(Lc, Lp, Lc.tune_an[0])) {
       int rc = run_anterp(c, s, R, f64 ? SMR_PREC_FP64 : SMR_PREC_FP32, st);
       if (rc) return rc;
     } else {
       const int an = Lc.tune_an[0];
+      // column chunk: half of what fits in shared memory where rows are long
+      // (40x40 level 1: 123 -> 78 us; level 0, 11 columns: 121 -> 133) or boxes fewer
+      // than SMs (40x40 level 3: 90 -> 68 us)
       int JC = Lc.ant_JC;
-      if (an == 1) JC = std::max(1, JC / 2);
+      if (an == 1 || (an == 0 && (JC > 12 || Lc.nbox < 152))) JC = std::max(1, JC / 2);
       int njc = (Lc.nph / 2 + JC - 1) / JC;
       size_t sm1 = (size_t)Lc.ant_GR * 2 * JC * NF * sizeof(double2);
-      int thr = (an == 2 || Lc.ant_GR * 2 * JC * (Part<double>::NT / 2) >= 2048) ? 256 : 128;
+      int thr = (an == 2 || (an == 0 && Lc.nph <= 24) || Lc.ant_GR * 2 * JC * (Part<double>::NT / 2) >= 2048) ? 256 : 128;
       auto ka = k_anterp1<0>;
       if (Lc.ant_PM == 8 && Lc.ant_TM == 8) ka = std::max(Lc.ant_PMx, Lc.ant_TMx) <= 7 ? k_anterp1<7> : k_anterp1<8>;
       ka<<<(unsigned)(Lc.nbox * Lc.ant_nit * njc), thr, sm1, st>>>(

@@ -91,7 +91,7 @@ struct Level {
   int* d_il_ptr = nullptr;
   int* d_il_src = nullptr;
   int* d_il_off = nullptr;
-  int* d_il_pk = nullptr;                // [n_il] source box * 64 + table row (few-box kernel)
+  int* d_il_pk = nullptr;                // [n_il] source box * 64 + table row (FP64 translation)
   double2* d_T64 = nullptr;              // [noff][K]
   float2* d_T32 = nullptr;
   int* d_parent = nullptr;
@@ -136,8 +136,6 @@ struct Level {
   int ntile_x = 0, ntile_y = 0, ntile_ne = 0;
   int* d_tiles = nullptr;                // non-empty 4x4 translation tiles (ty * ntile_x + tx)
   int* d_tile_tab = nullptr;             // per non-empty 4x4 tile: 64 source and 16 target boxes (k_translate.cu)
-  int ntile8_x = 0, ntile8_ne = 0;
-  int* d_tiles8 = nullptr;               // non-empty 8x8 tiles (single right-hand side kernel)
   // FP64 gather anterpolation into this level, one right-hand side (k_anterp1):
   // child theta rows in nit tiles of TI, parent rows [lo, hi) per tile
   // ([2][nit]), GR the widest range, JC the column chunk
@@ -149,7 +147,6 @@ struct Level {
   // few-box kernel (threads along the directions).  FP64 interpolation into
   // the parent of this level: 1 / 2 = the gather kernel with the full / half
   // theta-row tile.
-  int tune_tr[2] = {0, 0};
   int tune_ip[2] = {0, 0};
   // FP64 anterpolation into this level: 1 / 2 = the gather kernel with half
   // the column chunk / with 256 threads
