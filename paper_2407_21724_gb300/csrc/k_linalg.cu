@@ -25,8 +25,8 @@ __global__ void k_multidot_part(int J, long long n, int R, int rl, int nchunk, l
     long long i0 = chunk * rows_per, i1 = min(n, i0 + rows_per);
     for (long long i = i0 + a; i < i1; i += rl) {
       double2 x = v[i * R + r], y = w[i * R + r];
-      acc.x += x.x * y.x + x.y * y.y;
-      acc.y += x.x * y.y - x.y * y.x;
+      acc.x = fma(x.y, y.y, fma(x.x, y.x, acc.x));
+      acc.y = fma(-x.y, y.x, fma(x.x, y.y, acc.y));
     }
   }
   __shared__ double2 red[256];
@@ -70,15 +70,15 @@ __global__ void k_multi_axpy(int J, long long n, int R, const double2* __restric
     double2 v2 = V[(size_t)(j + 2) * ldv + t], v3 = V[(size_t)(j + 3) * ldv + t];
     double2 c0 = h[(size_t)j * R + r], c1 = h[(size_t)(j + 1) * R + r];
     double2 c2 = h[(size_t)(j + 2) * R + r], c3 = h[(size_t)(j + 3) * R + r];
-    acc.x += v0.x * c0.x - v0.y * c0.y + v1.x * c1.x - v1.y * c1.y;
-    acc.y += v0.x * c0.y + v0.y * c0.x + v1.x * c1.y + v1.y * c1.x;
-    acc2.x += v2.x * c2.x - v2.y * c2.y + v3.x * c3.x - v3.y * c3.y;
-    acc2.y += v2.x * c2.y + v2.y * c2.x + v3.x * c3.y + v3.y * c3.x;
+    acc.x = fma(-v1.y, c1.y, fma(v1.x, c1.x, fma(-v0.y, c0.y, fma(v0.x, c0.x, acc.x))));
+    acc.y = fma(v1.y, c1.x, fma(v1.x, c1.y, fma(v0.y, c0.x, fma(v0.x, c0.y, acc.y))));
+    acc2.x = fma(-v3.y, c3.y, fma(v3.x, c3.x, fma(-v2.y, c2.y, fma(v2.x, c2.x, acc2.x))));
+    acc2.y = fma(v3.y, c3.x, fma(v3.x, c3.y, fma(v2.y, c2.x, fma(v2.x, c2.y, acc2.y))));
   }
   for (; j < J; ++j) {
     double2 v = V[(size_t)j * ldv + t], c = h[(size_t)j * R + r];
-    acc.x += v.x * c.x - v.y * c.y;
-    acc.y += v.x * c.y + v.y * c.x;
+    acc.x = fma(-v.y, c.y, fma(v.x, c.x, acc.x));
+    acc.y = fma(v.y, c.x, fma(v.x, c.y, acc.y));
   }
   acc.x += acc2.x;
   acc.y += acc2.y;
@@ -189,10 +189,10 @@ __global__ void __launch_bounds__(256) k_gs_dot(int J, long long n, const double
     double ax = 0, ay = 0, bx = 0, by = 0;
 #pragma unroll
     for (int q = 0; q < GS_RPL; ++q) {
-      ax += a[q].x * wr[q].x + a[q].y * wr[q].y;
-      ay += a[q].x * wr[q].y - a[q].y * wr[q].x;
-      bx += b[q].x * wr[q].x + b[q].y * wr[q].y;
-      by += b[q].x * wr[q].y - b[q].y * wr[q].x;
+      ax = fma(a[q].y, wr[q].y, fma(a[q].x, wr[q].x, ax));
+      ay = fma(-a[q].y, wr[q].x, fma(a[q].x, wr[q].y, ay));
+      bx = fma(b[q].y, wr[q].y, fma(b[q].x, wr[q].x, bx));
+      by = fma(-b[q].y, wr[q].x, fma(b[q].x, wr[q].y, by));
     }
     ax = warp_sum(ax);
     ay = warp_sum(ay);
@@ -209,8 +209,8 @@ __global__ void __launch_bounds__(256) k_gs_dot(int J, long long n, const double
 #pragma unroll
     for (int q = 0; q < GS_RPL; ++q) {
       double2 a = (full || i0 + 32 * q < n) ? v0[32 * q] : make_double2(0, 0);
-      ax += a.x * wr[q].x + a.y * wr[q].y;
-      ay += a.x * wr[q].y - a.y * wr[q].x;
+      ax = fma(a.y, wr[q].y, fma(a.x, wr[q].x, ax));
+      ay = fma(-a.y, wr[q].x, fma(a.x, wr[q].y, ay));
     }
     ax = warp_sum(ax);
     ay = warp_sum(ay);
@@ -239,8 +239,8 @@ __global__ void __launch_bounds__(256) k_gs_axpy(int J, long long n, const doubl
     return full || i0 + 32 * q < n ? V[(size_t)jj * ldv + i0 + 32 * q] : make_double2(0, 0);
   };
   auto add = [&](double2& o, double2 a, double2 c0) {
-    o.x += a.x * c0.x - a.y * c0.y;
-    o.y += a.x * c0.y + a.y * c0.x;
+    o.x = fma(-a.y, c0.y, fma(a.x, c0.x, o.x));
+    o.y = fma(a.y, c0.x, fma(a.x, c0.y, o.y));
   };
   int j = 0;
   for (; j + JU <= J; j += JU) {
@@ -418,10 +418,10 @@ __global__ void __launch_bounds__(256) k_gs32_dot(int J, long long n, const floa
 #pragma unroll
     for (int q = 0; q < G32_RPL; ++q) {
       float4 u = wf[q];
-      ax += a[q].x * u.x + a[q].y * u.y + a[q].z * u.z + a[q].w * u.w;
-      ay += a[q].x * u.y - a[q].y * u.x + a[q].z * u.w - a[q].w * u.z;
-      bx += b[q].x * u.x + b[q].y * u.y + b[q].z * u.z + b[q].w * u.w;
-      by += b[q].x * u.y - b[q].y * u.x + b[q].z * u.w - b[q].w * u.z;
+      ax = fma(a[q].w, u.w, fma(a[q].z, u.z, fma(a[q].y, u.y, fma(a[q].x, u.x, ax))));
+      ay = fma(-a[q].w, u.z, fma(a[q].z, u.w, fma(-a[q].y, u.x, fma(a[q].x, u.y, ay))));
+      bx = fma(b[q].w, u.w, fma(b[q].z, u.z, fma(b[q].y, u.y, fma(b[q].x, u.x, bx))));
+      by = fma(-b[q].w, u.z, fma(b[q].z, u.w, fma(-b[q].y, u.x, fma(b[q].x, u.y, by))));
     }
     ax = warp_sumf(ax);
     ay = warp_sumf(ay);
@@ -438,8 +438,8 @@ __global__ void __launch_bounds__(256) k_gs32_dot(int J, long long n, const floa
 #pragma unroll
     for (int q = 0; q < G32_RPL; ++q) {
       float4 a = ld_pair(v0, i0 + 64 * q, n, full), u = wf[q];
-      ax += a.x * u.x + a.y * u.y + a.z * u.z + a.w * u.w;
-      ay += a.x * u.y - a.y * u.x + a.z * u.w - a.w * u.z;
+      ax = fma(a.w, u.w, fma(a.z, u.z, fma(a.y, u.y, fma(a.x, u.x, ax))));
+      ay = fma(-a.w, u.z, fma(a.z, u.w, fma(-a.y, u.x, fma(a.x, u.y, ay))));
     }
     ax = warp_sumf(ax);
     ay = warp_sumf(ay);
@@ -465,10 +465,10 @@ __global__ void __launch_bounds__(256) k_gs32_axpy(int J, long long n, const flo
 #pragma unroll
   for (int q = 0; q < RPL; ++q) acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
   auto add = [&](float4& o, float4 a, float2 c0) {
-    o.x += a.x * c0.x - a.y * c0.y;
-    o.y += a.x * c0.y + a.y * c0.x;
-    o.z += a.z * c0.x - a.w * c0.y;
-    o.w += a.z * c0.y + a.w * c0.x;
+    o.x = fma(-a.y, c0.y, fma(a.x, c0.x, o.x));
+    o.y = fma(a.y, c0.x, fma(a.x, c0.y, o.y));
+    o.z = fma(-a.w, c0.y, fma(a.z, c0.x, o.z));
+    o.w = fma(a.w, c0.x, fma(a.z, c0.y, o.w));
   };
   int j = 0;
   for (; j + JU <= J; j += JU) {
@@ -546,8 +546,8 @@ __global__ void k_gsr_dot(int J, long long n, int R, int rl, int nchunk, long lo
       float2 x = v[i * R + r];
       double2 yd = w[i * R + r];
       float2 y = make_float2((float)yd.x, (float)yd.y);
-      ax += x.x * y.x + x.y * y.y;
-      ay += x.x * y.y - x.y * y.x;
+      ax = fma(x.y, y.y, fma(x.x, y.x, ax));
+      ay = fma(-x.y, y.x, fma(x.x, y.y, ay));
     }
   }
   __shared__ double2 red[256];
@@ -591,15 +591,15 @@ __global__ void k_gsr_axpy(int J, long long n, int R, const float2* __restrict__
   for (; j + 2 <= J; j += 2) {
     float2 v0 = V[(size_t)j * ldv + t], v1 = V[(size_t)(j + 1) * ldv + t];
     float2 c0 = hf[(size_t)j * R + r], c1 = hf[(size_t)(j + 1) * R + r];
-    ax += v0.x * c0.x - v0.y * c0.y;
-    ay += v0.x * c0.y + v0.y * c0.x;
-    bx += v1.x * c1.x - v1.y * c1.y;
-    by += v1.x * c1.y + v1.y * c1.x;
+    ax = fma(-v0.y, c0.y, fma(v0.x, c0.x, ax));
+    ay = fma(v0.y, c0.x, fma(v0.x, c0.y, ay));
+    bx = fma(-v1.y, c1.y, fma(v1.x, c1.x, bx));
+    by = fma(v1.y, c1.x, fma(v1.x, c1.y, by));
   }
   if (j < J) {
     float2 v0 = V[(size_t)j * ldv + t], c0 = hf[(size_t)j * R + r];
-    ax += v0.x * c0.x - v0.y * c0.y;
-    ay += v0.x * c0.y + v0.y * c0.x;
+    ax = fma(-v0.y, c0.y, fma(v0.x, c0.x, ax));
+    ay = fma(v0.y, c0.x, fma(v0.x, c0.y, ay));
   }
   double2 o = w[t];
   o.x += sign * ((double)ax + (double)bx);

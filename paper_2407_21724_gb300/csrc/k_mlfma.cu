@@ -409,7 +409,7 @@ __global__ void __launch_bounds__(128) k_translate_il(int K, int NR, int nch, co
 }
 
 // ------------------------------------------------------------------ FP64 anterpolation, one right-hand side
-// For levels too small for the marching kernel to fill the SMs (run_level).
+// For the levels where it is ahead of the marching kernel (march_anterp).
 // Both adjoint passes fused.  CTA = (child c, tile of
 // child theta rows [i0, i0 + TI), column chunk [j0, j0 + JC) of the first
 // half of the phi grid together with the same chunk shifted by N/2, so that

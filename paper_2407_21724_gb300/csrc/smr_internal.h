@@ -142,11 +142,8 @@ struct Level {
   int ant_TI = 0, ant_nit = 0, ant_GR = 0, ant_JC = 0;
   int* d_ant_lo = nullptr;
   // launch variants chosen by smr_autotune per precision (FP64, FP32), one
-  // right-hand side; 0 = the built-in rule.  Translation: 1 / 2 = 8x8 target
-  // tiles with the full / half direction chunk, 3 = 4x4 tiles, 4 = the
-  // few-box kernel (threads along the directions).  FP64 interpolation into
-  // the parent of this level: 1 / 2 = the gather kernel with the full / half
-  // theta-row tile.
+  // right-hand side: 0 = built-in rule.  FP64 interpolation into the parent level: 1 / 2
+  // the gather kernel with the full / half theta-row tile, 3 the marching kernel.
   int tune_ip[2] = {0, 0};
   // FP64 anterpolation into this level: 1 / 2 = the gather kernel with half
   // the column chunk / with 256 threads
