@@ -23,8 +23,8 @@
 // Bound: instruction issue and shared-memory reads, both near half of their
 // peak with 12 to 14 warps per SM (the windows take the registers).  On the
 // 200x200 lens in FP32 (algorithmic bytes 259 and 414 MB at level 0, of
-// measured 6.68 TB/s): interpolation level 0 96 us, six levels 352 us;
-// anterpolation level 0 121 us, six levels 407 us.  With four fields a direction
+// measured 6.68 TB/s): interpolation level 0 88 us, six levels 313 us;
+// anterpolation level 0 111 us, six levels 378 us.  With four fields a direction
 // these took 168, 597, 235 and 808 us, and kernels that kept the phi-pass rows in
 // shared memory (a barrier and a round trip per row, 7 gathered taps per output)
 // 262, 955, 356 and 1369 us.  Measured with four fields: a thread per child pair
@@ -43,8 +43,15 @@ namespace {
 
 // threads of a CTA (at most), resident CTAs the register budget is set for,
 // copies of one input row per thread (at most)
-constexpr int INTERP_THREADS = 224, INTERP_CTAS = 2, INTERP_NK = 3;
-constexpr int ANTERP_THREADS = 192, ANTERP_CTAS = 2, ANTERP_NK = 4;
+// by precision: more and smaller CTAs wait less at their barriers (FP32, 200x200
+// lens: interpolation 352 us with 2 x 224 threads, 313 with 4 x 128; anterpolation 403
+// with 2 x 192, 378 with 3 x 128), in FP64 their shared rows cost more than that
+// (20x20, four columns, product: 1.24 ms with 4 x 128, 1.21 with 2 x 224)
+template <typename T> constexpr int INTERP_THREADS = sizeof(T) == 8 ? 224 : 128;
+template <typename T> constexpr int INTERP_CTAS = sizeof(T) == 8 ? 2 : 4;
+template <typename T> constexpr int ANTERP_THREADS = sizeof(T) == 8 ? 192 : 128;
+template <typename T> constexpr int ANTERP_CTAS = sizeof(T) == 8 ? 2 : 3;
+constexpr int INTERP_NK = 3, ANTERP_NK = 4;
 constexpr int MARCH_ROWS = 64;                 // parent rows of an interpolation tile, at most
 
 // 16 bytes global -> shared
@@ -254,7 +261,7 @@ __device__ __forceinline__ void stage_turned(const RowCopies<NK>& rc, int rowb, 
 // (the pole reflection, its sign folded into th_w).  ph_src[4 jp + 1]: the
 // child column at or before column jp.
 template <typename T>
-__global__ void __launch_bounds__(INTERP_THREADS, INTERP_CTAS) k_interp_march(
+__global__ void __launch_bounds__(INTERP_THREADS<T>, INTERP_CTAS<T>) k_interp_march(
     int nbox, int nthC, int nphC, int nthP, int nphP, int NT, int TR, MarchTile m, const int4* __restrict__ ch4,
     const int* __restrict__ vlast, const T* __restrict__ th_w, const int* __restrict__ ph_src,
     const T* __restrict__ ph_w, const typename Mp<T>::C* __restrict__ shift,
@@ -396,7 +403,7 @@ __global__ void __launch_bounds__(INTERP_THREADS, INTERP_CTAS) k_interp_march(
 // that no later entry reaches is added to the four children's incoming
 // spectra. 
 template <typename T, int PM, int NK = ANTERP_NK>
-__global__ void __launch_bounds__(ANTERP_THREADS, ANTERP_CTAS) k_anterp_march(
+__global__ void __launch_bounds__(ANTERP_THREADS<T>, ANTERP_CTAS<T>) k_anterp_march(
     int nbox, int nthC, int nphC, int nthP, int nphP, int NT, int TI, MarchTile m, const int4* __restrict__ ch4,
     const int* __restrict__ ent_ptr, const int* __restrict__ ent, const T* __restrict__ entw,
     const int* __restrict__ pst, const T* __restrict__ ptw, int pm, const typename Mp<T>::S* __restrict__ shift,
@@ -585,7 +592,7 @@ int interp_impl(Ctx* c, int s, int R, cudaStream_t st) {
   const bool f64 = sizeof(T) == 8;
   const Level &Lc = c->lev[s], &Lp = c->lev[s + 1];
   const int NT = P::HN * R;
-  const MarchTile m = march_tile(INTERP_THREADS, INTERP_NK, P::HN, P::HN, !f64, Lp.nbox, Lp.nph, NT, Lc.mi_start, 4, 4, 0);
+  const MarchTile m = march_tile(INTERP_THREADS<T>, INTERP_NK, P::HN, P::HN, !f64, Lp.nbox, Lp.nph, NT, Lc.mi_start, 4, 4, 0);
   // FP64: the two FP64 lanes of an SM are the bound, CTAs of one SM take turns
   const int TR = march_rows(m, Lp.nth, f64 ? 1 : 65536 / (128 * m.T), MARCH_ROWS);
   const size_t sm = (size_t)4 * 16 * m.nbx * 4 * m.cc * P::HN;
@@ -607,7 +614,7 @@ int anterp_impl(Ctx* c, int s, int R, cudaStream_t st) {
   const bool f64 = sizeof(T) == 8;
   const Level &Lc = c->lev[s], &Lp = c->lev[s + 1];
   const int NT = P::HN * R, sp = (int)sizeof(typename P::S) / 16;
-  const MarchTile m = march_tile(ANTERP_THREADS, Lc.ma_pm <= 8 ? ANTERP_NK : 16, P::HN, P::HN, !f64, Lp.nbox,
+  const MarchTile m = march_tile(ANTERP_THREADS<T>, Lc.ma_pm <= 8 ? ANTERP_NK : 16, P::HN, P::HN, !f64, Lp.nbox,
                                  Lc.nph, NT, Lc.ma_start, Lc.ma_pm, 1, sp);
   const int TI = march_rows(m, Lc.nth, f64 ? 1 : 65536 / (168 * m.T), Lc.nth);
   const size_t sm = (size_t)4 * 16 * m.cc * (m.nbx * P::HN + sp);
