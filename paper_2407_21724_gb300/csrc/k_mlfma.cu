@@ -709,18 +709,28 @@ __global__ void k_blocksparse(int nrow, int n2, int R, int rc, int nrc, const in
 }
 
 // ------------------------------------------------------------------ host drivers
+// Destroys the captured products for which stale(entry) holds: a graph replays on the
+// addresses of its capture, so it goes before the buffers it was built on do.
+template <typename F> static void drop_graphs(Ctx* c, F stale) {
+  for (size_t i = 0; i < c->graphs.size();) {
+    if (stale(c->graphs[i])) {
+      cudaGraphExecDestroy(c->graphs[i].exec);
+      c->graphs.erase(c->graphs.begin() + i);
+    } else {
+      ++i;
+    }
+  }
+}
+// products that run column by column, on d_split and the lanes' buffers
+static void drop_split_graphs(Ctx* c) {
+  drop_graphs(c, [](const Ctx::GraphEntry& g) { return g.prec == SMR_PREC_FP32 && g.R > 1; });
+}
+
 int ensure_spectra(Ctx* c, int R, int prec) {
   int p = (prec == SMR_PREC_FP64) ? 0 : 1;
   if (c->buf_R[p] != R) {
     // (re)allocate this precision's spectra; graphs built on them are dropped
-    for (size_t i = 0; i < c->graphs.size();) {
-      if (c->graphs[i].prec == prec) {
-        cudaGraphExecDestroy(c->graphs[i].exec);
-        c->graphs.erase(c->graphs.begin() + i);
-      } else {
-        ++i;
-      }
-    }
+    drop_graphs(c, [&](const Ctx::GraphEntry& g) { return g.prec == prec; });
     size_t es = (p == 0) ? sizeof(double2) : sizeof(float2);
     c->buf_R[p] = 0;
     for (int s = 0; s < c->nlev; ++s) {
@@ -1175,6 +1185,7 @@ bool split_columns(const Ctx* c, int R, int prec) { return R > 1 && prec == SMR_
 int ensure_split(Ctx* c, int R) {
   size_t need = (size_t)2 * R * 2 * c->npsi * c->p;
   if (c->split_elems >= need) return SMR_OK;
+  drop_split_graphs(c);
   if (c->d_split) cudaFree(c->d_split);
   c->d_split = nullptr;
   c->split_elems = 0;
@@ -1188,6 +1199,7 @@ int ensure_split(Ctx* c, int R) {
 }
 
 void free_lanes(Ctx* c) {
+  drop_split_graphs(c);
   for (size_t j = 1; j < c->lanes.size(); ++j) {
     Ctx::Lane& a = c->lanes[j];
     for (void* q : a.out) if (q) cudaFree(q);
