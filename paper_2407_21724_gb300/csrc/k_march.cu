@@ -35,6 +35,7 @@
 // the packed multiply-add takes for two fields they took 649 us.
 #include <algorithm>
 
+#include "march_tile.h"
 #include "smr_internal.h"
 
 namespace smr {
@@ -216,16 +217,6 @@ template <> struct Mp<double> {
   }
 };
 
-// Tile of a launch: a CTA takes nbx parent boxes, one chunk of ncol columns x
-// HN parts and one range of theta rows with T threads; the staged input
-// columns number cc.  mcc, mper: multiply-high reciprocals of cc and ncol
-// (exact for the small counts divided here).
-struct MarchTile {
-  int nbx, ncol, cc, T;
-  int nbg, nck, nhk;                           // box groups, column chunks, part chunks
-  unsigned mcc, mper;
-};
-
 __device__ __forceinline__ unsigned div_by(unsigned x, unsigned magic) { return magic ? __umulhi(x, magic) : x; }
 
 // A thread's copies of every input row: NK 16-byte chunks at ring offsets
@@ -397,17 +388,18 @@ __global__ void __launch_bounds__(INTERP_THREADS<T>, INTERP_CTAS<T>) k_interp_ma
 // ent_ptr[b] .. ent_ptr[b + 1], the parent's quadrature weight and the
 // child's inverse one folded in).  A stencil that reaches past a pole is a
 // second, reflected entry, half a turn around phi.  Per entry the
-// phi-transposed taps (PM consecutive parent columns from pst[j], weights
-// ptw) give the thread's child column the Re- and Im-weighted sums of both
-// conjugate pairs; the window scatters them to four child rows, and a row
-// that no later entry reaches is added to the four children's incoming
-// spectra. 
+// phi-transposed taps (consecutive parent columns from pst[j] + q0, weights
+// ptw [nph][pm]; PM of them, or `taps` if PM is 0) give the thread's child
+// column the Re- and Im-weighted sums of both conjugate pairs; the window
+// scatters them to four child rows, and a row that no later entry reaches is
+// added to the four children's incoming spectra.
 template <typename T, int PM, int NK = ANTERP_NK>
 __global__ void __launch_bounds__(ANTERP_THREADS<T>, ANTERP_CTAS<T>) k_anterp_march(
     int nbox, int nthC, int nphC, int nthP, int nphP, int NT, int TI, MarchTile m, const int4* __restrict__ ch4,
     const int* __restrict__ ent_ptr, const int* __restrict__ ent, const T* __restrict__ entw,
-    const int* __restrict__ pst, const T* __restrict__ ptw, int pm, const typename Mp<T>::S* __restrict__ shift,
-    const typename Mp<T>::H* __restrict__ inP, typename Mp<T>::H* __restrict__ inC) {
+    const int* __restrict__ pst, const T* __restrict__ ptw, int pm, int taps, int q0,
+    const typename Mp<T>::S* __restrict__ shift, const typename Mp<T>::H* __restrict__ inP,
+    typename Mp<T>::H* __restrict__ inC) {
   typedef Mp<T> P;
   typedef typename P::H H;
   typedef typename P::S S;
@@ -420,7 +412,7 @@ __global__ void __launch_bounds__(ANTERP_THREADS<T>, ANTERP_CTAS<T>) k_anterp_ma
   const int bg = bx / (m.nck * m.nhk);
   bx -= bg * m.nck * m.nhk;
   const int ck = bx / m.nhk, h0 = (bx - ck * m.nhk) * HN, p0 = ck * m.ncol, B0 = bg * m.nbx;
-  const int jp0 = pst[p0];                      // first staged parent column (before wrapping)
+  const int jp0 = pst[p0] + q0;                 // first staged parent column (before wrapping)
   constexpr int SP = sizeof(S) / 16;            // 16-byte pieces of a direction's shifts
   const int h = tid & (HN - 1);
   // chunk e of a row = (box, column, part), then the row's shifts
@@ -484,7 +476,7 @@ __global__ void __launch_bounds__(ANTERP_THREADS<T>, ANTERP_CTAS<T>) k_anterp_ma
   const unsigned kid[4] = {(unsigned)c4.x * Kc + j, (unsigned)c4.y * Kc + j, (unsigned)c4.z * Kc + j,
                            (unsigned)c4.w * Kc + j};
   const bool has[4] = {c4.x >= 0, c4.y >= 0, c4.z >= 0, c4.w >= 0};
-  const int tcol = pst[j] - jp0;
+  const int tcol = pst[j] + q0 - jp0;
   const H* tap = reinterpret_cast<const H*>(smem) + ((act ? lb : 0) * m.cc + tcol) * HN + h;
   const int stap = (Ev - ((act ? lb : 0) * m.cc + tcol) * HN - h) * 16 + tcol * (int)sizeof(S);
   T w[PM > 0 ? PM : 1];
@@ -514,7 +506,7 @@ __global__ void __launch_bounds__(ANTERP_THREADS<T>, ANTERP_CTAS<T>) k_anterp_ma
         G g;
         P::gzero(g);
 #pragma unroll
-        for (int q = 0; q < (PM > 0 ? PM : pm); ++q)
+        for (int q = 0; q < (PM > 0 ? PM : taps); ++q)
           P::tap(g, PM > 0 ? w[PM > 0 ? q : 0] : ptw[(size_t)j * pm + q], r[q * HN], rs + q);
 #pragma unroll
         for (int a = 0; a < 4; ++a) P::scatter(acc[(ph + a) & 3], tw[a], g);
@@ -529,61 +521,6 @@ __global__ void __launch_bounds__(ANTERP_THREADS<T>, ANTERP_CTAS<T>) k_anterp_ma
       P::gzero(acc[ph]);
     }
   }
-}
-
-unsigned magic_of(unsigned d) { return d > 1 ? (unsigned)(((1ull << 32) + d - 1) / d) : 0u; }
-
-// Columns and boxes of a CTA.  lanes: threads per column; start[j]: first
-// staged input column of output column j; width: input columns one output
-// column reads; per input column, `boxcopies` 16-byte copies per box and part
-// and `extra` more.  Whole rows where a row is short (of several boxes if
-// `pack`), chunks of columns where it is long; at most `most` threads and
-// nk copies per thread (threads without a column only copy).
-MarchTile march_tile(int most, int nk, int lanes, int hn, bool pack, int nbox, int nph, int NT, const std::vector<int>& start,
-                     int width, int boxcopies, int extra) {
-  MarchTile m;
-  m.nhk = NT / hn;
-  const int cols = most / lanes;
-  m.nck = (nph + cols - 1) / cols;
-  for (;; ++m.nck) {
-    m.ncol = (nph + m.nck - 1) / m.nck;
-    m.nck = (nph + m.ncol - 1) / m.ncol;
-    m.cc = 0;
-    for (int p = 0; p < nph; p += m.ncol)
-      m.cc = std::max(m.cc, start[std::min(nph, p + m.ncol) - 1] + width - start[p]);
-    m.nbx = !pack || m.nck > 1 ? 1 : std::max(1, std::min(nbox, most / (m.ncol * lanes)));
-    auto threads = [&]() {
-      const int E = m.cc * (m.nbx * boxcopies * hn + extra);
-      return std::max(m.nbx * m.ncol * lanes, (E + nk - 1) / nk);
-    };
-    while (m.nbx > 1 && threads() > most) --m.nbx;
-    m.T = (threads() + 31) / 32 * 32;
-    if (m.T <= most || m.ncol == 1) break;
-  }
-  m.nbg = (nbox + m.nbx - 1) / m.nbx;
-  m.mcc = magic_of(m.cc);
-  m.mper = magic_of(m.ncol);
-  return m;
-}
-
-// Theta rows of a CTA: the split of `rows` that finishes first when `per_sm`
-// CTAs of an SM run at full speed at a time.  A CTA costs its rows plus about
-// seven: the three stencil rows a range shares with its neighbour, and the
-// ring's start.
-int march_rows(const MarchTile& m, int rows, int per_sm, int most) {
-  const long long ctas = (long long)m.nbg * m.nck * m.nhk, slots = 152LL * std::max(1, per_sm);
-  int best = std::min(rows, most);
-  long long cost = -1;
-  for (int parts = 1; parts <= std::max(1, rows / 2); ++parts) {
-    const int t = (rows + parts - 1) / parts;
-    if (t > most) continue;
-    const long long k = (ctas * ((rows + t - 1) / t) + slots - 1) / slots * (t + 7);
-    if (cost < 0 || k < cost) {
-      cost = k;
-      best = t;
-    }
-  }
-  return best;
 }
 
 template <typename T>
@@ -614,19 +551,25 @@ int anterp_impl(Ctx* c, int s, int R, cudaStream_t st) {
   const bool f64 = sizeof(T) == 8;
   const Level &Lc = c->lev[s], &Lp = c->lev[s + 1];
   const int NT = P::HN * R, sp = (int)sizeof(typename P::S) / 16;
-  const MarchTile m = march_tile(ANTERP_THREADS<T>, Lc.ma_pm <= 8 ? ANTERP_NK : 16, P::HN, P::HN, !f64, Lp.nbox,
-                                 Lc.nph, NT, Lc.ma_start, Lc.ma_pm, 1, sp);
+  int taps;
+  const MarchTile m = anterp_tile(ANTERP_THREADS<T>, Lc.ma_pm <= 8 ? ANTERP_NK : 16, P::HN, P::HN, !f64, Lp.nbox,
+                                  Lc.nph, NT, Lc.ma_start, Lc.ma_pm, sp, &taps);
   const int TI = march_rows(m, Lc.nth, f64 ? 1 : 65536 / (168 * m.T), Lc.nth);
   const size_t sm = (size_t)4 * 16 * m.cc * (m.nbx * P::HN + sp);
   auto k = Lc.ma_pm == 7 ? k_anterp_march<T, 7> : Lc.ma_pm == 8 ? k_anterp_march<T, 8> : k_anterp_march<T, 0, 16>;
   cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
   dim3 g((unsigned)((long long)m.nbg * m.nck * m.nhk), (unsigned)((Lc.nth + TI - 1) / TI));
-  k<<<g, m.T, sm, st>>>(Lp.nbox, Lc.nth, Lc.nph, Lp.nth, Lp.nph, NT, TI, m, (const int4*)Lp.d_ch4, Lc.d_ma_ptr,
-                        Lc.d_ma_ent, (const T*)(f64 ? (void*)Lc.d_ma_w64 : (void*)Lc.d_ma_w32), Lc.d_ma_pst,
-                        (const T*)(f64 ? (void*)Lc.d_ma_pw64 : (void*)Lc.d_ma_pw32), Lc.ma_pm,
-                        (const typename P::S*)(f64 ? (void*)Lc.d_shiftp64 : (void*)Lc.d_shiftp32),
-                        (const typename P::H*)Lp.d_in, (typename P::H*)Lc.d_in);
-  SMR_LAUNCH(c);
+  // one launch but for stencils too wide for a CTA (above 768 parent columns in
+  // FP64, 1,024 in FP32), whose taps are divided: every launch adds its part
+  for (int q0 = 0; q0 < Lc.ma_pm; q0 += taps) {
+    k<<<g, m.T, sm, st>>>(Lp.nbox, Lc.nth, Lc.nph, Lp.nth, Lp.nph, NT, TI, m, (const int4*)Lp.d_ch4, Lc.d_ma_ptr,
+                          Lc.d_ma_ent, (const T*)(f64 ? (void*)Lc.d_ma_w64 : (void*)Lc.d_ma_w32), Lc.d_ma_pst,
+                          (const T*)(f64 ? (void*)Lc.d_ma_pw64 : (void*)Lc.d_ma_pw32) + q0, Lc.ma_pm,
+                          std::min(taps, Lc.ma_pm - q0), q0,
+                          (const typename P::S*)(f64 ? (void*)Lc.d_shiftp64 : (void*)Lc.d_shiftp32),
+                          (const typename P::H*)Lp.d_in, (typename P::H*)Lc.d_in);
+    SMR_LAUNCH(c);
+  }
   return SMR_OK;
 }
 
