@@ -1409,13 +1409,15 @@ void free_graphs(Ctx* c) {
 }
 
 int run_matvec_graph(Ctx* c, int R, int prec, const double2* x, double2* y, cudaStream_t st) {
+  const bool split = split_columns(c, R, prec);
   for (auto& g : c->graphs)
     if (g.x == x && g.y == y && g.R == R && g.prec == prec) {
       SMR_CUDA(c, cudaGraphLaunch(g.exec, st));
-      return SMR_OK;
+      // the last product's spectra are the replay's (its buffers are still the
+      // context's: a reallocation would have dropped the graph)
+      return ensure_spectra(c, split ? 1 : R, prec);
     }
   // allocations happen outside the capture
-  const bool split = split_columns(c, R, prec);
   int rc = ensure_spectra(c, split ? 1 : R, prec);
   if (!rc && split) rc = ensure_split(c, R);
   if (!rc && split) rc = ensure_lanes(c, lanes_for(c, R));

@@ -1,0 +1,38 @@
+"""smr_copy_level returns the spectra of the last product, whatever ran it."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+from paper_2407_21724_gb300 import smr, workloads
+
+from .test_gpu_parity import crandn, rel
+
+
+@pytest.fixture(scope="module")
+def scene():
+    ctx = smr.scene_from_workload(workloads.make("random", n=7, modes=6))
+    yield ctx, smr.smr_info(ctx)["n_unknowns"]
+    smr.smr_destroy(ctx)
+
+
+def test_replayed_product_is_the_last_one(scene):
+    """FP32 captured, FP64, FP32 replayed: the fields read are the FP32 product's,
+    the very bits read after its capture (the kernels sum in a fixed order)."""
+    ctx, n = scene
+    x, u = (torch.from_numpy(crandn(n, s)).cuda() for s in (1, 2))
+    y, v = torch.empty_like(x), torch.empty_like(x)
+    smr.smr_matvec_graph(ctx, x, y, smr.SMR_PREC_FP32)
+    smr.smr_sync(ctx)
+    want = [smr.smr_copy_level(ctx, 0, k) for k in (0, 1)]
+    smr.smr_matvec(ctx, u, v, smr.SMR_PREC_FP64)
+    other = smr.smr_copy_level(ctx, 0, 0)
+    smr.smr_matvec_graph(ctx, x, y, smr.SMR_PREC_FP32)
+    smr.smr_sync(ctx)
+    got = [smr.smr_copy_level(ctx, 0, k) for k in (0, 1)]
+    assert rel(got[0], other) > 0.1
+    assert all(np.array_equal(a, b) for a, b in zip(got, want))
