@@ -548,7 +548,14 @@ int smr_measure_peak(int kind, double* tflops);
  *    x_nu for y_mu (mu = nu: self block), same layout; SMR_E_INVALID_ARG if
  *    mu and nu are not a near pair;
  *  smr_copy_level: level-s outgoing (kind 0) or incoming (kind 1) spectra of
- *    the last product, [n_box][K_s][4][R] complex, in FP64. */
+ *    the last product, [n_box][K_s][4][R] complex, in FP64: the theta and phi
+ *    fields B0, B1 of the electric current and B2, B3 of the magnetic one.  The
+ *    product keeps v +- j u, v = B0 + B3 / zeta and u = -B1 + B2 / zeta, and the
+ *    fields returned combine to those as it left them; the share of each current
+ *    comes from two more far passes on the last product's coefficients.  These
+ *    take device scratch of the size of all levels' spectra (SMR_E_OOM if there
+ *    is none) and leave the product's spectra alone.  R as in the last product;
+ *    1 after an FP32 product with several columns (lane 0's last one). */
 int smr_copy_pattern(smr_ctx* ctx, int shape, double* out);
 int smr_copy_translation(smr_ctx* ctx, int level, int dx, int dy, double* out);
 int smr_copy_near_block(smr_ctx* ctx, int shape_m, int shape_n, int dx, int dy, double* out);

@@ -1482,47 +1482,82 @@ __global__ void k_one_current(long long n, int run, int cur, const double2* __re
 
 // A level's spectra of the last product in the four fields (theta and phi of
 // the electric and of the magnetic current's radiation), which the two circular
-// fields do not tell apart: the far pass once more for each current alone.
+// fields do not tell apart: the far pass once more for each current alone, in
+// scratch spectra, so that the product's stay as they are.  What the two passes
+// differ by from the stored fields is divided between the currents: the fields
+// returned combine to the spectra that the product left, whatever ran it.
 int copy_fields(Ctx* c, int level, int kind, double* out) {
-  const int prec = c->spec_prec, R = c->spec_R;
+  const int prec = c->spec_prec, R = c->spec_R, p = prec == SMR_PREC_FP64 ? 0 : 1;
   const Level& L = c->lev[level];
   const long long n = (long long)c->p * 2 * c->npsi * R;
   const size_t elems = (size_t)L.nbox * L.K * NF * R;
-  double2* buf = nullptr;
+  std::vector<double2> w[3];                     // electric current, magnetic current, as stored
+  auto read = [&](std::vector<double2>& v) -> int {
+    const void* src = kind == 0 ? L.d_out : L.d_in;
+    v.resize(elems);
+    if (p == 0) {
+      SMR_CUDA(c, cudaMemcpy(v.data(), src, elems * sizeof(double2), cudaMemcpyDeviceToHost));
+      return SMR_OK;
+    }
+    std::vector<float2> t(elems);
+    SMR_CUDA(c, cudaMemcpy(t.data(), src, elems * sizeof(float2), cudaMemcpyDeviceToHost));
+    for (size_t i = 0; i < elems; ++i) v[i] = make_double2(t[i].x, t[i].y);
+    return SMR_OK;
+  };
   SMR_CUDA(c, cudaDeviceSynchronize());
-  if (cudaMalloc((void**)&buf, 2 * n * sizeof(double2)) != cudaSuccess) {
-    cudaGetLastError();
-    c->err = "out of device memory for a level's fields";
-    return SMR_E_OOM;
+  int rc = read(w[2]);
+  if (!rc) rc = ensure_side(c, 1);
+  if (rc) return rc;
+  // scratch: the outgoing and incoming spectra of every level, x and y
+  std::vector<void*> own, scratch;
+  for (auto& l : c->lev) {
+    own.push_back(l.d_out);
+    own.push_back(l.d_in);
   }
-  int rc = ensure_side(c, 1);
-  std::vector<double2> w[2];
+  for (size_t i = 0; i <= own.size() && !rc; ++i) {
+    void* q = nullptr;
+    if (cudaMalloc(&q, i < own.size() ? c->lev[i / 2].buf_bytes[p] : 2 * n * sizeof(double2)) != cudaSuccess) {
+      cudaGetLastError();
+      c->err = "out of device memory for a level's fields";
+      rc = SMR_E_OOM;
+    }
+    scratch.push_back(q);
+  }
+  auto use = [&](const std::vector<void*>& b) {
+    for (size_t s = 0; s < c->lev.size(); ++s) {
+      c->lev[s].d_out = b[2 * s];
+      c->lev[s].d_in = b[2 * s + 1];
+    }
+  };
   std::vector<ProfRec>* prof = c->prof;
+  if (!rc) use(scratch);
   c->prof = nullptr;
   c->cur_side = 0;
   c->keep_x = true;
+  double2* buf = (double2*)scratch.back();
   for (int cur = 0; cur < 2 && !rc; ++cur) {
-    w[cur].resize(elems);
-    k_one_current<<<(unsigned)((n + 255) / 256), 256>>>(n, c->npsi * R, cur, c->d_xs[prec == SMR_PREC_FP64 ? 0 : 1], buf);
-    rc = run_far(c, R, prec, buf, buf + n, false, nullptr);
-    cudaError_t e = cudaDeviceSynchronize();
-    const void* src = kind == 0 ? L.d_out : L.d_in;
-    if (e == cudaSuccess && prec == SMR_PREC_FP64) {
-      e = cudaMemcpy(w[cur].data(), src, elems * sizeof(double2), cudaMemcpyDeviceToHost);
-    } else if (e == cudaSuccess) {
-      std::vector<float2> t(elems);
-      e = cudaMemcpy(t.data(), src, elems * sizeof(float2), cudaMemcpyDeviceToHost);
-      for (size_t i = 0; i < elems; ++i) w[cur][i] = make_double2(t[i].x, t[i].y);
-    }
+    k_one_current<<<(unsigned)((n + 255) / 256), 256>>>(n, c->npsi * R, cur, c->d_xs[p], buf);
+    rc = p == 0 ? far_impl<double>(c, R, buf, buf + n, false, nullptr)
+                : far_impl<float>(c, R, buf, buf + n, false, nullptr);
+    const cudaError_t e = cudaDeviceSynchronize();
     if (!rc && e != cudaSuccess) {
       c->err = std::string("level fields: ") + cudaGetErrorString(e);
       rc = SMR_E_CUDA;
     }
+    if (!rc) rc = read(w[cur]);
   }
+  use(own);
   c->keep_x = false;
   c->prof = prof;
-  cudaFree(buf);
+  for (void* q : scratch) cudaFree(q);
   if (rc) return rc;
+  for (size_t i = 0; i < elems; ++i) {
+    const double2 d = make_double2(0.5 * (w[2][i].x - w[0][i].x - w[1][i].x), 0.5 * (w[2][i].y - w[0][i].y - w[1][i].y));
+    for (int cur = 0; cur < 2; ++cur) {
+      w[cur][i].x += d.x;
+      w[cur][i].y += d.y;
+    }
+  }
   // electric current: W_+- = B0 -+ j B1; magnetic: W_+- = +-(j / z) (B2 -+ j B3)
   for (size_t d = 0; d < (size_t)L.nbox * L.K; ++d)
     for (int r = 0; r < R; ++r) {

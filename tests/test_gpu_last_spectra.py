@@ -36,3 +36,37 @@ def test_replayed_product_is_the_last_one(scene):
     got = [smr.smr_copy_level(ctx, 0, k) for k in (0, 1)]
     assert rel(got[0], other) > 0.1
     assert all(np.array_equal(a, b) for a, b in zip(got, want))
+
+
+@pytest.mark.parametrize("prec", [smr.SMR_PREC_FP64, smr.SMR_PREC_FP32])
+def test_fields_combine_to_the_stored_spectra(scene, prec):
+    """The fields read give the two combinations that the product stored, also when
+    the launches it would now run have changed (tensor cores off: other FP32
+    sums): equal to FP64 rounding of the few sums between, 1e-14, where another
+    FP32 product's are 1e-8 to 1e-6 off."""
+    ctx, n = scene
+    nlev = smr.smr_info(ctx)["n_levels"]
+    x = torch.from_numpy(crandn(n, 5)).cuda()
+    y = torch.empty_like(x)
+
+    def stored():
+        out = []
+        for s in range(nlev):
+            for k in (0, 1):
+                B = smr.smr_copy_level(ctx, s, k)[..., 0]
+                out.append(np.stack([B[:, :, 0] + B[:, :, 3], B[:, :, 2] - B[:, :, 1]]))
+        return out
+
+    try:
+        smr.smr_matvec_graph(ctx, x, y, prec)
+        smr.smr_sync(ctx)
+        want = stored()
+        smr.smr_set_tensor_cores(ctx, 0)
+        got = stored()
+        assert all(rel(a, b) < 1e-14 if np.any(b) else not np.any(a) for a, b in zip(got, want))
+        if prec == smr.SMR_PREC_FP32:
+            smr.smr_matvec(ctx, x, y, prec)
+            smr.smr_sync(ctx)
+            assert rel(stored()[0], want[0]) > 1e-9       # the change of launches does show
+    finally:
+        smr.smr_set_tensor_cores(ctx, 1)
