@@ -460,11 +460,12 @@ int smr_near_field(smr_ctx* ctx, int R, const void* x, int n_pt, const double* p
                    void* EH, void* stream);
 
 /* One product with a per-launch breakdown.  For each kernel launch of
- * smr_matvec, in launch order: its name, level (-1 if none), ALGORITHMIC
+ * smr_matvec, and for its one device copy ("keep": the coefficients stay with
+ * the spectra, for smr_copy_level), in launch order: its name, level (-1 if none), ALGORITHMIC
  * bytes (every operand read once, every result written once; tables
  * included) and flops of that launch, and its device time in ms from CUDA
  * events recorded on `stream` around the launch.  Fills at most n_max
- * entries of `out`, sets *n_out to the number of launches, and synchronises
+ * entries of `out`, sets *n_out to their number, and synchronises
  * `stream`.  Same arguments otherwise as smr_matvec. */
 typedef struct {
   char name[24];

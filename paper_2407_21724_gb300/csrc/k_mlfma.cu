@@ -869,7 +869,9 @@ static int far_impl(Ctx* c, int R, const double2* x, double2* y, bool accumulate
       SMR_CUDA(c, cudaEventRecord(sd->efork, st));
       SMR_CUDA(c, cudaStreamWaitEvent(sd->tr, sd->efork, 0));
     }
+    pbeg(c, st, "keep", -1, 2.0 * bytes, 0.0);
     SMR_CUDA(c, cudaMemcpyAsync(c->d_xs[f64 ? 0 : 1], x, bytes, cudaMemcpyDeviceToDevice, sd ? sd->tr : st));
+    pend(c, st);
   }
   // translation at every level (in the upward loop when it overlaps)
   auto translate = [&](int s, cudaStream_t ts) -> int {

@@ -70,3 +70,12 @@ def test_fields_combine_to_the_stored_spectra(scene, prec):
             assert rel(stored()[0], want[0]) > 1e-9       # the change of launches does show
     finally:
         smr.smr_set_tensor_cores(ctx, 1)
+
+
+@pytest.mark.parametrize("prec,R,columns", [(smr.SMR_PREC_FP64, 1, 1), (smr.SMR_PREC_FP64, 3, 3),
+                                            (smr.SMR_PREC_FP32, 1, 1), (smr.SMR_PREC_FP32, 3, 1)])
+def test_profile_lists_the_copy_of_the_coefficients(scene, prec, R, columns):
+    ctx, n = scene
+    x = torch.from_numpy(np.stack([crandn(n, r) for r in range(R)], axis=1)).cuda()
+    recs = [r for r in smr.smr_profile_matvec(ctx, x, torch.empty_like(x), prec, R=R) if r["name"] == "keep"]
+    assert [(r["level"], r["bytes"]) for r in recs] == [(-1, 2.0 * 16 * n * columns)] and recs[0]["ms"] > 0
