@@ -570,10 +570,11 @@ int smr_copy_level(smr_ctx* ctx, int level, int kind, double* out, size_t n_doub
  *  SMR_STEP_INTERPOLATE (into the parent of `level`): 0 built-in rule (FP32:
  *    the marching kernel; FP64: the gather kernel), 1 / 2 the gather kernel
  *    with the full / half theta-row tile (FP64), 3 the marching kernel;
- *  SMR_STEP_ANTERPOLATE (into `level`): 0 built-in rule (FP32: the marching
- *    kernel; FP64: that or the gather kernel by the level's size), 1 the gather
- *    kernel with half its column chunk, 2 with 256-thread CTAs (FP64), 4 and 5
- *    the marching kernel.
+ *  SMR_STEP_ANTERPOLATE (into `level`): 0 built-in rule (the marching or the
+ *    gather kernel by the level's size; in FP32 and for several columns the
+ *    gather kernel only where a child column has more than 8 taps), 1 the gather
+ *    kernel with half its column chunk, 2 with 256-thread CTAs, 4 and 5 the
+ *    marching kernel.
  * A variant that does not apply to a level falls back to the built-in rule.
  * Drops captured products.  No counterpart in the paper. */
 enum { SMR_STEP_TRANSLATE = 0, SMR_STEP_INTERPOLATE = 1, SMR_STEP_ANTERPOLATE = 2 };

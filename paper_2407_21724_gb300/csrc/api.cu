@@ -38,6 +38,7 @@ void free_scene(Ctx* c) {
     dfree(L.d_shiftp32); dfree(L.d_mi_vlast); dfree(L.d_ma_ptr); dfree(L.d_ma_ent);
     dfree(L.d_ma_w64); dfree(L.d_ma_w32); dfree(L.d_ma_pst); dfree(L.d_ma_pw64); dfree(L.d_ma_pw32);
     dfree(L.d_ant_lo); dfree(L.d_ant_pjp); dfree(L.d_ant_pw64); dfree(L.d_ant_ttp); dfree(L.d_ant_tw64);
+    dfree(L.d_ant_pw32); dfree(L.d_ant_tw32); dfree(L.d_wthp32); dfree(L.d_shift32);
     dfree(L.d_wthp64); dfree(L.d_boxmap); dfree(L.d_offid); dfree(L.d_tiles); dfree(L.d_tile_tab);
     for (int q = 0; q < 2; ++q) {
       if (L.buf_out[q]) cudaFree(L.buf_out[q]);
@@ -339,6 +340,11 @@ int build_interp(Ctx* c, Level& C, const Level& P) {
     if ((rc = upload(c, &C.d_ant_pjp, ppj)) || (rc = upload(c, &C.d_ant_pw64, ppw)) ||
         (rc = upload(c, &C.d_ant_ttp, tpk)) || (rc = upload(c, &C.d_ant_tw64, tpw)))
       return rc;
+    if (C.ma_pm > 8) {
+      const std::vector<float> pp(ppw.begin(), ppw.end()), tt(tpw.begin(), tpw.end()), wp(wpth.begin(), wpth.end());
+      if ((rc = upload(c, &C.d_ant_pw32, pp)) || (rc = upload(c, &C.d_ant_tw32, tt)) || (rc = upload(c, &C.d_wthp32, wp)))
+        return rc;
+    }
   }
   // shift tables exp(j k khat_p . (c_child - c_parent)), child offset (+-1/2) x child box
   std::vector<double2> sh(4 * (size_t)P.K);
@@ -356,6 +362,12 @@ int build_interp(Ctx* c, Level& C, const Level& P) {
       shp[(size_t)2 * k + q] = sh[(size_t)q * P.K + k];
       shp32[(size_t)2 * k + q] = make_float2((float)shp[(size_t)2 * k + q].x, (float)shp[(size_t)2 * k + q].y);
     }
+  C.ant_wide = C.ma_pm > 8;
+  if (C.ant_wide) {
+    std::vector<float2> sh32(sh.size());
+    for (size_t i = 0; i < sh.size(); ++i) sh32[i] = make_float2((float)sh[i].x, (float)sh[i].y);
+    if ((rc = upload(c, &C.d_shift32, sh32))) return rc;
+  }
   if ((rc = upload(c, &C.d_shiftp64, shp)) || (rc = upload(c, &C.d_shiftp32, shp32))) return rc;
   if ((rc = upload(c, &C.d_shift64, sh))) return rc;
   return SMR_OK;

@@ -58,10 +58,9 @@ template <typename V> __device__ __forceinline__ V cmul(V a, V b) {
 }
 
 // ------------------------------------------------------------------ 16-byte direction parts
-// The FP64 single right-hand side kernels give each thread one 16-byte part of a
-// direction (one field), so that
-// a warp instruction reads or writes one contiguous 512-byte run and shared
-// memory is accessed without bank conflicts.  NT threads share a direction.
+// The gather kernels work on 16-byte parts of a direction (one field in FP64, two in
+// FP32), so that a warp instruction reads or writes contiguous runs and shared memory
+// is accessed without bank conflicts.  NT parts make the fields of one column.
 template <typename T> struct Part;
 template <> struct Part<double> {
   typedef double2 H;
@@ -76,6 +75,25 @@ template <> struct Part<double> {
   static __device__ __forceinline__ void w4(const double* p, double* w) {
     double2 a = reinterpret_cast<const double2*>(p)[0], b = reinterpret_cast<const double2*>(p)[1];
     w[0] = a.x; w[1] = a.y; w[2] = b.x; w[3] = b.y;
+  }
+};
+template <> struct Part<float> {
+  typedef float4 H;
+  static constexpr int NT = NF / 2;
+  static __device__ __forceinline__ H zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
+  static __device__ __forceinline__ void rfma(H& a, float w, H v) {
+    a.x = fmaf(w, v.x, a.x); a.y = fmaf(w, v.y, a.y); a.z = fmaf(w, v.z, a.z); a.w = fmaf(w, v.w, a.w);
+  }
+  static __device__ __forceinline__ void cfma(H& a, float2 s, H v) {
+    a.x = fmaf(s.x, v.x, a.x); a.x = fmaf(-s.y, v.y, a.x);
+    a.y = fmaf(s.x, v.y, a.y); a.y = fmaf(s.y, v.x, a.y);
+    a.z = fmaf(s.x, v.z, a.z); a.z = fmaf(-s.y, v.w, a.z);
+    a.w = fmaf(s.x, v.w, a.w); a.w = fmaf(s.y, v.z, a.w);
+  }
+  static __device__ __forceinline__ void add(H& a, H v) { a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w; }
+  static __device__ __forceinline__ void w4(const float* p, float* w) {
+    const float4 a = *reinterpret_cast<const float4*>(p);
+    w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w;
   }
 };
 template <typename T>
@@ -408,35 +426,37 @@ __global__ void __launch_bounds__(128) k_translate_il(int K, int NR, int nch, co
   in[(size_t)b * n + e] = a;
 }
 
-// ------------------------------------------------------------------ FP64 anterpolation, one right-hand side
-// For the levels where it is ahead of the marching kernel (march_anterp).
+// ------------------------------------------------------------------ anterpolation by gathering
+// For the levels where it is ahead of the marching kernel (gather_anterp).
 // Both adjoint passes fused.  CTA = (child c, tile of
 // child theta rows [i0, i0 + TI), column chunk [j0, j0 + JC) of the first
 // half of the phi grid together with the same chunk shifted by N/2, so that
-// the pole reflection j -> j + N/2 stays inside the CTA).  The parent rows
+// the pole reflection j -> j + N/2 stays inside the CTA), one right-hand side
+// per blockIdx.y (MC).  The parent rows
 // [lo, hi) the tile draws on get the phi-transposed pass (conjugate shift and
 // parent theta weight) into shared memory; then the theta-transposed pass adds
-// into the child's incoming spectrum.  Transposed taps are padded to PM / TM
+// into the child's incoming spectrum.  A thread takes all fields of a direction.
+// Transposed taps are padded to PM / TM
 // per child column / row (zero weights), packed as (tp | refl << 16).
 // PMC > 0: tap tables padded to 8 per row (PM = TM = 8) and at most PMC
 // real taps per row, known at compile time (tap loops unrolled)
-template <int PMC>
-__global__ void __launch_bounds__(256) k_anterp1(int nthC, int nphC, int nthP, int nphP, int TI, int nit,
+template <typename T, int PMC, bool MC>
+__global__ void __launch_bounds__(256) k_anterp1(int nthC, int nphC, int nthP, int nphP, int R, int TI, int nit,
                                                  int JC, int njc, const int* __restrict__ parent,
                                                  const int* __restrict__ quad, const int* __restrict__ lo_row,
-                                                 int PM, const int* __restrict__ pjp, const double* __restrict__ pw,
-                                                 const double* __restrict__ wthp,
-                                                 const double2* __restrict__ shift,
-                                                 const double2* __restrict__ inP, int TM,
-                                                 const int* __restrict__ ttp, const double* __restrict__ tw,
-                                                 double2* __restrict__ inC) {
-  typedef double T;
-  typedef double2 V;
+                                                 int PM, const int* __restrict__ pjp, const T* __restrict__ pw,
+                                                 const T* __restrict__ wthp,
+                                                 const typename CV<T>::V* __restrict__ shift,
+                                                 const typename Part<T>::H* __restrict__ inP, int TM,
+                                                 const int* __restrict__ ttp, const T* __restrict__ tw,
+                                                 typename Part<T>::H* __restrict__ inC) {
+  typedef typename CV<T>::V V;
   typedef Part<T> P;
-  typedef P::H H;
+  typedef typename P::H H;
   constexpr int NT = P::NT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  V* Gt = reinterpret_cast<V*>(smem_raw);          // [GR][2 JC][NF]
+  H* Gt = reinterpret_cast<H*>(smem_raw);          // [GR][2 JC][NT]
+  const int nt = MC ? NT * R : NT;                 // parts of a direction
   int blk = blockIdx.x;
   int jcb = blk % njc;
   blk /= njc;
@@ -447,22 +467,26 @@ __global__ void __launch_bounds__(256) k_anterp1(int nthC, int nphC, int nthP, i
   int lo = lo_row[it], hi = lo_row[nit + it];
   int nr = hi - lo, W = 2 * nj;
   int Kp = nthP * nphP, Kc = nthC * nphC;
-  const V* srcP = inP + (size_t)parent[c] * Kp * NF;
+  const H* srcP = inP + (size_t)parent[c] * Kp * nt;
+  if (MC) {
+    srcP += blockIdx.y * NT;
+    inC += blockIdx.y * NT;
+  }
   const V* sh = shift + (size_t)quad[c] * Kp;
-  // each thread owns PPT consecutive 16-byte parts of a direction;
-  // (row, column) of its tasks stepped by the NTH tasks of one sweep of the
+  // (row, column) of a thread's tasks stepped by the tasks of one sweep of the
   // CTA without dividing per task
-  constexpr int PPT = 2, NT2 = NT / PPT;
-  const int NTH = blockDim.x / NT2, task0 = threadIdx.x / NT2, h = PPT * (threadIdx.x % NT2);
+  const int NTH = blockDim.x, task0 = threadIdx.x;
   const int r0 = task0 / W, u0 = task0 - r0 * W;
   const int dq = NTH / W, dr = NTH - dq * W;
   for (int r = r0, u = u0, task = task0; r < nr; task += NTH) {
     int j = (u < nj) ? j0 + u : j0 + half + (u - nj);
     int tp = lo + r;
     T wt = wthp[tp];
-    const V* prow = srcP + (size_t)tp * nphP * NF;
+    const H* prow = srcP + (size_t)tp * nphP * nt;
     const V* srow = sh + (size_t)tp * nphP;
-    H a = P::zero(), a1 = P::zero();
+    H a[NT];
+#pragma unroll
+    for (int h = 0; h < NT; ++h) a[h] = P::zero();
     const int pm = PMC > 0 ? 8 : PM;
 #pragma unroll
     for (int q = 0; q < (PMC > 0 ? PMC : PM); q += 4) {
@@ -476,12 +500,12 @@ __global__ void __launch_bounds__(256) k_anterp1(int nthC, int nphC, int nthP, i
         V s = srow[js[b]];
         T ww = w[b] * wt;
         const V cw = mkc(ww * s.x, -ww * s.y);
-        P::cfma(a, cw, ldp<T>(prow, js[b], h));
-        if (PPT == 2) P::cfma(a1, cw, ldp<T>(prow, js[b], h + 1));
+#pragma unroll
+        for (int h = 0; h < NT; ++h) P::cfma(a[h], cw, prow[(size_t)js[b] * nt + h]);
       }
     }
-    stp<T>(Gt, task, h, a);
-    if (PPT == 2) stp<T>(Gt, task, h + 1, a1);
+#pragma unroll
+    for (int h = 0; h < NT; ++h) Gt[task * NT + h] = a[h];
     u += dr;
     r += dq;
     if (u >= W) { u -= W; ++r; }
@@ -491,7 +515,9 @@ __global__ void __launch_bounds__(256) k_anterp1(int nthC, int nphC, int nthP, i
     int ur = u < nj ? u + nj : u - nj;             // column j + N/2 (mod N)
     int j = (u < nj) ? j0 + u : j0 + half + (u - nj);
     int i = i0 + il;
-    H a = P::zero(), a1 = P::zero();
+    H a[NT];
+#pragma unroll
+    for (int h = 0; h < NT; ++h) a[h] = P::zero();
     const int tm = PMC > 0 ? 8 : TM;
 #pragma unroll
     for (int q = 0; q < (PMC > 0 ? PMC : TM); q += 4) {
@@ -503,19 +529,17 @@ __global__ void __launch_bounds__(256) k_anterp1(int nthC, int nphC, int nthP, i
       for (int b = 0; b < 4; ++b) {
         if (PMC > 0 && q + b >= PMC) break;
         int r = (ps[b] & 0xffff) - lo;
-        const size_t g = (size_t)r * W + ((ps[b] >> 16) ? ur : u);
-        P::rfma(a, w[b], ldp<T>(Gt, g, h));
-        if (PPT == 2) P::rfma(a1, w[b], ldp<T>(Gt, g, h + 1));
+        const H* g = Gt + (size_t)(r * W + ((ps[b] >> 16) ? ur : u)) * NT;
+#pragma unroll
+        for (int h = 0; h < NT; ++h) P::rfma(a[h], w[b], g[h]);
       }
     }
-    size_t d = (size_t)c * Kc + (size_t)i * nphC + j;
-    H cur = ldp<T>(inC, d, h);
-    P::add(cur, a);
-    stp<T>(inC, d, h, cur);
-    if (PPT == 2) {
-      H cur1 = ldp<T>(inC, d, h + 1);
-      P::add(cur1, a1);
-      stp<T>(inC, d, h + 1, cur1);
+    H* d = inC + ((size_t)c * Kc + (size_t)i * nphC + j) * nt;
+#pragma unroll
+    for (int h = 0; h < NT; ++h) {
+      H cur = d[h];
+      P::add(cur, a[h]);
+      d[h] = cur;
     }
     u += dr;
     il += dq;
@@ -789,6 +813,55 @@ static bool march_anterp(const Level& Lc, const Level& Lp, int v) {
   if (v != 0) return v > 2;
   return Lc.nph > 24 && (size_t)Lp.nbox * Lp.K >= (Lc.nph <= 40 ? 2000000u : 240000u);
 }
+// FP32, or several columns: the marching kernel but for stencils wider than it is
+// compiled for (ant_wide), whose taps its threads walk one by one for every parent row
+// in turn, a chain that few boxes cannot hide.  The gather kernel's time grows with the
+// child boxes and the columns, the chain's with the taps: they cross near nbox K_p R =
+// 300,000 taps (FP32, orders 10 -> 38: 576 boxes 35 us against 78, 2,304 boxes 113
+// against 98; 16 -> 68: 144 boxes 43 against 104, 576 boxes 127 against 115; 2 -> 68:
+// 144 boxes 37 against 950; FP64, three columns, 4 -> 17: 576 boxes 125 against 227;
+// 12 -> 48: 576 boxes 798 against 650).  In FP64 rows of up to 10 columns leave the
+// marching kernel too few threads at any size (2 -> 11, 25,600 boxes, three columns:
+// 3.05 against 4.93 ms).
+constexpr size_t ANT_SMEM = 200 * 1024;
+static bool gather_anterp(const Level& Lc, const Level& Lp, bool f64, int R, int v) {
+  if (f64 && R == 1) return !march_anterp(Lc, Lp, v);
+  const bool few = (f64 && Lc.nph <= 10) || (double)Lc.nbox * Lp.K * R < 300000.0 * Lc.ma_pm;
+  return Lc.ant_wide && (v ? v <= 2 : few) &&
+         (size_t)Lc.ant_GR * 2 * NF * (f64 ? 16 : 8) <= ANT_SMEM;
+}
+
+// anterpolation of level Lp into Lc by gathering
+template <typename T> static int run_anterp_gather(Ctx* c, const Level& Lc, const Level& Lp, int R, int an, cudaStream_t st) {
+  typedef typename CV<T>::V V;
+  typedef typename Part<T>::H H;
+  const bool f64 = sizeof(T) == 8, one = f64 && R == 1;
+  // column chunk: half of the table's where rows are long (40x40 level 1: 123 ->
+  // 78 us; level 0, 11 columns: 121 -> 133) or boxes fewer than SMs (40x40 level 3:
+  // 90 -> 68 us); for wide stencils as many chunks as make two CTAs an SM
+  int JC = Lc.ant_JC;
+  if (an == 1 || (an == 0 && one && (JC > 12 || Lc.nbox < 152))) JC = std::max(1, JC / 2);
+  if (!one) JC = (int)std::max<long long>(1, std::min<long long>(JC, (long long)Lc.nph / 2 * Lc.nbox * Lc.ant_nit * R / 304));
+  const int njc = (Lc.nph / 2 + JC - 1) / JC;
+  const size_t sm = (size_t)Lc.ant_GR * 2 * JC * NF * sizeof(V);
+  const int thr = (an == 2 || (an == 0 && Lc.nph <= 24) || Lc.ant_GR * 2 * JC >= 2048) ? 256 : 128;
+  auto k = k_anterp1<T, 0, true>;
+  if constexpr (sizeof(T) == 8) {
+    if (one) {
+      k = k_anterp1<T, 0, false>;
+      if (Lc.ant_PM == 8 && Lc.ant_TM == 8) k = std::max(Lc.ant_PMx, Lc.ant_TMx) <= 7 ? k_anterp1<T, 7, false> : k_anterp1<T, 8, false>;
+    }
+  }
+  if (!one) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ANT_SMEM);
+  k<<<dim3((unsigned)(Lc.nbox * Lc.ant_nit * njc), (unsigned)R), thr, sm, st>>>(
+      Lc.nth, Lc.nph, Lp.nth, Lp.nph, R, Lc.ant_TI, Lc.ant_nit, JC, njc, Lc.d_parent, Lc.d_quad, Lc.d_ant_lo,
+      Lc.ant_PM, Lc.d_ant_pjp, (const T*)(f64 ? (void*)Lc.d_ant_pw64 : (void*)Lc.d_ant_pw32),
+      (const T*)(f64 ? (void*)Lc.d_wthp64 : (void*)Lc.d_wthp32),
+      (const V*)(f64 ? (void*)Lc.d_shift64 : (void*)Lc.d_shift32), (const H*)Lp.d_in, Lc.ant_TM, Lc.d_ant_ttp,
+      (const T*)(f64 ? (void*)Lc.d_ant_tw64 : (void*)Lc.d_ant_tw32), (H*)Lc.d_in);
+  SMR_LAUNCH(c);
+  return SMR_OK;
+}
 
 // Finest boxes made of cells.  Box b's outgoing spectrum is the sum of its
 // particles' spectra, and each particle receives its box's incoming
@@ -1017,27 +1090,11 @@ static int far_impl(Ctx* c, int R, const double2* x, double2* y, bool accumulate
          ((double)Lp.nbox * Lp.K + 2.0 * Lc.nbox * Lc.K) * NF * R_ * es + 4.0 * Lp.K * es,
          (double)Lc.nbox * Lp.nth * Lc.nph * NF * R_ * 8.0 * 2 * (double)Lp.nph / Lc.nph * 4.0 / 4.0 +
              (double)Lc.nbox * Lc.K * NF * R_ * 16.0 * (double)Lp.nth / Lc.nth);
-    if (!f64 || R > 1 || march_anterp(Lc, Lp, Lc.tune_an[0])) {
-      int rc = run_anterp(c, s, R, f64 ? SMR_PREC_FP64 : SMR_PREC_FP32, st);
-      if (rc) return rc;
-    } else {
-      const int an = Lc.tune_an[0];
-      // column chunk: half of what fits in shared memory where rows are long
-      // (40x40 level 1: 123 -> 78 us; level 0, 11 columns: 121 -> 133) or boxes fewer
-      // than SMs (40x40 level 3: 90 -> 68 us)
-      int JC = Lc.ant_JC;
-      if (an == 1 || (an == 0 && (JC > 12 || Lc.nbox < 152))) JC = std::max(1, JC / 2);
-      int njc = (Lc.nph / 2 + JC - 1) / JC;
-      size_t sm1 = (size_t)Lc.ant_GR * 2 * JC * NF * sizeof(double2);
-      int thr = (an == 2 || (an == 0 && Lc.nph <= 24) || Lc.ant_GR * 2 * JC * (Part<double>::NT / 2) >= 2048) ? 256 : 128;
-      auto ka = k_anterp1<0>;
-      if (Lc.ant_PM == 8 && Lc.ant_TM == 8) ka = std::max(Lc.ant_PMx, Lc.ant_TMx) <= 7 ? k_anterp1<7> : k_anterp1<8>;
-      ka<<<(unsigned)(Lc.nbox * Lc.ant_nit * njc), thr, sm1, st>>>(
-          Lc.nth, Lc.nph, Lp.nth, Lp.nph, Lc.ant_TI, Lc.ant_nit, JC, njc, Lc.d_parent, Lc.d_quad, Lc.d_ant_lo,
-          Lc.ant_PM, Lc.d_ant_pjp, Lc.d_ant_pw64, Lc.d_wthp64, Lc.d_shift64, (const double2*)Lp.d_in, Lc.ant_TM,
-          Lc.d_ant_ttp, Lc.d_ant_tw64, (double2*)Lc.d_in);
-      SMR_LAUNCH(c);
-    }
+    const int an = Lc.tune_an[f64 ? 0 : 1];
+    int rc;
+    if (gather_anterp(Lc, Lp, f64, R, an)) rc = run_anterp_gather<T>(c, Lc, Lp, R, an, st);
+    else rc = run_anterp(c, s, R, f64 ? SMR_PREC_FP64 : SMR_PREC_FP32, st);
+    if (rc) return rc;
     pend(c, st);
   }
   // receive

@@ -157,6 +157,11 @@ struct Level {
   double* d_ant_pw64 = nullptr;
   int* d_ant_ttp = nullptr;
   double* d_ant_tw64 = nullptr;
+  // stencils of more than 8 taps, wider than the marching kernel's compiled
+  // ones: the same tables in FP32, the parent's theta weights, the shifts
+  bool ant_wide = false;
+  float *d_ant_pw32 = nullptr, *d_ant_tw32 = nullptr, *d_wthp32 = nullptr;
+  float2* d_shift32 = nullptr;
   // spectra (allocated for the current R and precision)
   void* d_out = nullptr;                 // active spectra (the last product's precision)
   void* d_in = nullptr;
