@@ -43,22 +43,29 @@ __device__ __forceinline__ void cfma(double2& a, double2 x, double2 y) {
 
 // ------------------------------------------------------------------ far field
 // Rv[s][n][i][d] = sum_q w psi_n(q) exp(+j k u_d . r_q), the radiation vectors
-// along e1, e2 and u_d.  CTA = 16 directions (lanes) x 32 modes (4 per thread) of
-// one shape.  The phases of 64 surface points are computed once per CTA into
-// shared memory: a thread per (mode, direction) that recomputes them for each
-// mode spends 8 times more instructions on them than on the sums.  With few
-// directions the surface points are divided over blockIdx.y, one slice of Rv each
-// (a CTA's 512 points take some 0.5 ms whatever the number of CTAs).
-constexpr int RV_D = 16, RV_N = 4, RV_T = 128, RV_Q = 64;
+// along e1, e2 and u_d.  CTA = D directions x 32 modes (4 per thread) of one
+// shape; the threads of a direction and a mode group are T / (8 D) and take
+// every so manieth surface point.  The phases of 64 surface points are computed
+// once per CTA into shared memory: a thread per (mode, direction) that recomputes
+// them for each mode spends 8 times more instructions on them than on the sums.
+// With few directions the surface points are also divided over blockIdx.y, one
+// slice of Rv each (a CTA's 512 points take some 0.5 ms whatever the number of
+// CTAs).  D = 16 spends the FP64 rate on absent directions too; D = 4 is taken
+// where it spends it on at least an eighth fewer: 300 shapes of 32 modes, one
+// direction 1.41 -> 0.69 ms (20 directions 2.3 -> 1.6), a thread per mode and
+// direction 1.18.
+constexpr int RV_N = 4, RV_T = 128, RV_Q = 64, RV_M = 8 * RV_N;
 
+template <int D>
 __global__ void __launch_bounds__(RV_T) k_radvec(int npsi, int Q, int nd, int ndt, int nng,
                                                  const double* __restrict__ modes, const double* __restrict__ rq,
                                                  const double* __restrict__ dirs, double kw, size_t slice,
                                                  double2* __restrict__ Rv) {
-  __shared__ double2 ph[RV_Q][RV_D];
+  constexpr int SL = RV_T / (8 * D);               // threads that share a direction and a mode group
+  __shared__ double2 ph[RV_Q][D];
   const int dt = blockIdx.x % ndt, g = (blockIdx.x / ndt) % nng, s = blockIdx.x / (ndt * nng);
-  const int dl = threadIdx.x % RV_D, d = min(dt * RV_D + dl, nd - 1);
-  const int n0 = g * (RV_T / RV_D * RV_N) + threadIdx.x / RV_D * RV_N;
+  const int dl = threadIdx.x % D, d = min(dt * D + dl, nd - 1), sl = threadIdx.x / (8 * D);
+  const int n0 = g * RV_M + threadIdx.x / D % 8 * RV_N;
   const double u[3] = {dirs[3 * d], dirs[3 * d + 1], dirs[3 * d + 2]};
   const double* Rr = rq + (size_t)s * Q * 4;
   const double* M[RV_N];
@@ -70,7 +77,7 @@ __global__ void __launch_bounds__(RV_T) k_radvec(int npsi, int Q, int nd, int nd
   for (int q0 = (int)((long long)nch * blockIdx.y / gridDim.y) * RV_Q; q0 < qe; q0 += RV_Q) {
     const int nq = min(RV_Q, qe - q0);
     __syncthreads();
-    for (int q = threadIdx.x / RV_D; q < nq; q += RV_T / RV_D) {
+    for (int q = threadIdx.x / D; q < nq; q += RV_T / D) {
       const double* p = Rr + 4 * (q0 + q);
       double sn, cs;
       sincos(kw * (u[0] * p[0] + u[1] * p[1] + u[2] * p[2]), &sn, &cs);
@@ -78,7 +85,7 @@ __global__ void __launch_bounds__(RV_T) k_radvec(int npsi, int Q, int nd, int nd
     }
     __syncthreads();
 #pragma unroll 2
-    for (int q = 0; q < nq; ++q) {
+    for (int q = sl; q < nq; q += SL) {
       const double2 e = ph[q][dl];
 #pragma unroll
       for (int i = 0; i < RV_N; ++i) {
@@ -90,7 +97,21 @@ __global__ void __launch_bounds__(RV_T) k_radvec(int npsi, int Q, int nd, int nd
       }
     }
   }
-  if (dt * RV_D + dl >= nd) return;
+  if constexpr (SL > 1) {
+    __shared__ double2 red[SL][RV_N * 3][8 * D];
+    const int t = threadIdx.x % (8 * D);
+#pragma unroll
+    for (int i = 0; i < RV_N * 3; ++i) red[sl][i][t] = a[i / 3][i % 3];
+    __syncthreads();
+    if (sl) return;
+#pragma unroll
+    for (int i = 0; i < RV_N * 3; ++i)
+      for (int k = 1; k < SL; ++k) {
+        a[i / 3][i % 3].x += red[k][i][t].x;
+        a[i / 3][i % 3].y += red[k][i][t].y;
+      }
+  }
+  if (dt * D + dl >= nd) return;
   double t[3], e1[3], e2[3];
   dir_basis(u, t, e1, e2);
 #pragma unroll
@@ -247,7 +268,8 @@ int launch_far_field(Ctx* c, int R, const double2* x, int nd, const double* d_di
                                             std::max<long long>(1, 1216 / ((long long)tiles * R)));
   const int C = (c->p + want - 1) / want, nu = (c->p + C - 1) / C;
   double2 *Rv = nullptr, *part = nullptr;
-  const int ndt = (nd + RV_D - 1) / RV_D, nng = (c->npsi + RV_T / RV_D * RV_N - 1) / (RV_T / RV_D * RV_N);
+  const int d4 = (nd + 3) / 4 * 4, d16 = (nd + 15) / 16 * 16, D = 8 * d16 > 9 * d4 ? 4 : 16;
+  const int ndt = (nd + D - 1) / D, nng = (c->npsi + RV_M - 1) / RV_M;
   const long long ctas = (long long)c->S * nng * ndt;
   const int nqs = std::min((c->Q + RV_Q - 1) / RV_Q, ctas < 608 ? (int)(608 / ctas) : 1);
   const size_t slice = (size_t)c->S * c->npsi * nd * 3;
@@ -256,7 +278,8 @@ int launch_far_field(Ctx* c, int R, const double2* x, int nd, const double* d_di
   if (e != cudaSuccess) cudaFreeAsync(Rv, st);
   SMR_CUDA(c, e);
   const dim3 gr((unsigned)ctas, (unsigned)nqs);
-  k_radvec<<<gr, RV_T, 0, st>>>(c->npsi, c->Q, nd, ndt, nng, c->d_modes, c->d_rq, d_dirs, c->k, slice, Rv);
+  auto k = D == 4 ? k_radvec<4> : k_radvec<16>;
+  k<<<gr, RV_T, 0, st>>>(c->npsi, c->Q, nd, ndt, nng, c->d_modes, c->d_rq, d_dirs, c->k, slice, Rv);
   SMR_LAUNCH(c);
   if (nqs > 1) {
     k_rv_sum<<<(unsigned)((slice + 255) / 256), 256, 0, st>>>(slice, nqs, Rv);
