@@ -31,7 +31,7 @@ void free_scene(Ctx* c) {
   free_graphs(c);
   free_lanes(c);
   for (auto& L : c->lev) {
-    dfree(L.d_khat); dfree(L.d_w); dfree(L.d_il_ptr); dfree(L.d_il_src); dfree(L.d_il_off); dfree(L.d_il_pk);
+    dfree(L.d_khat); dfree(L.d_w); dfree(L.d_il_ptr); dfree(L.d_il_pk);
     dfree(L.d_T64); dfree(L.d_T32); dfree(L.d_parent); dfree(L.d_quad); dfree(L.d_ch_ptr);
     dfree(L.d_ch_idx); dfree(L.d_ch_quad); dfree(L.d_ch4); dfree(L.d_th_pk); dfree(L.d_th_ws64); dfree(L.d_th_ws32);
     dfree(L.d_ph_src); dfree(L.d_ph_w64); dfree(L.d_ph_w32); dfree(L.d_shift64); dfree(L.d_shiftp64);
@@ -62,7 +62,7 @@ void free_scene(Ctx* c) {
   dfree(c->d_tcn_mask); dfree(c->d_tcn_part); dfree(c->d_tc_part); dfree(c->d_Pinv64); dfree(c->d_Pinv32); dfree(c->d_pc_ptr);
   dfree(c->d_pc_col); dfree(c->d_pc_blk); dfree(c->d_tmp);
   dfree(c->d_arr);
-  dfree(c->d_tile_shape); dfree(c->d_tile_start); dfree(c->d_tile_count); dfree(c->d_perm);
+  dfree(c->d_perm);
   dfree(c->d_tc_rec); dfree(c->d_tc_agg); dfree(c->d_tc_perm); dfree(c->d_lpc); dfree(c->d_split);
   dfree(c->d_pcw);
   c->pcw_elems = 0;
@@ -285,7 +285,7 @@ int build_interp(Ctx* c, Level& C, const Level& P) {
           (rc = upload(c, &C.d_ma_ent, pk)) || (rc = upload(c, &C.d_ma_w64, w)) || (rc = upload(c, &C.d_ma_w32, w32)))
         return rc;
     }
-    // tiles of the FP64 gather anterpolation: child theta
+    // tiles of the gather anterpolation: child theta
     // rows in tiles of TI, each with the range [lo, hi) of parent rows its
     // transposed taps read; GR = the widest range
     C.ant_TI = C.nth <= 24 ? C.nth : 16;
@@ -304,7 +304,7 @@ int build_interp(Ctx* c, Level& C, const Level& P) {
       lohi[C.ant_nit + it] = hi;
       C.ant_GR = std::max(C.ant_GR, hi - lo);
     }
-    // column chunk: GR x 2 JC directions in 48 KB of shared memory
+    // column chunk: GR x 2 JC directions, 24 KB of shared memory in FP64
     C.ant_JC = std::max(1, std::min(C.nph / 2, (48 * 1024) / (C.ant_GR * 2 * 64)));
     if ((rc = upload(c, &C.d_ant_lo, lohi))) return rc;
     // padded transposed taps
@@ -624,8 +624,7 @@ int set_scene(Ctx* c, int p, const double* centres, const int* shape_ids, const 
     make_grid(L);
     int rc;
     if ((rc = upload(c, &L.d_khat, L.khat)) || (rc = upload(c, &L.d_w, L.w)) ||
-        (rc = upload(c, &L.d_il_ptr, L.il_ptr)) || (rc = upload(c, &L.d_il_src, L.il_src)) ||
-        (rc = upload(c, &L.d_il_off, L.il_off)) || (rc = upload(c, &L.d_parent, L.parent)) ||
+        (rc = upload(c, &L.d_il_ptr, L.il_ptr)) || (rc = upload(c, &L.d_parent, L.parent)) ||
         (rc = upload(c, &L.d_quad, L.quad)) || (rc = upload(c, &L.d_ch_ptr, L.ch_ptr)) ||
         (rc = upload(c, &L.d_ch_idx, L.ch_idx)) || (rc = upload(c, &L.d_ch_quad, L.ch_quad)))
       return rc;
@@ -666,22 +665,13 @@ int set_scene(Ctx* c, int p, const double* centres, const int* shape_ids, const 
         (rc = upload(c, &L.d_tiles, tiles)) || (rc = build_translate_tiles(c, L, tiles, bm)))
       return rc;
   }
-  // particles grouped by shape, tiles of at most 16
+  // particles grouped by shape
   {
-    std::vector<int> perm(p), tsh, tst, tcn;
+    std::vector<int> perm(p);
     for (int i = 0; i < p; ++i) perm[i] = i;
     std::stable_sort(perm.begin(), perm.end(), [&](int a, int b) { return c->sid[a] < c->sid[b]; });
-    for (int i = 0; i < p;) {
-      int s = c->sid[perm[i]], j = i;
-      while (j < p && c->sid[perm[j]] == s && j - i < 16) ++j;
-      tsh.push_back(s); tst.push_back(i); tcn.push_back(j - i);
-      i = j;
-    }
-    c->ntile = (int)tsh.size();
     int rc;
-    if ((rc = upload(c, &c->d_perm, perm)) || (rc = upload(c, &c->d_tile_shape, tsh)) ||
-        (rc = upload(c, &c->d_tile_start, tst)) || (rc = upload(c, &c->d_tile_count, tcn)))
-      return rc;
+    if ((rc = upload(c, &c->d_perm, perm))) return rc;
   }
   // ---- near lists: self + 8 lattice neighbours; block keys (sm, sn, dx, dy)
   // on a lattice; with displaced particles every exterior block is keyed by
@@ -1264,7 +1254,7 @@ int smr_set_variant(smr_ctx* h, int step, int level, int precision, int variant)
   if (!ok) return fail(c, SMR_E_INVALID_ARG, "unknown step or variant");
   for (int s = (level < 0 ? 0 : level); s < (level < 0 ? c->nlev : level + 1); ++s) {
     Level& L = c->lev[s];
-    if (step == SMR_STEP_INTERPOLATE) L.tune_ip[q] = variant;
+    if (step == SMR_STEP_INTERPOLATE && q == 0) L.tune_ip = variant;
     else if (step == SMR_STEP_ANTERPOLATE) L.tune_an[q] = variant;
   }
   free_graphs(c);                              // captured products used the old variants
@@ -1494,7 +1484,10 @@ int smr_autotune(smr_ctx* h, int R, int precision, void* stream) {
   // step: its trials 1 and 3 time the tensor cores and the CUDA cores
   for (int v = 1; v <= 3; ++v) {
     if (q == 1 && v == 2) continue;
-    for (auto& L : c->lev) L.tune_ip[q] = L.tune_an[q] = (q == 0 && v <= 2) ? v : 0;
+    for (auto& L : c->lev) {
+      L.tune_an[q] = (q == 0 && v <= 2) ? v : 0;
+      if (q == 0) L.tune_ip = L.tune_an[q];
+    }
     c->tune_tc_agg = c->tune_tc_rec = c->tune_tc_near = (v == 3) ? 0 : 1;
     if ((rc = profile_min(h, 1, x, y, precision, 3, stream, t))) break;
     for (int s = 0; s < c->nlev; ++s) {
@@ -1502,7 +1495,7 @@ int smr_autotune(smr_ctx* h, int R, int precision, void* stream) {
       const int av = c->lev[s].tune_an[q];
       if (an != t.end()) tan_[s][av] = std::min(tan_[s][av], an->second);
       auto ip = t.find({"interpolate", s});
-      const int iv = c->lev[s].tune_ip[q];
+      const int iv = q == 0 ? c->lev[s].tune_ip : 0;
       if (ip != t.end()) tip[s][iv] = std::min(tip[s][iv], ip->second);
     }
     int tc = (v == 3) ? 0 : 1;
@@ -1518,7 +1511,7 @@ int smr_autotune(smr_ctx* h, int R, int precision, void* stream) {
     int bi = 0;
     for (int v = 1; v <= 3; ++v)
       if (tip[s][v] < tip[s][bi]) bi = v;
-    L.tune_ip[q] = rc ? 0 : bi;
+    if (q == 0) L.tune_ip = rc ? 0 : bi;
     int ba = 0;
     for (int v = 1; v <= 3; ++v)
       if (tan_[s][v] < tan_[s][ba]) ba = v;

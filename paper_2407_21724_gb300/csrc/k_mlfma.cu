@@ -827,7 +827,7 @@ constexpr size_t ANT_SMEM = 200 * 1024;
 static bool gather_anterp(const Level& Lc, const Level& Lp, bool f64, int R, int v) {
   if (f64 && R == 1) return !march_anterp(Lc, Lp, v);
   const bool few = (f64 && Lc.nph <= 10) || (double)Lc.nbox * Lp.K * R < 300000.0 * Lc.ma_pm;
-  return Lc.ant_wide && (v ? v <= 2 : few) &&
+  return Lc.ant_wide && v <= 2 && (few || (v && !f64)) &&      // FP64's variant is for one column
          (size_t)Lc.ant_GR * 2 * NF * (f64 ? 16 : 8) <= ANT_SMEM;
 }
 
@@ -1038,7 +1038,7 @@ static int far_impl(Ctx* c, int R, const double2* x, double2* y, bool accumulate
     pbeg(c, st, "interpolate", s,
          ((double)Lc.nbox * Lc.K + (double)Lp.nbox * Lp.K) * NF * R_ * es + 4.0 * Lp.K * es,
          (double)Lc.nbox * Lp.nth * Lc.nph * NF * R_ * 16.0 + (double)Lc.nbox * Lp.K * NF * R_ * 24.0);
-    if (!f64 || R > 1 || march_interp(Lc.tune_ip[0]) || Lp.nph * Part<double>::NT > 256 * EM1) {
+    if (!f64 || R > 1 || march_interp(Lc.tune_ip) || Lp.nph * Part<double>::NT > 256 * EM1) {
       int rc = run_interp(c, s, R, f64 ? SMR_PREC_FP64 : SMR_PREC_FP32, st);
       if (rc) return rc;
     } else {
@@ -1047,8 +1047,8 @@ static int far_impl(Ctx* c, int R, const double2* x, double2* y, bool accumulate
       // has (levels of the 20x20 array 33 + 35 + 32 us with whole tiles, 23 + 21 + 19 so;
       // 40x40 80 + 60 + 56 + 44 and 79 + 49 + 42 + 36)
       const int most = std::max(1, std::min(Lp.nth, (256 * EM1) / (Lp.nph * Part<double>::NT)));
-      int TR = Lc.tune_ip[0] == 2 ? std::max(1, most / 2) : most;
-      if (Lc.tune_ip[0] == 0) {
+      int TR = Lc.tune_ip == 2 ? std::max(1, most / 2) : most;
+      if (Lc.tune_ip == 0) {
         long long cost = -1;
         for (int t = most; t >= 1; --t) {
           const long long w = ((long long)Lp.nbox * ((Lp.nth + t - 1) / t) + 303) / 304 * (t + 2);
@@ -1092,7 +1092,7 @@ static int far_impl(Ctx* c, int R, const double2* x, double2* y, bool accumulate
              (double)Lc.nbox * Lc.K * NF * R_ * 16.0 * (double)Lp.nth / Lc.nth);
     const int an = Lc.tune_an[f64 ? 0 : 1];
     int rc;
-    if (gather_anterp(Lc, Lp, f64, R, an)) rc = run_anterp_gather<T>(c, Lc, Lp, R, an, st);
+    if (gather_anterp(Lc, Lp, f64, R, an)) rc = run_anterp_gather<T>(c, Lc, Lp, R, f64 && R > 1 ? 0 : an, st);
     else rc = run_anterp(c, s, R, f64 ? SMR_PREC_FP64 : SMR_PREC_FP32, st);
     if (rc) return rc;
     pend(c, st);

@@ -89,8 +89,6 @@ struct Level {
   double* d_khat = nullptr;
   double* d_w = nullptr;
   int* d_il_ptr = nullptr;
-  int* d_il_src = nullptr;
-  int* d_il_off = nullptr;
   int* d_il_pk = nullptr;                // [n_il] source box * 64 + table row (FP64 translation)
   double2* d_T64 = nullptr;              // [noff][K]
   float2* d_T32 = nullptr;
@@ -136,17 +134,17 @@ struct Level {
   int ntile_x = 0, ntile_y = 0, ntile_ne = 0;
   int* d_tiles = nullptr;                // non-empty 4x4 translation tiles (ty * ntile_x + tx)
   int* d_tile_tab = nullptr;             // per non-empty 4x4 tile: 64 source and 16 target boxes (k_translate.cu)
-  // FP64 gather anterpolation into this level, one right-hand side (k_anterp1):
+  // gather anterpolation into this level (k_anterp1):
   // child theta rows in nit tiles of TI, parent rows [lo, hi) per tile
   // ([2][nit]), GR the widest range, JC the column chunk
   int ant_TI = 0, ant_nit = 0, ant_GR = 0, ant_JC = 0;
   int* d_ant_lo = nullptr;
-  // launch variants chosen by smr_autotune per precision (FP64, FP32), one
-  // right-hand side: 0 = built-in rule.  FP64 interpolation into the parent level: 1 / 2
+  // launch variants (smr_set_variant; smr_autotune chooses FP64's), one right-hand
+  // side: 0 = built-in rule.  FP64 interpolation into the parent level: 1 / 2
   // the gather kernel with the full / half theta-row tile, 3 the marching kernel.
-  int tune_ip[2] = {0, 0};
-  // FP64 anterpolation into this level: 1 / 2 = the gather kernel with half
-  // the column chunk / with 256 threads
+  int tune_ip = 0;
+  // anterpolation into this level (FP64, FP32): 1 / 2 = the gather kernel with half
+  // the column chunk / with 256 threads, 4 and 5 the marching kernel
   int tune_an[2] = {0, 0};
   // the transposed taps padded to fixed widths (multiples of 4, zero weights):
   // phi by child column [nph][PM] (parent column, weight x dphi_p / dphi_c),
@@ -256,11 +254,6 @@ struct Ctx {
   int* d_pc_ptr = nullptr;              // identity CSR for the block kernel
   int* d_pc_col = nullptr;
   int* d_pc_blk = nullptr;
-  // particles grouped by shape in tiles of at most 16 (aggregation / receive)
-  int ntile = 0;
-  int* d_tile_shape = nullptr;
-  int* d_tile_start = nullptr;
-  int* d_tile_count = nullptr;
   int* d_perm = nullptr;                // particles sorted by shape
   NN nn;
   // captured products: (x, y, R, precision) -> executable graph
