@@ -32,8 +32,9 @@ __device__ __forceinline__ float dsilu(float z) {
 // C tile of 64 x 64 per CTA, 256 threads of 4 x 4 results each, K in steps of 32
 // through two shared-memory buffers (the next step's values are loaded into
 // registers while this one is multiplied).  FP32 multiply-adds: a split-TF32
-// tensor-core version is a quarter faster, but its accumulators round toward
-// zero, which over a batch's rows put the gradient 6.3e-6 off, against 1.5e-7.
+// mma.sync version took 288 us a batch (below) against 323, but its one accumulator a
+// result rounds toward zero, which over a batch's rows put the gradient 6.3e-6 off,
+// against 1.7e-7; several accumulators, as in k_tc.cu, were not tried.
 // Bound: the grids are small (4,096 rows at width 256 make 256 such tiles), so
 // few warps per scheduler hide the shared-memory latency of two reads per 16
 // multiply-adds.  A 4096 x 256 x 256 layer takes 27 us; 8 x 4 results per

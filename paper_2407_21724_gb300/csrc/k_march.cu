@@ -21,7 +21,7 @@
 // Im parts once per pair instead of once per child.
 //
 // Bound: instruction issue and shared-memory reads, both near half of their
-// peak with 12 to 14 warps per SM (the windows take the registers).  On the
+// peak with 12 to 16 warps per SM (the windows take the registers).  On the
 // 200x200 lens in FP32 (algorithmic bytes 259 and 414 MB at level 0, of
 // measured 6.68 TB/s): interpolation level 0 88 us, six levels 313 us;
 // anterpolation level 0 111 us, six levels 378 us.  With four fields a direction

@@ -181,8 +181,8 @@ __device__ __forceinline__ void tmem_sum32(uint32_t t, float* v) {
 // split into TF32 hi / lo and stored swizzled.  One thread issues the 12 MMAs of
 // a chunk (4 K steps x 3 products) and commits them to the stage's barrier.
 // Bound: the producers' instructions (a warp takes about 80 for each 512-byte
-// row group of a chunk, at the latency of a few warps per scheduler); 8
-// producer warps instead of 16 take 248 us on the 200x200 lens against 243.
+// row group of a chunk, at the latency of a few warps per scheduler): 143 us on the
+// 200x200 lens (with four fields a direction 8 producer warps took 248 us, 16 243).
 // CTA (tile, s) of a grid with several s takes chunks s nK / S .. (s + 1) nK / S
 // and writes its partial rows (no accumulation) to y + s ystride.
 // A = coefficient images [nK][hi | lo][128 rows][32] (swizzled), one per
@@ -412,8 +412,8 @@ __global__ void __launch_bounds__(TC_PT + 32, 1) k_receive_tc(int nKall, int KB,
 // accumulators; one control thread streams the coefficient images of the M
 // tiles through a bulk-copy ring and issues the MMAs into two alternating
 // tensor-memory accumulators, so the epilogue of one M tile overlaps the MMAs
-// of the next.  Bound: the epilogue's stores (187 us on the 200x200 lens with 8
-// workers, 167 with 16).
+// of the next.  Bound: the epilogue's stores (125 us on the 200x200 lens; with four
+// fields a direction 187 with 8 workers, 167 with 16).
 constexpr int AG_NS = 3;                       // coefficient-image stages
 constexpr int AG_KCMAX = 4;                    // K chunks (K' <= 128)
 constexpr size_t AG_SMEM = (size_t)2 * AG_KCMAX * TC_BBYTES + (size_t)AG_NS * 2 * TC_ABYTES + 1024 + 1024;
@@ -722,7 +722,8 @@ int build_tc(Ctx* c) {
     c->tc_nMT = nMT;
     // CTAs along the M tiles of a particle tile, the number that finishes
     // first: a CTA costs its M tiles plus about three for its coefficients
-    // (1,600 particles in 18 tiles, 16 M tiles then: one 32 us, eight 20.6 us)
+    // (8 M tiles at order 10; 1,600 particles in 22 tiles: one CTA 42.8 us, these four
+    // 18.8, eight 24.4; 576 particles in 8 tiles: one 41.8, these eight 15.1)
     const int ntile = (int)tsh.size();
     long long cost = -1;
     for (int m = 1; m <= nMT; ++m) {
@@ -744,10 +745,10 @@ int build_tc(Ctx* c) {
   c->tc_nK = nK;
   c->tc_ntile = (int)tsh.size();
   // Splits of the receive's K chunks: with few tiles most SMs would idle while
-  // each CTA walks through all 61 chunks.  The number that finishes first,
-  // a split costing about six chunks of start and epilogue and the sum of the
-  // partial rows about ten (1,600 particles in 18 tiles: one split 76 us, eight
-  // 24.5 us; 24x24 with six tiles 90 and 30.5 us).
+  // each CTA walks through all chunks (31 at order 10).  The number that finishes
+  // first, a split costing about six chunks of start and epilogue and the sum of the
+  // partial rows about ten (1,600 particles in 22 tiles: one split 51.1 us, these six
+  // 20.5, eight 26.5; 576 particles in 8 tiles: one 49.1, eight 16.3, these eleven 18.3).
   c->tc_nsplit = 1;
   long long cost = -1;
   for (int S = 1; S <= std::max(1, std::min(32, nK / 2)); ++S) {
